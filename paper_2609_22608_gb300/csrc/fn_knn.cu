@@ -9,10 +9,16 @@
 // (KM = 8 or 16) in registers.  The node range is split over `nsplit` blocks
 // per query tile to fill the GPU; partial lists go to the caller's workspace
 // and a second kernel merges them.
+//
+// Searches of 256 nodes and more (knn_tc_wanted) filter with the tensor
+// cores instead (knn_tc.cuh): same lists.
 #include <cuda_runtime.h>
+
+#include <mutex>
 
 #include "fn_internal.h"
 #include "knn_core.cuh"
+#include "knn_tc.cuh"
 
 namespace fn {
 
@@ -101,6 +107,142 @@ __global__ void __launch_bounds__(256) k_knn_merge(int B, int nsplit, int k,
   }
 }
 
+// ---------------------------------------------------------------------------
+// tensor-core filter (knn_tc.cuh)
+// ---------------------------------------------------------------------------
+// a thread per operand row: nodes [first, N) in ntiles tiles, then (queries
+// of one batch) in tiles of 128
+__global__ void __launch_bounds__(128) k_knn_tc_pack(const float4* __restrict__ tree, int N,
+                                                     int first, int node_rows,
+                                                     const float4* __restrict__ queries, int B,
+                                                     float sw, uint8_t* __restrict__ nimg,
+                                                     float2* __restrict__ soa,
+                                                     uint8_t* __restrict__ qimg,
+                                                     int* __restrict__ err) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *err = 0;
+  float x[14];
+  if (i < node_rows) {
+    const bool have = i < N - first;
+    if (have) {
+      load_query(tree + 4 * (long)(first + i), x);
+      knn_store_soa(soa, i, x);
+    }
+    knn_pack_node(nimg + (long)(i / KT_ROWS) * KT_TILE, i % KT_ROWS, x, sw, have);
+  } else {
+    const int b = i - node_rows;   // the grid ends with the last query tile
+    const bool have = b < B;
+    if (have) load_query(queries + 4 * (long)b, x);
+    knn_pack_query(qimg + (long)(b / KT_ROWS) * KT_TILE, b % KT_ROWS, x, sw, have);
+  }
+}
+
+struct KnnTcWork {
+  const uint8_t* qimg;
+  const uint8_t* nimg;
+  float* gmin;
+  int ntiles, B;
+  __device__ __forceinline__ KtUnit operator()(long u) const {
+    const long qt = u / ntiles, stride = 4 * kt_row_f4(ntiles);
+    const int nt = (int)(u - qt * ntiles);
+    return KtUnit{qimg + qt * 2 * KT_TILE, nimg + (long)nt * KT_TILE, gmin + qt * KT_QT * stride,
+                  stride, (int)min((long)KT_QT, B - qt * KT_QT), nt, ntiles - 1 - nt};
+  }
+};
+
+__global__ void __launch_bounds__(KT_THREADS, 1) k_knn_tc_mins(KnnTcWork W, long units, int* err) {
+  extern __shared__ __align__(1024) uint8_t kt_smem[];
+  const long G = gridDim.x, b = blockIdx.x;
+  knn_mins(kt_smem, W, units * b / G, units * (b + 1) / G, err);
+}
+
+__global__ void __launch_bounds__(256, 4)
+    k_knn_tc_select(const float2* __restrict__ soa, int n, int first,
+                    const float4* __restrict__ queries, int B, int k, float w, float sw,
+                    const float* __restrict__ gmin, int ntiles, const int* __restrict__ err,
+                    float* __restrict__ out_d, int32_t* __restrict__ out_i) {
+  __shared__ unsigned long long list[8][KT_LIST];
+  const long b = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (b >= B) return;
+  const KeyList r = knn_select(soa, n, first, queries + 4 * b, k, w, sw,
+                               gmin + b * 4 * kt_row_f4(ntiles), ntiles, *err != 0,
+                               list[threadIdx.x >> 5]);
+  const int lane = threadIdx.x & 31;
+  if (lane < k) {
+    out_d[b * k + lane] = __uint_as_float((unsigned)(r.key >> 32));
+    out_i[b * k + lane] = r.key >= KT_NONE ? -1 : (int)(unsigned)r.key;
+  }
+}
+
+constexpr size_t kKtGminBytes = (size_t)64 << 20;   // group minima of one batch of queries, at most
+                                                    // (one tile of 256 queries if that is more)
+// Three launches cost about 17 us whatever they search; the scan in one or two
+// takes as long at 128 nodes (k = 8: 25 us for 32 queries or more, 15 us for
+// one) and 42 us at 256, where the filter takes 19.  From 256 nodes on the
+// filter is the faster one at every batch and k measured (1 to 8192 queries:
+// 1.2x at 256 nodes and one query, 2x at 32, 15x at 65536 nodes, 8192
+// queries and k = 16, 1906 -> 128 us).  States closer to one another than
+// the score's error (a tree of identical nodes) leave every group in reach:
+// the exact scoring of all of them takes up to 2.4x the scan's time.
+static bool knn_tc_wanted(int N) { return N >= 256; }
+
+struct KnnTcPlan {
+  int ntiles, batch;
+  size_t nimg, soa, qimg, gmin, total;   // offsets into the workspace
+};
+static KnnTcPlan knn_tc_plan(int B, int N) {
+  KnnTcPlan p;
+  p.ntiles = (N + KT_ROWS - 1) / KT_ROWS;
+  const size_t row = (size_t)kt_row_f4(p.ntiles) * sizeof(float4);
+  const long fit = std::max<long>(1, (long)(kKtGminBytes / row / KT_QT)) * KT_QT;
+  p.batch = (int)std::min<long>(fit, ((long)B + KT_QT - 1) / KT_QT * KT_QT);
+  p.nimg = 256;
+  p.soa = p.nimg + (size_t)p.ntiles * KT_TILE;
+  p.qimg = p.soa + (size_t)p.ntiles * (KT_ROWS / KT_GROUP) * KT_SOA * sizeof(float2);
+  p.gmin = p.qimg + (size_t)(p.batch / KT_ROWS) * KT_TILE;
+  p.total = p.gmin + (size_t)p.batch * row;
+  return p;
+}
+
+static fn_status knn_tc_launch(const float* tree, int N, int first, const float* queries, int B,
+                               int k, float w_vel, int32_t* idx, float* d2, void* workspace,
+                               cudaStream_t st) {
+  static std::once_flag once[64];
+  static bool attr_ok[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::call_once(once[dev & 63], [&] {
+    attr_ok[dev & 63] = cudaFuncSetAttribute(k_knn_tc_mins,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             kKtSmem) == cudaSuccess;
+  });
+  if (!attr_ok[dev & 63]) return FN_ECUDA;
+  const KnnTcPlan p = knn_tc_plan(B, N);
+  uint8_t* ws = (uint8_t*)workspace;
+  int* err = (int*)ws;
+  float2* soa = (float2*)(ws + p.soa);
+  float* gmin = (float*)(ws + p.gmin);
+  const float sw = std::sqrt(w_vel);
+  // tiles of the nodes actually searched (the plan holds room for all N)
+  const int ntiles = (N - first + KT_ROWS - 1) / KT_ROWS;
+  for (int b0 = 0; b0 < B; b0 += p.batch) {
+    const int nb = std::min(p.batch, B - b0);
+    const int qtiles = (nb + KT_QT - 1) / KT_QT;
+    const int nrows = b0 == 0 ? ntiles * KT_ROWS : 0;   // the node image serves every batch
+    const float4* q = (const float4*)queries + 4 * (long)b0;
+    k_knn_tc_pack<<<nrows / 128 + 2 * qtiles, 128, 0, st>>>((const float4*)tree, N, first, nrows, q,
+                                                            nb, sw, ws + p.nimg, soa, ws + p.qimg, err);
+    const long units = (long)qtiles * ntiles;
+    const KnnTcWork W{ws + p.qimg, ws + p.nimg, gmin, ntiles, nb};
+    k_knn_tc_mins<<<(unsigned)std::min<long>(units, num_sms()), KT_THREADS, kKtSmem, st>>>(W, units,
+                                                                                           err);
+    k_knn_tc_select<<<(nb + 7) / 8, 256, 0, st>>>(soa, N - first, first, q, nb, k, w_vel, sw, gmin,
+                                                  ntiles, err, d2 + (long)b0 * k,
+                                                  idx + (long)b0 * k);
+  }
+  return launch_status();
+}
+
 int knn_km(int k) { return k <= 8 ? 8 : 16; }
 
 // split count: about two blocks per SM, each split at least 4 tiles of
@@ -112,7 +254,8 @@ int knn_nsplit(int B, int N) {
   return std::max(1, std::min(std::min(want, chunks), 32));
 }
 
-size_t knn_ws_bytes(int B, int N, int k) {
+// workspace of the split pass
+static size_t knn_split_bytes(int B, int N, int k) {
   if (B <= 0 || N <= 0 || k < 1 || k > FN_MAX_KNN) return 0;
   const int ns = knn_nsplit(B, N);
   if (ns <= 1) return 0;
@@ -143,7 +286,11 @@ fn_status knn_launch(const float* tree, int N, int first, const float* queries, 
 
 using namespace fn;
 
-extern "C" size_t fn_knn_workspace_bytes(int B, int N, int k) { return knn_ws_bytes(B, N, k); }
+extern "C" size_t fn_knn_workspace_bytes(int B, int N, int k) {
+  const size_t split = knn_split_bytes(B, N, k);
+  if (B <= 0 || N <= 0 || k < 1 || k > FN_MAX_KNN || !knn_tc_wanted(N)) return split;
+  return std::max(split, knn_tc_plan(B, N).total);
+}
 
 extern "C" fn_status fn_knn_tree(const float* tree, int N, int first, const float* queries, int B,
                                  int k, float w_vel, int32_t* idx, float* d2, void* workspace,
@@ -156,7 +303,13 @@ extern "C" fn_status fn_knn_tree(const float* tree, int N, int first, const floa
   int nsplit = 1;
   float* part_d = nullptr;
   int32_t* part_i = nullptr;
-  const size_t need = knn_ws_bytes(B, N, k);
+  // the tensor-core filter where its workspace is given; a workspace that
+  // only holds the split pass still gets that
+  if (workspace && aligned256(workspace) && N > first && knn_tc_wanted(N - first) &&
+      workspace_bytes >= knn_tc_plan(B, N).total)
+    return knn_tc_launch(tree, N, first, queries, B, k, w_vel, idx, d2, workspace,
+                         (cudaStream_t)stream);
+  const size_t need = knn_split_bytes(B, N, k);
   if (workspace && need > 0) {
     if (workspace_bytes < need || !aligned256(workspace)) return FN_EINVAL;
     nsplit = knn_nsplit(B, N);

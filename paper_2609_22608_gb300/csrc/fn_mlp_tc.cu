@@ -23,6 +23,7 @@
 
 #include "fn_internal.h"
 #include "fn_mlp_tc.h"
+#include "fn_umma.cuh"
 
 namespace fn {
 
@@ -45,93 +46,10 @@ constexpr int kTcThreads = 512;
 
 constexpr int kRing = 4;
 constexpr int kTmemCols = 256;
-constexpr long long kWaitCycles = 2000000000LL;   // ~1 s at 2 GHz
-
 // instruction descriptor of tcgen05.mma kind::f16: FP32 accumulator,
 // bf16 A and B, both K-major, N = 256, M = 128
 constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
                             ((uint32_t)(kTcM >> 4) << 24);
-
-__device__ __forceinline__ uint32_t su32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-// shared-memory matrix descriptor: canonical K-major layout without swizzle
-// (start, leading = K-adjacent core matrices, stride = 8-row groups)
-__device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
-  uint64_t d = (uint64_t)((saddr >> 4) & 0x3FFFu);
-  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
-  d |= (uint64_t)((sbo >> 4) & 0x3FFFu) << 32;
-  d |= (uint64_t)1 << 46;   // descriptor version
-  return d;
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait for phase `parity` of the barrier to complete
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  const long long t0 = clock64();
-  while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > kWaitCycles) return false;
-  return true;
-}
-__device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t bytes,
-                                         uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::
-          "r"(dst),
-      "l"(src), "r"(bytes), "r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void umma(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(kIdesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint32_t bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
-      : "memory");
-}
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-}
-__device__ __forceinline__ void proxy_fence() {
-  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-}
-// 32 consecutive FP32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
-        "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
-        "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-}
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   const bf16 a = __float2bfloat16_rn(lo), b = __float2bfloat16_rn(hi);
@@ -256,8 +174,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       if (!fail) {
 #pragma unroll
         for (int s = 0; s < kTcK1 / 16; ++s)
-          umma(tmem, sdesc(a_base + s * 256, 128, kTcK1 * 16), sdesc(w1_base + s * 256, 128, kTcK1 * 16),
-               s > 0);
+          umma_f16(tmem, sdesc(a_base + s * 256, 128, kTcK1 * 16),
+                   sdesc(w1_base + s * 256, 128, kTcK1 * 16), kIdesc, s > 0);
         umma_commit(bar_layer);
       }
     }
@@ -309,8 +227,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const uint32_t bb = b_base + b * kTcChunkBytes;
 #pragma unroll
             for (int s = 0; s < kTcKc / 16; ++s)
-              umma(tmem, sdesc(a_base + (4 * c + s) * 256, 128, 256 * 16), sdesc(bb + s * 256, 128, kTcKc * 16),
-                   (c | s) != 0);
+              umma_f16(tmem, sdesc(a_base + (4 * c + s) * 256, 128, 256 * 16),
+                       sdesc(bb + s * 256, 128, kTcKc * 16), kIdesc, (c | s) != 0);
             umma_commit(bar_free(b));
             // refill the slot of the previous chunk (its MMAs are queued before
             // this chunk's) with the chunk RING - 1 ahead of this one
@@ -404,14 +322,6 @@ constexpr int kGScr = kGK * kGScrW * 2;             // 17 KB
 constexpr int kGSmem = 2 * kGStage + kGScr + 64;    // two stages, scratch, barriers
 constexpr uint32_t kGIdesc = (1u << 4) | (1u << 7) | (1u << 10) |
                              ((uint32_t)(kGN >> 3) << 17) | ((uint32_t)(kGM >> 4) << 24);
-
-__device__ __forceinline__ void umma_g(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-      " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(kGIdesc), "r"(acc)
-      : "memory");
-}
 
 // byte offset of element (row, k) of a 128 x 64 tile in the canonical
 // K-major layout: 8 x 8 core matrices of 128 B, K-adjacent ones 128 B apart,
@@ -542,8 +452,8 @@ __global__ void __launch_bounds__(128, 1)
       const uint32_t a = base + st * kGStage, b = a + kGTile;
 #pragma unroll
       for (int j = 0; j < kGK / 16; ++j)
-        umma_g(tmem, sdesc(a + j * 256, 128, (kGK / 8) * 128), sdesc(b + j * 256, 128, (kGK / 8) * 128),
-               (c | j) != 0);
+        umma_f16(tmem, sdesc(a + j * 256, 128, (kGK / 8) * 128),
+                 sdesc(b + j * 256, 128, (kGK / 8) * 128), kGIdesc, (c | j) != 0);
       umma_commit(bar0 + 8 * st);
     }
   }

@@ -63,3 +63,56 @@ def test_knn_full_size_sampled(ops, orc, arm):
     sel = np.random.default_rng(1).choice(B, 64, replace=False)
     ri, rd = orc.knn(tree, q[sel], k, 0.1)
     assert not knn_mismatches(ig[sel], dg[sel], ri, rd)
+
+
+def _scan(tree, q, k, first):
+    """fn_knn_tree without a workspace: the FP32 scan of every node."""
+    import ctypes as C
+
+    from paper_2609_22608_gb300._lib import lib
+    B = q.shape[0]
+    idx = torch.empty(B, k, dtype=torch.int32, device="cuda")
+    d2 = torch.empty(B, k, device="cuda")
+    st = lib().fn_knn_tree(C.c_void_p(tree.data_ptr()), tree.shape[0], first,
+                           C.c_void_p(q.data_ptr()), B, k, 0.1, C.c_void_p(idx.data_ptr()),
+                           C.c_void_p(d2.data_ptr()), None, 0,
+                           C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == 0
+    return idx, d2
+
+
+def _odd_states(kind, arm, N, B):
+    t, q = synth.random_states(arm, N, N), synth.random_states(arm, B, N + B)
+    rng = np.random.default_rng(N)
+    if kind == "copies":                      # ties everywhere
+        t = t[rng.integers(0, 9, N)]
+        q[::2] = t[rng.integers(0, N, len(q[::2]))]
+    elif kind == "tight":                     # clusters below the filter's resolution
+        t = t[rng.integers(0, 4, N)] + 1e-4 * rng.standard_normal((N, 16)).astype(np.float32)
+        q[:] = t[rng.integers(0, N, B)]
+    elif kind == "tiny":
+        t, q = t * np.float32(1e-4), q * np.float32(1e-4)
+    elif kind == "outside":                   # states the filter's operands cannot hold
+        t[5, 3], t[17, 0], t[40], t[N - 1, 9] = np.nan, np.inf, 1e20, -np.inf
+        t[60] *= 60
+        q[0, 2], q[1], q[2, 1] = np.nan, 1e20, np.inf
+        q[3], q[4] = t[40], q[4] * 1000
+    elif kind == "few":                       # fewer finite nodes than k
+        t[7:] = np.inf
+    return t.astype(np.float32), q.astype(np.float32)
+
+
+@pytest.mark.parametrize("kind", ["uniform", "copies", "tight", "tiny", "outside", "few"])
+@pytest.mark.parametrize("B,N,k,first", [(5, 257, 1, 1), (256, 384, 8, 0), (257, 2049, 16, 1),
+                                         (64, 4000, 7, 100), (700, 8320, 9, 1)])
+def test_knn_filter_is_the_scan(ops, arm, kind, B, N, k, first):
+    """The tensor-core filter's lists are the FP32 scan's bit for bit: sizes at
+    the edges of its groups, tiles and row blocks, and states where its scores
+    tie, coincide or do not exist."""
+    t, q = (dev(x) for x in _odd_states(kind, arm, N, B))
+    ws = torch.full((ops.knn_workspace_bytes(B, N, k) + 256,), 0xFF, dtype=torch.uint8,
+                    device="cuda")            # contents on entry do not matter (NaNs here)
+    idx, d2 = ops.knn_tree(t, q, k, 0.1, first=first, workspace=ws)
+    ri, rd = _scan(t, q, k, first)
+    assert torch.equal(idx, ri)
+    assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
