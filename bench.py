@@ -386,11 +386,12 @@ FLOP_PER_IK_START = 28267      # one damped-least-squares start, 24 iterations +
 # its launches in one iteration, as `achieved` is).  An entry holds only
 # while the kernel and the workload are the ones captured; it is removed
 # when either changes, and the roofline then reports null.
-MEASURED_DRAM_BYTES = {"k_plan_knn": 347392}
+MEASURED_DRAM_BYTES = {}
 # algorithmic bytes of one parent-search launch on this workload: the 4096
 # tree rows and the 2048 queries at 56 B (14 floats), the 2048 lists of 7
-# parents at 8 B per entry, halved over the iteration's two launches
-KNN_ALGO_BYTES = (56 * (4096 + 2048) + 8 * 2048 * 7) // 2
+# parents at 8 B per entry, over the iteration's four launches (group minima
+# and selection, free and goal queries)
+KNN_ALGO_BYTES = (56 * (4096 + 2048) + 8 * 2048 * 7) // 4
 
 
 def kernel_table(traced):
@@ -414,10 +415,11 @@ def roofline_from_trace(traced, work, workload="iteration"):
              "k_plan_edges_tm": (work["probe"] + work["mprobe"] + work["verify"], FLOP_PER_SAMPLE,
                                  "torque evaluations (splits, probes and checks)"),
              "k_plan_vstage": (None, FLOP_PER_SAMPLE, "torque evaluations"),
-             "k_plan_knn": (work["knn_pairs"], FLOP_PER_PAIR, "(query, node) pairs"),
+             "k_plan_knn": (work["knn_pairs"], FLOP_PER_PAIR, "(query, node) pairs, most of them scored on "
+                                                          "the tensor cores"),
              "k_plan_sample": (work["ik_starts"], FLOP_PER_IK_START,
-                               "IK starts (the goal chart's; the uniform draws and the tree "
-                               "mirror update in the same launch are not credited)")}
+                               "IK starts (the goal chart's; the uniform draws and the node "
+                               "images' update in the same launch are not credited)")}
     dom = max(tab, key=lambda k: tab[k]["ms"])
     peak = fp32_peak_tflops()
     total = sum(t["ms"] for t in tab.values())
@@ -454,7 +456,7 @@ def roofline_from_trace(traced, work, workload="iteration"):
         out["knn_memory"] = {"dram_gbs": None if b is None else b / t / 1e9,
                              "algorithmic_bytes_per_launch": KNN_ALGO_BYTES,
                              "algorithmic_gbs": KNN_ALGO_BYTES / t / 1e9,
-                             "note": "the tree and its mirror are L2-resident: the search is "
+                             "note": "the tree and its images are L2-resident: the search is "
                                      "bound by latency, not by HBM"}
     return out
 

@@ -10,9 +10,9 @@
 //   schedule : per-problem work offsets, work-queue resets
 //   sample   : goal chart (warp per candidate, lane-parallel IK) and
 //              uniform candidates (Philox counters); parent-search prep
-//              (tree mirror) in the same launch
-//   knn      : warps claim (problem, query, node split) items; the warp
-//              finishing a query's last split merges the split lists
+//              (operand images of the nodes and queries) in the same launch
+//   knn      : group minima of every query on the tensor cores, then a warp
+//              per query scores the groups in reach exactly (knn_tc.cuh)
 //   edges    : prep + item scan (eprep, escan, expand), probe of both end
 //              samples of every (edge, admissible duration), probe of four
 //              interior samples of the survivors (mprobe), verification
@@ -37,29 +37,10 @@
 #include "nary_core.cuh"
 #include "fn_mlp_tc.h"
 #include "fn_tune.h"
-#include "knn_core.cuh"
+#include "knn_tc.cuh"
 
-#define PL_NSPLIT_MAX 32
-#define PL_KNN_WARPS 4
-#ifndef PL_KNN_QW
-#define PL_KNN_QW 1                           // queries per warp
-#endif
-#define PL_KNN_SPAN 4096                      // nodes per split (at least)
-#ifndef PL_KNN_SPAN_GOAL
-#define PL_KNN_SPAN_GOAL 512                  // the same for goal queries (few, and late)
-#endif
-#ifndef PL_KNN_SPAN_MIN
-#define PL_KNN_SPAN_MIN 1024                  // smallest split of a free query's search
-#endif
-#ifndef PL_KNN_TW
-#define PL_KNN_TW 8                           // tiled search: free queries (one per warp) per CTA
-#endif
-#ifndef PL_KNN_TRING
-#define PL_KNN_TRING 4                        // tiled search: mirror blocks in the CTA's ring
-#endif
-#ifndef PL_KNN_TILE_NODES
-#define PL_KNN_TILE_NODES 32768               // tree capacity from which the tiled search is used
-#endif
+#define PL_KNN_BYTES ((size_t)2 << 30)        // group minima of one search launch, at most
+#define PL_KNN_SEL_WARPS 8
 #define PL_MAX_P 1024
 #define PL_MAX_KEV 40                         // launches traced per iteration
 #define PL_NCOUNT 14  // work counters: probe, verify, mid-probe, kNN pairs, IK starts,
@@ -96,25 +77,21 @@ struct Sched {
   unsigned tm_done;    // CTAs of k_plan_edges_tm finished (zero between bodies)
   int n_free_edges;   // free edges of all problems (the queue's first part)
   int n_edges;        // all edges
-  // parent-search items (problem, query group, split), one per warp, in two
-  // lists: [0] free queries, [1] goal queries (searched after the goal
-  // chart has decoded them, in smaller splits)
-  int knn_items[2];   // [1] unused: goal items come from the decoded-goal list
-  int knn_head[2];    // next unclaimed item of each list
+  // parent search, by kind of query ([0] free, [1] goal): tiles of KT_QT
+  // query rows (a problem's free candidates in order; its decoded goals in
+  // the order they were decoded, at most n_goal)
+  int knn_err;        // a bounded wait of the tensor-core filter ran out
   int gq_n;           // decoded goal queries appended to PlanDev::gq this round
-  int nsg_max;        // largest goal split count over the problems
+  int gq_cnt[PL_MAX_P];       // of them, problem p's
+  int qt_off[2][PL_MAX_P + 1];
   int free_off[PL_MAX_P + 1];
   int goal_off[PL_MAX_P + 1];
-  int knn_off[2][PL_MAX_P + 1];
-  int nsplit[2][PL_MAX_P];
-  int pack_lo[PL_MAX_P];      // first node of problem p to (re)pack into the mirror
-  int pack_off[PL_MAX_P + 1]; // flattened offsets of the nodes to pack
+  int pack_lo[PL_MAX_P];      // first operand row of problem p to (re)pack
+  int pack_off[PL_MAX_P + 1]; // flattened offsets of the rows to pack
 };
 
 struct PlanDev {  // device pointers, passed by value to the kernels
-  int P, NC, BM, KP, KN, KM, K, S, S_clear, G;
-  int knn_slots;      // resident warps (CTAs when tiled) of the free queries' search grid
-  int knn_tile;       // 1: the free queries' search is tiled (PL_KNN_TW queries share a CTA)
+  int P, NC, BM, KP, KN, K, S, S_clear, G;
   int att_wide;       // 1: attach over many blocks per problem (large batches, few problems)
   int32_t* att_idx;   // [P][BM] a candidate's index among its chunk's attached ones, or -1
   int32_t* att_blk;   // [P][ceil(BM/PL_ATT_T)] attached per chunk, then their offsets
@@ -135,9 +112,6 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   float* vrel;        // [P][BM]
   uint8_t* valid;     // [P][BM]
   int32_t* nn;        // [P][BM][KN]
-  float* part_d;      // [P][NSPLIT][BM][KM]
-  int32_t* part_i;
-  int32_t* knn_cnt;   // [P][BM] splits finished per query (zero between iterations)
   float* e_T;         // [P][BM][KP]
   float* e_rv;
   uint8_t* e_ok;
@@ -197,12 +171,19 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   float* cz;          // [P][BM][9] chart parameters of the goal candidates (NaN: unknown)
   float* zn;          // [P][NC][9] chart parameters of goal nodes, written at attach
   int32_t* glist;     // [P][BM] the round's valid goal candidates, in order
-  int2* gq;           // [P * BM] (problem, slot) of the round's decoded goal queries
+  int4* gq;           // [P * BM] (problem, slot, row) of the round's decoded goal queries
   fn_sampler_cfg_t scfg;
-  // parents: node mirror laid out for lane-contiguous loads (see knn_mirror_index)
-  float4* mir;        // [P][NB][7][32]
-  int32_t* packed;    // [P] leading nodes whose mirror entries are current
-  int NB;             // 64-node blocks per problem
+  // parents (knn_tc.cuh): operand images and exact values of the non-root
+  // nodes (row r: node r + 1), of the queries, and the group minima of one
+  // launch's query tiles, by kind of query
+  uint8_t* nimg;      // [P][NT][KT_TILE]
+  float2* soa;        // [P][4 NT][KT_SOA]
+  uint8_t* qimg[2];   // [query tiles][2][KT_TILE]
+  float* gmin[2];     // [tiles of a launch][KT_QT][4 kt_row_f4(NT)]
+  int32_t* packed;    // [P] leading nodes whose images are current
+  int NT;             // node tiles per problem
+  int knn_tiles;      // query tiles of one launch
+  float sw_vel;       // sqrt(w_vel)
 };
 
 // Programmatic dependent launch: a kernel launched with programmatic
@@ -303,63 +284,40 @@ __global__ void k_plan_schedule(PlanDev D) {
   __syncthreads();
   if (threadIdx.x != 0) return;
   Sched* S = D.sched;
-  // free queries over all problems: with fewer query groups than resident
-  // warps of the parent search, each query's nodes are split further so
-  // that every warp gets an item (splits of at least PL_KNN_SPAN_MIN nodes)
-  // (groups of PL_KNN_TW queries, one CTA item each, when the search is tiled)
-  const int qg = D.knn_tile ? PL_KNN_TW : PL_KNN_QW;
-  int qf = 0;
-  for (int p = 0; p < D.P; ++p) {
-    const int B = min(max(D.prob[p].batch, 0), D.BM);
-    const int G = min(max(D.prob[p].n_goal, 0), B);
-    if (D.KN > 0 && D.n_nodes[p] > 1) qf += (B - G + qg - 1) / qg;
-  }
-  const int fill = qf > 0 ? max(1, D.knn_slots / qf) : 1;
-  int fo = 0, go = 0, ko = 0, kg = 0, po = 0, nsg_max = 1;
+  int fo = 0, go = 0, qf = 0, qg = 0, po = 0;
   for (int p = 0; p < D.P; ++p) {
     const fn_problem_t& P = D.prob[p];
     const int B = min(max(P.batch, 0), D.BM);
     const int G = min(max(P.n_goal, 0), B);
     S->free_off[p] = fo;
     S->goal_off[p] = go;
-    S->knn_off[0][p] = ko;
-    S->knn_off[1][p] = kg;
+    S->qt_off[0][p] = qf;
+    S->qt_off[1][p] = qg;
+    S->gq_cnt[p] = 0;
     fo += (B - G) * D.KP;
     go += G * D.KP;
-    const int span = D.n_nodes[p] - 1;  // non-root nodes
-    int ns = 1, nsg = 1;
-    if (D.KN > 0 && span > 0) {
-      ns = max((span + PL_KNN_SPAN - 1) / PL_KNN_SPAN, min(fill, span / PL_KNN_SPAN_MIN));
-      ns = min(PL_NSPLIT_MAX, ns);
-      nsg = min(PL_NSPLIT_MAX, (span + PL_KNN_SPAN_GOAL - 1) / PL_KNN_SPAN_GOAL);
-    }
-    S->nsplit[0][p] = ns;
-    S->nsplit[1][p] = nsg;
-    nsg_max = max(nsg_max, nsg);
-    if (D.KN > 0 && span > 0) {
-      ko += ((B - G + qg - 1) / qg) * ns;
-      kg += ((G + PL_KNN_QW - 1) / PL_KNN_QW) * nsg;
+    const int N = D.n_nodes[p];
+    if (N > 1) {
+      qf += (B - G + KT_QT - 1) / KT_QT;
+      qg += (G + KT_QT - 1) / KT_QT;
     }
     D.added[p] = 0;
-    const int lo = min(D.packed[p], D.n_nodes[p]);
+    // rows of the nodes past the packed ones, to the end of their last tile
+    const int lo = max(min(D.packed[p], N), 1) - 1;
     S->pack_lo[p] = lo;
     S->pack_off[p] = po;
-    po += D.n_nodes[p] - lo;
-    D.packed[p] = D.n_nodes[p];
+    if (N - 1 > lo) po += (N - 1 + KT_ROWS - 1) / KT_ROWS * KT_ROWS - lo;
+    D.packed[p] = N;
   }
   S->pack_off[D.P] = po;
   S->free_off[D.P] = fo;
   S->goal_off[D.P] = go;
-  S->knn_off[0][D.P] = ko;
-  S->knn_off[1][D.P] = kg;
+  S->qt_off[0][D.P] = qf;
+  S->qt_off[1][D.P] = qg;
   S->n_free_edges = fo;
   S->n_edges = fo + (D.goal_split ? 0 : go);
-  S->knn_items[0] = ko;
-  S->knn_items[1] = kg;
-  S->knn_head[0] = 0;
-  S->knn_head[1] = 0;
+  S->knn_err = 0;
   S->gq_n = 0;
-  S->nsg_max = nsg_max;
   if (D.sur_n) *D.sur_n = 0;
   S->queue_head = 0u;
   S->n_dyn = 0;
@@ -425,6 +383,21 @@ __device__ __forceinline__ void density_z(const fn_density_t& th, unsigned long 
   for (int i = 0; i < 9; ++i) z[i] = z_fold(i, fmaf(th.sd[m][i], nrm[i], th.mu[m][i]));
 }
 
+// row r of the query images of a kind for problem p, from a state's values
+__device__ __forceinline__ void pack_query_row(const PlanDev& D, int kind, int p, int r,
+                                               const float* q, const float* qd) {
+  const int t = D.sched->qt_off[kind][p] + r / KT_QT;
+  if (t >= D.sched->qt_off[kind][p + 1]) return;   // a single-node tree: no search
+  float x[14];
+#pragma unroll
+  for (int j = 0; j < 7; ++j) {
+    x[j] = q[j];
+    x[7 + j] = qd[j];
+  }
+  knn_pack_query(D.qimg[kind] + ((long)t * 2 + (r % KT_QT) / KT_ROWS) * KT_TILE, r % KT_ROWS, x,
+                 D.sw_vel, true);
+}
+
 // Free candidate (p, b): uniform in the box, |qd| <= vel_frac qdbar.
 __device__ __forceinline__ void sample_free(const PlanDev& D, const ArmK& A, int p, int b) {
   const fn_problem_t& P = D.prob[p];
@@ -447,6 +420,7 @@ __device__ __forceinline__ void sample_free(const PlanDev& D, const ArmK& A, int
   o4[1] = make_float4(q[4], q[5], q[6], 0.f);
   o4[2] = make_float4(qd[0], qd[1], qd[2], qd[3]);
   o4[3] = make_float4(qd[4], qd[5], qd[6], 0.f);
+  pack_query_row(D, 0, p, b - min(max(P.n_goal, 0), min(max(P.batch, 0), D.BM)), q, qd);
 }
 
 __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stride);
@@ -454,13 +428,14 @@ __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stri
 __device__ __forceinline__ void sample_goal(const PlanDev& D, const ArmK& A, int p, int b, int dens);
 
 // a goal query of this round: a decoded (valid) one joins the goal list of
-// the parent search; the others get empty parent lists here
+// the parent search and its problem's query rows; the others get empty
+// parent lists here
 __device__ __forceinline__ void goal_query(const PlanDev& D, int p, int b, bool valid) {
-  if (D.KN <= 0) return;
   const long ci = (long)p * D.BM + b;
   if (valid && D.n_nodes[p] > 1) {
-    const int v = atomicAdd(&D.sched->gq_n, 1);
-    D.gq[v] = make_int2(p, b);
+    const int r = atomicAdd(&D.sched->gq_cnt[p], 1);
+    D.gq[atomicAdd(&D.sched->gq_n, 1)] = make_int4(p, b, r, 0);
+    pack_query_row(D, 1, p, r, D.cand + ci * 16, D.cand + ci * 16 + 8);
   } else {
     for (int j = 0; j < D.KN; ++j) D.nn[ci * D.KN + j] = -1;
   }
@@ -469,7 +444,7 @@ __device__ __forceinline__ void goal_query(const PlanDev& D, int p, int b, bool 
 // Sampling launches: warp w < nslots (P * b_max, or 0 when the caller gives
 // the candidates) owns candidate slot (p, b).
 //   role 0: a free slot is drawn by lane 0; the warps past the slots prepare
-//           the parent search (parents_prep: tree mirror, empty lists);
+//           the parent search (parents_prep: node images, empty lists);
 //   role 1: a goal slot is decoded by the whole warp (sample_goal).
 __global__ void __launch_bounds__(128) k_plan_sample(PlanDev D, ArmK A, long nslots,
                                                      int prep_warps, int dens, int role) {
@@ -488,11 +463,13 @@ __global__ void __launch_bounds__(128) k_plan_sample(PlanDev D, ArmK A, long nsl
     } else if (gid - nsw < prep_warps) {
       const long i = (gid - nsw) * 32 + lane, stride = (long)prep_warps * 32;
       parents_prep(D, i, stride);
-      if (nslots == 0)                                // external candidates: list their goals
+      if (nslots == 0)                                // external candidates: their queries
         for (long x = i; x < (long)D.P * D.BM; x += stride) {
           const int p = (int)(x / D.BM), b = (int)(x - (long)p * D.BM);
           const int B = min(max(D.prob[p].batch, 0), D.BM);
-          if (b < min(max(D.prob[p].n_goal, 0), B)) goal_query(D, p, b, D.valid[x] != 0);
+          const int G = min(max(D.prob[p].n_goal, 0), B);
+          if (b < G) goal_query(D, p, b, D.valid[x] != 0);
+          else if (b < B) pack_query_row(D, 0, p, b - G, D.cand + x * 16, D.cand + x * 16 + 8);
         }
     }
   } else if (gid < nslots) {
@@ -556,435 +533,129 @@ __device__ __forceinline__ void sample_goal(const PlanDev& D, const ArmK& A, int
 }
 
 // ---------------------------------------------------------------------------
-// parents: (problem, query group, split) items over all problems, claimed
-// by warps one at a time.  A warp takes PL_KNN_QW queries and sweeps the
-// split's nodes 64 at a time; the k best
-// (d, index) pairs live across lanes 0..KM-1 in ascending order, and only
-// nodes that beat the current k-th pair enter the list, one at a time (a
-// ballot finds them; a shuffle-up opens their slot), or by a warp merge
-// when a ballot holds many of them.
+// parents (knn_tc.cuh): group minima of query tiles [t0, t1) of a kind on the
+// tensor cores, then a warp per query.  The lists are those of an FP32 scan
+// of the tree, which these launches replaced: a warp per query (or a CTA
+// sharing the node blocks among eight) swept every node on the FP32 pipe,
+// bound by L2 on small trees and by issue on large ones.  Both searches of a
+// round, before and after: 64 uneven problems (287 M pairs) 1010 -> 185 us,
+// 8192 queries on 28 k nodes (k = 16) 770 -> 96 us, 2048 queries on 4096
+// nodes 57 -> 34 us (four launches' latency, of which half runs beside the
+// inverse kinematics).  Planners of all sizes take them; a window of query
+// tiles bounds the minima's memory.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ int knn_rows(const PlanDev& D, int kind, int p) {
+  if (D.n_nodes[p] <= 1) return 0;
+  if (kind == 1) return D.sched->gq_cnt[p];
+  const int B = min(max(D.prob[p].batch, 0), D.BM);
+  return B - min(max(D.prob[p].n_goal, 0), B);
+}
+__device__ __forceinline__ int knn_node_tiles(const PlanDev& D, int p) {
+  return (D.n_nodes[p] - 1 + KT_ROWS - 1) / KT_ROWS;
+}
 
-template <int KM>
-struct WarpTopK {
-  float d = INFINITY;                         // lane j < KM: j-th best
-  int i = 0x7fffffff;
-  float td = INFINITY;                        // the k-th best, on every lane
-  int ti = 0x7fffffff;
-  // Offer the candidates (cd, ci) of the lanes in m (each beat the k-th
-  // pair when m was formed): in lane order, a candidate still better than
-  // the current k-th pair takes its sorted slot and the tail shifts down.
-  // Branch-free in the candidate (a candidate that no longer qualifies
-  // gets pos = 32, which moves nothing).
-  __device__ __forceinline__ void insert(unsigned m, float cd, int ci) {
-    const int lane = threadIdx.x & 31;
-    while (m) {
-      const int src = __ffs(m) - 1;
-      m &= m - 1u;
-      const float nd = __shfl_sync(0xffffffffu, cd, src);
-      const int ni = __shfl_sync(0xffffffffu, ci, src);
-      const bool ok = knn_less(nd, ni, td, ti);
-      const unsigned lt = __ballot_sync(0xffffffffu, knn_less(d, i, nd, ni)) & ((1u << KM) - 1u);
-      const int pos = ok ? __popc(lt) : 32;
-      const float ud = __shfl_up_sync(0xffffffffu, d, 1);
-      const int ui = __shfl_up_sync(0xffffffffu, i, 1);
-      d = lane < pos ? d : (lane == pos ? nd : ud);
-      i = lane < pos ? i : (lane == pos ? ni : ui);
-      td = __shfl_sync(0xffffffffu, d, KM - 1);
-      ti = __shfl_sync(0xffffffffu, i, KM - 1);
-    }
-  }
-  // The same for many candidates at once (the first block of a split fills
-  // an empty list): the KM smallest of the list and the offered candidates
-  // by KM rounds of a warp argmin, each winner taken out by its owner (node
-  // indices are distinct; the empty entries (inf, max) are all alike).
-  __device__ __forceinline__ void merge(unsigned m, float cd, int ci) {
-    const int lane = threadIdx.x & 31;
-    const bool mine = (m >> lane) & 1u;
-    float ld = lane < KM ? d : INFINITY, xd = mine ? cd : INFINITY;
-    int li = lane < KM ? i : 0x7fffffff, xi = mine ? ci : 0x7fffffff;
-    float nd = INFINITY;
-    int ni = 0x7fffffff;
-#pragma unroll
-    for (int r = 0; r < KM; ++r) {
-      const bool fl = knn_less(ld, li, xd, xi);
-      float bd = fl ? ld : xd;
-      int bi = fl ? li : xi;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float od = __shfl_xor_sync(0xffffffffu, bd, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (knn_less(od, oi, bd, bi)) { bd = od; bi = oi; }
-      }
-      if (lane == r) { nd = bd; ni = bi; }
-      if (ld == bd && li == bi) { ld = INFINITY; li = 0x7fffffff; }
-      else if (xd == bd && xi == bi) { xd = INFINITY; xi = 0x7fffffff; }
-    }
-    d = nd;
-    i = ni;
-    td = __shfl_sync(0xffffffffu, d, KM - 1);
-    ti = __shfl_sync(0xffffffffu, i, KM - 1);
-  }
-  // one at a time for a few candidates, else the merge
-  __device__ __forceinline__ void offer(unsigned m, float cd, int ci) {
-    if (__popc(m) >= 2 * KM) merge(m, cd, ci);
-    else insert(m, cd, ci);
+struct PlanKnnWork {
+  const PlanDev& D;
+  const int* uo;   // [P + 1] units before each problem
+  int kind, t0;
+  __device__ __forceinline__ KtUnit operator()(long u) const {
+    const int p = find_problem(uo, D.P, (int)u);
+    const int* qt = D.sched->qt_off[kind];
+    const int nt = knn_node_tiles(D, p), local = (int)u - uo[p], qi = local / nt;
+    const int t = max(qt[p], t0) + qi, n = local - qi * nt;
+    const long stride = 4 * (long)kt_row_f4(D.NT);
+    return KtUnit{D.qimg[kind] + (long)t * 2 * KT_TILE, D.nimg + ((long)p * D.NT + n) * KT_TILE,
+                  D.gmin[kind] + (long)(t - t0) * KT_QT * stride, stride,
+                  min(KT_QT, knn_rows(D, kind, p) - (t - qt[p]) * KT_QT), n, nt - 1 - n};
   }
 };
 
-// Merge of a query's split lists (run by the warp that finishes its last
-// split): lane s < ns holds split s's list; KN rounds of a warp argmin.
-template <int KM>
-__device__ __forceinline__ void knn_merge_query(const PlanDev& D, int p, int b, int ns) {
-  const int lane = threadIdx.x & 31;
-  float d[KM];
-  int id[KM];
-#pragma unroll
-  for (int j = 0; j < KM; ++j) { d[j] = INFINITY; id[j] = 0x7fffffff; }
-  if (lane < ns) {
-    const long off = (((long)p * PL_NSPLIT_MAX + lane) * D.BM + b) * KM;
-#pragma unroll
-    for (int j = 0; j < KM; ++j) { d[j] = __ldcg(D.part_d + off + j); id[j] = __ldcg(D.part_i + off + j); }
-  }
-  const long out = ((long)p * D.BM + b) * D.KN;
-  for (int r = 0; r < D.KN; ++r) {
-    float md = d[0];
-    int mi = id[0];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float od = __shfl_xor_sync(0xffffffffu, md, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
-      if (knn_less(od, oi, md, mi)) { md = od; mi = oi; }
-    }
-    if (lane == 0) D.nn[out + r] = mi == 0x7fffffff ? -1 : mi;
-    if (id[0] == mi && mi != 0x7fffffff) {
-#pragma unroll
-      for (int j = 0; j + 1 < KM; ++j) { d[j] = d[j + 1]; id[j] = id[j + 1]; }
-      d[KM - 1] = INFINITY;
-      id[KM - 1] = 0x7fffffff;
-    }
-  }
-}
+constexpr int kPlanKnnSmem = kKtSmem + (PL_MAX_P + 1) * (int)sizeof(int);
+static_assert(kPlanKnnSmem <= 227 * 1024, "parent search: shared-memory layout");
 
-// asynchronous 16-byte global -> shared copy (completion tracked per thread)
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() {
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-}
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
-
-#ifndef PL_KNN_RING
-#define PL_KNN_RING 3   // mirror blocks per warp in flight (shared-memory ring)
-#endif
-constexpr int kKnnSmem = PL_KNN_WARPS * PL_KNN_RING * 7 * 32 * 16;
-
-// One warp per (query group, split): lane j takes nodes 2j and 2j+1 of each
-// 64-node block of the split from the mirror and scores both against the
-// warp's queries with paired FP32 operations (each half rounds exactly like
-// the scalar knn_dist: t = q - x, dq and dv accumulated in component order,
-// d = w dv + dq).  The mirror blocks stream through a per-warp ring in
-// shared memory, PL_KNN_RING - 1 blocks ahead; each lane copies (cp.async)
-// and later reads only its own 16-byte words, so the ring needs no barrier.
-template <int KM>
-__global__ void __launch_bounds__(32 * PL_KNN_WARPS) k_plan_knn(PlanDev D, int kind) {
+__global__ void __launch_bounds__(KT_THREADS, 1) k_plan_knn_mins(PlanDev D, int kind, int t0,
+                                                                 int t1) {
   pdl_begin();
-  extern __shared__ float4 knn_ring[];   // [warp][slot][7][32]
-  const Sched* S = D.sched;
-  const int items = kind == 0 ? S->knn_items[0] : S->gq_n * S->nsg_max;
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float4* ring = knn_ring + (long)w * PL_KNN_RING * 7 * 32 + lane;
-  const float2 w2 = make_float2(D.w_vel, D.w_vel);
-  Sched* Sw = D.sched;
-  // warp g's first item is g; later ones are claimed from a counter past the
-  // grid's warps (a claim per warp at launch would queue every warp on one
-  // address)
-  const int nw = gridDim.x * PL_KNN_WARPS;
-  for (int round = 0;; ++round) {
-    int item = blockIdx.x * PL_KNN_WARPS + w;
-    if (round > 0) {
-      if (lane == 0) item = nw + atomicAdd(&Sw->knn_head[kind], 1);
-      item = __shfl_sync(0xffffffffu, item, 0);
+  extern __shared__ __align__(1024) uint8_t kt_smem[];
+  int* uo = reinterpret_cast<int*>(kt_smem + kKtSmem);
+  if (threadIdx.x < 32) {   // units of every problem's query tiles in the window
+    const int lane = threadIdx.x;
+    const int* qt = D.sched->qt_off[kind];
+    int total = 0;
+    for (int b = 0; b < D.P; b += 32) {
+      const int p = b + lane;
+      int n = 0;
+      if (p < D.P) {
+        const int rows = knn_rows(D, kind, p);
+        const int lo = max(qt[p], t0), hi = min(qt[p] + (rows + KT_QT - 1) / KT_QT, t1);
+        if (hi > lo) n = (hi - lo) * knn_node_tiles(D, p);
+      }
+      int x = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      if (p < D.P) uo[p] = total + x - n;
+      total += __shfl_sync(0xffffffffu, x, 31);
     }
-    if (item >= items) break;
-    int p, ns, split, b0, B;
-    if (kind == 0) {   // free queries [G, B) of problem p, PL_KNN_QW per item
-      p = find_problem(S->knn_off[0], D.P, item);
-      const int local = item - S->knn_off[0][p];
-      ns = S->nsplit[0][p];
-      const int g = local / ns;
-      split = local - g * ns;
-      B = min(max(D.prob[p].batch, 0), D.BM);
-      b0 = min(max(D.prob[p].n_goal, 0), B) + g * PL_KNN_QW;
-    } else {           // one decoded goal query per item: (list entry, split)
-      const int v = item / S->nsg_max;
-      split = item - v * S->nsg_max;
-      const int2 e = D.gq[v];
+    if (lane == 0) uo[D.P] = total;
+  }
+  __syncthreads();
+  const long units = uo[D.P], G = gridDim.x, b = blockIdx.x;
+  knn_mins(kt_smem, PlanKnnWork{D, uo, kind, t0}, units * b / G, units * (b + 1) / G,
+           &D.sched->knn_err);
+}
+
+__global__ void __launch_bounds__(32 * PL_KNN_SEL_WARPS, 4) k_plan_knn_select(PlanDev D, int kind,
+                                                                              int t0, int t1) {
+  pdl_begin();
+  __shared__ unsigned long long list[PL_KNN_SEL_WARPS][KT_LIST];
+  const Sched* S = D.sched;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int* qt = S->qt_off[kind];
+  const int items = kind == 0 ? (min(qt[D.P], t1) - t0) * KT_QT : S->gq_n;
+  const long stride = 4 * (long)kt_row_f4(D.NT);
+  const bool all = S->knn_err != 0;
+  unsigned long long pairs = 0;
+  for (int i = blockIdx.x * PL_KNN_SEL_WARPS + w; i < items; i += gridDim.x * PL_KNN_SEL_WARPS) {
+    int p, b, t, r;
+    if (kind == 0) {
+      t = t0 + i / KT_QT;
+      r = i % KT_QT;
+      p = find_problem(qt, D.P, t);
+      const int row = (t - qt[p]) * KT_QT + r;
+      if (row >= knn_rows(D, 0, p)) continue;          // warp-uniform
+      b = min(max(D.prob[p].n_goal, 0), D.BM) + row;
+    } else {
+      const int4 e = D.gq[i];
       p = e.x;
-      ns = S->nsplit[1][p];
-      if (split >= ns) continue;                 // warp-uniform: a smaller tree
-      b0 = e.y;
-      B = e.y + 1;
+      b = e.y;
+      t = qt[p] + e.z / KT_QT;
+      r = e.z % KT_QT;
+      if (t < t0 || t >= t1) continue;                 // warp-uniform
     }
-    // candidates whose decoding failed get no parents (their edges are
-    // invalid whatever the lists hold)
-    bool wact = false;                         // warp-uniform
-#pragma unroll
-    for (int a = 0; a < PL_KNN_QW; ++a)
-      wact |= b0 + a < B && D.valid[(long)p * D.BM + b0 + a];
-    const int N = D.n_nodes[p];
-    const int span = N - 1;
-    const int per = (span + ns - 1) / ns;
-    const int lo = 1 + split * per, hi = min(N, lo + per);
-    float2 q2[PL_KNN_QW][14];
-#pragma unroll
-    for (int a = 0; a < PL_KNN_QW; ++a) {
-      float qv[14];
-      load_query(reinterpret_cast<const float4*>(D.cand) + 4 * ((long)p * D.BM + min(b0 + a, B - 1)),
-                 qv);
-#pragma unroll
-      for (int c = 0; c < 14; ++c) q2[a][c] = make_float2(qv[c], qv[c]);
+    const long ci = (long)p * D.BM + b;
+    if (!D.valid[ci]) {                                // no edges, whatever the list holds
+      if (lane < D.KN) D.nn[ci * D.KN + lane] = -1;
+      continue;
     }
-    WarpTopK<KM> top[PL_KNN_QW];
-    const float4* mir = D.mir + (long)p * D.NB * 7 * 32 + lane;
-    const int blk0 = lo >> 6, nblk = wact ? ((hi + 63) >> 6) - blk0 : 0;
-#pragma unroll
-    for (int r = 0; r < PL_KNN_RING - 1; ++r) {   // prologue: blocks 0 .. RING-2
-      if (r < nblk)
-#pragma unroll
-        for (int cc = 0; cc < 7; ++cc)
-          cp_async16(ring + (r * 7 + cc) * 32, mir + ((blk0 + r) * 7 + cc) * 32);
-      cp_async_commit();
-    }
-    for (int r = 0; r < nblk; ++r) {
-      __syncwarp();   // last round's reads of the slot precede its refill
-      {
-        const int rn = r + PL_KNN_RING - 1;         // refill the slot freed last round
-        if (rn < nblk) {
-          const int slot = rn % PL_KNN_RING;
-#pragma unroll
-          for (int cc = 0; cc < 7; ++cc)
-            cp_async16(ring + (slot * 7 + cc) * 32, mir + ((blk0 + rn) * 7 + cc) * 32);
-        }
-        cp_async_commit();
-      }
-      cp_async_wait<PL_KNN_RING - 1>();             // this lane's copies of block r landed
-      float4 x[7];
-      const int slot = r % PL_KNN_RING;
-#pragma unroll
-      for (int cc = 0; cc < 7; ++cc) x[cc] = ring[(slot * 7 + cc) * 32];
-      const int blk = blk0 + r;
-      const int n0 = blk * 64 + 2 * lane;
-      const bool v0 = n0 >= lo && n0 < hi, v1 = n0 + 1 >= lo && n0 + 1 < hi;
-      float2 d[PL_KNN_QW];
-#pragma unroll
-      for (int a = 0; a < PL_KNN_QW; ++a) {
-        float2 dq = make_float2(0.f, 0.f), dv = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 14; ++c) {
-          const float4 v = x[c >> 1];
-          const float2 nv = (c & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-          const float2 t = __fadd2_rn(q2[a][c], nv);
-          if (c < 7) dq = __ffma2_rn(t, t, dq);
-          else dv = __ffma2_rn(t, t, dv);
-        }
-        d[a] = __ffma2_rn(w2, dv, dq);
-      }
-#pragma unroll
-      for (int a = 0; a < PL_KNN_QW; ++a) {
-        top[a].offer(__ballot_sync(0xffffffffu, v0 && knn_less(d[a].x, n0, top[a].td, top[a].ti)),
-                     d[a].x, n0);
-        top[a].offer(__ballot_sync(0xffffffffu, v1 && knn_less(d[a].y, n0 + 1, top[a].td, top[a].ti)),
-                     d[a].y, n0 + 1);
-      }
-    }
-    cp_async_wait<0>();
-    if (D.samples && lane == 0 && wact) {
-      int nq = 0;
-#pragma unroll
-      for (int a = 0; a < PL_KNN_QW; ++a) nq += b0 + a < B && D.valid[(long)p * D.BM + b0 + a];
-      atomicAdd(D.samples + 3, (unsigned long long)nq * (unsigned long long)max(hi - lo, 0));
-    }
-#pragma unroll
-    for (int a = 0; a < PL_KNN_QW; ++a) {
-      const int b = b0 + a;
-      if (b >= B || lane >= KM) continue;
-      const int id = D.valid[(long)p * D.BM + b] ? top[a].i : 0x7fffffff;
-      if (ns == 1) {
-        if (lane < D.KN) D.nn[((long)p * D.BM + b) * D.KN + lane] = id == 0x7fffffff ? -1 : id;
-      } else {
-        const long off = (((long)p * PL_NSPLIT_MAX + split) * D.BM + b) * KM + lane;
-        D.part_d[off] = top[a].d;
-        D.part_i[off] = id;
-      }
-    }
-    if (ns > 1) {
-      // the warp that completes a query's last split merges its lists
-#pragma unroll
-      for (int a = 0; a < PL_KNN_QW; ++a) {
-        const int b = b0 + a;
-        if (b >= B) continue;
-        // every lane's split-list stores are fenced, and the warp has passed
-        // its fences, before lane 0 counts the split as finished
-        __threadfence();
-        __syncwarp();
-        int last = 0;
-        if (lane == 0) {
-          int* cnt = D.knn_cnt + (long)p * D.BM + b;
-          last = atomicAdd(cnt, 1) == ns - 1;
-          if (last) *cnt = 0;   // ready for the next iteration
-        }
-        if (__shfl_sync(0xffffffffu, last, 0)) {
-          __threadfence();
-          knn_merge_query<KM>(D, p, b, ns);
-        }
-      }
-    }
+    const int n = D.n_nodes[p] - 1;
+    const KeyList best =
+        knn_select(D.soa + (long)p * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA, n, 1,
+                   reinterpret_cast<const float4*>(D.cand) + 4 * ci, D.KN, D.w_vel, D.sw_vel,
+                   D.gmin[kind] + ((long)(t - t0) * KT_QT + r) * stride, knn_node_tiles(D, p), all,
+                   list[w]);
+    if (lane < D.KN)
+      D.nn[ci * D.KN + lane] = best.key >= KT_NONE ? -1 : (int)(unsigned)best.key;
+    pairs += n;
   }
-}
-
-
-// Tiled search of the free queries (planners whose tree capacity is at
-// least PL_KNN_TILE_NODES): a CTA of PL_KNN_TW warps claims (problem, group
-// of PL_KNN_TW queries, split) items, warp w takes query w of the group.
-// The CTA's threads copy each 64-node mirror block of the split once into a
-// shared ring (cp.async, PL_KNN_TRING - 1 blocks ahead, one barrier per
-// block) and every warp scores it from there as k_plan_knn does (the same
-// paired arithmetic, list and tie rule), so a split's nodes leave L2 once
-// per PL_KNN_TW queries: on large trees the per-warp search is bound by the
-// L2 reads of every query streaming the whole split.  Warps whose query is
-// not valid keep to the copies and barriers.
-constexpr int kKnnTileSmem = PL_KNN_TRING * 7 * 32 * 16;
-
-template <int KM>
-__global__ void __launch_bounds__(32 * PL_KNN_TW) k_plan_knn_tile(PlanDev D) {
-  pdl_begin();
-  extern __shared__ float4 knn_tring[];   // [slot][7][32]
-  __shared__ int s_item;
-  const Sched* S = D.sched;
-  const int items = S->knn_items[0];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const float2 w2 = make_float2(D.w_vel, D.w_vel);
-  Sched* Sw = D.sched;
-  for (;;) {
-    __syncthreads();   // the last item's ring reads and s_item reads are done
-    if (threadIdx.x == 0) s_item = atomicAdd(&Sw->knn_head[0], 1);
-    __syncthreads();
-    const int item = s_item;
-    if (item >= items) break;                  // block-uniform
-    const int p = find_problem(S->knn_off[0], D.P, item);
-    const int local = item - S->knn_off[0][p];
-    const int ns = S->nsplit[0][p];
-    const int g = local / ns, split = local - g * ns;
-    const int B = min(max(D.prob[p].batch, 0), D.BM);
-    const int b = min(max(D.prob[p].n_goal, 0), B) + g * PL_KNN_TW + w;
-    const bool mine = b < B;                                    // warp-uniform
-    const bool wact = mine && D.valid[(long)p * D.BM + b];     // warp-uniform
-    const int N = D.n_nodes[p];
-    const int span = N - 1;
-    const int per = (span + ns - 1) / ns;
-    const int lo = 1 + split * per, hi = min(N, lo + per);
-    float2 q2[14];
-    {
-      float qv[14];
-      load_query(reinterpret_cast<const float4*>(D.cand) + 4 * ((long)p * D.BM + (mine ? b : B - 1)),
-                 qv);
-#pragma unroll
-      for (int c = 0; c < 14; ++c) q2[c] = make_float2(qv[c], qv[c]);
-    }
-    WarpTopK<KM> top;
-    const float4* mir = D.mir + (long)p * D.NB * 7 * 32;
-    const int blk0 = lo >> 6, nblk = hi > lo ? ((hi + 63) >> 6) - blk0 : 0;   // block-uniform
-    auto issue = [&](int r) {   // block r of the split into ring slot r % PL_KNN_TRING
-      if (r < nblk) {
-        const float4* src = mir + (long)(blk0 + r) * 7 * 32;
-        float4* dst = knn_tring + (r % PL_KNN_TRING) * 7 * 32;
-        for (int i = threadIdx.x; i < 7 * 32; i += 32 * PL_KNN_TW) cp_async16(dst + i, src + i);
-      }
-      cp_async_commit();
-    };
-#pragma unroll
-    for (int r = 0; r < PL_KNN_TRING - 1; ++r) issue(r);
-    for (int r = 0; r < nblk; ++r) {
-      cp_async_wait<PL_KNN_TRING - 2>();   // this thread's copies of block r landed
-      __syncthreads();                     // everyone's copies of block r; slot of r - 1 read
-      issue(r + PL_KNN_TRING - 1);         // into the slot block r - 1 held
-      if (wact) {
-        const float4* sl = knn_tring + (r % PL_KNN_TRING) * 7 * 32 + lane;
-        float4 x[7];
-#pragma unroll
-        for (int cc = 0; cc < 7; ++cc) x[cc] = sl[cc * 32];
-        const int n0 = (blk0 + r) * 64 + 2 * lane;
-        const bool v0 = n0 >= lo && n0 < hi, v1 = n0 + 1 >= lo && n0 + 1 < hi;
-        float2 dq = make_float2(0.f, 0.f), dv = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 14; ++c) {
-          const float4 v = x[c >> 1];
-          const float2 nv = (c & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
-          const float2 t = __fadd2_rn(q2[c], nv);
-          if (c < 7) dq = __ffma2_rn(t, t, dq);
-          else dv = __ffma2_rn(t, t, dv);
-        }
-        const float2 d = __ffma2_rn(w2, dv, dq);
-        top.offer(__ballot_sync(0xffffffffu, v0 && knn_less(d.x, n0, top.td, top.ti)), d.x, n0);
-        top.offer(__ballot_sync(0xffffffffu, v1 && knn_less(d.y, n0 + 1, top.td, top.ti)), d.y,
-                  n0 + 1);
-      }
-    }
-    cp_async_wait<0>();
-    if (D.samples && lane == 0 && wact)
-      atomicAdd(D.samples + 3, (unsigned long long)max(hi - lo, 0));
-    if (!mine) continue;                       // warp-uniform
-    if (lane < KM) {
-      const int id = wact ? top.i : 0x7fffffff;
-      if (ns == 1) {
-        if (lane < D.KN) D.nn[((long)p * D.BM + b) * D.KN + lane] = id == 0x7fffffff ? -1 : id;
-      } else {
-        const long off = (((long)p * PL_NSPLIT_MAX + split) * D.BM + b) * KM + lane;
-        D.part_d[off] = top.d;
-        D.part_i[off] = id;
-      }
-    }
-    if (ns > 1) {
-      // every lane's split-list stores are fenced, and the warp has passed
-      // its fences, before lane 0 counts the split as finished
-      __threadfence();
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) {
-        int* cnt = D.knn_cnt + (long)p * D.BM + b;
-        last = atomicAdd(cnt, 1) == ns - 1;
-        if (last) *cnt = 0;   // ready for the next iteration
-      }
-      if (__shfl_sync(0xffffffffu, last, 0)) {
-        __threadfence();
-        knn_merge_query<KM>(D, p, b, ns);
-      }
-    }
-  }
-}
-
-
-// Mirror of the tree for the parent search: node n sits in 64-node block
-// n / 64 at pair slot j = (n % 64) / 2, half h = n % 2; for component pair
-// cc (components 2cc, 2cc+1 of (q_1..q_7, qd_1..qd_7)) the float4
-// (x_2j[2cc], x_2j+1[2cc], x_2j[2cc+1], x_2j+1[2cc+1]) holds the values
-// negated, so that lane j loads its two nodes' component pairs with seven
-// 16-byte loads (512 contiguous bytes per warp instruction) and forms
-// q - x as q + (-x), exactly.
-__device__ __forceinline__ float* knn_mirror_slot(const PlanDev& D, int p, int n, int cc) {
-  const long f4 = (((long)p * D.NB + (n >> 6)) * 7 + cc) * 32 + ((n >> 1) & 31);
-  return reinterpret_cast<float*>(D.mir + f4) + (n & 1);
+  if (D.samples && lane == 0 && pairs) atomicAdd(D.samples + 3, pairs);
 }
 
 // parents prep (thread i of `stride`): neighbour lists of single-node trees
 // are empty; tree nodes added (or moved) since the last iteration enter the
-// mirror
+// images, with the empty rows that end their last tile
 __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stride) {
   if (stride <= 0 || i < 0 || i >= stride) return;
   const long n = (long)D.P * D.BM * D.KN;
@@ -996,15 +667,15 @@ __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stri
   const int total = S->pack_off[D.P];
   for (long x = i; x < total; x += stride) {
     const int p = find_problem(S->pack_off, D.P, (int)x);
-    const int node = S->pack_lo[p] + (int)(x - S->pack_off[p]);
-    const float* r = D.st + ((long)p * D.NC + node) * 16;
-#pragma unroll
-    for (int cc = 0; cc < 7; ++cc) {
-      const int c0 = 2 * cc, c1 = 2 * cc + 1;
-      float* slot = knn_mirror_slot(D, p, node, cc);
-      slot[0] = -r[c0 < 7 ? c0 : c0 + 1];
-      slot[2] = -r[c1 < 7 ? c1 : c1 + 1];
+    const int row = S->pack_lo[p] + (int)(x - S->pack_off[p]);
+    const bool have = row + 1 < D.n_nodes[p];
+    float v[14];
+    if (have) {
+      load_query(reinterpret_cast<const float4*>(D.st) + 4 * ((long)p * D.NC + row + 1), v);
+      knn_store_soa(D.soa + (long)p * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA, row, v);
     }
+    knn_pack_node(D.nimg + ((long)p * D.NT + row / KT_ROWS) * KT_TILE, row % KT_ROWS, v, D.sw_vel,
+                  have);
   }
 }
 
@@ -1998,6 +1669,7 @@ __global__ void __launch_bounds__(PL_CHORD_THREADS) k_plan_chord(PlanDev D, ArmK
     o4[1] = make_float4(q[4], q[5], q[6], 0.f);
     o4[2] = make_float4(qd[0], qd[1], qd[2], qd[3]);
     o4[3] = make_float4(qd[4], qd[5], qd[6], 0.f);
+    pack_query_row(D, 0, p, b - G, q, qd);
   }
 }
 
@@ -2833,7 +2505,7 @@ __global__ void __launch_bounds__(PL_PRUNE_T) k_prune_copy(PlanDev D) {
   if (ch == 0 && threadIdx.x == 0) {
     const int N = D.n_nodes[p];
     D.n_nodes[p] = total;
-    if (total != N) D.packed[p] = 0;   // indices moved: repack the mirror
+    if (total != N) D.packed[p] = 0;   // indices moved: repack the images
     const Incumbent in = D.inc[p];
     if (in.id >= 0 && in.id < N) {
       Incumbent o = in;
@@ -2919,7 +2591,7 @@ __global__ void __launch_bounds__(PL_ATTACH_THREADS) k_plan_prune(PlanDev D, Arm
   __syncthreads();
   if (threadIdx.x == 0) {
     D.n_nodes[p] = total;
-    if (total != N) D.packed[p] = 0;   // indices moved: repack the mirror
+    if (total != N) D.packed[p] = 0;   // indices moved: repack the images
     if (in.id >= 0) {
       Incumbent o = in;
       o.id = D.newidx[nb + in.id];
@@ -3146,48 +2818,8 @@ static void pl_launch(void (*k)(KArgs...), unsigned grid, unsigned block, size_t
   pl_launch_pdl(true, k, grid, block, smem, st, args...);
 }
 
-template <int KM>
-static int knn_blocks(fn_planner* pl) {
-  (void)pl;
-  static int blocks[64] = {0};   // per device: resident blocks of k_plan_knn<KM>
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) dev = 0;
-  if (blocks[dev] == 0) {
-    cudaFuncSetAttribute(k_plan_knn<KM>, cudaFuncAttributeMaxDynamicSharedMemorySize, kKnnSmem);
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plan_knn<KM>, 32 * PL_KNN_WARPS,
-                                                      kKnnSmem) != cudaSuccess ||
-        per_sm < 1)
-      per_sm = 1;
-    blocks[dev] = per_sm * num_sms();
-  }
-  return blocks[dev];
-}
-
-// resident CTAs of the tiled free-query search (its persistent grid)
-template <int KM>
-static int knn_tile_blocks() {
-  static int blocks[64] = {0};
-  int dev = 0;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= 64) dev = 0;
-  if (blocks[dev] == 0) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plan_knn_tile<KM>,
-                                                      32 * PL_KNN_TW, kKnnTileSmem) !=
-            cudaSuccess ||
-        per_sm < 1)
-      per_sm = 1;
-    blocks[dev] = per_sm * num_sms();
-  }
-  return blocks[dev];
-}
-
-// sampling and parents: candidates of every problem (unless given by the
-// caller), then their nearest tree nodes (mark(2) between the two)
 // the shared-memory request of the planner's tensor-memory kernels (the
-// warp-per-edge body, the goal edges), set once per device
+// warp-per-edge body, the goal edges, the parent search), set once per device
 static bool plan_tm_ready() {
   static std::once_flag once[64];
   static bool ok[64];
@@ -3198,11 +2830,15 @@ static bool plan_tm_ready() {
         cudaFuncSetAttribute(k_plan_edges_tm, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)kTmSmem) == cudaSuccess &&
         cudaFuncSetAttribute(k_plan_goal_edges, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kTmSmem) == cudaSuccess;
+                             (int)kTmSmem) == cudaSuccess &&
+        cudaFuncSetAttribute(k_plan_knn_mins, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kPlanKnnSmem) == cudaSuccess;
   });
   return ok[dev & 63];
 }
 
+// sampling and parents: candidates of every problem (unless given by the
+// caller), then their nearest tree nodes (mark(2) between the two)
 template <class Mark>
 static void enqueue_front(fn_planner* pl, unsigned flags, cudaStream_t st, Mark&& mark) {
   PlanDev& D = pl->D;
@@ -3218,25 +2854,18 @@ static void enqueue_front(fn_planner* pl, unsigned flags, cudaStream_t st, Mark&
   auto search = [&](int kind, cudaStream_t s) {
     if (!knn) return;
     const bool pdl = s != pl->side;
-    // the goal list is short (the decoded goals): a small grid claims it
-    const int gb = 2 * num_sms();
-    if (kind == 0 && D.knn_tile) {   // large trees: the tiled search
-      if (D.KM == 8)
-        pl_launch_pdl(pdl, k_plan_knn_tile<8>, knn_tile_blocks<8>(), 32 * PL_KNN_TW, kKnnTileSmem,
-                      s, D);
-      else
-        pl_launch_pdl(pdl, k_plan_knn_tile<16>, knn_tile_blocks<16>(), 32 * PL_KNN_TW,
-                      kKnnTileSmem, s, D);
-    } else if (D.KM == 8) {
-      pl_launch_pdl(pdl, k_plan_knn<8>,
-                    kind == 0 ? knn_blocks<8>(pl) : std::min(gb, knn_blocks<8>(pl)),
-                    32 * PL_KNN_WARPS, kKnnSmem, s, D, kind);
-    } else {
-      pl_launch_pdl(pdl, k_plan_knn<16>,
-                    kind == 0 ? knn_blocks<16>(pl) : std::min(gb, knn_blocks<16>(pl)),
-                    32 * PL_KNN_WARPS, kKnnSmem, s, D, kind);
+    // one pass unless the group minima of all query tiles exceed PL_KNN_BYTES
+    const int tiles = P * ((D.BM + KT_QT - 1) / KT_QT);
+    for (int t0 = 0; t0 < tiles; t0 += D.knn_tiles) {
+      const int t1 = std::min(tiles, t0 + D.knn_tiles);
+      pl_launch_pdl(pdl, k_plan_knn_mins, num_sms(), KT_THREADS, kPlanKnnSmem, s, D, kind, t0, t1);
+      trace(pl, s, "k_plan_knn");
+      const long warps = (long)(t1 - t0) * KT_QT;
+      pl_launch_pdl(pdl, k_plan_knn_select,
+                    (unsigned)std::min<long>(4L * num_sms(), (warps + PL_KNN_SEL_WARPS - 1) / PL_KNN_SEL_WARPS),
+                    32 * PL_KNN_SEL_WARPS, 0, s, D, kind, t0, t1);
+      trace(pl, s, "k_plan_knn");
     }
-    trace(pl, s, "k_plan_knn");
   };
   auto goals = [&](cudaStream_t s) {
     pl_launch_pdl(s != pl->side, k_plan_sample, (unsigned)((32 * n + 127) / 128), 128, 0, s, D,
@@ -3439,23 +3068,18 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
   PlanDev& D = pl->D;
   memset(&D, 0, sizeof(D));
   D.P = c.P; D.NC = c.n_cap; D.BM = c.b_max; D.KP = c.k; D.KN = std::max(c.k - 1, 1);
-  D.KM = (c.k - 1) <= 8 ? 8 : 16;
-  D.knn_tile = c.n_cap >= PL_KNN_TILE_NODES ? 1 : 0;
   D.att_wide = c.b_max >= PL_ATT_WIDE_B && c.P <= PL_ATT_WIDE_P ? 1 : 0;
-  D.knn_slots = D.knn_tile ? (D.KM == 8 ? knn_tile_blocks<8>() : knn_tile_blocks<16>())
-                           : (D.KM == 8 ? knn_blocks<8>(pl) : knn_blocks<16>(pl)) * PL_KNN_WARPS;
   D.vstages = (long)c.P * c.b_max * c.k >= PL_VSTAGE_EDGES ? 2 : 1;
   D.goal_split = 1;
   D.K = c.K; D.S = c.S; D.S_clear = c.S_clear; D.G = c.reach_grid;
   D.w_vel = c.w_vel; D.vel_frac = c.vel_frac; D.margin = c.clear_margin;
-  const size_t P = c.P, NC = c.n_cap, BM = c.b_max, KP = c.k, KN = D.KN, KM = D.KM;
+  const size_t P = c.P, NC = c.n_cap, BM = c.b_max, KP = c.k, KN = D.KN;
   fn_status rc = FN_OK;
 #define A_(ptr, n) if (rc == FN_OK) rc = pl_alloc_n(pl, &(ptr), (n))
   A_(D.st, P * NC * 16); A_(D.t, P * NC); A_(D.par, P * NC); A_(D.J, P * NC);
   A_(D.nu, P * NC); A_(D.eT, P * NC); A_(D.n_nodes, P);
   A_(D.cand, P * BM * 16); A_(D.treq, P * BM); A_(D.vrel, P * BM); A_(D.valid, P * BM);
   A_(D.nn, P * BM * KN);
-  A_(D.part_d, P * PL_NSPLIT_MAX * BM * KM); A_(D.part_i, P * PL_NSPLIT_MAX * BM * KM);
   A_(D.e_T, P * BM * KP); A_(D.e_rv, P * BM * KP); A_(D.e_ok, P * BM * KP);
   A_(D.e_k, P * BM * KP);
   A_(D.inc, P); A_(D.prob, P); A_(D.sched, 1); A_(D.out, P); A_(D.iter, 1);
@@ -3484,13 +3108,22 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
   A_(D.pend, (size_t)D.Emax * 2);
   D.surv_cap = (int)std::min<long>((long)D.Emax * 16, 1L << 26);
   A_(D.surv, (size_t)D.surv_cap);
-  D.NB = (NC + 63) / 64;
-  A_(D.mir, (size_t)P * D.NB * 7 * 32);
+  D.NT = (c.n_cap - 1 + KT_ROWS - 1) / KT_ROWS;
+  D.sw_vel = std::sqrt(c.w_vel);
+  {
+    const size_t tiles = P * ((BM + KT_QT - 1) / KT_QT);
+    const size_t per = (size_t)KT_QT * kt_row_f4(D.NT) * sizeof(float4);
+    D.knn_tiles = (int)std::max<size_t>(1, std::min(tiles, PL_KNN_BYTES / per));
+    A_(D.nimg, P * D.NT * KT_TILE); A_(D.soa, P * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA);
+    for (int i = 0; i < 2; ++i) {
+      A_(D.qimg[i], tiles * 2 * KT_TILE);
+      A_(D.gmin[i], (size_t)D.knn_tiles * per / sizeof(float));
+    }
+  }
   A_(D.packed, (size_t)P);
   D.sur = 0;
   D.sur_list = nullptr;
   A_(D.sur_n, 1);
-  A_(D.knn_cnt, P * BM);
   A_(D.dens, P); A_(D.arch, P); A_(D.cz, P * BM * 9); A_(D.zn, P * NC * 9); A_(D.glist, P * BM); A_(D.gq, P * BM);
   D.scfg = default_sampler_cfg();
   if (rc == FN_OK) {
@@ -3505,7 +3138,6 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
         cudaMemset(D.zn, 0xff, sizeof(float) * P * NC * 9) != cudaSuccess)
       rc = FN_ECUDA;
   }
-  if (rc == FN_OK && cudaMemset(D.knn_cnt, 0, sizeof(int32_t) * P * BM) != cudaSuccess) rc = FN_ECUDA;
   if (rc == FN_OK && cudaMemset(D.packed, 0, sizeof(int32_t) * P) != cudaSuccess) rc = FN_ECUDA;
 #undef A_
   if (rc == FN_OK) {

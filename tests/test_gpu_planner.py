@@ -557,3 +557,54 @@ def test_plan_round_nary_refinement(P, orc, arm):
         explained += ok
         assert ok, f"candidate {b} differs from the oracle's refined round outside the margin class"
     assert total >= 10 and same + explained == total, (same, explained, total)
+
+
+def _scan_lists(states, cand, k, w_vel):
+    """Parent lists of the standalone FP32 scan (fn_knn_tree without a workspace)."""
+    import ctypes as C
+
+    import torch
+
+    from paper_2609_22608_gb300._lib import lib
+    t, q = torch.from_numpy(states).cuda(), torch.from_numpy(cand).cuda()
+    idx = torch.empty(len(cand), k, dtype=torch.int32, device="cuda")
+    d2 = torch.empty(len(cand), k, device="cuda")
+    st = lib().fn_knn_tree(C.c_void_p(t.data_ptr()), len(states), 1, C.c_void_p(q.data_ptr()),
+                           len(cand), k, w_vel, C.c_void_p(idx.data_ptr()),
+                           C.c_void_p(d2.data_ptr()), None, 0,
+                           C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert st == 0
+    return idx.cpu().numpy()
+
+
+@pytest.mark.parametrize("k,bm,cap", [(8, 600, 4000), (17, 257, 3000),
+                                      (4, 65536, 1 << 19)])   # two windows of query tiles
+def test_parent_lists_are_the_scan(P, arm, k, bm, cap):
+    """The planner's parent lists are the FP32 scan's bit for bit, over uneven
+    problems (a tree of two nodes, tiles' edges, goal and free queries), in a
+    round after which the trees shrink (rows of the earlier trees must not be
+    seen), and where the group minima of all query tiles take two passes."""
+    sizes = [[2, 130, 2900], [3, 2500, 129]] if bm < 1000 else [[3000], [700]]
+    Bs = [5, min(bm, 300), min(bm, 257)] if bm < 1000 else [bm]
+    n = len(Bs)
+    root = synth.random_states(arm, 1, 77)[0]
+    pr = synth.make_problem(synth.random_toss(arm, 21), root=root)
+    pl = P.Planner(arm, P=n, n_cap=cap, b_max=bm, k=k, K=4, S=4, w_vel=0.1)
+    goals = [min(b, 90) if p != 1 else 0 for p, b in enumerate(Bs)]
+    probs = [P.problem_struct(pr, Bs[p], goals[p], root=root) for p in range(n)]
+    for r, Ns in enumerate(sizes):
+        pl.reset(probs)
+        trees = []
+        for p in range(n):
+            states, parent, t = synth.random_tree(arm, Ns[p], 31 + p + 7 * r, root=root)
+            cand = synth.random_states(arm, Bs[p], 50 + p + 7 * r)
+            cand[0] = states[Ns[p] - 1]
+            pl.load_tree(p, states, t, parent)
+            pl.set_candidates(p, cand, goals[p], np.full(goals[p], 0.5, np.float32),
+                              np.full(goals[p], 4.0, np.float32))
+            trees.append((states, cand))
+        pl.iterate(probs, 0, P.FN_PLAN_EXTERNAL)
+        for p, (states, cand) in enumerate(trees):
+            assert np.array_equal(pl.get_parents(p, Bs[p]),
+                                  _scan_lists(states, cand, k - 1, 0.1)), (r, p)
+    pl.close()
