@@ -320,6 +320,235 @@ __device__ __forceinline__ bool ik_solve_group(const ArmK& A, const float* Rg, c
   return tr > 1.f;
 }
 
+// ---------------------------------------------------------------------------
+// The same runs with a lane to two starts (the halves of the paired FP32
+// instructions) instead of eight lanes to one.  The group form passes every
+// frame product, Jacobian column and pivot row through warp shuffles, 111 an
+// iteration, and a SM does one a clock: 33 thousand goals' starts took 512 us
+// of which the shuffles alone are 313.  Here a lane holds everything, the
+// frames are formed by the products of the group form's scan (each in its
+// order, those that nothing reads left out), and each half's arithmetic is
+// the group form's, rounding for rounding: the same starts converge to the
+// same bits.  33 thousand goals: XX us.
+// ---------------------------------------------------------------------------
+#define FN_IK_TAB_F4 4
+struct IkTab {
+  const float4* p;   // [7][FN_IK_TAB_F4] (ca ca sa sa) (px px py py) (pz pz th0 th0) (lo lo hi hi)
+};
+__device__ __forceinline__ void fill_ik_tab(const ArmK& A, float4* t, int j) {
+  if (j >= 7) return;
+  t[4 * j + 0] = make_float4(A.ca[j], A.ca[j], A.sa[j], A.sa[j]);
+  t[4 * j + 1] = make_float4(A.px[j], A.px[j], A.py[j], A.py[j]);
+  t[4 * j + 2] = make_float4(A.pz[j], A.pz[j], A.th0[j], A.th0[j]);
+  t[4 * j + 3] = make_float4(A.q_lo[j], A.q_lo[j], A.q_hi[j], A.q_hi[j]);
+}
+
+struct Frame2 {        // pairs: rotation columns x, y, z and the origin
+  float2 x[3], y[3], z[3], o[3];
+};
+
+// link j's local transform (z: the constants (0, -sa, ca); o: p_j)
+__device__ __forceinline__ void ik_local(const IkTab& T, int j, float2 q, Frame2& f) {
+  const float4 t0 = T.p[4 * j], t1 = T.p[4 * j + 1], t2 = T.p[4 * j + 2];
+  const float2 ca = lo2(t0), sa = hi2(t0), th = add2(q, hi2(t2));
+  float2 s, c;
+  __sincosf(th.x, &s.x, &c.x);
+  __sincosf(th.y, &s.y, &c.y);
+  f.x[0] = c;
+  f.y[0] = neg2(s);
+  f.x[1] = mul2(s, ca);
+  f.y[1] = mul2(c, ca);
+  f.x[2] = mul2(s, sa);
+  f.y[2] = mul2(c, sa);
+  f.z[0] = dup2(0.f);
+  f.z[1] = neg2(sa);
+  f.z[2] = ca;
+  f.o[0] = lo2(t1);
+  f.o[1] = hi2(t1);
+  f.o[2] = lo2(t2);
+}
+// l's rotation times v: fmaf(x, v0, fmaf(y, v1, z v2)) per row
+__device__ __forceinline__ void ik_rot(const Frame2& l, const float2 (&v)[3], float2 (&r)[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    r[k] = fma2(l.x[k], v[0], fma2(l.y[k], v[1], mul2(l.z[k], v[2])));
+}
+// z and o of the product l f (r may be f)
+__device__ __forceinline__ void ik_mul_zo(const Frame2& l, const Frame2& f, Frame2& r) {
+  float2 z[3], o[3];
+  ik_rot(l, f.z, z);
+  ik_rot(l, f.o, o);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    r.z[k] = z[k];
+    r.o[k] = add2(l.o[k], o[k]);
+  }
+}
+// the whole product l f; kLocal: f is a local transform (its z's first entry is 0)
+template <bool kLocal>
+__device__ __forceinline__ void ik_mul(const Frame2& l, const Frame2& f, Frame2& r) {
+  float2 x[3], y[3];
+  ik_rot(l, f.x, x);
+  ik_rot(l, f.y, y);
+  if (kLocal) {
+    float2 z[3], o[3];
+    ik_rot(l, f.o, o);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) z[k] = fma2(l.y[k], f.z[1], mul2(l.z[k], f.z[2]));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      r.z[k] = z[k];
+      r.o[k] = add2(l.o[k], o[k]);
+    }
+  } else {
+    ik_mul_zo(l, f, r);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    r.x[k] = x[k];
+    r.y[k] = y[k];
+  }
+}
+__device__ __forceinline__ float2 rcp2(float2 a) {
+  return make_float2(rcp_approx(a.x), rcp_approx(a.y));
+}
+
+// Starts 2 h and 2 h + 1 on this lane: found.x, found.y whether they
+// converged, q[0..5] their final joints.  The target (Rg, pg), q7 and h may
+// differ from lane to lane.
+__device__ __forceinline__ void ik_solve_pair(const IkTab& T, float flange, const float* Rg,
+                                              const float* pg, float q7, int h, float2 (&q)[6],
+                                              bool& found_x, bool& found_y) {
+#pragma unroll
+  for (int s = 0; s < 6; ++s) {
+    const float4 t = T.p[4 * s + 3];
+    const float c = 0.5f * (t.x + t.z), hr = 0.5f * (t.z - t.x);
+    // starts 0, 1: 0 and (0, .5, 0, -.5, 0, .5); 2, 3: its negative and (0, -.5, 0, -.5, 0, -.5)
+    const float p1 = (s & 1) ? (s == 3 ? -0.5f : 0.5f) : 0.f;
+    const float px = h ? -p1 : 0.f, py = h ? ((s & 1) ? -0.5f : 0.f) : p1;
+    q[s] = make_float2(fmaf(px, hr, c), fmaf(py, hr, c));
+    if (s == 0) q[s] = dup2(fminf(fmaxf(atan2f(pg[1], pg[0]), t.x), t.z));
+  }
+  bool fail_x = false, fail_y = false;
+  float2 ep[3], er[3], Ree[9];
+#pragma unroll 1
+  for (int it = 0;; ++it) {
+    float2 z[6][3], o[6][3];   // axes and origins of joints 1..6 (frames of the scan)
+    Frame2 e;                  // end effector
+    {
+      Frame2 t0, t1, a1, a2, a3, b3, f, g;
+      ik_local(T, 0, q[0], t0);
+      ik_local(T, 1, q[1], t1);
+      ik_mul<true>(t0, t1, a1);                 // 0..1
+      ik_local(T, 2, q[2], f);
+      ik_mul<true>(t1, f, a2);                  // 1..2
+      ik_mul_zo(t0, a2, g);                     // 0..2
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        z[0][k] = t0.z[k]; o[0][k] = t0.o[k];
+        z[1][k] = a1.z[k]; o[1][k] = a1.o[k];
+        z[2][k] = g.z[k];  o[2][k] = g.o[k];
+      }
+      ik_local(T, 3, q[3], t1);
+      ik_mul<true>(f, t1, a3);                  // 2..3
+      ik_mul<false>(a1, a3, b3);                // 0..3
+      ik_local(T, 4, q[4], f);
+      ik_mul<true>(t1, f, g);                   // 3..4
+      ik_mul_zo(a2, g, g);                      // 1..4
+      ik_mul_zo(t0, g, g);                      // 0..4
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        z[3][k] = b3.z[k]; o[3][k] = b3.o[k];
+        z[4][k] = g.z[k];  o[4][k] = g.o[k];
+      }
+      ik_local(T, 5, q[5], t1);
+      ik_mul<true>(f, t1, g);                   // 4..5
+      ik_mul_zo(a3, g, f);                      // 2..5
+      ik_mul_zo(a1, f, f);                      // 0..5
+#pragma unroll
+      for (int k = 0; k < 3; ++k) { z[5][k] = f.z[k]; o[5][k] = f.o[k]; }
+      ik_local(T, 6, dup2(q7), t1);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)               // 6..flange: the rotation is link 7's
+        t1.o[k] = add2(t1.o[k], mul2(t1.z[k], dup2(flange)));
+      ik_mul<false>(g, t1, f);                  // 4..flange
+      ik_mul<false>(b3, f, e);                  // 0..flange
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      ep[k] = add2(dup2(pg[k]), neg2(e.o[k]));
+      er[k] = dup2(0.f);
+      Ree[3 * k] = e.x[k];
+      Ree[3 * k + 1] = e.y[k];
+      Ree[3 * k + 2] = e.z[k];
+    }
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      float2 x[3];
+      cross2(Ree[c], Ree[3 + c], Ree[6 + c], dup2(Rg[c]), dup2(Rg[3 + c]), dup2(Rg[6 + c]), x[0],
+             x[1], x[2]);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) er[k] = fma2(dup2(0.5f), x[k], er[k]);
+    }
+    if (it == FN_IK_ITERS) break;
+    // N = J^T J + lambda^2 I (symmetric before the elimination) and J^T e
+    float2 N[6][6], gr[6];
+    {
+      float2 J[6][6];   // J[m]: column of joint m
+#pragma unroll
+      for (int m = 0; m < 6; ++m) {
+        cross2(z[m][0], z[m][1], z[m][2], add2(e.o[0], neg2(o[m][0])),
+               add2(e.o[1], neg2(o[m][1])), add2(e.o[2], neg2(o[m][2])), J[m][0], J[m][1], J[m][2]);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) J[m][3 + k] = z[m][k];
+      }
+#pragma unroll
+      for (int m = 0; m < 6; ++m) {
+#pragma unroll
+        for (int n = m; n < 6; ++n) {
+          float2 a = dup2(n == m ? FN_IK_LAMBDA * FN_IK_LAMBDA : 0.f);
+#pragma unroll
+          for (int i = 0; i < 6; ++i) a = fma2(J[m][i], J[n][i], a);
+          N[m][n] = a;
+          N[n][m] = a;
+        }
+        float2 a = dup2(0.f);
+#pragma unroll
+        for (int i = 0; i < 6; ++i) a = fma2(J[m][i], i < 3 ? ep[i] : er[i - 3], a);
+        gr[m] = a;
+      }
+    }
+    float2 ip[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      fail_x |= !(N[k][k].x > 0.f);
+      fail_y |= !(N[k][k].y > 0.f);
+      ip[k] = rcp2(N[k][k]);
+#pragma unroll
+      for (int r = 0; r < 6; ++r) {
+        if (r == k) continue;
+        const float2 f = neg2(mul2(N[r][k], ip[k]));
+#pragma unroll
+        for (int j = k + 1; j < 6; ++j) N[r][j] = fma2(f, N[k][j], N[r][j]);
+        gr[r] = fma2(f, gr[k], gr[r]);
+      }
+    }
+#pragma unroll
+    for (int s = 0; s < 6; ++s) {
+      const float4 t = T.p[4 * s + 3];
+      const float2 n = fma2(gr[s], ip[s], q[s]);
+      q[s] = make_float2(fminf(fmaxf(n.x, t.x), t.z), fminf(fmaxf(n.y, t.x), t.z));
+    }
+  }
+  float2 tr = dup2(0.f);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) tr = fma2(dup2(Rg[i]), Ree[i], tr);
+  const float px[3] = {ep[0].x, ep[1].x, ep[2].x}, rx[3] = {er[0].x, er[1].x, er[2].x};
+  const float py[3] = {ep[0].y, ep[1].y, ep[2].y}, ry[3] = {er[0].y, er[1].y, er[2].y};
+  found_x = !fail_x && norm3(px) < FN_IK_POS_TOL && norm3(rx) < FN_IK_ROT_TOL && tr.x > 1.f;
+  found_y = !fail_y && norm3(py) < FN_IK_POS_TOL && norm3(ry) < FN_IK_ROT_TOL && tr.y > 1.f;
+}
+
 // Eq. (ballistic) at flight time t
 __device__ __forceinline__ void flight(const fn_problem_t& P, float t, float* x, float* xd) {
 #pragma unroll

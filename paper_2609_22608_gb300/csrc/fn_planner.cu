@@ -8,8 +8,8 @@
 // captured as a CUDA graph.  One iteration is a fixed sequence of launches
 // over all problems (each launched with programmatic dependent launch):
 //   schedule : per-problem work offsets, work-queue resets
-//   sample   : goal chart (warp per candidate, lane-parallel IK) and
-//              uniform candidates (Philox counters); parent-search prep
+//   goals    : goal chart (two lanes per candidate, two IK starts a lane)
+//   sample   : uniform candidates (Philox counters); parent-search prep
 //              (operand images of the nodes and queries) in the same launch
 //   knn      : group minima of every query on the tensor cores, then a warp
 //              per query scores the groups in reach exactly (knn_tc.cuh)
@@ -425,8 +425,6 @@ __device__ __forceinline__ void sample_free(const PlanDev& D, const ArmK& A, int
 
 __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stride);
 
-__device__ __forceinline__ void sample_goal(const PlanDev& D, const ArmK& A, int p, int b, int dens);
-
 // a goal query of this round: a decoded (valid) one joins the goal list of
 // the parent search and its problem's query rows; the others get empty
 // parent lists here
@@ -441,95 +439,109 @@ __device__ __forceinline__ void goal_query(const PlanDev& D, int p, int b, bool 
   }
 }
 
-// Sampling launches: warp w < nslots (P * b_max, or 0 when the caller gives
-// the candidates) owns candidate slot (p, b).
-//   role 0: a free slot is drawn by lane 0; the warps past the slots prepare
-//           the parent search (parents_prep: node images, empty lists);
-//   role 1: a goal slot is decoded by the whole warp (sample_goal).
+// Sampling launch: a lane per candidate slot (nslots = P * b_max, or 0 when
+// the caller gives the candidates) draws the free ones; the warps past the
+// slots prepare the parent search (parents_prep: node images, empty lists).
 __global__ void __launch_bounds__(128) k_plan_sample(PlanDev D, ArmK A, long nslots,
-                                                     int prep_warps, int dens, int role) {
+                                                     int prep_warps) {
   pdl_begin();
   const long gid = ((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
-  if (role == 0) {
-    const long nsw = (nslots + 31) / 32;              // slot warps: one lane per slot
-    if (gid < nsw) {
-      const long x = gid * 32 + lane;
-      if (x < nslots) {
+  const long nsw = (nslots + 31) / 32;              // slot warps
+  if (gid < nsw) {
+    const long x = gid * 32 + lane;
+    if (x < nslots) {
+      const int p = (int)(x / D.BM), b = (int)(x - (long)p * D.BM);
+      const int B = min(max(D.prob[p].batch, 0), D.BM);
+      if (b >= min(max(D.prob[p].n_goal, 0), B) && b < B) sample_free(D, A, p, b);
+    }
+  } else if (gid - nsw < prep_warps) {
+    const long i = (gid - nsw) * 32 + lane, stride = (long)prep_warps * 32;
+    parents_prep(D, i, stride);
+    if (nslots == 0)                                // external candidates: their queries
+      for (long x = i; x < (long)D.P * D.BM; x += stride) {
         const int p = (int)(x / D.BM), b = (int)(x - (long)p * D.BM);
         const int B = min(max(D.prob[p].batch, 0), D.BM);
-        if (b >= min(max(D.prob[p].n_goal, 0), B) && b < B) sample_free(D, A, p, b);
+        const int G = min(max(D.prob[p].n_goal, 0), B);
+        if (b < G) goal_query(D, p, b, D.valid[x] != 0);
+        else if (b < B) pack_query_row(D, 0, p, b - G, D.cand + x * 16, D.cand + x * 16 + 8);
       }
-    } else if (gid - nsw < prep_warps) {
-      const long i = (gid - nsw) * 32 + lane, stride = (long)prep_warps * 32;
-      parents_prep(D, i, stride);
-      if (nslots == 0)                                // external candidates: their queries
-        for (long x = i; x < (long)D.P * D.BM; x += stride) {
-          const int p = (int)(x / D.BM), b = (int)(x - (long)p * D.BM);
-          const int B = min(max(D.prob[p].batch, 0), D.BM);
-          const int G = min(max(D.prob[p].n_goal, 0), B);
-          if (b < G) goal_query(D, p, b, D.valid[x] != 0);
-          else if (b < B) pack_query_row(D, 0, p, b - G, D.cand + x * 16, D.cand + x * 16 + 8);
-        }
-    }
-  } else if (gid < nslots) {
-    const int p = (int)(gid / D.BM);
-    const int b = (int)(gid - (long)p * D.BM);
-    const int B = min(max(D.prob[p].batch, 0), D.BM);
-    if (b < min(max(D.prob[p].n_goal, 0), B)) sample_goal(D, A, p, b, dens);   // warp-uniform
   }
 }
 
-// A goal slot: every lane decodes the chart pose, lane groups 0-3 (8 lanes
-// each) run the four IK starts in parallel (ik_solve_group) and the lowest
-// start that converges wins, the same result as trying the starts in order.
-// The draw's outcome (defined, or the condition that left phi undefined) is
-// counted in work counters 8..13.
-__device__ __forceinline__ void sample_goal(const PlanDev& D, const ArmK& A, int p, int b,
-                                            int dens) {
-  const int lane = threadIdx.x & 31;
-  const fn_problem_t& P = D.prob[p];
-  const long ci = (long)p * D.BM + b;
-  const int it = *D.iter;
-  float u[12], z[9];
+// Goal slots: two lanes to a goal, each decoding the chart pose and running
+// two of the four IK starts (ik_solve_pair); the lowest start that converges
+// wins, the same result as trying them in order.  Blocks of one warp, so
+// that a small batch spreads over the SMs.  The draws' outcomes (defined, or
+// the condition that left phi undefined) are counted in work counters 8..13.
+__global__ void __launch_bounds__(32) k_plan_goals(PlanDev D, ArmK A, int dens) {
+  pdl_begin();
+  __shared__ float4 tab[7 * FN_IK_TAB_F4];
+  const int lane = threadIdx.x, h = lane & 1;
+  fill_ik_tab(A, tab, lane);
+  __syncwarp();
+  const Sched* S = D.sched;
+  const int total = S->goal_off[D.P] / D.KP, it = *D.iter;
+  for (int base = blockIdx.x * 16; base < total; base += gridDim.x * 16) {   // warp-uniform
+    const int item = min(base + (lane >> 1), total - 1);
+    const bool mine = base + (lane >> 1) < total && h == 0;   // writes the goal
+    const int p = find_problem(S->goal_off, D.P, item * D.KP);
+    const int b = item - S->goal_off[p] / D.KP;
+    const fn_problem_t& P = D.prob[p];
+    const long ci = (long)p * D.BM + b;
+    float u[12], z[9];
 #pragma unroll
-  for (int s = 0; s < 3; ++s) philox_u4(P.seed, b, it, p, 8 + s, u + 4 * s);
+    for (int s = 0; s < 3; ++s) philox_u4(P.seed, b, it, p, 8 + s, u + 4 * s);
 #pragma unroll
-  for (int i = 0; i < 9; ++i) z[i] = u[i];
-  if (dens) density_z(D.dens[p], P.seed, b, it, p, z);
+    for (int i = 0; i < 9; ++i) z[i] = u[i];
+    if (dens) density_z(D.dens[p], P.seed, b, it, p, z);
+    if (mine)
 #pragma unroll
-  for (int i = 0; i < 9; ++i)
-    if (lane == i) D.cz[ci * 9 + i] = z[i];
-  ChartPose o;
-  float q[7], qd[7];
-  const int why = warp_decode_goal(A, P, z, o, q, qd);
-  if (lane != 0) return;
-  if (D.samples) {
-    if (why != CHART_SPEED) atomicAdd(D.samples + 4, (unsigned long long)FN_IK_STARTS);
-    atomicAdd(D.samples + 8 + why, 1ull);
-  }
-  if (why == CHART_SPEED || why == CHART_IK) {   // undefined before the velocity part
+      for (int i = 0; i < 9; ++i) D.cz[ci * 9 + i] = z[i];
+    ChartPose o = {};
+    float2 q2[6];
+    bool fx, fy;
+    int why = chart_pose(A, P, z, o) ? CHART_OK : CHART_SPEED;
+    ik_solve_pair(IkTab{tab}, A.flange_d, o.Rg, o.pg, o.q7, h, q2, fx, fy);
+    // the pair's lowest converged start
+    const unsigned own = (fx ? 1u : 0u) | (fy ? 2u : 0u);
+    const unsigned other = __shfl_xor_sync(0xffffffffu, own, 1);
+    const unsigned won = h ? other | own << 2 : own | other << 2;
+    const int start = __ffs(won) - 1;                  // -1: none
+    float q[7], qd[7];
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      const float a = (start & 1) ? q2[j].y : q2[j].x;
+      const float c = __shfl_xor_sync(0xffffffffu, a, 1);
+      q[j] = (start >> 1) == h ? a : c;
+    }
+    q[6] = o.q7;
+    if (why == CHART_OK) why = won ? chart_velocity(A, o, q, qd) : CHART_IK;
+    if (D.samples) {
+      const unsigned tried = __ballot_sync(0xffffffffu, mine && why != CHART_SPEED);
+      if (lane == 0 && tried)
+        atomicAdd(D.samples + 4, (unsigned long long)FN_IK_STARTS * __popc(tried));
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const unsigned m = __ballot_sync(0xffffffffu, mine && why == c);
+        if (lane == 0 && m) atomicAdd(D.samples + 8 + c, (unsigned long long)__popc(m));
+      }
+    }
+    if (!mine) continue;
+    const bool ok = why == CHART_OK;
+    if (!ok)   // phi is undefined
+#pragma unroll
+      for (int j = 0; j < 7; ++j) q[j] = qd[j] = 0.f;
     D.treq[ci] = o.T;
     D.vrel[ci] = o.vrel;
-    D.valid[ci] = 0;
+    D.valid[ci] = ok ? 1 : 0;
     float4* o4 = reinterpret_cast<float4*>(D.cand + ci * 16);
-    o4[0] = o4[1] = o4[2] = o4[3] = make_float4(0.f, 0.f, 0.f, 0.f);
-    goal_query(D, p, b, false);
-    return;
+    o4[0] = make_float4(q[0], q[1], q[2], q[3]);
+    o4[1] = make_float4(q[4], q[5], q[6], 0.f);
+    o4[2] = make_float4(qd[0], qd[1], qd[2], qd[3]);
+    o4[3] = make_float4(qd[4], qd[5], qd[6], 0.f);
+    goal_query(D, p, b, ok);
   }
-  const bool ok = why == CHART_OK;
-  if (!ok)
-#pragma unroll
-    for (int j = 0; j < 7; ++j) q[j] = qd[j] = 0.f;
-  D.treq[ci] = o.T;
-  D.vrel[ci] = o.vrel;
-  D.valid[ci] = ok ? 1 : 0;
-  float4* o4 = reinterpret_cast<float4*>(D.cand + ci * 16);
-  o4[0] = make_float4(q[0], q[1], q[2], q[3]);
-  o4[1] = make_float4(q[4], q[5], q[6], 0.f);
-  o4[2] = make_float4(qd[0], qd[1], qd[2], qd[3]);
-  o4[3] = make_float4(qd[4], qd[5], qd[6], 0.f);
-  goal_query(D, p, b, ok);
 }
 
 // ---------------------------------------------------------------------------
@@ -2868,8 +2880,9 @@ static void enqueue_front(fn_planner* pl, unsigned flags, cudaStream_t st, Mark&
     }
   };
   auto goals = [&](cudaStream_t s) {
-    pl_launch_pdl(s != pl->side, k_plan_sample, (unsigned)((32 * n + 127) / 128), 128, 0, s, D,
-                  pl->arm, n, 0, dens, 1);
+    pl_launch_pdl(s != pl->side, k_plan_goals,
+                  (unsigned)std::min<long>((n + 15) / 16, 16L * num_sms()), 32, 0, s, D, pl->arm,
+                  dens);
     trace(pl, s, "k_plan_sample");
   };
   auto goal_edges = [&](cudaStream_t s) {   // after the goal queries' parent search
@@ -2878,22 +2891,28 @@ static void enqueue_front(fn_planner* pl, unsigned flags, cudaStream_t st, Mark&
                   pl->arm);
     trace(pl, s, "k_plan_goal_edges");
   };
+  // two branches: the free queries' parent search (and, after this function,
+  // the free edges) on the caller's stream; the goal chart's IK, the goal
+  // queries' search and the goal edges on the side stream, joined before the
+  // attach.  The IK needs the schedule only; the goal search also the nodes
+  // that the sampling launch packs.
+  const bool fork = n > 0 && knn && D.goal_split && !(flags & FN_PLAN_CHORD) && pl->allow_fork;
+  if (fork) {
+    cudaEventRecord(pl->ev_fork, st);
+    cudaStreamWaitEvent(pl->side, pl->ev_fork, 0);
+    goals(pl->side);
+  }
   if (n + prep > 0) {
     const long warps = (n + 31) / 32 + prep;
     pl_launch(k_plan_sample, (unsigned)((32 * warps + 127) / 128), 128, 0, st, D, pl->arm, n,
-              prep, dens, 0);
+              prep);
     trace(pl, st, "k_plan_prep");
   }
-  if (n > 0 && knn && D.goal_split && !(flags & FN_PLAN_CHORD) && pl->allow_fork) {
-    // two branches: the free queries' parent search (and, after this
-    // function, the free edges) on the caller's stream; the goal chart's IK,
-    // the goal queries' search and the goal edges on the side stream, joined
-    // before the attach
+  if (fork) {
     mark(2);
     cudaEventRecord(pl->ev_fork, st);
     cudaStreamWaitEvent(pl->side, pl->ev_fork, 0);
     search(0, st);
-    goals(pl->side);
     search(1, pl->side);
     goal_edges(pl->side);
     cudaEventRecord(pl->ev_join, pl->side);

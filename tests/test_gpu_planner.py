@@ -608,3 +608,30 @@ def test_parent_lists_are_the_scan(P, arm, k, bm, cap):
             assert np.array_equal(pl.get_parents(p, Bs[p]),
                                   _scan_lists(states, cand, k - 1, 0.1)), (r, p)
     pl.close()
+
+
+@pytest.mark.parametrize("goals", [[1, 0, 15, 2], [0, 16, 17, 0], [33, 0, 0, 250], [0, 0, 0, 1]])
+def test_goal_draws_do_not_depend_on_the_batch(P, arm, goals):
+    """A goal slot's draw is a function of its problem and index alone: uneven
+    problems (with no goals among them, and goals that leave a warp's lanes
+    empty) give the slots of a round in which every problem draws 250."""
+    n = len(goals)
+    probs = []
+    for p in range(n):
+        root = synth.random_states(arm, 1, 60 + p)[0]
+        probs.append((synth.make_problem(synth.random_toss(arm, 40 + p), root=root), root))
+    pl = P.Planner(arm, P=n, n_cap=600, b_max=260, k=3, K=4, S=4)
+
+    def draws(gs):
+        ps = [P.problem_struct(pr, 260, g, root=root, seed=5 + i)
+              for i, ((pr, root), g) in enumerate(zip(probs, gs))]
+        pl.reset(ps)
+        pl.iterate(ps, 3, 0)
+        return [pl.get_candidates(p, 260) for p in range(n)]
+
+    ref, got = draws([250] * n), draws(goals)
+    pl.close()
+    assert sum(int(r["valid"][:250].sum()) for r in ref) > 0
+    for p, g in enumerate(goals):
+        for f in ("states", "T_req", "v_rel", "valid"):
+            assert got[p][f][:g].tobytes() == ref[p][f][:g].tobytes(), (p, f)
