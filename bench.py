@@ -409,8 +409,8 @@ def roofline_from_trace(traced, work, workload="iteration"):
     iteration: its algorithmic FLOP (work counter x FLOP per unit) over its
     own event-timed duration, against the derived FP32 peak."""
     tab = kernel_table(traced)
-    units = {"k_plan_expand": (work["probe"], FLOP_PER_SAMPLE,
-                               "torque evaluations (the end-sample split, three per edge end)"),
+    units = {"k_plan_probe": (work["probe"], FLOP_PER_SAMPLE,
+                              "torque evaluations (the end-sample split, three per edge end)"),
              "k_plan_mprobe": (work["mprobe"], FLOP_PER_SAMPLE, "torque evaluations"),
              "k_plan_edges_tm": (work["probe"] + work["mprobe"] + work["verify"], FLOP_PER_SAMPLE,
                                  "torque evaluations (splits, probes and checks)"),
@@ -442,7 +442,7 @@ def roofline_from_trace(traced, work, workload="iteration"):
                     "flop_per_unit": f})
     # the edge-timing kernels (the RNEA hot path) for reference
     edge = {}
-    for k in ("k_plan_expand", "k_plan_mprobe", "k_plan_edges_tm"):
+    for k in ("k_plan_probe", "k_plan_mprobe", "k_plan_edges_tm"):
         if k in tab:
             n, f, _ = units[k]
             edge[k] = {"ms": tab[k]["ms"], "tflops": n * f / (tab[k]["ms"] / 1e3) / 1e12}

@@ -13,8 +13,8 @@
 //              (operand images of the nodes and queries) in the same launch
 //   knn      : group minima of every query on the tensor cores, then a warp
 //              per query scores the groups in reach exactly (knn_tc.cuh)
-//   edges    : prep + item scan (eprep, escan, expand), probe of both end
-//              samples of every (edge, admissible duration), probe of four
+//   edges    : prep (eprep), end-sample split and probe of both end samples
+//              of every (edge, admissible duration) (probe), probe of four
 //              interior samples of the survivors (mprobe), verification
 //              (vinit, two packed stages + selections, leftover stage),
 //              rho_v and clearance at the accepted duration
@@ -67,11 +67,9 @@ struct Incumbent {
 
 struct Sched {
   unsigned int queue_head;
-  int n_items;        // probe items of the packed edge phase
   int n_pend[2];      // lengths of the two pending-edge lists
   int n_surv;         // probe survivors appended (may exceed surv_cap)
   int n_dyn;          // edges with probe items listed by the prep (zero between bodies)
-  unsigned prep_done; // blocks of k_plan_eprep finished (zero between iterations)
   unsigned att_done;  // blocks of k_attach_scan finished (zero between iterations)
   unsigned prune_done;  // blocks of k_prune_walk finished (zero between iterations)
   unsigned tm_done;    // CTAs of k_plan_edges_tm finished (zero between bodies)
@@ -148,16 +146,13 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   int32_t* e_par;     // [E] parent node (-1: invalid edge)
   float* e_Tp;        // [E] goal: fixed duration; free: cap
   uint8_t* e_j;       // [E] parent slot | 0x80 for goal edges
-  int32_t* e_cnt;     // [E] probe items; then local exclusive offsets
-  int32_t* e_klo;     // [E] grid index of the edge's first probe item
-  int32_t* blk_off;   // [ceil(E/PL_SCAN)] block offsets of the item scan
+  int32_t* e_cnt;     // [E] durations to probe (0: decided by the prep)
+  int32_t* e_klo;     // [E] grid index of the first of them
   uint32_t* mask;     // [E][8] surviving grid indices of the probe
-  int32_t* owner;     // [E*K] probe item -> edge
   int32_t* cur_k;     // [E] duration under verification (grid index; 0 for goals)
   uint32_t* fail;     // [E] a sample of cur_k violated a limit
   int32_t* pend;      // [2][E] edges pending verification (ping-pong lists)
   int2* surv;         // [surv_cap] probe survivors (edge, grid index)
-  float* edyn;        // [Emax][2][28] end-sample torque split (alpha, beta, gamma, qd) per end
   int32_t* dyn_list;  // [Emax] edges with probe items (order of listing)
   int Emax, Kmax, surv_cap;
   // duration surrogate: free edges with admissible durations routed to the
@@ -761,33 +756,20 @@ __device__ __forceinline__ void list_dyn_edge(const PlanDev& D, int e, bool has_
   if (has_items) D.dyn_list[base + __popc(m & ((1u << lane) - 1u))] = e;
 }
 
-// exclusive scan of the per-block item totals (one block of PL_SCAN threads)
-__device__ __forceinline__ void scan_block_totals(const PlanDev& D, int* sh) {
-  Sched* S = D.sched;
-  const int nb = (S->n_edges + PL_SCAN - 1) / PL_SCAN;
-  int carry = 0;
-  for (int base = 0; base < nb; base += PL_SCAN) {
-    const int i = base + threadIdx.x;
-    const int v = i < nb ? __ldcg(D.blk_off + i) : 0;
-    int tot;
-    const int ex = block_scan(v, sh, &tot);
-    if (i < nb) D.blk_off[i] = carry + ex;
-    carry += tot;
-  }
-  if (threadIdx.x == 0) {
-    S->n_items = carry;
-    S->queue_head = 0u;
-    S->n_pend[0] = S->n_pend[1] = 0;   // verification lists and probe survivors
-    S->n_surv = 0;
-  }
+// the lists that the body appends to, emptied by the prep before it
+__device__ __forceinline__ void clear_body_lists(Sched* S) {
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  S->queue_head = 0u;
+  S->n_pend[0] = S->n_pend[1] = 0;
+  S->n_surv = 0;
 }
 
 __global__ void __launch_bounds__(PL_SCAN) k_plan_eprep(PlanDev D, GridKP Gr) {
   pdl_begin();
   __shared__ float sT[FN_MAX_GRID];
-  __shared__ int sh[32];
   for (int i = threadIdx.x; i < D.K; i += blockDim.x) sT[i] = Gr.T[i];
   __syncthreads();
+  clear_body_lists(D.sched);
   const Sched* S = D.sched;
   const int E = S->n_edges;
   const int e = blockIdx.x * PL_SCAN + threadIdx.x;
@@ -828,6 +810,7 @@ __global__ void __launch_bounds__(PL_SCAN) k_plan_eprep(PlanDev D, GridKP Gr) {
     D.e_Tp[e] = Tp;
     D.e_j[e] = (uint8_t)(j | (goal ? 0x80 : 0));
     D.e_klo[e] = 0;
+    D.e_cnt[e] = cnt;
 #pragma unroll
     for (int w = 0; w < 8; ++w) D.mask[8L * e + w] = 0u;
     if (cnt == 0 && !routed) {   // decided without dynamics: invalid or no admissible duration
@@ -838,126 +821,121 @@ __global__ void __launch_bounds__(PL_SCAN) k_plan_eprep(PlanDev D, GridKP Gr) {
     }
   }
   list_dyn_edge(D, e, e < E && cnt > 0);
-  // block-local exclusive scan of the item counts
-  int tot;
-  const int ex = block_scan(cnt, sh, &tot);
-  if (e < E) D.e_cnt[e] = ex;
-  // the block that finishes last scans the block totals (the planner's
-  // k_plan_escan folded into this launch): each block's total is fenced
-  // before the block is counted
-  __shared__ bool s_last;
-  if (threadIdx.x == 0) {
-    D.blk_off[blockIdx.x] = tot;
-    __threadfence();
-    const unsigned done = atomicAdd(&D.sched->prep_done, 1u);
-    s_last = done == gridDim.x - 1;
-    if (s_last) D.sched->prep_done = 0u;   // ready for the next iteration
-  }
-  __syncthreads();
-  if (s_last) {
-    __threadfence();
-    scan_block_totals(D, sh);
-  }
 }
 
-__global__ void __launch_bounds__(PL_SCAN) k_plan_escan(PlanDev D) {
+// Split and probe of the listed edges, five to a warp at a time.  Lanes
+// (edge, end, part) evaluate the end-sample torque split (end_torque_part's
+// decomposition: three torque evaluations per end instead of two per
+// duration) with the rolled recursion, whose one-link body is fetched once
+// where each lane evaluates Eq. (torque) about once; then, edge by edge, the
+// lanes take 32 grid durations each and check both end samples (u = 0, 1)
+// from the split in shared memory.  A duration whose ends pass is marked in
+// the edge's survivor mask and appended to the survivor list, whose counter
+// gets one atomic per five edges.  Goal edges have one item: their fixed
+// duration.
+// The split and the probe were two launches, the probe a lane per (edge,
+// duration) item: a map from item to edge, a scan of the item counts, the
+// split's 224 bytes an edge through memory, and an atomic on one counter per
+// 32 items, each behind the last's latency.  65 thousand edges (anytime
+// loop): 34 + 129 us before, XX now; 130 thousand (64 problems) 75 + 149,
+// XX now.
+#define PL_PR_WARPS 3
+#define PL_PR_EDGES 5
+__global__ void __launch_bounds__(32 * PL_PR_WARPS) k_plan_probe(PlanDev D, ArmK A, GridKP Gr) {
   pdl_begin();
-  __shared__ int sh[32];
-  scan_block_totals(D, sh);
-}
-
-__device__ __forceinline__ int item_off(const PlanDev& D, int e) {
-  return D.e_cnt[e] + D.blk_off[e / PL_SCAN];
-}
-
-// For every listed edge with probe items, one lane per (edge, end, part):
-// the item -> owning edge map (the edge's six lanes share its items) and the
-// end-sample torque split (end_torque_part's decomposition): three torque
-// evaluations per end replace two per item.  The evaluation is the rolled
-// recursion (torque_at_rolled) of a cubic whose u = 0 sample is the item's
-// (q, qd, qdd), with its coefficients and per-link records in the lane's
-// shared-memory columns: each lane evaluates Eq. (torque) about once, so
-// the one-link body, fetched once, replaces seven unrolled links the
-// instruction cache would fetch cold.  Warps loop in step (every lane of a
-// warp makes the same calls); sized to the resident blocks.
-#define PL_EXP_WARPS 3
-__global__ void __launch_bounds__(32 * PL_EXP_WARPS) k_plan_expand(PlanDev D, ArmK A) {
-  pdl_begin();
-  __shared__ float sCoef[PL_EXP_WARPS][FN_CUBIC_WORDS * 32];
-  __shared__ float sWr[PL_EXP_WARPS][FN_LINK_WORDS * 32];
+  __shared__ float sT[FN_MAX_GRID];
+  __shared__ float sCoef[PL_PR_WARPS][FN_CUBIC_WORDS * 32];
+  __shared__ float sWr[PL_PR_WARPS][FN_LINK_WORDS * 32];
+  __shared__ float sEs[PL_PR_WARPS][PL_PR_EDGES * 32];
+  __shared__ __align__(16) float sSplit[PL_PR_WARPS][PL_PR_EDGES * FN_SPLIT_WORDS];
+  __shared__ uint32_t sBits[PL_PR_WARPS][PL_PR_EDGES * 8];
   __shared__ float4 sLink[7 * FN_LINK_F4];
   fill_links(A, sLink);
+  for (int i = threadIdx.x; i < D.K; i += blockDim.x) sT[i] = Gr.T[i];
   __syncthreads();
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const CubicLane cb{&sCoef[w][lane]};
-  const LaneLink wr{&sWr[w][lane]};
-  const LinkTab L{sLink};
-  const Sched* S = D.sched;
-  const int E = S->n_edges;
-  const int nd = min(S->n_dyn, E);
-  const long n = 6L * nd;
+  const ScalarCore core{LinkTab{sLink}, CubicLane{&sCoef[w][lane]}, LaneLink{&sWr[w][lane]}};
+  float* es = sEs[w];
+  float* split = sSplit[w];
+  uint32_t* bits = sBits[w];
+  Sched* S = D.sched;
+  const int nd = min(S->n_dyn, S->n_edges);
+  const int stride = gridDim.x * PL_PR_WARPS * PL_PR_EDGES;
   unsigned nsamp = 0;
-  const long stride = (long)gridDim.x * blockDim.x;
-  for (long x0 = (long)blockIdx.x * blockDim.x + 32 * w; x0 < n; x0 += stride) {
-    const long x = x0 + lane;
-    const bool act = x < n;
-    const int r = (int)(x % 6), end = r / 3, part = r - 3 * end;
-    Cubic c;
-    float* out = nullptr;
-    c.iT = c.iT2 = 1.f;
-    if (act) {
-      const int e = D.dyn_list[x / 6];
-      const int o = item_off(D, e);
-      const int cnt = (e + 1 < E ? item_off(D, e + 1) : S->n_items) - o;
-      for (int t = r; t < cnt; t += 6) D.owner[o + t] = e;
-      const int p = D.e_ci[e] / D.BM;
-      const float4* r0 = reinterpret_cast<const float4*>(D.st + ((long)p * D.NC + D.e_par[e]) * 16);
-      const float4* r1 = reinterpret_cast<const float4*>(D.cand + (long)D.e_ci[e] * 16);
-      float q0[7], qd0[7], q1[7], qd1[7];
-      load_state(r0, q0, qd0);
-      load_state(r1, q1, qd1);
-      out = D.edyn + (2L * e + end) * 28;
+  for (int x0 = (blockIdx.x * PL_PR_WARPS + w) * PL_PR_EDGES; x0 < nd; x0 += stride) {
+    const int ne = min(PL_PR_EDGES, nd - x0);
+    // lane i < ne: edge i's record
+    const int e = D.dyn_list[x0 + min(lane, ne - 1)];
+    const int ci = D.e_ci[e], par = D.e_par[e], klo = D.e_klo[e], cnt = D.e_cnt[e];
+    const bool goal = D.e_j[e] & 0x80;
+    const float Tp = D.e_Tp[e];
+    const long row0 = (long)(ci / D.BM) * D.NC + par;
+    float v[PL_PR_EDGES];
 #pragma unroll
-      for (int j = 0; j < 7; ++j) {   // end_torque_part's (q, qd, qdd) as a cubic at u = 0
-        const float d = q1[j] - q0[j];
-        const float qa = end ? -6.0f * d : 6.0f * d;
-        const float qb = end ? fmaf(4.0f, qd1[j], 2.0f * qd0[j]) : -fmaf(4.0f, qd0[j], 2.0f * qd1[j]);
-        c.q0[j] = end ? q1[j] : q0[j];
-        c.b1[j] = part == 0 ? (end ? qd1[j] : qd0[j]) : 0.f;
-        c.b2[j] = 0.5f * (part == 0 ? 0.f : (part == 1 ? qa : qb));
-        c.b3[j] = 0.f;
-        if (part == 0) out[21 + j] = c.b1[j];   // the end velocity
-      }
-      ++nsamp;
-    } else {
-#pragma unroll
-      for (int j = 0; j < 7; ++j) c.q0[j] = c.b1[j] = c.b2[j] = c.b3[j] = 0.f;
+    for (int i = 0; i < PL_PR_EDGES; ++i) {
+      const long r0 = __shfl_sync(0xffffffffu, row0, i), r1 = __shfl_sync(0xffffffffu, ci, i);
+      v[i] = i < ne ? (lane < 16 ? __ldg(D.st + r0 * 16 + lane) : __ldg(D.cand + r1 * 16 + lane - 16))
+                    : 0.f;
     }
-    cb.store(c);
-    const float on = part == 0 ? 1.f : 0.f;   // parts 1, 2: M + I_m only
-    const int o = part == 0 ? 14 : 7 * (part - 1);
-    torque_at_rolled(
-        A, L, cb, 0.f,
-        [&](int j, float tau, float, float) {
-          if (act) out[o + j] = tau;
-        },
-        wr, on, on);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < PL_PR_EDGES; ++i) es[32 * i + lane] = v[i];
+    if (lane < PL_PR_EDGES * 8) bits[lane] = 0u;
+    if (lane < PL_PR_EDGES * 8 - 32) bits[32 + lane] = 0u;
+    __syncwarp();
+    split_group(A, core, es, split, ne, nsamp);
+    for (int i = 0; i < ne; ++i) {
+      const int k0 = __shfl_sync(0xffffffffu, klo, i);
+      const int k1 = k0 + __shfl_sync(0xffffffffu, cnt, i);
+      const bool gl = __shfl_sync(0xffffffffu, (int)goal, i) != 0;
+      const float Tg = __shfl_sync(0xffffffffu, Tp, i);
+      for (int b = k0 & ~31; b < k1; b += 32) {
+        const int k = b + lane;
+        const bool in = k >= k0 && k < k1;
+        bool f0;
+        const bool pass =
+            in && end_probe_pass(A, split + FN_SPLIT_WORDS * i, gl ? Tg : sT[in ? k : k0], f0);
+        const unsigned m = __ballot_sync(0xffffffffu, pass);
+        if (lane == 0 && m) bits[8 * i + (b >> 5)] = m;
+      }
+    }
+    __syncwarp();
+    // the masks, and the survivors in one append
+    const uint32_t m0 = bits[lane], m1 = lane < PL_PR_EDGES * 8 - 32 ? bits[32 + lane] : 0u;
+    const int e0 = __shfl_sync(0xffffffffu, e, lane >> 3), e1 = __shfl_sync(0xffffffffu, e, 4);
+    if ((lane >> 3) < ne && m0) D.mask[8L * e0 + (lane & 7)] = m0;
+    if (m1) D.mask[8L * e1 + lane] = m1;
+    const int n0 = __popc(m0), n = n0 + __popc(m1);
+    int at = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, at, o);
+      if (lane >= o) at += y;
+    }
+    const int tot = __shfl_sync(0xffffffffu, at, 31);
+    if (tot == 0) continue;                       // warp-uniform
+    int first = 0;
+    if (lane == 0) first = atomicAdd(&S->n_surv, tot);
+    at += __shfl_sync(0xffffffffu, first, 0) - n;
+    for (uint32_t m = m0; m; m &= m - 1u, ++at)
+      if (at < D.surv_cap) D.surv[at] = make_int2(e0, 32 * (lane & 7) + __ffs(m) - 1);
+    for (uint32_t m = m1; m; m &= m - 1u, ++at)
+      if (at < D.surv_cap) D.surv[at] = make_int2(e1, 32 * lane + __ffs(m) - 1);
   }
   // one counter update per warp (tens of thousands of same-address atomics
   // from single lanes would serialise at the L2)
-  const unsigned tot = __reduce_add_sync(0xffffffffu, nsamp);
-  if (D.samples && lane == 0 && tot) atomicAdd(D.samples + 0, (unsigned long long)tot);
+  if (D.samples && lane == 0 && nsamp) atomicAdd(D.samples + 0, (unsigned long long)nsamp);
 }
 
-static int expand_blocks() {
-  static int blocks[64] = {0};   // per device: resident blocks of k_plan_expand
+static int probe_blocks() {
+  static int blocks[64] = {0};   // per device: resident blocks of k_plan_probe
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev < 0 || dev >= 64) dev = 0;
   if (blocks[dev] == 0) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plan_expand, 32 * PL_EXP_WARPS,
-                                                      0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_plan_probe, 32 * PL_PR_WARPS, 0) !=
+            cudaSuccess ||
         per_sm < 1)
       per_sm = 1;
     blocks[dev] = per_sm * num_sms();
@@ -965,64 +943,14 @@ static int expand_blocks() {
   return blocks[dev];
 }
 
-// Probe: one lane per (edge, grid duration) item checks both end samples
-// (u = 0, u = 1) from the edge's end-sample torque split: tau = alpha / T^2
-// + beta / T + gamma per joint, then rho_tau and rho_P at the end velocity;
-// a duration whose ends pass is marked in the edge's survivor mask.  Goal
-// edges have one item: their fixed duration.
-template <int MINB>
-__global__ void __launch_bounds__(32 * PL_EDGE_WARPS, MINB) k_plan_probe(PlanDev D, ArmK A,
-                                                                         GridKP Gr) {
-  pdl_begin();
-  __shared__ float sT[FN_MAX_GRID];
-  for (int i = threadIdx.x; i < D.K; i += blockDim.x) sT[i] = Gr.T[i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const Sched* S = D.sched;
-  const int n_items = S->n_items;
-  const long W = (long)gridDim.x * PL_EDGE_WARPS;
-  for (long c = (long)blockIdx.x * PL_EDGE_WARPS + w; c * 32 < n_items; c += W) {
-    const int i = (int)(c * 32) + lane;
-    const bool live = i < n_items;
-    int e = 0, k = 0;
-    bool pass = live;
-    if (live) {
-      e = D.owner[i];
-      k = D.e_klo[e] + (i - item_off(D, e));
-      const bool goal = D.e_j[e] & 0x80;
-      const float T = goal ? D.e_Tp[e] : sT[k];
-      const float iT = 1.0f / T, iT2 = iT * iT;
+// an edge's two states, as stage_rows lays them out, in eight 16-byte loads
+__device__ __forceinline__ void load_rows(const float* row0, const float* row1, float (&es)[32]) {
 #pragma unroll
-      for (int end = 0; end < 2; ++end) {
-        const float4* c4 = reinterpret_cast<const float4*>(D.edyn) + (2L * e + end) * 7;
-        float f[28];
-#pragma unroll
-        for (int v = 0; v < 7; ++v) {
-          const float4 t = __ldg(c4 + v);
-          f[4 * v] = t.x; f[4 * v + 1] = t.y; f[4 * v + 2] = t.z; f[4 * v + 3] = t.w;
-        }
-        float r = 0.f, pw = 0.f;
-#pragma unroll
-        for (int j = 0; j < 7; ++j) {
-          const float tau = fmaf(f[j], iT2, fmaf(f[7 + j], iT, f[14 + j]));
-          r = fmaxf(r, fabsf(tau) * A.inv_tau[j]);
-          pw = fmaf(tau, f[21 + j], pw);
-        }
-        pass = pass && r <= 1.f && fabsf(pw) * A.inv_w <= 1.f;
-      }
-    }
-    const unsigned pm = __ballot_sync(0xffffffffu, pass);
-    int slot0 = 0;
-    if (lane == 0 && pm) slot0 = atomicAdd(&D.sched->n_surv, __popc(pm));
-    slot0 = __shfl_sync(0xffffffffu, slot0, 0);
-    if (pass) {
-      // one atomic per mask word among the warp's passing lanes
-      const unsigned grp = __match_any_sync(pm, (unsigned long long)(8L * e + (k >> 5)));
-      const unsigned bits = __reduce_or_sync(grp, 1u << (k & 31));
-      if (lane == __ffs(grp) - 1) atomicOr(&D.mask[8L * e + (k >> 5)], bits);
-      const int slot = slot0 + __popc(pm & ((1u << lane) - 1u));
-      if (slot < D.surv_cap) D.surv[slot] = make_int2(e, k);
-    }
+  for (int m = 0; m < 4; ++m) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(row0) + m);
+    const float4 b = __ldg(reinterpret_cast<const float4*>(row1) + m);
+    es[4 * m] = a.x; es[4 * m + 1] = a.y; es[4 * m + 2] = a.z; es[4 * m + 3] = a.w;
+    es[16 + 4 * m] = b.x; es[17 + 4 * m] = b.y; es[18 + 4 * m] = b.z; es[19 + 4 * m] = b.w;
   }
 }
 
@@ -1058,11 +986,8 @@ __global__ void __launch_bounds__(32 * PL_EDGE_WARPS, MINB) k_plan_mprobe(PlanDe
       const bool goal = D.e_j[e] & 0x80;
       const float T = goal ? D.e_Tp[e] : sT[k];
       const int p = D.e_ci[e] / D.BM;
-      const float* r0 = D.st + ((long)p * D.NC + D.e_par[e]) * 16;
-      const float* r1 = D.cand + (long)D.e_ci[e] * 16;
       float es[32];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) { es[m] = __ldg(r0 + m); es[16 + m] = __ldg(r1 + m); }
+      load_rows(D.st + ((long)p * D.NC + D.e_par[e]) * 16, D.cand + (long)D.e_ci[e] * 16, es);
       Cubic cc;
       cubic_coef_sh<false>(es, T, cc);
       cb.store(cc);
@@ -1097,10 +1022,9 @@ __global__ void k_plan_vinit(PlanDev D) {
   pdl_begin();
   Sched* S = D.sched;
   const int E = S->n_edges;
-  if (blockIdx.x == 0 && threadIdx.x == 0) S->n_dyn = 0;   // the expand consumed the list
+  if (blockIdx.x == 0 && threadIdx.x == 0) S->n_dyn = 0;   // the probe consumed the list
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < E; e += gridDim.x * blockDim.x) {
-    const int c = (e + 1 < E ? item_off(D, e + 1) : S->n_items) - item_off(D, e);
-    if (c == 0) continue;   // decided in prep
+    if (D.e_cnt[e] == 0) continue;   // decided in prep
     const int k = next_survivor(D, e, 0);
     D.fail[e] = 0u;
     if (k < 0) {
@@ -1152,11 +1076,8 @@ __global__ void __launch_bounds__(32 * PL_EDGE_WARPS, MINB) k_plan_vstage(PlanDe
       const bool goal = D.e_j[e] & 0x80;
       const float T = goal ? D.e_Tp[e] : sT[D.cur_k[e]];
       const int p = D.e_ci[e] / D.BM;
-      const float* r0 = D.st + ((long)p * D.NC + D.e_par[e]) * 16;
-      const float* r1 = D.cand + (long)D.e_ci[e] * 16;
       float es[32];
-#pragma unroll
-      for (int m = 0; m < 16; ++m) { es[m] = __ldg(r0 + m); es[16 + m] = __ldg(r1 + m); }
+      load_rows(D.st + ((long)p * D.NC + D.e_par[e]) * 16, D.cand + (long)D.e_ci[e] * 16, es);
       Cubic cc;
       cubic_coef_sh<true>(es, T, cc);
       cb.store(cc);
@@ -2751,13 +2672,6 @@ static fn_status pl_alloc_n(fn_planner* pl, T** p, size_t n) {
 }
 
 typedef void (*PlanEdgeKernel)(PlanDev, ArmK, GridKP);
-static PlanEdgeKernel plan_probe_variant(int v) {
-  switch (v) {
-    case 0: return k_plan_probe<2>;
-    case 1: return k_plan_probe<3>;
-    default: return k_plan_probe<4>;
-  }
-}
 static PlanEdgeKernel plan_mprobe_variant(int v) {
   switch (v) {
     case 0: return k_plan_mprobe<2>;
@@ -2802,7 +2716,7 @@ static int resident_stage(PlanStageKernel k) {
 
 static int plan_edge_blocks(fn_planner* pl, int v) {
   (void)pl;
-  return std::min(resident(plan_probe_variant(v)),
+  return std::min(resident(plan_mprobe_variant(v)),
                   std::min(resident_stage(plan_vstage_variant(v)),
                            resident_stage(plan_vseq_variant(v))));
 }
@@ -2962,20 +2876,14 @@ static int vstages(const PlanDev& D) {
   return D.vstages >= 2 ? 2 : (D.goal_split ? PL_VSTAGES_SMALL : 1);
 }
 
-// the packed edge phase after the per-edge prep: item scan, probe, verify
+// the packed edge phase after the per-edge prep: split and probe, verify
 // (over the edges of the view D; mark(i) records the phase boundaries when
 // timing)
 template <class Mark>
 static void enqueue_edge_body(fn_planner* pl, const PlanDev& D, int v, int blocks, cudaStream_t st,
-                              Mark&& mark, bool scan = true) {
-  if (scan) {   // k_plan_eprep scans the block totals itself
-    pl_launch(k_plan_escan, 1, PL_SCAN, 0, st, D);
-    trace(pl, st, "k_plan_escan");
-  }
-  pl_launch(k_plan_expand, expand_blocks(), 32 * PL_EXP_WARPS, 0, st, D, pl->arm);
-  trace(pl, st, "k_plan_expand");
+                              Mark&& mark) {
   mark(4);
-  pl_launch(plan_probe_variant(v), blocks, 32 * PL_EDGE_WARPS, 0, st, D, pl->arm, pl->grid);
+  pl_launch(k_plan_probe, probe_blocks(), 32 * PL_PR_WARPS, 0, st, D, pl->arm, pl->grid);
   trace(pl, st, "k_plan_probe");
   pl_launch(plan_mprobe_variant(v), blocks, 32 * PL_EDGE_WARPS, 0, st, D, pl->arm, pl->grid);
   trace(pl, st, "k_plan_mprobe");
@@ -3017,7 +2925,7 @@ static void enqueue_edges(fn_planner* pl, int v, int blocks, cudaStream_t st, Ma
     mark(5);
     return;
   }
-  enqueue_edge_body(pl, D, v, blocks, st, mark, false);
+  enqueue_edge_body(pl, D, v, blocks, st, mark);
 }
 
 extern "C" fn_status fn_planner_destroy(fn_planner_t* pl) {
@@ -3116,11 +3024,8 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
   A_(D.e_ci, (size_t)D.Emax); A_(D.e_par, (size_t)D.Emax); A_(D.e_Tp, (size_t)D.Emax);
   A_(D.e_klo, (size_t)D.Emax);
   A_(D.e_j, (size_t)D.Emax); A_(D.e_cnt, (size_t)D.Emax);
-  A_(D.blk_off, (size_t)(D.Emax + PL_SCAN - 1) / PL_SCAN + 1);
   A_(D.mask, (size_t)D.Emax * 8);
   D.Kmax = c.K;
-  A_(D.owner, (size_t)D.Emax * c.K);
-  A_(D.edyn, (size_t)D.Emax * 56);
   A_(D.dyn_list, (size_t)D.Emax);
   A_(D.cur_k, (size_t)D.Emax);
   A_(D.fail, (size_t)D.Emax);
@@ -3810,9 +3715,9 @@ __global__ void __launch_bounds__(PL_SCAN) k_edges_prep(PlanDev D, GridKP Gr, in
                                                         int2* __restrict__ win) {
   pdl_begin();
   __shared__ float sT[FN_MAX_GRID];
-  __shared__ int sh[32];
   for (int i = threadIdx.x; i < D.K; i += blockDim.x) sT[i] = Gr.T[i];
   __syncthreads();
+  clear_body_lists(D.sched);
   const int n = n_list ? min(*n_list, E) : E;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     D.sched->n_edges = n;
@@ -3853,6 +3758,7 @@ __global__ void __launch_bounds__(PL_SCAN) k_edges_prep(PlanDev D, GridKP Gr, in
     D.e_Tp[e] = c;
     D.e_j[e] = 0;
     D.e_klo[e] = klo;
+    D.e_cnt[e] = cnt;
 #pragma unroll
     for (int w = 0; w < 8; ++w) D.mask[8L * e + w] = 0u;
     if (cnt == 0) {
@@ -3863,10 +3769,6 @@ __global__ void __launch_bounds__(PL_SCAN) k_edges_prep(PlanDev D, GridKP Gr, in
     }
   }
   list_dyn_edge(D, e, e < n && cnt > 0);
-  int tot;
-  const int ex = block_scan(cnt, sh, &tot);
-  if (e < n) D.e_cnt[e] = ex;
-  if (threadIdx.x == 0) D.blk_off[blockIdx.x] = tot;
 }
 
 // Window certificate (exact under monotone rho_tau, rho_P): the first
