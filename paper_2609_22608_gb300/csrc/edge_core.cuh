@@ -189,7 +189,9 @@ __device__ __forceinline__ unsigned lowest_bits(unsigned x, int n) {
 // eval() is called by every lane of the warp (tensor-memory records are
 // warp-collective); sink(j, tau, qd, 1 / tau_max_j) gets pairs, whose .y
 // half is meaningful only for NS = 2; gs, fs scale gravity and friction per
-// half.  store2 gives the halves different cubics (the scalar core keeps x).
+// half; back: lanes from the column of the lane's cubic (0: its own; see
+// cubic_store_shared).  store2 gives the halves different cubics (the scalar
+// core keeps x).
 struct ScalarCore {
   static constexpr int NS = 1;
   LinkTab L;
@@ -198,10 +200,10 @@ struct ScalarCore {
   __device__ __forceinline__ void store(const Cubic& c) const { cb.store(c); }
   __device__ __forceinline__ void store2(const Cubic& cx, const Cubic&) const { cb.store(cx); }
   template <class Sink>
-  __device__ __forceinline__ void eval(const ArmK& A, float2 u, float2 gs, float2 fs,
-                                       Sink&& sink) const {
+  __device__ __forceinline__ void eval(const ArmK& A, float2 u, float2 gs, float2 fs, Sink&& sink,
+                                       int back = 0) const {
     torque_at_rolled(
-        A, L, cb, u.x,
+        A, L, cb.back(back), u.x,
         [&](int j, float tau, float v, float inv_tau) {
           sink(j, make_float2(tau, 0.f), make_float2(v, 0.f), inv_tau);
         },
@@ -220,9 +222,9 @@ struct PairCore {
     cb.store2(cx, cy);
   }
   template <class Sink>
-  __device__ __forceinline__ void eval(const ArmK& A, float2 u, float2 gs, float2 fs,
-                                       Sink&& sink) const {
-    torque_at_pair(A, L, cb, u, sink, st, gs, fs);
+  __device__ __forceinline__ void eval(const ArmK& A, float2 u, float2 gs, float2 fs, Sink&& sink,
+                                       int back = 0) const {
+    torque_at_pair(A, L, cb.back(back), u, sink, st, gs, fs);
   }
 };
 
@@ -349,6 +351,7 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
   unsigned sel = 0u;    // PROBE_MID: the durations being probed
   float mt = 0.f, mp = 0.f;
   bool bad = false;
+  int back = 0;         // lanes from the column that holds this lane's cubic
   bool w_pending = wmode == 2 && w_in > 0 && w_in < S - 1;   // interior witness of the caller
   const int cap = scan_pass_cap(fixed ? 1 : max(Kadm - k_begin, 1), S);
   int passes = 0;
@@ -366,23 +369,25 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
   for (;;) {
     if (++passes > cap) return FN_SCAN_ABORT;   // warp-uniform
     if (coef != COEF_NONE) {           // the single coefficient-build site
-      Cubic c;
-      if (coef == COEF_SPLIT) {
-        // lane l < 6: end l / 3, part l % 3
-        const int end = lane >= 3 ? 1 : 0;
-        split_cubic(es, end, lane - 3 * end, c);
-      } else if (coef == COEF_PLAIN) {
-        if (cdur >= 0) {
-          cubic_coef_sh<false>(es, sT[cdur], c);
-        } else {                       // an idle lane: any finite cubic
-          c.iT = c.iT2 = 1.f;
-#pragma unroll
-          for (int j = 0; j < 7; ++j) c.q0[j] = c.b1[j] = c.b2[j] = c.b3[j] = 0.f;
-        }
+      if (coef == COEF_EXACT) {        // one duration for the whole warp
+        cubic_store_shared<true>(core.cb, es, fixed ? Tfix : sT[kk], 32);
+        back = lane;
+      } else if (coef == COEF_PLAIN && packed) {   // one for four lanes (idle ones: any)
+        cubic_store_shared<false>(core.cb, es, cdur >= 0 ? sT[cdur] : 1.f, 4);
+        back = lane & 3;
       } else {
-        cubic_coef_sh<true>(es, fixed ? Tfix : sT[kk], c);
+        Cubic c;
+        if (coef == COEF_SPLIT) {
+          // lane l < 6: end l / 3, part l % 3
+          const int end = lane >= 3 ? 1 : 0;
+          split_cubic(es, end, lane - 3 * end, c);
+        } else {
+          cubic_coef_sh<false>(es, cdur >= 0 ? sT[cdur] : 1.f, c);   // idle lanes: any
+        }
+        __syncwarp();                  // shared columns may still be read
+        core.store(c);
+        back = 0;
       }
-      core.store(c);
       coef = COEF_NONE;
     }
     bool decide = false;  // choose the next step from (cand, mpr)
@@ -444,7 +449,7 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
           ry = fmaxf(ry, fabsf(tau.y) * inv_tau);
           py = fmaf(tau.y, v.y, py);
         }
-      });
+      }, back);
       const float bx = fabsf(px) * A.inv_w, by = fabsf(py) * A.inv_w;
       const bool pass_x = ax && rx <= 1.f && bx <= 1.f;
       const bool pass_y = ay && ry <= 1.f && by <= 1.f;

@@ -170,6 +170,8 @@ struct CubicLane {
     p[32 * 28] = c.iT;
     p[32 * 29] = c.iT2;
   }
+  __device__ __forceinline__ void put(int f, float v) const { p[32 * f] = v; }
+  __device__ __forceinline__ CubicLane back(int lanes) const { return CubicLane{p - lanes}; }
 };
 
 __device__ __forceinline__ void cubic_eval(const CubicLane& c, int j, float u, float& q, float& v,
@@ -488,6 +490,13 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 __device__ __forceinline__ float2 lo2(float4 v) { return make_float2(v.x, v.y); }
 __device__ __forceinline__ float2 hi2(float4 v) { return make_float2(v.z, v.w); }
 
+// a b + c d with three roundings: the assembler contracts a mul2 into the
+// add2 that follows it, the scalar forms it leaves as they are
+__device__ __forceinline__ float2 sum2(float2 a, float2 b, float2 c, float2 d) {
+  return make_float2(__fadd_rn(__fmul_rn(a.x, b.x), __fmul_rn(c.x, d.x)),
+                     __fadd_rn(__fmul_rn(a.y, b.y), __fmul_rn(c.y, d.y)));
+}
+
 // a x b - the pair form of the scalar cross products (a_y b_z - a_z b_y, ...)
 __device__ __forceinline__ void cross2(float2 ax, float2 ay, float2 az, float2 bx, float2 by,
                                        float2 bz, float2& cx, float2& cy, float2& cz) {
@@ -564,27 +573,57 @@ struct CubicLane2 {
     p[32 * 28] = make_float2(cx.iT, cy.iT);
     p[32 * 29] = make_float2(cx.iT2, cy.iT2);
   }
+  __device__ __forceinline__ void put(int f, float v) const { p[32 * f] = make_float2(v, v); }
+  __device__ __forceinline__ CubicLane2 back(int lanes) const { return CubicLane2{p - lanes}; }
 };
+
+// One cubic for a group of `width` lanes (4 or 32, aligned): each lane builds
+// its share of the joints' coefficients into the column of the group's first
+// lane, from which all of them then read (cb.back(lane in group)).  A check
+// of one duration by the whole warp built the same seven joints on every
+// lane: 250 of the 2463 instructions of its pass.
+template <bool ACC, class CB>
+__device__ __forceinline__ void cubic_store_shared(const CB& cb, const float* es, float T,
+                                                   int width) {
+  const int r = threadIdx.x & (width - 1);
+  const CB c = cb.back(r);
+  __syncwarp();   // the column's last readers are done
+  for (int j = r; j < 8; j += width) {
+    if (j == 7) {
+      const float iT = 1.0f / T;
+      c.put(28, iT);
+      c.put(29, iT * iT);
+    } else {
+      float b1, b2, b3;
+      joint_coef<ACC>(es[j], es[8 + j], es[16 + j], es[24 + j], T, b1, b2, b3);
+      c.put(j, es[j]);
+      c.put(7 + j, b1);
+      c.put(14 + j, b2);
+      c.put(21 + j, b3);
+    }
+  }
+  __syncwarp();
+}
 
 // sink(j, tau_j, qd_j, 1 / tau_max_j) in the inward order j = 6..0, tau_j and
 // qd_j as pairs; gs, fs: per-half gravity and friction scales.  Stash:
 // store(j, rec) / stored() / load(j, rec) (LaneLink2, or a tensor-memory
 // column block); every lane of the warp must call this.
+// The first link outward (w = dw = 0 below it), the last one (its record
+// stays in registers) and the first one inward (only its torque is wanted)
+// stand outside the loops: a tenth of the recursion's operations.
 template <class Sink, class Stash>
 __device__ __forceinline__ void torque_at_pair(const ArmK& A, LinkTab2 L, CubicLane2 c, float2 u,
                                                Sink&& sink, Stash W, float2 gs = {1.f, 1.f},
                                                float2 fs2 = {1.f, 1.f}) {
-  float2 wx = dup2(0.f), wy = dup2(0.f), wz = dup2(0.f);
-  float2 dwx = dup2(0.f), dwy = dup2(0.f), dwz = dup2(0.f);
+  float2 wx = dup2(0.f), wy = dup2(0.f), wz, dwx = dup2(0.f), dwy = dup2(0.f), dwz;
   float2 ax = mul2(dup2(A.g0x), gs), ay = mul2(dup2(A.g0y), gs), az = mul2(dup2(A.g0z), gs);
   const float2 iT = c.iT(), iT2 = c.iT2();
-#pragma unroll 1
-  for (int j = 0; j < 7; ++j) {
-    const float4* t = L.p + FN_LINK2_F4 * j;
-    const float4 t0 = t[0], t1 = t[1], t2 = t[2], t3 = t[3], t4 = t[4];
-    const float4 t5 = t[5], t6 = t[6], t7 = t[7], t8 = t[8];
-    const float2 ca = lo2(t0), sa = hi2(t0), px = lo2(t1), py = hi2(t1), pz = lo2(t2);
-    float2 rec[FN_REC2];
+  float2 rec[FN_REC2];
+  // joint j's motion: cos, sin, velocity and armature + friction into the
+  // record; the acceleration is returned
+  auto motion = [&](int j, const float4* t) {
+    const float4 t2 = t[2], t6 = t[6], t7 = t[7], t8 = t[8];
     // sigma, sigma_dot, sigma_ddot at both samples
     const float2 b1 = c.b1(j), b2 = c.b2(j), b3 = c.b3(j), tb2 = add2(b2, b2);
     const float2 q = fma2(fma2(fma2(b3, u, b2), u, b1), u, c.q0(j));
@@ -599,14 +638,38 @@ __device__ __forceinline__ void torque_at_pair(const ArmK& A, LinkTab2 L, CubicL
     const float2 rc = make_float2(fn_rcp(1.0f + ex), fn_rcp(1.0f + ey));
     rec[9] = fma2(hi2(t6), acc, mul2(fs2, fma2(lo2(t7), rc, neg2(hi2(t8)))));
     rec[8] = v;
-    float2 s_, c_;
-    {
-      const float2 th = add2(q, hi2(t2));
-      fn_sincos(th.x, &s_.x, &c_.x);
-      fn_sincos(th.y, &s_.y, &c_.y);
-    }
-    rec[6] = c_;
-    rec[7] = s_;
+    const float2 th = add2(q, hi2(t2));
+    fn_sincos(th.x, &rec[7].x, &rec[6].x);
+    fn_sincos(th.y, &rec[7].y, &rec[6].y);
+    return acc;
+  };
+  {   // link 1
+    const float4* t = L.p;
+    const float4 t0 = t[0], t3 = t[3], t4 = t[4], t6 = t[6];
+    const float2 acc = motion(0, t), v = rec[8], c_ = rec[6], s_ = rec[7];
+    const float2 ca = lo2(t0), sa = hi2(t0);
+    const float2 r1 = fma2(ca, ay, mul2(sa, az)), r2 = fma2(neg2(sa), ay, mul2(ca, az));
+    const float2 ux = ax;
+    ax = fma2(c_, ux, mul2(s_, r1));
+    ay = fma2(neg2(s_), ux, mul2(c_, r1));
+    az = r2;
+    wz = v;
+    dwz = acc;
+    const float2 cx = hi2(t3), cy = lo2(t4), m = lo2(t3), Iz = lo2(t6);
+    const float2 wcx = neg2(mul2(wz, cy)), wcy = mul2(wz, cx);
+    rec[0] = mul2(m, add2(neg2(sum2(dwz, cy, wz, wcy)), ax));
+    rec[1] = mul2(m, add2(sum2(dwz, cx, wz, wcx), ay));
+    rec[2] = rec[3] = rec[4] = dup2(0.f);   // (F_z, N_x, N_y of link 1 are not read)
+    rec[5] = mul2(Iz, dwz);
+    W.store(0, rec);
+  }
+#pragma unroll 1
+  for (int j = 1; j < 7; ++j) {
+    const float4* t = L.p + FN_LINK2_F4 * j;
+    const float4 t0 = t[0], t1 = t[1], t2 = t[2], t3 = t[3], t4 = t[4];
+    const float4 t5 = t[5], t6 = t[6];
+    const float2 ca = lo2(t0), sa = hi2(t0), px = lo2(t1), py = hi2(t1), pz = lo2(t2);
+    const float2 acc = motion(j, t), v = rec[8], c_ = rec[6], s_ = rec[7];
     // u = dw_prev x p + w_prev x (w_prev x p) + dv_prev   (frame j-1)
     float2 tx, ty, tz, gx, gy, gz, hx, hy, hz;
     cross2(wx, wy, wz, px, py, pz, tx, ty, tz);
@@ -648,19 +711,26 @@ __device__ __forceinline__ void torque_at_pair(const ArmK& A, LinkTab2 L, CubicL
     rec[3] = fma2(Ix, dwx, kx);
     rec[4] = fma2(Iy, dwy, ky);
     rec[5] = fma2(Iz, dwz, kz);
-    W.store(j, rec);
+    if (j < 6) W.store(j, rec);
   }
   W.stored();
-  float2 fx = dup2(0.f), fy = dup2(0.f), fz = dup2(0.f);
-  float2 nx = dup2(0.f), ny = dup2(0.f), nz = dup2(0.f);
-  float2 cn = dup2(1.f), sn = dup2(0.f);   // cos, sin of joint j + 1 (any value for j = 6)
+  float2 fx, fy, fz, nx, ny, nz;
+  {   // link 7: no wrench beyond it
+    const float4* m = L.p + FN_LINK2_F4 * 6;
+    const float4 m3 = m[3], m4 = m[4];
+    cross2(hi2(m3), lo2(m4), hi2(m4), rec[0], rec[1], rec[2], nx, ny, nz);
+    fx = rec[0]; fy = rec[1]; fz = rec[2];
+    nx = add2(rec[3], nx);
+    ny = add2(rec[4], ny);
+    nz = add2(rec[5], nz);
+    sink(6, add2(nz, rec[9]), rec[8], m[9].x);
+  }
+  float2 cn = rec[6], sn = rec[7];   // cos, sin of joint j + 1
 #pragma unroll 1
-  for (int j = 6; j >= 0; --j) {
-    float2 rec[FN_REC2];
+  for (int j = 5; j > 0; --j) {
     W.load(j, rec);
-    // R_{j+1} (f, n) and p_{j+1} x R_{j+1} f; zero for the last link (f = n = 0)
-    const int jc = j < 6 ? j + 1 : 6;
-    const float4* t = L.p + FN_LINK2_F4 * jc;
+    // R_{j+1} (f, n) and p_{j+1} x R_{j+1} f
+    const float4* t = L.p + FN_LINK2_F4 * (j + 1);
     const float4 k0 = t[0], k1 = t[1], k2 = t[2];
     const float2 ca = lo2(k0), sa = hi2(k0), nsa = neg2(sa), ns = neg2(sn);
     float2 u0 = fma2(cn, fx, mul2(ns, fy)), u1 = fma2(sn, fx, mul2(cn, fy)), u2 = fz;
@@ -680,6 +750,21 @@ __device__ __forceinline__ void torque_at_pair(const ArmK& A, LinkTab2 L, CubicL
     cn = rec[6];
     sn = rec[7];
     sink(j, add2(nz, rec[9]), rec[8], m[9].x);
+  }
+  {   // link 1: its torque only
+    W.load(0, rec);
+    const float4* t = L.p + FN_LINK2_F4;
+    const float4 k0 = t[0], k1 = t[1];
+    const float2 ca = lo2(k0), sa = hi2(k0), nsa = neg2(sa), ns = neg2(sn);
+    float2 u1 = fma2(sn, fx, mul2(cn, fy));
+    const float2 Rfx = fma2(cn, fx, mul2(ns, fy)), Rfy = fma2(ca, u1, mul2(nsa, fz));
+    u1 = fma2(sn, nx, mul2(cn, ny));
+    const float2 Rnz = fma2(sa, u1, mul2(ca, nz));
+    const float2 pRz = fma2(lo2(k1), Rfy, neg2(mul2(hi2(k1), Rfx)));
+    const float4 m3 = L.p[3], m4 = L.p[4];
+    const float2 cFz = fma2(hi2(m3), rec[1], neg2(mul2(lo2(m4), rec[0])));
+    nz = add2(add2(add2(rec[5], Rnz), cFz), pRz);
+    sink(0, add2(nz, rec[9]), rec[8], L.p[9].x);
   }
 }
 

@@ -329,7 +329,8 @@ __device__ __forceinline__ bool ik_solve_group(const ArmK& A, const float* Rg, c
 // frames are formed by the products of the group form's scan (each in its
 // order, those that nothing reads left out), and each half's arithmetic is
 // the group form's, rounding for rounding: the same starts converge to the
-// same bits.  33 thousand goals: XX us.
+// same bits.  33 thousand goals: 113 us; 1024 goals (64 warps, one to an
+// SM): 37 us either way, the chain of one warp.
 // ---------------------------------------------------------------------------
 #define FN_IK_TAB_F4 4
 struct IkTab {

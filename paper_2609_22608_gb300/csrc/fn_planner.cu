@@ -837,8 +837,9 @@ __global__ void __launch_bounds__(PL_SCAN) k_plan_eprep(PlanDev D, GridKP Gr) {
 // duration) item: a map from item to edge, a scan of the item counts, the
 // split's 224 bytes an edge through memory, and an atomic on one counter per
 // 32 items, each behind the last's latency.  65 thousand edges (anytime
-// loop): 34 + 129 us before, XX now; 130 thousand (64 problems) 75 + 149,
-// XX now.
+// loop): 34 + 129 us before, 77 now; 130 thousand (64 problems) 73 + 157,
+// 168 now (785 thousand torque evaluations are some 95 of them at the scalar
+// recursion's rate).
 #define PL_PR_WARPS 3
 #define PL_PR_EDGES 5
 __global__ void __launch_bounds__(32 * PL_PR_WARPS) k_plan_probe(PlanDev D, ArmK A, GridKP Gr) {
@@ -1278,30 +1279,27 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_goal_edges(PlanDev D,
       gs = __shfl_sync(0xffffffffu, gs, 0);
       if (g0 >= nl) break;                           // warp-uniform
       const int n = min(gs, nl - g0);
-      long my_ei = 0;
-      int my_p = 0;
-      float my_Tp = 0.f;
-      for (int i = 0; i < n; ++i) {
-        const GoalEdge g = decode_goal_edge(D, S, list[g0 + i]);
-        stage_rows(D.st + ((long)g.p * D.NC + g.pr) * 16, D.cand + g.ci * 16, es_g + 32 * i);
-        if (lane == i) { my_ei = g.ei; my_p = g.p; my_Tp = g.Tp; }
+      // lane i < n decodes edge i; the rows of all come in together
+      const GoalEdge mine = decode_goal_edge(D, S, list[g0 + min(lane, n - 1)]);
+      const long my_ei = mine.ei, my_row = (long)mine.p * D.NC + mine.pr, my_ci = mine.ci;
+      const int my_p = mine.p;
+      const float my_Tp = mine.Tp;
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const long r0 = __shfl_sync(0xffffffffu, my_row, i), r1 = __shfl_sync(0xffffffffu, my_ci, i);
+        v[i] = i < n ? __ldg(lane < 16 ? D.st + r0 * 16 + lane : D.cand + r1 * 16 + lane - 16) : 0.f;
       }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) es_g[32 * i + lane] = v[i];
+      __syncwarp();
       unsigned probed = n > 1 ? 0u : 1u;   // a lone edge goes straight to its check
       if (n > 1) {
         const int q = lane >> 2;
         const bool act = q < n;
         const float T = __shfl_sync(0xffffffffu, my_Tp, act ? q : 0);
-        {
-          Cubic c;
-          if (act) {
-            cubic_coef_sh<true>(es_g + 32 * q, T, c);
-          } else {                                   // an idle lane: any finite cubic
-            c.iT = c.iT2 = 1.f;
-#pragma unroll
-            for (int m = 0; m < 7; ++m) c.q0[m] = c.b1[m] = c.b2[m] = c.b3[m] = 0.f;
-          }
-          core.store(c);
-        }
+        cubic_store_shared<true>(core.cb, es_g + 32 * (act ? q : 0), T, 4);
         const float2 u = make_float2(sample_u(goal_probe_index(lane & 3, D.S), D.S),
                                      sample_u(goal_probe_index((lane & 3) + 4, D.S), D.S));
         float rx = 0.f, px = 0.f, ry = 0.f, py = 0.f;
@@ -1310,7 +1308,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_goal_edges(PlanDev D,
           px = fmaf(tau.x, v.x, px);
           ry = fmaxf(ry, fabsf(tau.y) * inv_tau);
           py = fmaf(tau.y, v.y, py);
-        });
+        }, lane & 3);
         const bool okl = act && rx <= 1.f && fabsf(px) * A.inv_w <= 1.f && ry <= 1.f &&
                          fabsf(py) * A.inv_w <= 1.f;
         const unsigned ok = __ballot_sync(0xffffffffu, okl);

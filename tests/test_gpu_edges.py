@@ -223,3 +223,19 @@ def test_full_size_sampled(ops, orc, arm):
     ref = orc.time_edges(arm, s0[sel], s1[sel], grid, 64)
     bad = kstar_mismatches(orc, arm, s0[sel], s1[sel], grid, 64, k[sel], ref["k_star"])
     assert not bad
+
+
+@pytest.mark.parametrize("E,S", [(1, 2), (13, 3), (200, 31), (200, 33), (301, 64), (301, 65), (77, 255)])
+def test_paired_check_is_the_scalar_one(arm, E, S):
+    """The fixed-duration check on the paired core (coefficients shared by the
+    warp, first and last link outside its loops) gives the scalar core's
+    ratios bit for bit, whatever part of the last pass of 64 samples is used."""
+    from paper_2609_22608_gb300 import ops
+    s0, s1 = (torch.from_numpy(a).cuda() for a in synth.random_edges(arm, E, 41 + S))
+    T = torch.from_numpy(np.random.default_rng(S).uniform(0.06, 1.8, E).astype(np.float32)).cuda()
+    got = []
+    for v in (2, 3):
+        ops.set_time_edges_variant(1, E, 1, S, v)
+        r = ops.time_edges(arm, s0, s1, S=S, mode=ops.FN_MODE_FIXED, T_fixed=T)
+        got.append({k: x.cpu().numpy().tobytes() for k, x in r.items()})
+    assert got[0] == got[1]
