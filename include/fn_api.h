@@ -872,8 +872,8 @@ fn_status fn_mlp_destroy(fn_mlp_t* m);
 fn_status fn_mlp_predict(fn_mlp_t* m, const fn_arm_t* arm, const float* s0, const float* s1,
                          int E, float* Y, void* stream);
 
-/* The same forward on the training kernels' path (mma.sync GEMMs through
- * the model's workspace, chunks of max_batch).  Same rounding points; the
+/* The same forward layer by layer (one GEMM each through the model's
+ * workspace, chunks of max_batch), the fused kernels' reference.  Same rounding points; the
  * two differ only by FP32 summation order. */
 fn_status fn_mlp_predict_ref(fn_mlp_t* m, const fn_arm_t* arm, const float* s0, const float* s1,
                              int E, float* Y, void* stream);

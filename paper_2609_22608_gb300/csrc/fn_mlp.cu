@@ -10,10 +10,10 @@
 // Adam keeps FP32 master weights and refreshes the bf16 copies after every
 // step.
 //
-// The contractions use mma.sync.m16n8k16 (bf16 in, f32 accumulate) in a
-// tiled 64x64x32 kernel with optional transposed operands, which serves the
-// forward pass (h W), the input gradients (dz W^T) and the weight gradients
-// (h^T dz).
+// Inference and training are fused tcgen05 kernels (fn_mlp_tc.cu,
+// fn_mlp_train.cu); this file holds the reference forward, layer by layer
+// through memory, with the two-column layer 4 on mma.sync.m16n8k16, and the
+// model's state.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -56,10 +56,8 @@ __global__ void k_mlp_features(ArmK A, const float* __restrict__ s0, const float
 }
 
 // ---------------------------------------------------------------------------
-// C (M x N) = act(A (M x K) B (K x N) + bias), bf16 operands, f32 accumulate.
-// A(m, k) = A[m lda + k] (TA: A[k lda + m]); B(k, n) = B[k ldb + n]
-// (TB: B[n ldb + k]).  Outputs: Cf (f32, optionally accumulated) and/or Cb
-// (bf16).  Tiles: 64 x 64 per block, 32 along K; 4 warps of 32 x 32.
+// C (M x N, f32) = A (M x K) B (K x N) + bias, bf16 operands, f32 accumulate.
+// Tiles: 64 x 64 per block, 32 along K; 4 warps of 32 x 32.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint32_t* b) {
   asm volatile(
@@ -69,13 +67,11 @@ __device__ __forceinline__ void mma_bf16(float* d, const uint32_t* a, const uint
       : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-template <bool TA, bool TB>
 __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K,
                                                    const bf16* __restrict__ A, int lda,
                                                    const bf16* __restrict__ B, int ldb,
-                                                   const float* __restrict__ bias, int relu,
-                                                   int accumulate, float* __restrict__ Cf,
-                                                   int ldcf, bf16* __restrict__ Cb, int ldcb) {
+                                                   const float* __restrict__ bias,
+                                                   float* __restrict__ C, int ldc) {
   __shared__ __align__(16) bf16 As[64][40];  // [m][k]
   __shared__ __align__(16) bf16 Bs[64][40];  // [n][k]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -91,19 +87,17 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K,
       for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
   for (int k0 = 0; k0 < K; k0 += 32) {
     for (int t = tid; t < 64 * 32; t += 128) {
-      int r, c;  // (m, k) with the contiguous global index fastest
-      if (TA) { r = t & 63; c = t >> 6; } else { r = t >> 5; c = t & 31; }
+      const int r = t >> 5, c = t & 31;   // (m, k)
       const int gm = m0 + r, gk = k0 + c;
       bf16 v = zero;
-      if (gm < M && gk < K) v = TA ? A[(long)gk * lda + gm] : A[(long)gm * lda + gk];
+      if (gm < M && gk < K) v = A[(long)gm * lda + gk];
       As[r][c] = v;
     }
     for (int t = tid; t < 64 * 32; t += 128) {
-      int r, c;  // (n, k)
-      if (TB) { r = t >> 5; c = t & 31; } else { r = t & 63; c = t >> 6; }
+      const int r = t & 63, c = t >> 6;   // (n, k)
       const int gn = n0 + r, gk = k0 + c;
       bf16 v = zero;
-      if (gn < N && gk < K) v = TB ? B[(long)gn * ldb + gk] : B[(long)gk * ldb + gn];
+      if (gn < N && gk < K) v = B[(long)gk * ldb + gn];
       Bs[r][c] = v;
     }
     __syncthreads();
@@ -144,85 +138,8 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K,
           const int row = m0 + wm * 32 + mi * 16 + g + 8 * h;
           const int col = n0 + wn * 32 + ni * 8 + 2 * tg + cc;
           if (row >= M || col >= N) continue;
-          float v = acc[mi][ni][2 * h + cc] + (bias ? bias[col] : 0.f);
-          if (relu) v = fmaxf(v, 0.f);
-          if (Cf) {
-            float* o = Cf + (long)row * ldcf + col;
-            *o = accumulate ? *o + v : v;
-          }
-          if (Cb) Cb[(long)row * ldcb + col] = __float2bfloat16_rn(v);
+          C[(long)row * ldc + col] = acc[mi][ni][2 * h + cc] + bias[col];
         }
-}
-
-// The training GEMMs with a 256-wide output (and 16-byte aligned rows) run
-// on the tensor cores (tcgen05, gemm_tc); the two-column ones of layer 4 on
-// mma.sync tiles.
-template <bool TA, bool TB>
-static void gemm(int M, int N, int K, const bf16* A, int lda, const bf16* B, int ldb,
-                 const float* bias, bool relu, bool accumulate, float* Cf, int ldcf, bf16* Cb,
-                 int ldcb, int* err, cudaStream_t st) {
-  if (N >= 128 && lda % 8 == 0 && ldb % 8 == 0 && aligned16(A) && aligned16(B)) {
-    gemm_tc<TA, TB>(M, N, K, A, lda, B, ldb, bias, relu, accumulate, Cf, ldcf, Cb, ldcb, err, st);
-    return;
-  }
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
-  k_gemm_bf16<TA, TB><<<grid, 128, 0, st>>>(M, N, K, A, lda, B, ldb, bias, relu ? 1 : 0,
-                                            accumulate ? 1 : 0, Cf, ldcf, Cb, ldcb);
-}
-
-// loss L = (1/n) sum_i [ f_i (y_i0 - log T*_i)^2 + BCE(y_i1, f_i) ] and dL/dy
-__global__ void k_mlp_loss(const float* __restrict__ Y, const int32_t* __restrict__ kstar,
-                           const float* __restrict__ logT, int n, float* __restrict__ dY,
-                           bf16* __restrict__ dYb, float* __restrict__ loss) {
-  __shared__ float red[256];
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  float L = 0.f;
-  if (i < n) {
-    const int k = kstar[i];
-    const float f = k >= 0 ? 1.f : 0.f;
-    const float y0 = Y[2 * i], y1 = Y[2 * i + 1];
-    const float d = k >= 0 ? y0 - logT[k] : 0.f;
-    const float s = 1.f / (1.f + expf(-y1));
-    L = f * d * d + fmaxf(y1, 0.f) - y1 * f + log1pf(expf(-fabsf(y1)));
-    const float g0 = 2.f * f * d / (float)n, g1 = (s - f) / (float)n;
-    dY[2 * i] = g0;
-    dY[2 * i + 1] = g1;
-    dYb[2 * i] = __float2bfloat16_rn(g0);
-    dYb[2 * i + 1] = __float2bfloat16_rn(g1);
-  }
-  red[threadIdx.x] = L;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) atomicAdd(loss, red[0] / (float)n);
-}
-
-// dz = dh * 1[h > 0] -> bf16, and the column sums of dz (bias gradient)
-__global__ void k_mlp_relu_back(const float* __restrict__ dH, const bf16* __restrict__ Hb, int n,
-                                int width, bf16* __restrict__ dZb, float* __restrict__ gb) {
-  const int c = threadIdx.x;  // blockDim.x = width
-  const int rows = (n + gridDim.x - 1) / gridDim.x;
-  const int r0 = blockIdx.x * rows, r1 = min(n, r0 + rows);
-  float sum = 0.f;
-  for (int r = r0; r < r1; ++r) {
-    const long idx = (long)r * width + c;
-    const float z = __bfloat162float(Hb[idx]) > 0.f ? dH[idx] : 0.f;
-    dZb[idx] = __float2bfloat16_rn(z);
-    sum += z;
-  }
-  atomicAdd(gb + c, sum);
-}
-
-// column sums of a [n][w] f32 matrix into gb (w <= 32)
-__global__ void k_mlp_colsum(const float* __restrict__ D, int n, int w, float* __restrict__ gb) {
-  float sum = 0.f;
-  const int c = threadIdx.x % w;
-  for (long r = (long)blockIdx.x * (blockDim.x / w) + threadIdx.x / w; r < n;
-       r += (long)gridDim.x * (blockDim.x / w))
-    sum += D[r * w + c];
-  atomicAdd(gb + c, sum);
 }
 
 // Adam on FP32 master weights; bf16 copy refreshed
@@ -262,21 +179,21 @@ struct fn_mlp {
   float* gW[MLP_LAYERS]; float* gb[MLP_LAYERS];
   int step;
   // workspace for one batch
-  bf16* X;        // [n][32]
-  bf16* Hb[3];    // [n][256]
+  bf16* X;        // [n][32]: features, row by row (reference forward) or as an image (training)
+  bf16* Hb[3];    // [n][256]: activations, likewise
+  bf16* dZ[3];    // [n][256]: the images of dz3, dz2, dz1
+  bf16* dYb;      // [2][n]: dL/dy
+  size_t rows;    // max_batch up to whole tiles, which the workspace holds
   float* Y;       // [n][2]
-  float* dY;      // [n][2]
-  bf16* dYb;      // [n][2]
-  float* dH;      // [n][256]
-  bf16* dZb;      // [n][256]
+  float* grads;   // gW, gb and the loss in one piece
+  size_t n_grads;
   float* loss;    // [1]
-  float* logT;    // [FN_MAX_GRID]
-  // tensor-core inference: layers 1-3 packed for tcgen05 (refreshed lazily
-  // after any weight change) and the kernel's error flag
+  // the weights packed for tcgen05 (refreshed lazily after any weight change;
+  // `packed` matrices: 3, with the transposes 5) and the kernels' error flag
   bf16* W1p;      // [16 KB]
-  bf16* W23p;     // [256 KB]
+  bf16* Wp;       // [512 KB]
   int* tc_err;    // [1]
-  bool packed;
+  int packed;
   std::vector<void*> allocs;
 };
 
@@ -307,16 +224,31 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
     A((void**)&m->W[l], nw * 4); A((void**)&m->b[l], nb * 4); A((void**)&m->Wb[l], nw * 2);
     A((void**)&m->mW[l], nw * 4); A((void**)&m->vW[l], nw * 4);
     A((void**)&m->mb[l], nb * 4); A((void**)&m->vb[l], nb * 4);
-    A((void**)&m->gW[l], nw * 4); A((void**)&m->gb[l], nb * 4);
   }
-  const size_t n = max_batch;
+  // every gradient tensor a multiple of 16 bytes into the piece
+  m->n_grads = 4;
+  for (int l = 0; l < MLP_LAYERS; ++l)
+    m->n_grads += (size_t)kDims[l] * kDims[l + 1] + (kDims[l + 1] + 3) / 4 * 4;
+  A((void**)&m->grads, m->n_grads * 4);
+  if (rc == FN_OK) {
+    float* g = m->grads;
+    for (int l = 0; l < MLP_LAYERS; ++l) {
+      m->gW[l] = g;
+      g += (size_t)kDims[l] * kDims[l + 1];
+      m->gb[l] = g;
+      g += (kDims[l + 1] + 3) / 4 * 4;
+    }
+    m->loss = g;
+  }
+  const size_t n = ((size_t)max_batch + kTcM - 1) / kTcM * kTcM;
+  m->rows = n;
   A((void**)&m->X, n * 32 * 2);
   for (int l = 0; l < 3; ++l) A((void**)&m->Hb[l], n * MLP_H * 2);
-  A((void**)&m->Y, n * 2 * 4); A((void**)&m->dY, n * 2 * 4); A((void**)&m->dYb, n * 2 * 2);
-  A((void**)&m->dH, n * MLP_H * 4); A((void**)&m->dZb, n * MLP_H * 2);
-  A((void**)&m->loss, 4); A((void**)&m->logT, FN_MAX_GRID * 4);
-  A((void**)&m->W1p, kTcW1Bytes); A((void**)&m->W23p, kTcW23Bytes); A((void**)&m->tc_err, 4);
-  m->packed = false;
+  for (int l = 0; l < 3; ++l) A((void**)&m->dZ[l], n * MLP_H * 2);
+  A((void**)&m->dYb, n * 2 * 2);
+  A((void**)&m->Y, n * 2 * 4);
+  A((void**)&m->W1p, kTcW1Bytes); A((void**)&m->Wp, kTcWpBytes); A((void**)&m->tc_err, 4);
+  m->packed = 0;
   if (rc != FN_OK) {
     fn_mlp_destroy(m);
     return rc;
@@ -349,14 +281,19 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
 
 // forward pass of n rows whose features are in m->X; Y = output
 static void mlp_forward(fn_mlp* m, int n, cudaStream_t st) {
-  gemm<false, false>(n, 256, 32, m->X, 32, m->Wb[0], 256, m->b[0], true, false, nullptr, 0,
-                     m->Hb[0], 256, m->tc_err, st);
-  gemm<false, false>(n, 256, 256, m->Hb[0], 256, m->Wb[1], 256, m->b[1], true, false, nullptr, 0,
-                     m->Hb[1], 256, m->tc_err, st);
-  gemm<false, false>(n, 256, 256, m->Hb[1], 256, m->Wb[2], 256, m->b[2], true, false, nullptr, 0,
-                     m->Hb[2], 256, m->tc_err, st);
-  gemm<false, false>(n, 2, 256, m->Hb[2], 256, m->Wb[3], 2, m->b[3], false, false, m->Y, 2,
-                     nullptr, 0, m->tc_err, st);
+  for (int l = 0; l < 3; ++l)
+    gemm_tc(n, 256, kDims[l], l ? m->Hb[l - 1] : m->X, kDims[l], m->Wb[l], 256, m->b[l], true,
+            m->Hb[l], 256, m->tc_err, st);
+  k_gemm_bf16<<<dim3(1, (n + 63) / 64), 128, 0, st>>>(n, 2, 256, m->Hb[2], 256, m->Wb[3], 2,
+                                                      m->b[3], m->Y, 2);
+}
+
+// the packed weights up to date on the stream (the transposes for training)
+static void mlp_pack(fn_mlp* m, bool transposed, cudaStream_t st) {
+  const int want = transposed ? 5 : 3;
+  if (m->packed >= want) return;
+  mlp_tc_pack(m->Wb[0], m->Wb[1], m->Wb[2], transposed, m->W1p, m->Wp, st);
+  m->packed = want;
 }
 
 static fn_status mlp_features(fn_mlp* m, const fn_arm_t* arm, const float* s0, const float* s1,
@@ -377,13 +314,8 @@ extern "C" fn_status fn_mlp_predict(fn_mlp_t* m, const fn_arm_t* arm, const floa
   ArmK A;
   if (!make_armk(arm, &A)) return FN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  if (!m->packed) {
-    mlp_tc_pack(m->Wb[0], 32, kTcK1, m->W1p, st);
-    mlp_tc_pack(m->Wb[1], 256, kTcKc, m->W23p, st);
-    mlp_tc_pack(m->Wb[2], 256, kTcKc, m->W23p + kTcW23Bytes / 4, st);
-    m->packed = true;
-  }
-  return mlp_tc_forward(A, s0, s1, E, m->W1p, m->W23p, m->b[0], m->b[1], m->b[2], m->Wb[3],
+  mlp_pack(m, false, st);
+  return mlp_tc_forward(A, s0, s1, E, m->W1p, m->Wp, m->b[0], m->b[1], m->b[2], m->Wb[3],
                         m->b[3], Y, m->tc_err, st);
 }
 
@@ -392,19 +324,13 @@ fn_status mlp_forward_rows(fn_mlp* m, const ArmK& A, const float* s0, const floa
                            const int* E_dev, float* Y, cudaStream_t st) {
   if (!m || E_max < 0) return FN_EINVAL;
   if (E_max == 0) return FN_OK;
-  if (!m->packed) {
-    mlp_tc_pack(m->Wb[0], 32, kTcK1, m->W1p, st);
-    mlp_tc_pack(m->Wb[1], 256, kTcKc, m->W23p, st);
-    mlp_tc_pack(m->Wb[2], 256, kTcKc, m->W23p + kTcW23Bytes / 4, st);
-    m->packed = true;
-  }
-  return mlp_tc_forward(A, s0, s1, E_max, m->W1p, m->W23p, m->b[0], m->b[1], m->b[2], m->Wb[3],
+  mlp_pack(m, false, st);
+  return mlp_tc_forward(A, s0, s1, E_max, m->W1p, m->Wp, m->b[0], m->b[1], m->b[2], m->Wb[3],
                         m->b[3], Y, m->tc_err, st, E_dev);
 }
 }  // namespace fn
 
-// the same forward on the mma.sync path (the training kernels), E <= max_batch
-// per internal batch
+// the same forward layer by layer, E <= max_batch per internal batch
 extern "C" fn_status fn_mlp_predict_ref(fn_mlp_t* m, const fn_arm_t* arm, const float* s0,
                                         const float* s1, int E, float* Y, void* stream) {
   if (!m || E < 0 || !Y || (E > 0 && (!s0 || !s1))) return FN_EINVAL;
@@ -428,56 +354,40 @@ extern "C" fn_status fn_mlp_error(fn_mlp_t* m, int* flag, int reset) {
   return FN_OK;
 }
 
-// forward + loss + backward into m->gW / m->gb (no update)
-static fn_status mlp_backward(fn_mlp* m, int n, const int32_t* kstar, cudaStream_t st) {
-  mlp_forward(m, n, st);
-  cudaMemsetAsync(m->loss, 0, 4, st);
-  k_mlp_loss<<<(n + 255) / 256, 256, 0, st>>>(m->Y, kstar, m->logT, n, m->dY, m->dYb, m->loss);
-  for (int l = 0; l < MLP_LAYERS; ++l) {
-    cudaMemsetAsync(m->gb[l], 0, kDims[l + 1] * 4, st);
-  }
-  // layer 4 (linear): dz4 = dy
-  gemm<true, false>(256, 2, n, m->Hb[2], 256, m->dYb, 2, nullptr, false, false, m->gW[3], 2,
-                    nullptr, 0, m->tc_err, st);
-  k_mlp_colsum<<<64, 256, 0, st>>>(m->dY, n, 2, m->gb[3]);
-  gemm<false, true>(n, 256, 2, m->dYb, 2, m->Wb[3], 2, nullptr, false, false, m->dH, 256, nullptr,
-                    0, m->tc_err, st);
-  const int rb = std::max(1, std::min(512, (n + 63) / 64));
-  for (int l = 2; l >= 0; --l) {
-    // dz_l = dh_l * 1[h_l > 0]; dW_l = h_{l-1}^T dz_l; dh_{l-1} = dz_l W_l^T
-    k_mlp_relu_back<<<rb, 256, 0, st>>>(m->dH, m->Hb[l], n, 256, m->dZb, m->gb[l]);
-    const bf16* hin = l == 0 ? m->X : m->Hb[l - 1];
-    const int nin = kDims[l];
-    gemm<true, false>(nin, 256, n, hin, nin, m->dZb, 256, nullptr, false, false, m->gW[l], 256,
-                      nullptr, 0, m->tc_err, st);
-    if (l > 0)
-      gemm<false, true>(n, 256, 256, m->dZb, 256, m->Wb[l], 256, nullptr, false, false, m->dH, 256,
-                        nullptr, 0, m->tc_err, st);
-  }
-  return launch_status();
-}
-
-static fn_status set_logT(fn_mlp* m, const float* T_grid, int K, cudaStream_t st) {
-  if (!T_grid || K < 1 || K > FN_MAX_GRID) return FN_EINVAL;
-  float lg[FN_MAX_GRID];
-  for (int k = 0; k < K; ++k) {
-    if (!(T_grid[k] > 0.f)) return FN_EINVAL;
-    lg[k] = std::log(T_grid[k]);
-  }
-  if (cudaMemcpyAsync(m->logT, lg, K * 4, cudaMemcpyHostToDevice, st) != cudaSuccess)
-    return FN_ECUDA;
-  return cudaStreamSynchronize(st) == cudaSuccess ? FN_OK : FN_ECUDA;
-}
-
 extern "C" fn_status fn_mlp_backward(fn_mlp_t* m, const fn_arm_t* arm, const float* s0,
                                      const float* s1, const int32_t* k_star, const float* T_grid,
                                      int K, int E, float* loss, void* stream) {
   if (!m || E < 1 || E > m->max_batch || !s0 || !s1 || !k_star) return FN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  fn_status rc = set_logT(m, T_grid, K, st);
+  if (!T_grid || K < 1 || K > FN_MAX_GRID) return FN_EINVAL;
+  MlpLogT logT = {};
+  for (int k = 0; k < K; ++k) {
+    if (!(T_grid[k] > 0.f)) return FN_EINVAL;
+    logT.v[k] = std::log(T_grid[k]);
+  }
+  ArmK A;
+  if (!make_armk(arm, &A)) return FN_EINVAL;
+  // not part of a graph: a replay would not count Adam's steps
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
+    return FN_ECUDA;
+  mlp_pack(m, true, st);
+  if (cudaMemsetAsync(m->grads, 0, m->n_grads * 4, st) != cudaSuccess) return FN_ECUDA;
+  MlpTrain p;
+  p.s0 = s0; p.s1 = s1; p.kstar = k_star; p.E = E;
+  p.W1p = m->W1p; p.Wp = m->Wp; p.W4b = m->Wb[3];
+  for (int l = 0; l < MLP_LAYERS; ++l) {
+    p.b[l] = m->b[l]; p.gW[l] = m->gW[l]; p.gb[l] = m->gb[l];
+  }
+  p.img[0] = m->X;
+  for (int l = 0; l < 3; ++l) {
+    p.img[1 + l] = m->Hb[l];
+    p.img[4 + l] = m->dZ[l];
+  }
+  p.dy = m->dYb; p.dy_pitch = (long)m->rows;
+  p.loss = m->loss; p.err = m->tc_err;
+  const fn_status rc = mlp_tc_train(A, logT, p, st);
   if (rc != FN_OK) return rc;
-  if ((rc = mlp_features(m, arm, s0, s1, E, st)) != FN_OK) return rc;
-  if ((rc = mlp_backward(m, E, k_star, st)) != FN_OK) return rc;
   if (loss) {
     if (cudaMemcpyAsync(loss, m->loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
@@ -490,7 +400,7 @@ extern "C" fn_status fn_mlp_adam_step(fn_mlp_t* m, float lr, void* stream) {
   if (!m || !(lr >= 0.f)) return FN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   m->step += 1;
-  m->packed = false;
+  m->packed = 0;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = (float)(1.0 - std::pow(0.9, m->step));
   const float c2 = (float)(1.0 - std::pow(0.999, m->step));
@@ -536,7 +446,7 @@ extern "C" fn_status fn_mlp_set_params(fn_mlp_t* m, int l, const float* W, const
   if (W && cudaMemcpy(m->W[l], W, nw * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
   if (b && cudaMemcpy(m->b[l], b, nb * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
   k_to_bf16<<<(unsigned)((nw + 255) / 256), 256>>>(m->W[l], m->Wb[l], (long)nw);
-  m->packed = false;
+  m->packed = 0;
   return cudaDeviceSynchronize() == cudaSuccess ? FN_OK : FN_ECUDA;
 }
 

@@ -22,49 +22,25 @@
 #include <cstdint>
 
 #include "fn_internal.h"
-#include "fn_mlp_tc.h"
-#include "fn_umma.cuh"
+#include "mlp_tc.cuh"
 
 namespace fn {
 
-typedef __nv_bfloat16 bf16;
-
-// shared memory map (bytes)
-constexpr int kSA = 0;                          // A operand: 128 x 256 bf16 (64 KB)
-constexpr int kSB = 65536;                      // weight ring: 4 x 32 KB
-constexpr int kSW1 = kSB + 4 * kTcChunkBytes;   // packed W1 (16 KB)
-constexpr int kSBias = kSW1 + kTcW1Bytes;       // b1, b2, b3 (3 x 256 f32)
-constexpr int kSW4 = kSBias + 3 * 256 * 4;      // W4 [256][2] f32
-constexpr int kSBar = kSW4 + 512 * 4;           // mbarriers + TMEM address
-constexpr int kSY = kSBar + 128;                // layer-4 partial sums [4][128][2] f32
-constexpr int kTcSmem = kSY + 4 * kTcM * 2 * 4;
-
-// 16 warps: warp w reads TMEM lane quarter w % 4 (the tcgen05 access rule)
-// and column group w / 4 (64 of the 256 accumulator columns) in the
-// epilogues, so that four warps share each scheduler.
-constexpr int kTcThreads = 512;
-
-constexpr int kRing = 4;
-constexpr int kTmemCols = 256;
-// instruction descriptor of tcgen05.mma kind::f16: FP32 accumulator,
-// bf16 A and B, both K-major, N = 256, M = 128
-constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTcN >> 3) << 17) |
-                            ((uint32_t)(kTcM >> 4) << 24);
-
-__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const bf16 a = __float2bfloat16_rn(lo), b = __float2bfloat16_rn(hi);
-  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
-}
-
-// weights [K][256] bf16 -> packed chunks of Kt columns
-__global__ void k_mlp_tc_pack(const bf16* __restrict__ W, int K, int Kt, bf16* __restrict__ out) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long)K * kTcN) return;
-  const int k = (int)(i / kTcN), n = (int)(i - (long)k * kTcN);
+// bf16 weights -> packed chunks (mlp_pack): blockIdx.y picks the matrix, W1,
+// W2, W3 and for training W3^T, W2^T
+__global__ void k_mlp_tc_pack(const bf16* __restrict__ W1, const bf16* __restrict__ W2,
+                              const bf16* __restrict__ W3, bf16* __restrict__ W1p,
+                              bf16* __restrict__ Wp) {
+  const int mat = blockIdx.y, K = mat == 0 ? kTcK1 : 256, Kt = mat == 0 ? kTcK1 : kTcKc;
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= K * kTcN) return;
+  const bf16* W = mat == 0 ? W1 : (mat == 1 || mat == 4 ? W2 : W3);
+  bf16* out = mat == 0 ? W1p : Wp + (mat - 1) * 256 * kTcN;
+  int k = i / kTcN, n = i - k * kTcN;
+  if (mat >= 3) { const int t = k; k = n; n = t; }   // W^T: its element (n, k) is W's (k, n)
   const int c = k / Kt, kk = k - c * Kt;
-  const long off = (long)c * kTcN * Kt +
-                   ((long)((n >> 3) * (Kt >> 3) + (kk >> 3)) * 128 + (n & 7) * 16 + (kk & 7) * 2) / 2;
-  out[off] = W[i];
+  out[c * kTcN * Kt +
+      (((n >> 3) * (Kt >> 3) + (kk >> 3)) * 128 + (n & 7) * 16 + (kk & 7) * 2) / 2] = W[i];
 }
 
 __global__ void __launch_bounds__(kTcThreads, 1)
@@ -92,8 +68,6 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   volatile int* s_fail = reinterpret_cast<volatile int*>(smem + kSBar + 84);
   const uint32_t a_base = su32(sA), b_base = su32(smem + kSB), w1_base = su32(smem + kSW1);
   const uint32_t bar_base = su32(bars);
-  auto bar_w = [&](int b) { return bar_base + 8u * b; };
-  auto bar_free = [&](int b) { return bar_base + 8u * (4 + b); };
   const uint32_t bar_layer = bar_base + 64u, bar_w1 = bar_base + 72u;
 
   for (int i = tid; i < 768; i += blockDim.x)
@@ -117,54 +91,20 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = *s_tmem;
   const uint32_t tmem_lane = tmem + ((uint32_t)(lq * 32) << 16);   // this warp's 32 lanes
 
-  const long total = (long)my_tiles * 8;   // streamed chunks (layers 2 and 3 of every tile)
-  int issued[kRing] = {0, 0, 0, 0};        // thread 0: copies in flight per slot
-  uint32_t ph_w[kRing] = {0, 0, 0, 0}, ph_free[kRing] = {0, 0, 0, 0};
+  TcRing ring(bar_base, b_base, W23p, 8, my_tiles);   // thread 0: layers 2 and 3 of every tile
   uint32_t ph_layer = 0;
-  long g = 0;                              // next chunk to multiply (thread 0)
   bool fail = false;
   if (tid == 0) {
     mbar_expect_tx(bar_w1, kTcW1Bytes);
     bulk_g2s(w1_base, W1p, kTcW1Bytes, bar_w1);
-    for (int c = 0; c < kRing && c < total; ++c) {
-      mbar_expect_tx(bar_w(c), kTcChunkBytes);
-      bulk_g2s(b_base + c * kTcChunkBytes, W23p + (long)(c % 8) * (kTcChunkBytes / 2),
-               kTcChunkBytes, bar_w(c));
-      issued[c] = 1;
-    }
+    ring.start();
   }
 
   for (int it = 0; it < my_tiles; ++it) {
     const long row = ((long)blockIdx.x + (long)it * gridDim.x) * kTcM + trow;
     // ---- features -> A (K = 32 layout: 4 core matrices per 8-row group):
     // warps 0-3, whose thread tid owns row tid (= trow)
-    if (tid < kTcM) {
-      float f[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) f[j] = 0.f;
-      if (row < E) {
-        const float* p0 = s0 + 16 * row;
-        const float* p1 = s1 + 16 * row;
-#pragma unroll
-        for (int j = 0; j < 7; ++j) {
-          const float c = 0.5f * (A.q_lo[j] + A.q_hi[j]);
-          const float h = 0.5f * (A.q_hi[j] - A.q_lo[j]);
-          f[j] = (p0[j] - c) / h;
-          f[7 + j] = p0[8 + j] / A.qd_max[j];
-          f[14 + j] = (p1[j] - c) / h;
-          f[21 + j] = p1[8 + j] / A.qd_max[j];
-        }
-      }
-#pragma unroll
-      for (int kb = 0; kb < 4; ++kb) {
-        uint4 v;
-        v.x = pack_bf16x2(f[8 * kb + 0], f[8 * kb + 1]);
-        v.y = pack_bf16x2(f[8 * kb + 2], f[8 * kb + 3]);
-        v.z = pack_bf16x2(f[8 * kb + 4], f[8 * kb + 5]);
-        v.w = pack_bf16x2(f[8 * kb + 6], f[8 * kb + 7]);
-        *reinterpret_cast<uint4*>(sA + ((tid >> 3) * 4 + kb) * 128 + (tid & 7) * 16) = v;
-      }
-    }
+    if (tid < kTcM) tc_features(A, s0 + 16 * row, s1 + 16 * row, row < E, sA, tid);
     proxy_fence();
     __syncthreads();
     // ---- layer 1
@@ -219,30 +159,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         // ---- layers 2, 3: four streamed chunks of 64 K columns each
         if (tid == 0 && !fail) {
           tc_fence_after();
-          for (int c = 0; c < 4 && !fail; ++c, ++g) {
-            const int b = (int)(g % kRing);
-            if (!mbar_wait(bar_w(b), ph_w[b])) { fail = true; break; }
-            ph_w[b] ^= 1;
-            issued[b] = 0;
-            const uint32_t bb = b_base + b * kTcChunkBytes;
-#pragma unroll
-            for (int s = 0; s < kTcKc / 16; ++s)
-              umma_f16(tmem, sdesc(a_base + (4 * c + s) * 256, 128, 256 * 16),
-                       sdesc(bb + s * 256, 128, kTcKc * 16), kIdesc, (c | s) != 0);
-            umma_commit(bar_free(b));
-            // refill the slot of the previous chunk (its MMAs are queued before
-            // this chunk's) with the chunk RING - 1 ahead of this one
-            if (g >= 1 && g + kRing - 1 < total) {
-              const int pb = (int)((g - 1) % kRing);
-              if (!mbar_wait(bar_free(pb), ph_free[pb])) { fail = true; break; }
-              ph_free[pb] ^= 1;
-              const long nc = g + kRing - 1;
-              mbar_expect_tx(bar_w(pb), kTcChunkBytes);
-              bulk_g2s(b_base + pb * kTcChunkBytes, W23p + (nc % 8) * (kTcChunkBytes / 2),
-                       kTcChunkBytes, bar_w(pb));
-              issued[pb] = 1;
-            }
-          }
+          fail = !ring.layer(tmem, a_base);
           if (!fail) umma_commit(bar_layer);
           else *s_fail = 1;
         }
@@ -288,8 +205,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if (*s_fail || fail) {
     if (tid == 0) {
       atomicExch(err, 1);
-      for (int b = 0; b < kRing; ++b)
-        if (issued[b]) mbar_wait(bar_w(b), ph_w[b]);
+      ring.drain();
     }
     __syncthreads();
   }
@@ -301,18 +217,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 }
 
 // ---------------------------------------------------------------------------
-// General BF16 GEMM on the tensor cores for the surrogate's training:
-//   C[M][N] = op(A)[M][K] op(B)[K][N] (+ bias, ReLU), FP32 accumulation in
-//   tensor memory; op(A) = A [M][K] (row-major, lda) or, TA, A^T with A
-//   [K][M]; op(B) = B [K][N] or, TB, B^T with B [N][K].
-// A CTA computes a 128 x 128 tile over the K range of its grid z slice:
-// 128 threads stage 64-column K chunks of both operands into shared memory
-// in the canonical K-major layout with 16-byte loads (stage_tile), two
-// stages deep; one thread issues four tcgen05.mma (K = 16) per chunk and commits
-// them to the stage's barrier; the epilogue reads the accumulator back
-// (warp w: lanes 32w..32w+31) and stores FP32 and / or BF16, or adds FP32
-// partial sums atomically when the K range is split.  Waits are bounded as
-// in the fused forward.
+// BF16 GEMM on the tensor cores for the reference forward, layer by layer:
+//   C[M][N] = A[M][K] B[K][N] (+ bias, ReLU), FP32 accumulation in tensor
+//   memory, C rounded to BF16.
+// A CTA computes a 128 x 128 tile: 128 threads stage 64-column K chunks of
+// both operands into shared memory in the canonical K-major layout with
+// 16-byte loads (stage_tile), two stages deep; one thread issues four
+// tcgen05.mma (K = 16) per chunk and commits them to the stage's barrier; the
+// epilogue reads the accumulator back (warp w: lanes 32w..32w+31).  Waits are
+// bounded as in the fused forward.
 // ---------------------------------------------------------------------------
 constexpr int kGM = 128, kGN = 128, kGK = 64;
 constexpr int kGTile = kGM * kGK * 2;               // 16 KB per operand tile
@@ -396,17 +309,13 @@ __device__ __forceinline__ void stage_tile(uint8_t* dst, const bf16* __restrict_
   }
 }
 
-template <bool TA, bool TB>
 __global__ void __launch_bounds__(128, 1)
-    k_gemm_tc(int M, int N, int K, int kslice, const bf16* __restrict__ A, int lda,
+    k_gemm_tc(int M, int N, int K, const bf16* __restrict__ A, int lda,
               const bf16* __restrict__ B, int ldb, const float* __restrict__ bias, int relu,
-              int accumulate, int atomic, float* __restrict__ Cf, int ldcf, bf16* __restrict__ Cb,
-              int ldcb, int* __restrict__ err) {
+              bf16* __restrict__ C, int ldc, int* __restrict__ err) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m0 = blockIdx.y * kGM, n0 = blockIdx.x * kGN;
-  const int k0 = blockIdx.z * kslice, k1 = min(K, k0 + kslice);
-  if (k0 >= k1) return;                              // block-uniform, before any barrier
   bf16* scr = reinterpret_cast<bf16*>(smem + 2 * kGStage);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + 2 * kGStage + kGScr);
   volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + 2 * kGStage + kGScr + 32);
@@ -430,7 +339,7 @@ __global__ void __launch_bounds__(128, 1)
   tc_fence_after();
   const uint32_t tmem = *s_tmem;
   const bf16 zero = __float2bfloat16_rn(0.f);
-  const int nk = (k1 - k0 + kGK - 1) / kGK;
+  const int nk = (K + kGK - 1) / kGK;
   for (int c = 0; c < nk; ++c) {
     const int st = c & 1;
     // the MMAs that read this stage two chunks ago must be done (a block
@@ -442,9 +351,9 @@ __global__ void __launch_bounds__(128, 1)
     }
     uint8_t* sa = smem + st * kGStage;
     uint8_t* sb = sa + kGTile;
-    const int kc = k0 + c * kGK;
-    stage_tile<!TA>(sa, A, lda, m0, M, kc, k1, scr, tid);   // (m, k)
-    stage_tile<TB>(sb, B, ldb, n0, N, kc, k1, scr, tid);    // (n, k)
+    const int kc = c * kGK;
+    stage_tile<true>(sa, A, lda, m0, M, kc, K, scr, tid);    // (m, k)
+    stage_tile<false>(sb, B, ldb, n0, N, kc, K, scr, tid);   // (n, k)
     proxy_fence();
     __syncthreads();
     if (tid == 0) {
@@ -475,12 +384,7 @@ __global__ void __launch_bounds__(128, 1)
           if (col >= N) continue;
           float x = __uint_as_float(v[j]) + (bias ? bias[col] : 0.f);
           if (relu) x = fmaxf(x, 0.f);
-          if (Cf) {
-            float* o = Cf + (long)row * ldcf + col;
-            if (atomic) atomicAdd(o, x);
-            else *o = accumulate ? *o + x : x;
-          }
-          if (Cb) Cb[(long)row * ldcb + col] = __float2bfloat16_rn(x);
+          C[(long)row * ldc + col] = __float2bfloat16_rn(x);
         }
       }
     }
@@ -495,48 +399,22 @@ __global__ void __launch_bounds__(128, 1)
                  : "memory");
 }
 
-template <bool TA, bool TB>
 void gemm_tc(int M, int N, int K, const bf16* A, int lda, const bf16* B, int ldb,
-             const float* bias, bool relu, bool accumulate, float* Cf, int ldcf, bf16* Cb,
-             int ldcb, int* err, cudaStream_t st) {
+             const float* bias, bool relu, bf16* C, int ldc, int* err, cudaStream_t st) {
   static bool attr[64] = {false};
   int dev = 0;
   cudaGetDevice(&dev);
   if (dev >= 0 && dev < 64 && !attr[dev]) {
-    cudaFuncSetAttribute(k_gemm_tc<TA, TB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
+    cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
     attr[dev] = true;
   }
-  const int gx = (N + kGN - 1) / kGN, gy = (M + kGM - 1) / kGM;
-  // split a long K over the grid's z so that every SM gets a CTA; the
-  // slices add FP32 partial sums atomically into a zeroed C
-  int slices = 1;
-  const int want = num_sms() / std::max(1, gx * gy);
-  if (want > 1 && K > 8 * kGK && !Cb && Cf && !bias && !relu) {
-    slices = std::min(want, (K + 4 * kGK - 1) / (4 * kGK));
-    if (slices > 1 && !accumulate) {
-      if (ldcf == N)
-        cudaMemsetAsync(Cf, 0, sizeof(float) * (size_t)M * N, st);
-      else
-        for (int r = 0; r < M; ++r) cudaMemsetAsync(Cf + (long)r * ldcf, 0, sizeof(float) * N, st);
-    }
-  }
-  const int kslice = slices > 1 ? ((K + slices - 1) / slices + kGK - 1) / kGK * kGK : K;
-  slices = (K + kslice - 1) / kslice;
-  k_gemm_tc<TA, TB><<<dim3(gx, gy, slices), 128, kGSmem, st>>>(
-      M, N, K, kslice, A, lda, B, ldb, bias, relu ? 1 : 0, accumulate ? 1 : 0, slices > 1 ? 1 : 0,
-      Cf, ldcf, Cb, ldcb, err);
+  k_gemm_tc<<<dim3((N + kGN - 1) / kGN, (M + kGM - 1) / kGM), 128, kGSmem, st>>>(
+      M, N, K, A, lda, B, ldb, bias, relu ? 1 : 0, C, ldc, err);
 }
 
-template void gemm_tc<false, false>(int, int, int, const bf16*, int, const bf16*, int, const float*,
-                                    bool, bool, float*, int, bf16*, int, int*, cudaStream_t);
-template void gemm_tc<true, false>(int, int, int, const bf16*, int, const bf16*, int, const float*,
-                                   bool, bool, float*, int, bf16*, int, int*, cudaStream_t);
-template void gemm_tc<false, true>(int, int, int, const bf16*, int, const bf16*, int, const float*,
-                                   bool, bool, float*, int, bf16*, int, int*, cudaStream_t);
-
-void mlp_tc_pack(const bf16* W, int K, int Kt, bf16* out, cudaStream_t st) {
-  const long n = (long)K * kTcN;
-  k_mlp_tc_pack<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(W, K, Kt, out);
+void mlp_tc_pack(const bf16* W1, const bf16* W2, const bf16* W3, bool transposed, bf16* W1p,
+                 bf16* Wp, cudaStream_t st) {
+  k_mlp_tc_pack<<<dim3(256, transposed ? 5 : 3), 256, 0, st>>>(W1, W2, W3, W1p, Wp);
 }
 
 fn_status mlp_tc_forward(const ArmK& A, const float* s0, const float* s1, int E, const bf16* W1p,

@@ -20,11 +20,13 @@ constexpr int kTcK1 = 32;              // layer-1 inputs (28 features + 4 zeros)
 constexpr int kTcKc = 64;              // K columns per streamed weight chunk
 constexpr int kTcChunkBytes = kTcN * kTcKc * 2;         // 32 KB
 constexpr int kTcW1Bytes = kTcN * kTcK1 * 2;            // 16 KB
-constexpr int kTcW23Bytes = 2 * 4 * kTcChunkBytes;      // layers 2 and 3: 8 chunks
+constexpr int kTcWpBytes = 4 * 4 * kTcChunkBytes;       // W2, W3, W3^T, W2^T: 16 chunks
 
-// Pack bf16 weights W [K][256] (row-major over the outputs) into chunks of
-// Kt columns (K a multiple of Kt).
-void mlp_tc_pack(const __nv_bfloat16* W, int K, int Kt, __nv_bfloat16* out, cudaStream_t st);
+// Pack the bf16 weights W [K][256] (row-major over the outputs): layer 1 as
+// one chunk of 32 columns, layers 2 and 3 and, with `transposed`, W3^T and
+// W2^T (the backward pass) as chunks of kTcKc columns.
+void mlp_tc_pack(const __nv_bfloat16* W1, const __nv_bfloat16* W2, const __nv_bfloat16* W3,
+                 bool transposed, __nv_bfloat16* W1p, __nv_bfloat16* Wp, cudaStream_t st);
 
 // Y[e] = MLP(features(s0[e], s1[e])) for e < E with the packed layers 1-3,
 // the bf16 layer-4 weights W4b [256][2] and the FP32 biases.  *err is set
@@ -36,16 +38,31 @@ fn_status mlp_tc_forward(const ArmK& A, const float* s0, const float* s1, int E,
                          const float* b4, float* Y, int* err, cudaStream_t st,
                          const int* E_dev = nullptr);
 
-// General BF16 GEMM on the tensor cores (FP32 accumulation):
-// C = op(A) op(B) (+ bias, ReLU), op = transpose when TA / TB (see
-// fn_mlp_tc.cu); C as FP32 (Cf, overwritten or, `accumulate`, added to) and
-// / or BF16 (Cb).  A long K without bias, ReLU or BF16 output is split over
-// CTAs whose FP32 partial sums are added atomically.  *err is set to 1 if a
-// wait on the tensor core timed out.
-template <bool TA, bool TB>
+// C = A B (+ bias, ReLU) in BF16 with FP32 accumulation on the tensor cores
+// (fn_mlp_tc.cu): A [M][K], B [K][N], C [M][N] rounded to BF16.  *err is set
+// to 1 if a wait on the tensor core timed out.
 void gemm_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb,
-             const float* bias, bool relu, bool accumulate, float* Cf, int ldcf,
-             __nv_bfloat16* Cb, int ldcb, int* err, cudaStream_t st);
+             const float* bias, bool relu, __nv_bfloat16* C, int ldc, int* err, cudaStream_t st);
+
+// One gradient (fn_mlp_train.cu).  img: the operand images of ceil(E / 128)
+// tiles, X (8 KB a tile), h1, h2, h3, dz3, dz2, dz1 (64 KB a tile); row r, column
+// c of a tile of width w at byte ((r / 8) * (w / 8) + c / 8) * 128 +
+// (r % 8) * 16 + (c % 8) * 2.  loss, gW and gb are added
+// to (zero before a gradient).
+struct MlpTrain {
+  const float *s0, *s1;                       // [E][16]
+  const int32_t* kstar;                       // [E]
+  int E;
+  const __nv_bfloat16 *W1p, *Wp, *W4b;
+  const float* b[4];
+  __nv_bfloat16* img[7];
+  __nv_bfloat16* dy;                          // dL/dy by columns, dy_pitch (whole tiles) apart
+  long dy_pitch;
+  float *gW[4], *gb[4], *loss;
+  int* err;
+};
+struct MlpLogT { float v[FN_MAX_GRID]; };     // log of the grid's durations
+fn_status mlp_tc_train(const ArmK& A, const MlpLogT& logT, const MlpTrain& p, cudaStream_t st);
 
 }  // namespace fn
 

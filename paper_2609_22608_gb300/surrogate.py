@@ -87,7 +87,7 @@ class MLP:
         return out
 
     def predict_ref(self, arm, s0, s1, out=None, stream=None):
-        """fn_mlp_predict_ref: the forward on the training kernels' path."""
+        """fn_mlp_predict_ref: the forward layer by layer."""
         E = s0.shape[0]
         if out is None:
             out = torch.empty(E, 2, device=s0.device)

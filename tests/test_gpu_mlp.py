@@ -140,6 +140,36 @@ def test_gradient_parity(S, orc, arm):
     mlp.close()
 
 
+@pytest.mark.parametrize("E", [1, 63, 64, 65, 128, 129, 513, 152 * 128 + 77])
+def test_gradient_of_ragged_batches(S, arm, E):
+    """One row, the edges of the 64-row blocks, 128-row tiles and 512-row
+    stages, and more tiles than SMs, in a workspace of exactly E rows, with
+    feasible and infeasible labels: norm-wise within 1e-3 of the FP64 reference
+    with the same rounding points (a rounding that falls the other way moves a
+    tensor by up to 2^-9 / sqrt(E)); a second call gives the same again."""
+    mlp = S.MLP(max_batch=E)
+    ps = seeded_params(21)
+    load(mlp, ps)
+    s0, s1 = synth.random_edges(arm, E, 22)
+    grid = synth.duration_grid(48)
+    lab = np.random.default_rng(23).integers(-1, 48, E).astype(np.int32)
+    lab[0] = 7
+    P64 = [(W.astype(np.float64), b.astype(np.float64)) for W, b in ps]
+    y, cache = M.forward(P64, M.features(arm, s0, s1))
+    logT = np.log(grid.astype(np.float64))[np.clip(lab, 0, None)]
+    L, dy = M.loss_and_grad_y(y, logT, lab >= 0)
+    grads = M.backward(P64, cache, dy)
+    for _ in range(2):
+        loss = mlp.backward(arm, dev(s0), dev(s1), dev(lab), grid)
+        assert mlp.error() == 0
+        assert loss == pytest.approx(L, rel=1e-3)
+        for l in range(4):
+            gW, gb = mlp.get_grads(l)
+            tol = max(1e-3, 2.0 ** -9 / np.sqrt(E))
+            assert relerr(gW, grads[l][0]) < tol and relerr(gb, grads[l][1]) < tol, l
+    mlp.close()
+
+
 def test_adam_step_parity(S, arm):
     mlp = S.MLP(max_batch=64)
     ps = seeded_params(2)
