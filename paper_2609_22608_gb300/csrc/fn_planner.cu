@@ -1980,83 +1980,163 @@ __global__ void k_attach_final(PlanDev D, int output) {
 
 // ---------------------------------------------------------------------------
 // goal density (FN_PLAN_DENSITY / FN_PLAN_REFIT): one block per problem after
-// attach.  Thread 0 inserts the round's new rendezvous nodes whose chart
-// parameters are known into the best-plans archive (best J first, a new
-// entry after equal ones, at most n_fit); with `refit`, p_theta is refit to
-// the archive by EM with diagonal covariances (E-step: thread per plan;
-// M-step: thread per (component, parameter)).
+// attach.  The round's new rendezvous nodes whose chart parameters are known
+// go, in node order, into the best-plans archive (best J first, a new entry
+// after equal ones, at most n_fit); with `refit`, p_theta is refit to the
+// archive by EM with diagonal covariances (E-step: thread per plan and
+// component; M-step: thread per (component, parameter)).
+//
+// Insertion: the block looks at PL_DN_TURN nodes at a time and lists those that
+// the archive of before the turn would take (its last J only rises, so none is
+// missed); warp 0 inserts the few listed ones, the archive's J in registers, two
+// entries to a lane; z follows once at the end.  One thread walking the nodes,
+// each waiting for its J from memory, made the kernel 186 us in an anytime cycle
+// with 8192 samples; now 24, the eight EM iterations most of it.
 // ---------------------------------------------------------------------------
-#define PL_DENSITY_THREADS 64   // >= FN_ARCHIVE_MAX and >= 9 * FN_DENSITY_MAX_C
+#define PL_DENSITY_THREADS 256   // = FN_ARCHIVE_MAX * FN_DENSITY_MAX_C, >= 9 * FN_DENSITY_MAX_C
+#define PL_DN_TURN (4 * PL_DENSITY_THREADS)
 
 __global__ void __launch_bounds__(PL_DENSITY_THREADS) k_plan_density(PlanDev D, int refit) {
   pdl_begin();
   __shared__ float sz[FN_ARCHIVE_MAX][9];
   __shared__ float sr[FN_ARCHIVE_MAX][FN_DENSITY_MAX_C];
   __shared__ fn_density_t th;
-  __shared__ int sn;
+  __shared__ int sn, scount[4][PL_DENSITY_THREADS / 32], ssrc[FN_ARCHIVE_MAX];
+  __shared__ float slast, sJ[PL_DN_TURN];
+  __shared__ int snode[PL_DN_TURN];
   const int p = blockIdx.x;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
   Archive& ar = D.arch[p];
-  if (t == 0) {
-    const int N1 = D.n_nodes[p], add = D.added[p];
-    const long nb = (long)p * D.NC;
-    const int cap = min(max(D.scfg.n_fit, 1), FN_ARCHIVE_MAX);
-    int n = min(max(ar.n, 0), cap);
-    for (int nd = max(N1 - add, 0); nd < N1; ++nd) {
-      const float J = D.J[nb + nd];
-      const float* z = D.zn + (nb + nd) * 9;
-      bool known = isfinite(J);
-      for (int i = 0; i < 9; ++i) known = known && isfinite(z[i]);
-      if (!known) continue;
-      int pos = n;
-      for (int i = 0; i < n; ++i)
-        if (J > ar.J[i]) {
-          pos = i;
-          break;
-        }
-      if (pos >= cap) continue;
-      for (int i = min(n, cap - 1); i > pos; --i) {
-        ar.J[i] = ar.J[i - 1];
-        for (int k = 0; k < 9; ++k) ar.z[i][k] = ar.z[i - 1][k];
-      }
-      ar.J[pos] = J;
-      for (int k = 0; k < 9; ++k) ar.z[pos][k] = z[k];
-      n = min(n + 1, cap);
+  const int N1 = D.n_nodes[p], add = D.added[p];
+  const long nb = (long)p * D.NC;
+  const int cap = min(max(D.scfg.n_fit, 1), FN_ARCHIVE_MAX);
+  int n = min(max(ar.n, 0), cap);
+  // warp 0: entries lane and lane + 32, J and where z is (-1 - slot: this archive, else a node)
+  float aJ[2] = {0.f, 0.f};
+  int src[2] = {-1 - lane, -33 - lane};
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+    if (w == 0 && lane + 32 * i < n) aJ[i] = ar.J[lane + 32 * i];
+  if (t == 0) th = D.dens[p];
+  if (t == 0) slast = n == cap ? ar.J[cap - 1] : -INFINITY;
+  __syncthreads();
+  bool changed = false;
+  for (int base = max(N1 - add, 0); base < N1; base += PL_DN_TURN) {
+    const float last = slast;        // every finite J is above -inf: an archive with room
+    float J[4];
+    unsigned take[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int nd = base + j * PL_DENSITY_THREADS + t;
+      J[j] = nd < N1 ? D.J[nb + nd] : NAN;
     }
-    ar.n = n;
-    sn = n;
-    th = D.dens[p];
-    if (refit && n > 0 && th.C <= 0) {       // first fit: the best min(C, n) plans
-      const int C = min(max(D.scfg.C, 1), min(n, FN_DENSITY_MAX_C));
-      th.C = C;
-      for (int m = 0; m < C; ++m) {
-        th.pi[m] = 1.f / (float)C;
-        for (int k = 0; k < 9; ++k) {
-          th.mu[m][k] = ar.z[m][k];
-          th.sd[m][k] = D.scfg.sd_init;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int nd = base + j * PL_DENSITY_THREADS + t;
+      bool known = isfinite(J[j]) && J[j] > last;
+      if (known)
+        for (int i = 0; i < 9; ++i) known = known && isfinite(D.zn[(nb + nd) * 9 + i]);
+      take[j] = __ballot_sync(0xffffffffu, known);
+      if (lane == 0) scount[j][w] = __popc(take[j]);
+    }
+    __syncthreads();
+    int total = 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      for (int v = 0; v < PL_DENSITY_THREADS / 32; ++v) {
+        if (v == w && (take[j] >> lane & 1u)) {
+          const int at = total + __popc(take[j] & ((1u << lane) - 1u));
+          sJ[at] = J[j];
+          snode[at] = base + j * PL_DENSITY_THREADS + t;
         }
+        total += scount[j][v];
+      }
+    __syncthreads();
+    if (w == 0) {
+      for (int c = 0; c < total; ++c) {
+        const float Jc = sJ[c];
+        const int pos = __popc(__ballot_sync(0xffffffffu, lane < n && aJ[0] >= Jc)) +
+                        __popc(__ballot_sync(0xffffffffu, lane + 32 < n && aJ[1] >= Jc));
+        if (pos >= cap) continue;
+        const float J0 = __shfl_up_sync(0xffffffffu, aJ[0], 1);
+        const float J1 = __shfl_up_sync(0xffffffffu, aJ[1], 1);
+        const float Jm = __shfl_sync(0xffffffffu, aJ[0], 31);
+        const int s0 = __shfl_up_sync(0xffffffffu, src[0], 1);
+        const int s1 = __shfl_up_sync(0xffffffffu, src[1], 1);
+        const int sm = __shfl_sync(0xffffffffu, src[0], 31);
+        if (lane == pos) {
+          aJ[0] = Jc;
+          src[0] = snode[c];
+        } else if (lane > pos) {
+          aJ[0] = J0;
+          src[0] = s0;
+        }
+        if (lane + 32 == pos) {
+          aJ[1] = Jc;
+          src[1] = snode[c];
+        } else if (lane + 32 > pos) {
+          aJ[1] = lane ? J1 : Jm;
+          src[1] = lane ? s1 : sm;
+        }
+        n = min(n + 1, cap);
+      }
+      const float l = __shfl_sync(0xffffffffu, cap > 32 ? aJ[1] : aJ[0], (cap - 1) & 31);
+      if (lane == 0) slast = n == cap ? l : -INFINITY;
+    }
+    changed = changed || total > 0;
+    __syncthreads();
+  }
+  if (w == 0) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      ssrc[lane + 32 * i] = src[i];
+      if (changed && lane + 32 * i < n) ar.J[lane + 32 * i] = aJ[i];
+    }
+    if (lane == 0) sn = ar.n = n;
+  }
+  __syncthreads();
+  n = sn;
+  // the plans' parameters from where they lie, then back into the archive
+  for (int i = t; i < 9 * n; i += PL_DENSITY_THREADS) {
+    const int e = i / 9, k = i - 9 * e, from = ssrc[e];
+    sz[e][k] = from < 0 ? ar.z[-1 - from][k] : D.zn[(nb + from) * 9 + k];
+  }
+  __syncthreads();
+  if (changed)
+    for (int i = t; i < 9 * n; i += PL_DENSITY_THREADS) ar.z[i / 9][i % 9] = sz[i / 9][i % 9];
+  if (!refit || n == 0) return;
+  if (t == 0 && th.C <= 0) {                 // first fit: the best min(C, n) plans
+    const int C = min(max(D.scfg.C, 1), min(n, FN_DENSITY_MAX_C));
+    th.C = C;
+    for (int m = 0; m < C; ++m) {
+      th.pi[m] = 1.f / (float)C;
+      for (int k = 0; k < 9; ++k) {
+        th.mu[m][k] = sz[m][k];
+        th.sd[m][k] = D.scfg.sd_init;
       }
     }
   }
   __syncthreads();
-  const int n = sn;
-  if (!refit || n == 0) return;
-  if (t < n)
-    for (int k = 0; k < 9; ++k) sz[t][k] = ar.z[t][k];
-  __syncthreads();
   const int C = th.C;
   const float floor2 = D.scfg.sd_floor * D.scfg.sd_floor;
   for (int itn = 0; itn < D.scfg.em_iters; ++itn) {
-    if (t < n) {                              // E-step: responsibilities of plan t
-      float lp[FN_DENSITY_MAX_C], top = -INFINITY;
-      for (int m = 0; m < C; ++m) {
+    {                                        // E-step: log weight of plan e under component m
+      const int e = t % FN_ARCHIVE_MAX, m = t / FN_ARCHIVE_MAX;
+      if (e < n && m < C) {
         float a = th.pi[m] > 0.f ? logf(th.pi[m]) : -INFINITY;
         for (int k = 0; k < 9; ++k) {
-          const float d = (sz[t][k] - th.mu[m][k]) / th.sd[m][k];
+          const float d = (sz[e][k] - th.mu[m][k]) / th.sd[m][k];
           a -= 0.5f * d * d + logf(th.sd[m][k]);
         }
-        lp[m] = a;
-        top = fmaxf(top, a);
+        sr[e][m] = a;
+      }
+    }
+    __syncthreads();
+    if (t < n) {                             // responsibilities of plan t
+      float lp[FN_DENSITY_MAX_C], top = -INFINITY;
+      for (int m = 0; m < C; ++m) {
+        lp[m] = sr[t][m];
+        top = fmaxf(top, lp[m]);
       }
       float sum = 0.f;
       for (int m = 0; m < C; ++m) {
