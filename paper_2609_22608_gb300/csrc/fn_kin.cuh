@@ -742,24 +742,42 @@ __device__ __forceinline__ float objective(const fn_problem_t& P, float T, float
          P.w_x * log_arm;
 }
 
-// Eq. (reach) on a G-point grid: first grid index g with
-// t_n + |p_n - x(T_g + t_offset)| / V_tip <= T_g, p_n the closest point of the
-// node's blade edge; -1 if none.
-__device__ __forceinline__ int reach_index(const ArmK& A, const fn_problem_t& P, const float* q,
-                                           float t_n, int G) {
+// Eq. (reach) on a G-point grid, REACH_LANES consecutive lanes of a warp to a
+// node (all 32 lanes call it; `live` is the same over a node's lanes): whether
+// the first grid time T_g with t_n + |p_n - x(T_g + t_offset)| / V_tip <= T_g,
+// p_n the closest point of the node's blade edge, is at most t_best.  The lanes
+// take neighbouring g; on a rising grid the times past t_best decide nothing.
+#define REACH_LANES 8
+__device__ __forceinline__ bool reach_by(const ArmK& A, const fn_problem_t& P, const float* q,
+                                         float t_n, int G, float t_best, bool live) {
+  const int l = threadIdx.x & (REACH_LANES - 1), l0 = (threadIdx.x & 31) - l;
   float Ree[9], oee[3], b0[3], b1[3];
   fk_frames(A, q, Ree, oee, [](int, const float*, const float*) {});
   blade_world(A, Ree, oee, b0, b1);
   const float step = (P.t_fall - P.t_enter) / (float)(G - 1);
-  for (int g = 0; g < G; ++g) {
+  const bool rising = step >= 0.f;
+  bool keep = false, open = live;
+  for (int g0 = 0; __any_sync(0xffffffffu, open); g0 += REACH_LANES) {
+    const int g = g0 + l;
     const float T = fmaf((float)g, step, P.t_enter);
-    float x[3], p[3];
-    flight(P, T + P.t_offset, x, nullptr);
-    seg_closest(b0, b1, x, p);
-    const float d[3] = {p[0] - x[0], p[1] - x[1], p[2] - x[2]};
-    if (t_n + norm3(d) / P.v_tip <= T) return g;
+    bool hit = false;
+    if (open && g < G && !(rising && !(T <= t_best))) {
+      float x[3], p[3];
+      flight(P, T + P.t_offset, x, nullptr);
+      seg_closest(b0, b1, x, p);
+      const float d[3] = {p[0] - x[0], p[1] - x[1], p[2] - x[2]};
+      hit = t_n + norm3(d) / P.v_tip <= T;
+    }
+    const unsigned hits = __ballot_sync(0xffffffffu, hit) >> l0 & ((1u << REACH_LANES) - 1u);
+    if (open && hits) {
+      keep = fmaf((float)(g0 + __ffs(hits) - 1), step, P.t_enter) <= t_best;
+      open = false;
+    }
+    // the next eight: past the grid, or past t_best from their first on
+    const int gn = g0 + REACH_LANES;
+    if (gn >= G || (rising && !(fmaf((float)gn, step, P.t_enter) <= t_best))) open = false;
   }
-  return -1;
+  return keep;
 }
 
 // minimum over links and spheres of |centre - capsule axis| - r_link - r_obs

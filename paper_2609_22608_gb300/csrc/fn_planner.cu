@@ -2369,29 +2369,29 @@ __global__ void __launch_bounds__(32 * PL_GR_WARPS) k_plan_grefine(PlanDev D, Ar
 // ---------------------------------------------------------------------------
 // prune (Eq. (reach)): one block per problem
 // ---------------------------------------------------------------------------
-// Eq. (reach) for every node of every problem (one thread per node): keep
-// the root and the nodes that can reach the object by t_best
-__global__ void __launch_bounds__(128) k_plan_reach(PlanDev D, ArmK A) {
+// Eq. (reach) for every node of every problem: keep the root and the nodes
+// that can reach the object by t_best.  A chain of up to G roots and divisions
+// per node with few nodes in flight: eight lanes to a node, and nothing past
+// t_best, take 16 us where a thread per node and the whole grid took 47 (the
+// tree of an anytime cycle with 65536 slots).
+#define PL_REACH_T 256
+__global__ void __launch_bounds__(PL_REACH_T) k_plan_reach(PlanDev D, ArmK A) {
   pdl_begin();
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long gid = ((long)blockIdx.x * PL_REACH_T + threadIdx.x) / REACH_LANES;
   const int p = (int)(gid / D.NC);
   const int i = (int)(gid - (long)p * D.NC);
-  if (p >= D.P || i >= D.n_nodes[p]) return;
-  const long nb = (long)p * D.NC;
-  bool keep = i == 0;
-  if (!keep) {
-    const fn_problem_t& P = D.prob[p];
-    float q[7];
+  const bool live = p < D.P && i < D.n_nodes[min(p, D.P - 1)];
+  if (!__any_sync(0xffffffffu, live)) return;
+  const long n = (long)(live ? p : 0) * D.NC + (live ? i : 0);   // a slot that exists
+  const fn_problem_t& P = D.prob[live ? p : 0];
+  float q[7];
 #pragma unroll
-    for (int j = 0; j < 7; ++j) q[j] = D.st[(nb + i) * 16 + j];
-    const int g = reach_index(A, P, q, D.t[nb + i], D.G);
-    if (g >= 0) {
-      const float Tg = fmaf((float)g, (P.t_fall - P.t_enter) / (float)(D.G - 1), P.t_enter);
-      keep = Tg <= D.inc[p].t_best;
-    }
+  for (int j = 0; j < 7; ++j) q[j] = D.st[n * 16 + j];
+  const bool keep = reach_by(A, P, q, D.t[n], D.G, D.inc[live ? p : 0].t_best, live && i > 0);
+  if (live && (threadIdx.x & (REACH_LANES - 1)) == 0) {
+    D.alive[n] = keep || i == 0 ? 1 : 0;
+    D.ptr[n] = D.par[n];
   }
-  D.alive[nb + i] = keep ? 1 : 0;
-  D.ptr[nb + i] = D.par[nb + i];
 }
 
 // Multi-block prune after k_plan_reach (which leaves alive_i = the node's
@@ -3347,7 +3347,8 @@ static fn_status enqueue_iteration(fn_planner* pl, unsigned flags, cudaStream_t 
   mark(7);
   if (flags & FN_PLAN_PRUNE) {
     const long nn = (long)P * D.NC;
-    pl_launch(k_plan_reach, (unsigned)((nn + 127) / 128), 128, 0, st, D, pl->arm);
+    pl_launch(k_plan_reach, (unsigned)((nn * REACH_LANES + PL_REACH_T - 1) / PL_REACH_T),
+              PL_REACH_T, 0, st, D, pl->arm);
     trace(pl, st, "k_plan_reach");
     pl_launch(k_prune_path, (unsigned)((P + 127) / 128), 128, 0, st, D);
     trace(pl, st, "k_plan_prune");
