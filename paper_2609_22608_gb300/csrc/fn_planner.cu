@@ -46,7 +46,6 @@
 #define PL_NCOUNT 14  // work counters: probe, verify, mid-probe, kNN pairs, IK starts,
                       // surrogate-routed edges, surrogate rescans, refine evaluations,
                       // goal draws by outcome (defined, speed, IK, box, singular, taper)
-#define PL_CHORD_THREADS 1024
 
 namespace fn {
 
@@ -165,7 +164,6 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   struct Archive* arch;  // [P] best plans of the current tree
   float* cz;          // [P][BM][9] chart parameters of the goal candidates (NaN: unknown)
   float* zn;          // [P][NC][9] chart parameters of goal nodes, written at attach
-  int32_t* glist;     // [P][BM] the round's valid goal candidates, in order
   int4* gq;           // [P * BM] (problem, slot, row) of the round's decoded goal queries
   fn_sampler_cfg_t scfg;
   // parents (knn_tc.cuh): operand images and exact values of the non-root
@@ -1549,59 +1547,83 @@ __global__ void __launch_bounds__(32 * PL_EDGE_WARPS, MINB) k_plan_vseq(PlanDev 
   if (D.samples && lane == 0 && nsamp) atomicAdd(D.samples + 1, (unsigned long long)nsamp);
 }
 
-// Chord sampler (FN_PLAN_CHORD), one block per problem after the sampling
-// launch: the round's valid goals in candidate order, then every free
-// candidate whose chord draw succeeds (probability w_chord) is replaced by
-// q0 + lambda (q_g - q0) + chord_sigma * half-range * n (clamped to the box)
-// toward a goal chosen uniformly; its velocity as for a uniform draw.  Philox
-// streams: 0-3 as the uniform draw, 4 (choice, goal, lambda), 5-6 normals.
-__global__ void __launch_bounds__(PL_CHORD_THREADS) k_plan_chord(PlanDev D, ArmK A) {
+// Chord sampler (FN_PLAN_CHORD), after the goal chart: the round's valid goals
+// in candidate order, then every free candidate whose chord draw succeeds
+// (probability w_chord) is replaced by q0 + lambda (q_g - q0) + chord_sigma *
+// half-range * n (clamped to the box) toward a goal chosen uniformly; its
+// velocity as for a uniform draw.  Philox streams: 0-3 as the uniform draw, 4
+// (choice, goal, lambda), 5-6 normals.  A block takes PL_CHORD_T free
+// candidates of one problem and makes its own bitmap of the problem's valid
+// goals (a byte each from L2, at most 2048 words) to pick from: the draws, eight
+// Philox blocks and eight logarithms each, then use the whole chip.  One block
+// for a problem's draws took 28 us at 4096 of them; now 14.
+#define PL_CHORD_T 256
+__global__ void __launch_bounds__(PL_CHORD_T) k_plan_chord(PlanDev D, ArmK A) {
   pdl_begin();
   __shared__ int sh[32];
-  const int p = blockIdx.x;
+  __shared__ unsigned sbits[(1 << 16) / 32];
+  __shared__ int sbase[(1 << 16) / 32];   // valid goals before the word
+  const int chunks = (D.BM + PL_CHORD_T - 1) / PL_CHORD_T;
+  const int p = blockIdx.x / chunks;
   const fn_problem_t& P = D.prob[p];
   const int B = min(max(P.batch, 0), D.BM);
   const int G = min(max(P.n_goal, 0), B);
+  const int b0 = G + (blockIdx.x - p * chunks) * PL_CHORD_T;
+  if (b0 >= B) return;                 // block-uniform, before any barrier
   const long cb = (long)p * D.BM;
-  const int per = (G + blockDim.x - 1) / blockDim.x;
-  const int c0 = min(G, threadIdx.x * per), c1 = min(G, c0 + per);
-  int cnt = 0;
-  for (int b = c0; b < c1; ++b) cnt += D.valid[cb + b] ? 1 : 0;
-  int nv;
-  int r = block_scan(cnt, sh, &nv);
-  for (int b = c0; b < c1; ++b)
-    if (D.valid[cb + b]) D.glist[cb + r++] = b;
-  __syncthreads();
-  if (nv == 0) return;                 // the free candidates keep their uniform draws
-  const int it = *D.iter;
-  for (int b = G + threadIdx.x; b < B; b += blockDim.x) {
-    float uc[4];
-    philox_u4(P.seed, b, it, p, 4, uc);
-    if (!(uc[0] < D.scfg.w_chord)) continue;
-    const int g = min((int)floorf(uc[1] * (float)nv), nv - 1);
-    const float* qg = D.cand + (cb + D.glist[cb + g]) * 16;
-    float u[16], un[8], nrm[8];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) philox_u4(P.seed, b, it, p, k, u + 4 * k);
-#pragma unroll
-    for (int k = 0; k < 2; ++k) philox_u4(P.seed, b, it, p, 5 + k, un + 4 * k);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) box_muller(un[2 * k], un[2 * k + 1], nrm[2 * k], nrm[2 * k + 1]);
-    float q[7], qd[7];
-#pragma unroll
-    for (int j = 0; j < 7; ++j) {
-      const float lo = A.q_lo[j], hi = A.q_hi[j];
-      const float x = P.q0[j] + uc[2] * (qg[j] - P.q0[j]) + D.scfg.chord_sigma * 0.5f * (hi - lo) * nrm[j];
-      q[j] = fminf(fmaxf(x, lo), hi);
-      qd[j] = fmaf(2.f, u[7 + j], -1.f) * (D.vel_frac * taper(A, j, q[j]));
-    }
-    float4* o4 = reinterpret_cast<float4*>(D.cand + (cb + b) * 16);
-    o4[0] = make_float4(q[0], q[1], q[2], q[3]);
-    o4[1] = make_float4(q[4], q[5], q[6], 0.f);
-    o4[2] = make_float4(qd[0], qd[1], qd[2], qd[3]);
-    o4[3] = make_float4(qd[4], qd[5], qd[6], 0.f);
-    pack_query_row(D, 0, p, b - G, q, qd);
+  const int lane = threadIdx.x & 31, nw = (G + 31) / 32;
+#pragma unroll 4
+  for (int i = threadIdx.x >> 5; i < nw; i += PL_CHORD_T / 32) {
+    const int b = 32 * i + lane;
+    const unsigned m = __ballot_sync(0xffffffffu, b < G && D.valid[cb + b]);
+    if (lane == 0) sbits[i] = m;
   }
+  __syncthreads();
+  const int per = (nw + PL_CHORD_T - 1) / PL_CHORD_T;
+  const int w0 = min(nw, (int)threadIdx.x * per), w1 = min(nw, w0 + per);
+  int cnt = 0;
+  for (int i = w0; i < w1; ++i) cnt += __popc(sbits[i]);
+  int nv;
+  int r0 = block_scan(cnt, sh, &nv);
+  for (int i = w0; i < w1; ++i) {
+    sbase[i] = r0;
+    r0 += __popc(sbits[i]);
+  }
+  __syncthreads();
+  const int b = b0 + threadIdx.x;
+  if (nv == 0 || b >= B) return;       // without goals they keep their uniform draws
+  const int it = *D.iter;
+  float uc[4];
+  philox_u4(P.seed, b, it, p, 4, uc);
+  if (!(uc[0] < D.scfg.w_chord)) return;
+  const int g = min((int)floorf(uc[1] * (float)nv), nv - 1);
+  int wd = 0;                        // the word of the g-th valid goal, then its bit
+  for (int o = 1 << 11; o > 0; o >>= 1)
+    if (wd + o < nw && sbase[wd + o] <= g) wd += o;
+  unsigned m = sbits[wd];
+  for (int r = sbase[wd]; r < g; ++r) m &= m - 1u;
+  const float* qg = D.cand + (cb + 32 * wd + __ffs(m) - 1) * 16;
+  float u[16], un[8], nrm[8];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) philox_u4(P.seed, b, it, p, k, u + 4 * k);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) philox_u4(P.seed, b, it, p, 5 + k, un + 4 * k);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) box_muller(un[2 * k], un[2 * k + 1], nrm[2 * k], nrm[2 * k + 1]);
+  float q[7], qd[7];
+#pragma unroll
+  for (int j = 0; j < 7; ++j) {
+    const float lo = A.q_lo[j], hi = A.q_hi[j];
+    const float x = P.q0[j] + uc[2] * (qg[j] - P.q0[j]) + D.scfg.chord_sigma * 0.5f * (hi - lo) * nrm[j];
+    q[j] = fminf(fmaxf(x, lo), hi);
+    qd[j] = fmaf(2.f, u[7 + j], -1.f) * (D.vel_frac * taper(A, j, q[j]));
+  }
+  float4* o4 = reinterpret_cast<float4*>(D.cand + (cb + b) * 16);
+  o4[0] = make_float4(q[0], q[1], q[2], q[3]);
+  o4[1] = make_float4(q[4], q[5], q[6], 0.f);
+  o4[2] = make_float4(qd[0], qd[1], qd[2], qd[3]);
+  o4[3] = make_float4(qd[4], qd[5], qd[6], 0.f);
+  pack_query_row(D, 0, p, b - G, q, qd);
 }
 
 // N-ary refinement (FN_PLAN_NARY), after the verification stages: every free
@@ -2912,17 +2934,22 @@ static void enqueue_front(fn_planner* pl, unsigned flags, cudaStream_t st, Mark&
     return;
   }
   if (n > 0) goals(st);
+  // chord states make the free candidates wait for the goal chart (and
+  // caller-given candidates have none): the goal queries' search and the goal
+  // edges still run beside the chord states, the free queries' search and the
+  // free edges
+  const bool fork_late = knn && D.goal_split && pl->allow_fork;
+  if (fork_late) {
+    cudaEventRecord(pl->ev_fork, st);
+    cudaStreamWaitEvent(pl->side, pl->ev_fork, 0);
+  }
   if (n > 0 && (flags & FN_PLAN_CHORD)) {
-    pl_launch(k_plan_chord, P, PL_CHORD_THREADS, 0, st, D, pl->arm);
+    const long blocks = (long)P * ((D.BM + PL_CHORD_T - 1) / PL_CHORD_T);
+    pl_launch(k_plan_chord, (unsigned)blocks, PL_CHORD_T, 0, st, D, pl->arm);
     trace(pl, st, "k_plan_chord");
   }
   mark(2);
-  if (knn && D.goal_split && pl->allow_fork) {
-    // chord states make the free candidates wait for the goal chart (and
-    // caller-given candidates have none): the goal queries' search and the
-    // goal edges still run beside the free queries' search and free edges
-    cudaEventRecord(pl->ev_fork, st);
-    cudaStreamWaitEvent(pl->side, pl->ev_fork, 0);
+  if (fork_late) {
     search(0, st);
     search(1, pl->side);
     goal_edges(pl->side);
@@ -3126,7 +3153,7 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
   D.sur = 0;
   D.sur_list = nullptr;
   A_(D.sur_n, 1);
-  A_(D.dens, P); A_(D.arch, P); A_(D.cz, P * BM * 9); A_(D.zn, P * NC * 9); A_(D.glist, P * BM); A_(D.gq, P * BM);
+  A_(D.dens, P); A_(D.arch, P); A_(D.cz, P * BM * 9); A_(D.zn, P * NC * 9); A_(D.gq, P * BM);
   D.scfg = default_sampler_cfg();
   if (rc == FN_OK) {
     std::vector<fn_density_t> th(P);
