@@ -1138,7 +1138,11 @@ __device__ __forceinline__ void finish_edge(const PlanDev& D, const ArmK& A, int
 
 // after a stage: edges whose duration passed are finished; the others move
 // to their next survivor (next list) or end with no feasible duration
-__global__ void __launch_bounds__(128) k_plan_vselect(PlanDev D, ArmK A, GridKP Gr, int list) {
+// A warp's edge is one long chain (forward kinematics, then seven capsules
+// against every obstacle), so the grid is what 96 registers let an SM hold: 5
+// blocks of an SM take 32 us in an anytime cycle with five obstacles, 2 took 42.
+#define PL_VSEL_BLOCKS 5
+__global__ void __launch_bounds__(128, PL_VSEL_BLOCKS) k_plan_vselect(PlanDev D, ArmK A, GridKP Gr, int list) {
   pdl_begin();
   __shared__ float sEs[4][32];
   Sched* S = D.sched;
@@ -3000,7 +3004,7 @@ static void enqueue_edge_body(fn_planner* pl, const PlanDev& D, int v, int block
   for (int stage = 0; stage < vstages(D); ++stage) {
     pl_launch(plan_vstage_variant(v), blocks, 32 * PL_EDGE_WARPS, 0, st, D, pl->arm, pl->grid, list);
     trace(pl, st, "k_plan_vstage");
-    pl_launch(k_plan_vselect, tb, 128, 0, st, D, pl->arm, pl->grid, list);
+    pl_launch(k_plan_vselect, PL_VSEL_BLOCKS * num_sms(), 128, 0, st, D, pl->arm, pl->grid, list);
     trace(pl, st, "k_plan_vselect");
     list ^= 1;
   }
