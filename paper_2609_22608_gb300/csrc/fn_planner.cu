@@ -3346,6 +3346,7 @@ static fn_status enqueue_iteration(fn_planner* pl, unsigned flags, cudaStream_t 
     cudaStreamWaitEvent(st, pl->ev_join, 0);
     pl->forked = false;
   }
+  const bool can_fork = pl->allow_fork;
   pl->allow_fork = false;
   if (flags & FN_PLAN_NARY) {
     pl_launch(k_plan_refine, 4 * num_sms(), 32 * PL_REFINE_WARPS, 0, st, D, pl->arm, pl->grid,
@@ -3366,9 +3367,20 @@ static fn_status enqueue_iteration(fn_planner* pl, unsigned flags, cudaStream_t 
     pl_launch(k_plan_attach, P, PL_ATTACH_THREADS, 0, st, D, late ? 0 : 1);
     trace(pl, st, "k_plan_attach");
   }
-  if (flags & (FN_PLAN_DENSITY | FN_PLAN_REFIT)) {
-    pl_launch(k_plan_density, P, PL_DENSITY_THREADS, 0, st, D, (flags & FN_PLAN_REFIT) ? 1 : 0);
+  // the density reads the round's new nodes where the attach put them, which
+  // the prune only changes in its last steps: its single block (24 us) runs
+  // beside the prune's first ones unless the refinement comes between
+  const bool dens = flags & (FN_PLAN_DENSITY | FN_PLAN_REFIT);
+  const bool dens_side = dens && (flags & FN_PLAN_PRUNE) && !(flags & FN_PLAN_GREFINE) && can_fork;
+  if (dens_side) {
+    cudaEventRecord(pl->ev_fork, st);
+    cudaStreamWaitEvent(pl->side, pl->ev_fork, 0);
+  }
+  if (dens) {
+    pl_launch_pdl(!dens_side, k_plan_density, P, PL_DENSITY_THREADS, 0, dens_side ? pl->side : st,
+                  D, (flags & FN_PLAN_REFIT) ? 1 : 0);
     trace(pl, st, "k_plan_density");
+    if (dens_side) cudaEventRecord(pl->ev_join, pl->side);
   }
   if (flags & FN_PLAN_GREFINE) {
     pl_launch(k_plan_grefine, P, 32 * PL_GR_WARPS, 0, st, D, pl->arm, pl->gr_iters, pl->gr_eta0,
@@ -3378,8 +3390,10 @@ static fn_status enqueue_iteration(fn_planner* pl, unsigned flags, cudaStream_t 
   mark(7);
   if (flags & FN_PLAN_PRUNE) {
     const long nn = (long)P * D.NC;
-    pl_launch(k_plan_reach, (unsigned)((nn * REACH_LANES + PL_REACH_T - 1) / PL_REACH_T),
-              PL_REACH_T, 0, st, D, pl->arm);
+    // (its blocks, launched early, would keep the density's off the SMs)
+    pl_launch_pdl(!dens_side, k_plan_reach,
+                  (unsigned)((nn * REACH_LANES + PL_REACH_T - 1) / PL_REACH_T), PL_REACH_T, 0, st, D,
+                  pl->arm);
     trace(pl, st, "k_plan_reach");
     pl_launch(k_prune_path, (unsigned)((P + 127) / 128), 128, 0, st, D);
     trace(pl, st, "k_plan_prune");
@@ -3388,6 +3402,7 @@ static fn_status enqueue_iteration(fn_planner* pl, unsigned flags, cudaStream_t 
     trace(pl, st, "k_plan_prune");
     pl_launch(k_prune_scatter, pb, PL_PRUNE_T, 0, st, D);
     trace(pl, st, "k_plan_prune");
+    if (dens_side) cudaStreamWaitEvent(st, pl->ev_join, 0);
     pl_launch(k_prune_copy, pb, PL_PRUNE_T, 0, st, D);
     trace(pl, st, "k_plan_prune");
     pl_launch(k_plan_prune, P, PL_ATTACH_THREADS, 0, st, D, pl->arm);   // deep chains only
