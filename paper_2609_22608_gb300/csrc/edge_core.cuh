@@ -153,6 +153,35 @@ __device__ __forceinline__ bool end_probe_pass(const ArmK& A, const float* split
   return pass;
 }
 
+// The same for two durations of one edge (x, y): the split is read once for
+// both and the torques are paired FP32 operations with the scalar roundings.
+__device__ __forceinline__ void end_probe_pass2(const ArmK& A, const float* split, float2 T,
+                                                bool& px, bool& py) {
+  const float2 iT = make_float2(1.0f / T.x, 1.0f / T.y), iT2 = mul2(iT, iT);
+  px = py = true;
+#pragma unroll
+  for (int end = 0; end < 2; ++end) {
+    const float4* c4 = reinterpret_cast<const float4*>(split + 28 * end);
+    float f[28];
+#pragma unroll
+    for (int v = 0; v < 7; ++v) {
+      const float4 t = c4[v];
+      f[4 * v] = t.x; f[4 * v + 1] = t.y; f[4 * v + 2] = t.z; f[4 * v + 3] = t.w;
+    }
+    float2 r = make_float2(0.f, 0.f), pw = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 7; ++j) {
+      const float2 tau = fma2(dup2(f[j]), iT2, fma2(dup2(f[7 + j]), iT, dup2(f[14 + j])));
+      const float2 t = mul2(tau, dup2(A.inv_tau[j]));
+      r.x = fmaxf(r.x, fabsf(t.x));
+      r.y = fmaxf(r.y, fabsf(t.y));
+      pw = fma2(tau, dup2(f[21 + j]), pw);
+    }
+    px = px && r.x <= 1.f && fabsf(pw.x) * A.inv_w <= 1.f;
+    py = py && r.y <= 1.f && fabsf(pw.y) * A.inv_w <= 1.f;
+  }
+}
+
 // position of the i-th lowest set bit of x (i = 0: the lowest); -1 if x has
 // at most i set bits
 __device__ __forceinline__ int nth_bit(unsigned x, int i) {

@@ -888,14 +888,18 @@ __global__ void __launch_bounds__(32 * PL_PR_WARPS) k_plan_probe(PlanDev D, ArmK
       const int k1 = k0 + __shfl_sync(0xffffffffu, cnt, i);
       const bool gl = __shfl_sync(0xffffffffu, (int)goal, i) != 0;
       const float Tg = __shfl_sync(0xffffffffu, Tp, i);
-      for (int b = k0 & ~31; b < k1; b += 32) {
-        const int k = b + lane;
-        const bool in = k >= k0 && k < k1;
-        bool f0;
-        const bool pass =
-            in && end_probe_pass(A, split + FN_SPLIT_WORDS * i, gl ? Tg : sT[in ? k : k0], f0);
-        const unsigned m = __ballot_sync(0xffffffffu, pass);
+      const float* sp = split + FN_SPLIT_WORDS * i;
+      for (int b = k0 & ~31; b < k1; b += 64) {
+        const int k = b + lane, k2 = k + 32;
+        const bool in = k >= k0 && k < k1, in2 = k2 < k1;
+        const float T = gl ? Tg : sT[in ? k : k0];
+        bool px, py = false, f0;
+        if (b + 32 < k1) end_probe_pass2(A, sp, make_float2(T, sT[in2 ? k2 : k0]), px, py);
+        else px = end_probe_pass(A, sp, T, f0);
+        const unsigned m = __ballot_sync(0xffffffffu, in && px);
+        const unsigned m2 = __ballot_sync(0xffffffffu, in2 && py);
         if (lane == 0 && m) bits[8 * i + (b >> 5)] = m;
+        if (lane == 0 && m2) bits[8 * i + (b >> 5) + 1] = m2;
       }
     }
     __syncwarp();
