@@ -333,10 +333,8 @@ static fn_status launch_time_edges_tm(const ArmK& A, const GridK* G, int K, int 
                                              (int)kTmSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
-  const long want = ((long)E + TM_WARPS - 1) / TM_WARPS;
-  const int blocks = (int)std::max<long>(1, std::min<long>(want, num_sms()));
   static GridK empty;
-  k_time_edges_tm<<<blocks, 32 * TM_WARPS, kTmSmem, st>>>(A, G ? *G : empty, K, S, mode, s0, s1, E,
+  k_time_edges_tm<<<tm_blocks(E), 32 * TM_WARPS, kTmSmem, st>>>(A, G ? *G : empty, K, S, mode, s0, s1, E,
                                                            Tparam, k_star, T_star, rho3, ok,
                                                            counter);
   return launch_status();
@@ -357,9 +355,7 @@ static fn_status launch_time_window_tm(const ArmK& A, const GridK& G, int K, int
                                              (int)kTmSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
-  const long want = ((long)E + TM_WARPS - 1) / TM_WARPS;
-  const int blocks = (int)std::max<long>(1, std::min<long>(want, num_sms()));
-  k_time_window_tm<<<blocks, 32 * TM_WARPS, kTmSmem, st>>>(A, G, K, S, s0, s1, E, Y, W, logT0,
+  k_time_window_tm<<<tm_blocks(E), 32 * TM_WARPS, kTmSmem, st>>>(A, G, K, S, s0, s1, E, Y, W, logT0,
                                                             dlog, k_star, T_star, rho3, ok, path,
                                                             counter);
   return launch_status();

@@ -14,7 +14,10 @@
 
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "edge_core.cuh"
+#include "fn_internal.h"
 #include "fn_tmem.cuh"
 
 namespace fn {
@@ -68,10 +71,16 @@ struct TmBlock {
   }
 };
 
+// CTAs for E items: one per SM, fewer only when there are fewer items.  A
+// range of up to TM_WARPS items then costs its slowest item alone (tm_claim):
+// 256 edges at K = 64 take 23 us on 152 SMs, and took 36 as pairs on the six
+// warps of 22.
+inline int tm_blocks(long E) { return (int)std::max<long>(1, std::min<long>(E, num_sms())); }
+
 // Claim of a run by a warp of the CTA whose range holds `len` items: about
-// (range left) / (2 TM_WARPS) items, at least two and at most TM_GROUP, so
-// that runs shrink towards the end of the range and the warps finish
-// together.  Returns the run's first item (relative to the range) and its
+// (range left) / (2 TM_WARPS) items, at least two (one where there is a warp
+// for every item) and at most TM_GROUP, so that runs shrink towards the end of
+// the range and the warps finish together.  Returns the run's first item (relative to the range) and its
 // length n (0: the range is done), the same on every lane.
 __device__ __forceinline__ int tm_claim(int* next, int len, int& n) {
   const int lane = threadIdx.x & 31;
@@ -79,7 +88,7 @@ __device__ __forceinline__ int tm_claim(int* next, int len, int& n) {
   n = 0;
   if (lane == 0) {
     const int seen = atomicAdd(next, 0);
-    const int want = min(TM_GROUP, max(2, (len - seen) / (2 * TM_WARPS)));
+    const int want = min(TM_GROUP, max(len <= TM_WARPS ? 1 : 2, (len - seen) / (2 * TM_WARPS)));
     first = atomicAdd(next, want);
     n = max(0, min(want, len - first));
   }
