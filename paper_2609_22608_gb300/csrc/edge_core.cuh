@@ -330,11 +330,12 @@ __device__ __forceinline__ void split_group(const ArmK& A, const Core& core, flo
 //              (alpha, beta: gravity, velocity and friction off)
 //   PROBE_END: lanes = grid durations base+lane, both end samples from the
 //              split (no torque evaluation)
-//   PROBE_MID: interior samples mid_probe_index(j, S, 4 NS), j < 4 NS, of the
+//   PROBE_MID: interior samples mid_probe_index(j, S, n), j < n, n = 4 NS
+//              (wmode > 0: 4, the same with every core), of the
 //              lowest survivors not yet probed there: packed (wmode 0), the
 //              lowest eight survivors x 4 NS samples in one pass, lane = 4 i +
 //              j (x: sample j, y: sample j + 4); otherwise lanes = durations,
-//              NS samples per pass
+//              four samples, NS per pass
 //   PROBE_W  : (wmode 2) one sample, the witness, at the remaining survivors
 //              (plain coefficients): after a failed verify, that duration's
 //              first violating sample; on the first chunk, the caller's w_in
@@ -368,10 +369,10 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
   enum { SPLIT = 0, PROBE_END = 1, PROBE_W = 2, PROBE_MID = 3, VERIFY = 4 };
   enum { COEF_NONE = 0, COEF_PLAIN = 1, COEF_EXACT = 2, COEF_SPLIT = 3 };
   constexpr int NS = Core::NS;
-  constexpr int NMID = FN_MID_PROBES * NS;   // interior probe samples per survivor
+  const int nmid = FN_MID_PROBES * (wmode == 0 ? NS : 1);   // interior probe samples per survivor
   constexpr int BATCH = 32 * NS;             // verification samples per pass
   const int lane = threadIdx.x & 31;
-  const bool packed = wmode == 0;       // interior probes of 8 survivors x NMID samples per pass
+  const bool packed = wmode == 0;       // interior probes of 8 survivors x nmid samples per pass
   int mode = PROBE_END, base = k_begin, kk = 0, s0 = 0, mj = 0, sw = 0, coef = COEF_NONE;
   int cdur = -1;        // COEF_PLAIN: this lane's grid index (-1: none)
   int kill = -1;        // wmode > 0: sample that proved duration base + lane infeasible
@@ -451,13 +452,13 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
       } else if (mode == PROBE_MID && packed) {
         ax = cdur >= 0;
         ay = NS == 2 && ax;
-        sx = mid_probe_index(lane & 3, S, NMID);
-        sy = mid_probe_index((lane & 3) + 4, S, NMID);
+        sx = mid_probe_index(lane & 3, S, nmid);
+        sy = mid_probe_index((lane & 3) + 4, S, nmid);
       } else if (mode == PROBE_MID) {   // lanes = durations, NS samples per pass
         ax = ((sel & cand) >> lane) & 1u;
         ay = NS == 2 && ax;
-        sx = mid_probe_index(mj, S, NMID);
-        sy = mid_probe_index(mj + 1, S, NMID);
+        sx = mid_probe_index(mj, S, nmid);
+        sy = mid_probe_index(mj + 1, S, nmid);
       } else {              // PROBE_W
         ax = (cand >> lane) & 1u;
         sx = sw;
@@ -518,7 +519,7 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
         else if (wmode > 0 && ay && !pass_y) kill = sy;
         cand &= ~(fail_x | fail_y);
         mj += NS;
-        if (mj < NMID && (sel & cand)) continue;
+        if (mj < nmid && (sel & cand)) continue;
         mpr |= sel;
         decide = true;
       } else {                         // VERIFY

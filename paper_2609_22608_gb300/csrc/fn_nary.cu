@@ -6,7 +6,8 @@
 // kept, until the bracket is no wider than eps.  rho_v is checked once, at
 // the refined duration.
 //
-// One warp per edge.  A round is the grid scan's own probe/verify machinery
+// One warp per edge, on the paired core with its records in tensor memory
+// (tm_scan.cuh) unless a scalar variant of the grid scan was chosen.  A round is the grid scan's own probe/verify machinery
 // (edge_core.cuh) run over a 31-entry duration list in the warp's shared
 // slot, so the kernel keeps a single torque-evaluation call site: the grid
 // pass and every round go through the same edge_scan call in one loop.  The
@@ -17,8 +18,11 @@
 #include <cuda_runtime.h>
 
 #include "fn_internal.h"
-#include "nary_core.cuh"
+#include <mutex>
+
 #include "fn_tune.h"
+#include "nary_core.cuh"
+#include "tm_scan.cuh"
 
 namespace fn {
 
@@ -29,16 +33,38 @@ struct NaryGrid {
 #define NARY_WARPS 3   // as the grid scan: static shared memory within 48 KB
 #define NARY_MAX_ROUNDS 16
 
+struct NaryOut {
+  int32_t* k_star;
+  float *T_star, *T_lo, *rho3;
+  uint8_t* ok;
+  int32_t* rounds;
+};
+
+// edge e's results (the warp's staged edge es; o.k = -2: invalid states)
+__device__ __forceinline__ void nary_write(const ArmK& A, const float* es, long e,
+                                           const NaryEdge& o, const NaryOut& out) {
+  const bool found = o.k >= 0;
+  const float rv = found ? warp_rho_v(A, es, o.b) : NAN;
+  if ((threadIdx.x & 31) == 0) {
+    out.k_star[e] = o.k;
+    out.T_star[e] = found ? o.b : (o.k == -1 ? INFINITY : NAN);   // -2 invalid, -3 aborted
+    if (out.T_lo) out.T_lo[e] = found ? o.a : NAN;
+    out.rho3[3 * e + 0] = found ? o.rt : NAN;
+    out.rho3[3 * e + 1] = found ? o.rp : NAN;
+    out.rho3[3 * e + 2] = rv;
+    out.ok[e] = (found && rv <= 1.f) ? 1 : 0;
+    if (out.rounds) out.rounds[e] = o.r;
+  }
+}
+
 // Persistent: warp w takes edges w, w + W, ...  MINB sets the register
 // budget, as for the grid scan's kernel, whose tuned variant it follows.
 template <int MINB>
 __global__ void __launch_bounds__(32 * NARY_WARPS, MINB)
     k_time_edges_nary(ArmK A, NaryGrid G, int K, int S, const float* __restrict__ s0,
                       const float* __restrict__ s1, int E, const float* __restrict__ T_cap,
-                      float eps, int max_rounds, int32_t* __restrict__ k_star,
-                      float* __restrict__ T_star, float* __restrict__ T_lo,
-                      float* __restrict__ rho3, uint8_t* __restrict__ ok,
-                      int32_t* __restrict__ rounds, unsigned long long* __restrict__ counter) {
+                      float eps, int max_rounds, NaryOut out,
+                      unsigned long long* __restrict__ counter) {
   __shared__ float sT[FN_MAX_GRID];
   __shared__ float sSub[NARY_WARPS][32];
   __shared__ float sEdge[NARY_WARPS][32];
@@ -60,53 +86,87 @@ __global__ void __launch_bounds__(32 * NARY_WARPS, MINB)
   for (long e = (long)blockIdx.x * NARY_WARPS + w; e < E; e += W) {
     const bool finite = stage_rows(s0 + 16 * e, s1 + 16 * e, es);
     const float Tp = T_cap ? __ldg(T_cap + e) : INFINITY;
-    int k = -2, r = 0;
-    float a = NAN, b = NAN, rt = NAN, rp = NAN, rv = NAN;
-    if (finite) {
-      const float* dur = sT;                 // the grid, then each round's points
-      int n = grid_prefix(sT, K, Tp);
-      int wit = -1;                          // sample that proved a infeasible
-      for (;;) {
-        float t_rt = NAN, t_rp = NAN;
-        int w_out = -1;
-        const bool grid = dur == sT;
-        const int idx = edge_scan(A, ScalarCore{L, cb, wr}, es, sSplit[w], dur, n, S, false, 0.f, false, t_rt, t_rp, nsamp,
-                                  0, grid ? 1 : 2, wit, &w_out);
-        if (idx == FN_SCAN_ABORT) {          // the scan's pass bound (never expected)
-          k = FN_SCAN_ABORT;
-          break;
-        }
-        if (grid) {
-          k = idx;
-          if (idx < 0) break;
-          a = idx > 0 ? sT[idx - 1] : 0.f;
-          b = sT[idx];
-          wit = idx > 0 ? w_out : -1;
-          rt = t_rt;
-          rp = t_rp;
-        } else {
-          nary_bracket(sub, idx, w_out, t_rt, t_rp, a, b, wit, rt, rp);
-          ++r;
-        }
-        if (r >= max_rounds || !(b - a > eps)) break;
-        nary_points(sub, a, b);
-        dur = sub;
-        n = NARY_N - 1;
-      }
-      if (k >= 0) rv = warp_rho_v(A, es, b);
-    }
-    if (lane == 0) {
-      k_star[e] = k;
-      T_star[e] = k >= 0 ? b : (k == -1 ? INFINITY : NAN);   // -2 invalid, -3 aborted
-      if (T_lo) T_lo[e] = k >= 0 ? a : NAN;
-      rho3[3 * e + 0] = k >= 0 ? rt : NAN;
-      rho3[3 * e + 1] = k >= 0 ? rp : NAN;
-      rho3[3 * e + 2] = rv;
-      ok[e] = (k >= 0 && rv <= 1.f) ? 1 : 0;
-      if (rounds) rounds[e] = r;
+    NaryEdge o{-2, 0, NAN, NAN, NAN, NAN};
+    if (finite)
+      o = nary_edge(A, ScalarCore{L, cb, wr}, es, sSplit[w], sub, sT, grid_prefix(sT, K, Tp), S,
+                    eps, max_rounds, nsamp);
+    nary_write(A, es, e, o, out);
+  }
+  if (counter && lane == 0 && nsamp) atomicAdd(counter, (unsigned long long)nsamp);
+}
+
+// The same on tm_scan.cuh's block layout: runs of edges claimed by the CTA's
+// warps, the splits of a run in one pass, then an edge at a time.  A pass
+// checks 64 samples of a duration (two of the four interior probes of 32) where
+// the scalar core checks 32 (one), and finds the same first violating sample,
+// so the rounds are the scalar core's bit for bit.  The paired passes and the
+// shared splits bound it as the grid scan: 65536 edges at K = 128, S = 64, eps =
+// 1e-4 take 2.20 ms, the scalar variant 2.99.
+constexpr size_t kNarySub = TM_WARPS * 32 * sizeof(float);
+static_assert(kTmUsed + kNarySub <= kTmSmem, "the warps' points beside the scan's layout");
+__global__ void __launch_bounds__(32 * TM_WARPS, 1)
+    k_time_nary_tm(ArmK A, NaryGrid G, int K, int S, const float* __restrict__ s0,
+                   const float* __restrict__ s1, int E, const float* __restrict__ T_cap,
+                   float eps, int max_rounds, NaryOut out,
+                   unsigned long long* __restrict__ counter) {
+  extern __shared__ float4 tm_smem[];
+  const TmBlock blk(tm_smem);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  float* sT = blk.grid;
+  float* sub = reinterpret_cast<float*>(reinterpret_cast<char*>(tm_smem) + kTmUsed) + 32 * w;
+  fill_links2(A, blk.link);
+  const long per = ((long)E + gridDim.x - 1) / gridDim.x;
+  const long r_lo = std::min<long>((long)blockIdx.x * per, E), r_hi = std::min<long>(r_lo + per, E);
+  if (threadIdx.x == 0) *blk.next = 0;
+  for (int i = threadIdx.x; i < K; i += blockDim.x) sT[i] = G.T[i];
+  if (w == 0) tmem_alloc(blk.tmem, kTmCols);
+  tmem_sync_block();
+  const uint32_t tmem = *blk.tmem;
+  const PairCore<TmemStash> core = blk.core(tmem, w, lane);
+  float* es_g = blk.edges_of(w);
+  float* split_g = blk.splits_of(w);
+  unsigned nsamp = 0;
+  for (;;) {
+    int n;
+    const int first = tm_claim(blk.next, (int)(r_hi - r_lo), n);
+    if (n == 0) break;                               // warp-uniform
+    const long e0 = r_lo + first;
+    unsigned fin = 0u;
+    for (int i = 0; i < n; ++i)
+      if (stage_rows(s0 + 16 * (e0 + i), s1 + 16 * (e0 + i), es_g + 32 * i)) fin |= 1u << i;
+    split_group(A, core, es_g, split_g, n, nsamp);
+    for (int i = 0; i < n; ++i) {
+      float* es = es_g + 32 * i;
+      const float Tp = T_cap ? __ldg(T_cap + e0 + i) : INFINITY;
+      NaryEdge o{-2, 0, NAN, NAN, NAN, NAN};
+      if ((fin >> i) & 1u)
+        o = nary_edge(A, core, es, split_g + FN_SPLIT_WORDS * i, sub, sT, grid_prefix(sT, K, Tp),
+                      S, eps, max_rounds, nsamp);
+      nary_write(A, es, e0 + i, o, out);
     }
   }
   if (counter && lane == 0 && nsamp) atomicAdd(counter, (unsigned long long)nsamp);
+  tmem_sync_block();   // every warp's tensor-memory accesses precede the release
+  if (w == 0) tmem_dealloc(tmem, kTmCols);
+}
+
+static fn_status launch_nary_tm(const ArmK& A, const NaryGrid& G, int K, int S, const float* s0,
+                                const float* s1, int E, const float* T_cap, float eps,
+                                int max_rounds, const NaryOut& out, unsigned long long* counter,
+                                cudaStream_t st) {
+  static std::once_flag once[64];
+  static bool attr_ok[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::call_once(once[dev & 63], [&] {
+    attr_ok[dev & 63] = cudaFuncSetAttribute(k_time_nary_tm,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kTmSmem) == cudaSuccess;
+  });
+  if (!attr_ok[dev & 63]) return FN_ECUDA;
+  k_time_nary_tm<<<tm_blocks(E), 32 * TM_WARPS, kTmSmem, st>>>(A, G, K, S, s0, s1, E, T_cap, eps,
+                                                               max_rounds, out, counter);
+  return launch_status();
 }
 
 }  // namespace fn
@@ -135,10 +195,12 @@ extern "C" fn_status fn_time_edges_nary(const fn_arm_t* arm, const float* s0, co
   if (!s0 || !s1 || !k_star || !T_star || !rho3 || !ok) return FN_EINVAL;
   if (!aligned16(s0) || !aligned16(s1)) return FN_EINVAL;
   typedef void (*Kern)(ArmK, NaryGrid, int, int, const float*, const float*, int, const float*,
-                       float, int, int32_t*, float*, float*, float*, uint8_t*, int32_t*,
-                       unsigned long long*);
-  const int vt = tuned_variant(TUNE_EDGES_FULL, E, K, S);   // its register budget
-  const int v = vt < kEdgeVariants ? vt : kDefaultEdgeVariant;
+                       float, int, NaryOut, unsigned long long*);
+  const NaryOut out{k_star, T_star, T_lo, rho3, ok, rounds};
+  const int v = tuned_variant(TUNE_EDGES_FULL, E, K, S);    // the grid scan's core and budget
+  if (v == kPairEdgeVariant)
+    return launch_nary_tm(A, G, K, S, s0, s1, E, T_cap, eps, max_rounds, out, sample_count,
+                          (cudaStream_t)stream);
   Kern kern = v == 0 ? k_time_edges_nary<2> : (v == 1 ? k_time_edges_nary<3> : k_time_edges_nary<4>);
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NARY_WARPS, 0) !=
@@ -147,7 +209,6 @@ extern "C" fn_status fn_time_edges_nary(const fn_arm_t* arm, const float* s0, co
   const long want = ((long)E + NARY_WARPS - 1) / NARY_WARPS;
   const int blocks = (int)std::max<long>(1, std::min<long>(want, (long)per_sm * num_sms()));
   kern<<<blocks, 32 * NARY_WARPS, 0, (cudaStream_t)stream>>>(A, G, K, S, s0, s1, E, T_cap, eps,
-                                                             max_rounds, k_star, T_star, T_lo,
-                                                             rho3, ok, rounds, sample_count);
+                                                             max_rounds, out, sample_count);
   return launch_status();
 }

@@ -67,4 +67,49 @@ __device__ __forceinline__ int nary_rounds(const ArmK& A, const Core& core, floa
   return r;
 }
 
+// The grid scan of one staged edge over its n admissible durations sT and the
+// rounds after it, both through one edge_scan call site.  k: the first
+// feasible grid index (-1 none, FN_SCAN_ABORT); (a, b]: the final bracket with
+// the ratios rt, rp at b; r: rounds run.
+struct NaryEdge {
+  int k, r;
+  float a, b, rt, rp;
+};
+template <class Core>
+__device__ __forceinline__ NaryEdge nary_edge(const ArmK& A, const Core& core, float* es,
+                                              float* split, float* sub, const float* sT, int n,
+                                              int S, float eps, int max_rounds, unsigned& nsamp) {
+  NaryEdge o{-1, 0, NAN, NAN, NAN, NAN};
+  const float* dur = sT;                 // the grid, then each round's points
+  int wit = -1;                          // sample that proved a infeasible
+  for (;;) {
+    float t_rt = NAN, t_rp = NAN;
+    int w_out = -1;
+    const bool grid = dur == sT;
+    const int idx = edge_scan(A, core, es, split, dur, n, S, false, 0.f, false, t_rt, t_rp, nsamp,
+                              0, grid ? 1 : 2, wit, &w_out);
+    if (idx == FN_SCAN_ABORT) {          // the scan's pass bound (never expected)
+      o.k = FN_SCAN_ABORT;
+      break;
+    }
+    if (grid) {
+      o.k = idx;
+      if (idx < 0) break;
+      o.a = idx > 0 ? sT[idx - 1] : 0.f;
+      o.b = sT[idx];
+      wit = idx > 0 ? w_out : -1;
+      o.rt = t_rt;
+      o.rp = t_rp;
+    } else {
+      nary_bracket(sub, idx, w_out, t_rt, t_rp, o.a, o.b, wit, o.rt, o.rp);
+      ++o.r;
+    }
+    if (o.r >= max_rounds || !(o.b - o.a > eps)) break;
+    nary_points(sub, o.a, o.b);
+    dur = sub;
+    n = NARY_N - 1;
+  }
+  return o;
+}
+
 }  // namespace fn

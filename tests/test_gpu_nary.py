@@ -187,3 +187,21 @@ def test_nary_full_size_sampled(ops, orc, arm):
     sample = np.random.default_rng(12).choice(65536, 192, replace=False)
     res = _check(ops, orc, arm, s0, s1, synth.duration_grid(128), 64, 1e-4, sample=sample)
     assert res["same"].sum() >= 60
+
+
+@pytest.mark.parametrize("E,K,S,eps", [(1, 1, 2, 1e-3), (5, 33, 5, 1e-4), (257, 64, 32, 1e-3),
+                                       (2000, 128, 65, 1e-4), (300, 40, 200, 1e-5)])
+def test_paired_rounds_are_the_scalar_ones(ops, arm, E, K, S, eps):
+    """The refinement on the paired core (64 samples or two interior probes to a
+    pass) keeps the scalar core's brackets, witnesses and ratios bit for bit."""
+    s0, s1 = (torch.from_numpy(a).cuda() for a in synth.random_edges(arm, E, 61 + S))
+    grid = synth.duration_grid(K)
+    got = []
+    try:
+        for v in (2, 3):
+            ops.set_time_edges_variant(0, E, K, S, v)
+            r = ops.time_edges_nary(arm, s0, s1, grid, S, eps)
+            got.append({k: x.cpu().numpy().tobytes() for k, x in r.items()})
+    finally:
+        ops.set_time_edges_variant(0, E, K, S, 3)
+    assert got[0] == got[1]
