@@ -16,6 +16,8 @@
 
 namespace fn {
 
+using Tm = TmBlock<16>;
+
 struct GridK {
   float T[FN_MAX_GRID];
 };
@@ -71,21 +73,21 @@ __global__ void __launch_bounds__(32 * EDGE_WARPS, MINB)
 
 // The paired scan (two samples per lane, PairCore) with the per-link records
 // of the torque evaluation in tensor memory, on tm_scan.cuh's block layout
-// (one CTA of TM_WARPS warps per SM).  CTA b owns a contiguous range of the
+// (one CTA of Tm::kWarps warps per SM).  CTA b owns a contiguous range of the
 // edges, which its warps claim in runs that shrink towards the end of the
 // range (tm_claim): an edge's cost varies with the passes it needs, and
 // shrinking runs keep the warps busy until the range is done.  A warp
 // stages its run, computes the end-sample splits in one pass (split_group:
 // up to sixty (edge, end, part) items on the lanes' two halves), then scans
 // the edges one by one.
-__global__ void __launch_bounds__(32 * TM_WARPS, 1)
+__global__ void __launch_bounds__(32 * Tm::kWarps, 1)
     k_time_edges_tm(ArmK A, GridK G, int K, int S, int mode, const float* __restrict__ s0,
                     const float* __restrict__ s1, int E, const float* __restrict__ Tparam,
                     int32_t* __restrict__ k_star, float* __restrict__ T_star,
                     float* __restrict__ rho3, uint8_t* __restrict__ ok,
                     unsigned long long* __restrict__ counter) {
   extern __shared__ float4 tm_smem[];
-  const TmBlock blk(tm_smem);
+  const Tm blk(tm_smem);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float* sT = blk.grid;
   fill_links2(A, blk.link);
@@ -105,7 +107,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1)
   unsigned nsamp = 0;
   for (;;) {
     int n;
-    const int first = tm_claim(blk.next, len, n);
+    const int first = tm_claim<Tm::kWarps>(blk.next, len, n);
     if (n == 0) break;                               // warp-uniform
     const long e0 = r_lo + first;
     unsigned fin = 0u;
@@ -153,7 +155,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1)
 // full scan.  The block layout and the run claiming are those of
 // k_time_edges_tm.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(32 * TM_WARPS, 1)
+__global__ void __launch_bounds__(32 * Tm::kWarps, 1)
     k_time_window_tm(ArmK A, GridK G, int K, int S, const float* __restrict__ s0,
                      const float* __restrict__ s1, int E, const float* __restrict__ Y, int Wn,
                      float logT0, float dlog, int32_t* __restrict__ k_star,
@@ -161,7 +163,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1)
                      uint8_t* __restrict__ ok, uint8_t* __restrict__ path,
                      unsigned long long* __restrict__ counter) {
   extern __shared__ float4 tm_smem[];
-  const TmBlock blk(tm_smem);
+  const Tm blk(tm_smem);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float* sT = blk.grid;
   fill_links2(A, blk.link);
@@ -179,7 +181,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1)
   unsigned nsamp = 0;
   for (;;) {
     int n;
-    const int first = tm_claim(blk.next, len, n);
+    const int first = tm_claim<Tm::kWarps>(blk.next, len, n);
     if (n == 0) break;                               // warp-uniform
     const long e0 = r_lo + first;
     unsigned fin = 0u;
@@ -330,11 +332,11 @@ static fn_status launch_time_edges_tm(const ArmK& A, const GridK* G, int K, int 
   std::call_once(once[dev & 63], [&] {
     attr_ok[dev & 63] = cudaFuncSetAttribute(k_time_edges_tm,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTmSmem) == cudaSuccess;
+                                             (int)Tm::kSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
   static GridK empty;
-  k_time_edges_tm<<<tm_blocks(E), 32 * TM_WARPS, kTmSmem, st>>>(A, G ? *G : empty, K, S, mode, s0, s1, E,
+  k_time_edges_tm<<<tm_blocks(E), 32 * Tm::kWarps, Tm::kSmem, st>>>(A, G ? *G : empty, K, S, mode, s0, s1, E,
                                                            Tparam, k_star, T_star, rho3, ok,
                                                            counter);
   return launch_status();
@@ -352,10 +354,10 @@ static fn_status launch_time_window_tm(const ArmK& A, const GridK& G, int K, int
   std::call_once(once[dev & 63], [&] {
     attr_ok[dev & 63] = cudaFuncSetAttribute(k_time_window_tm,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTmSmem) == cudaSuccess;
+                                             (int)Tm::kSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
-  k_time_window_tm<<<tm_blocks(E), 32 * TM_WARPS, kTmSmem, st>>>(A, G, K, S, s0, s1, E, Y, W, logT0,
+  k_time_window_tm<<<tm_blocks(E), 32 * Tm::kWarps, Tm::kSmem, st>>>(A, G, K, S, s0, s1, E, Y, W, logT0,
                                                             dlog, k_star, T_star, rho3, ok, path,
                                                             counter);
   return launch_status();

@@ -26,6 +26,8 @@
 
 namespace fn {
 
+using Tm = TmBlock<16>;
+
 struct NaryGrid {
   float T[FN_MAX_GRID];
 };
@@ -102,18 +104,18 @@ __global__ void __launch_bounds__(32 * NARY_WARPS, MINB)
 // so the rounds are the scalar core's bit for bit.  The paired passes and the
 // shared splits bound it as the grid scan: 65536 edges at K = 128, S = 64, eps =
 // 1e-4 take 2.20 ms, the scalar variant 2.99.
-constexpr size_t kNarySub = TM_WARPS * 32 * sizeof(float);
-static_assert(kTmUsed + kNarySub <= kTmSmem, "the warps' points beside the scan's layout");
-__global__ void __launch_bounds__(32 * TM_WARPS, 1)
+constexpr size_t kNarySub = Tm::kWarps * 32 * sizeof(float);
+static_assert(Tm::kUsed + kNarySub <= Tm::kSmem, "the warps' points beside the scan's layout");
+__global__ void __launch_bounds__(32 * Tm::kWarps, 1)
     k_time_nary_tm(ArmK A, NaryGrid G, int K, int S, const float* __restrict__ s0,
                    const float* __restrict__ s1, int E, const float* __restrict__ T_cap,
                    float eps, int max_rounds, NaryOut out,
                    unsigned long long* __restrict__ counter) {
   extern __shared__ float4 tm_smem[];
-  const TmBlock blk(tm_smem);
+  const Tm blk(tm_smem);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   float* sT = blk.grid;
-  float* sub = reinterpret_cast<float*>(reinterpret_cast<char*>(tm_smem) + kTmUsed) + 32 * w;
+  float* sub = reinterpret_cast<float*>(reinterpret_cast<char*>(tm_smem) + Tm::kUsed) + 32 * w;
   fill_links2(A, blk.link);
   const long per = ((long)E + gridDim.x - 1) / gridDim.x;
   const long r_lo = std::min<long>((long)blockIdx.x * per, E), r_hi = std::min<long>(r_lo + per, E);
@@ -128,7 +130,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1)
   unsigned nsamp = 0;
   for (;;) {
     int n;
-    const int first = tm_claim(blk.next, (int)(r_hi - r_lo), n);
+    const int first = tm_claim<Tm::kWarps>(blk.next, (int)(r_hi - r_lo), n);
     if (n == 0) break;                               // warp-uniform
     const long e0 = r_lo + first;
     unsigned fin = 0u;
@@ -161,10 +163,10 @@ static fn_status launch_nary_tm(const ArmK& A, const NaryGrid& G, int K, int S, 
   std::call_once(once[dev & 63], [&] {
     attr_ok[dev & 63] = cudaFuncSetAttribute(k_time_nary_tm,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)kTmSmem) == cudaSuccess;
+                                             (int)Tm::kSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
-  k_time_nary_tm<<<tm_blocks(E), 32 * TM_WARPS, kTmSmem, st>>>(A, G, K, S, s0, s1, E, T_cap, eps,
+  k_time_nary_tm<<<tm_blocks(E), 32 * Tm::kWarps, Tm::kSmem, st>>>(A, G, K, S, s0, s1, E, T_cap, eps,
                                                                max_rounds, out, counter);
   return launch_status();
 }

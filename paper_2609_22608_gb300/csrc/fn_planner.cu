@@ -49,6 +49,8 @@
 
 namespace fn {
 
+using Tm = TmBlock<12>;
+
 // best plans of a problem's tree: (J, z) best first, at most n_fit entries
 struct Archive {
   int n;
@@ -1234,10 +1236,10 @@ __device__ __forceinline__ void goal_edge_fail(const PlanDev& D, const GoalEdge&
   D.e_rv[g.ei] = NAN;
   D.e_k[g.ei] = -1;
 }
-__global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_goal_edges(PlanDev D, ArmK A) {
+__global__ void __launch_bounds__(32 * Tm::kWarps, 1) k_plan_goal_edges(PlanDev D, ArmK A) {
   pdl_begin();
   extern __shared__ float4 tm_smem[];
-  const TmBlock blk(tm_smem);
+  const Tm blk(tm_smem);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const Sched* S = D.sched;
   const int E = S->goal_off[D.P];
@@ -1245,7 +1247,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_goal_edges(PlanDev D,
   const int per = (E + (int)gridDim.x - 1) / (int)gridDim.x;
   const int r_lo = min((int)blockIdx.x * per, E), r_hi = min(r_lo + per, E);
   int* list = reinterpret_cast<int*>(blk.split);   // the live edges (the splits' room)
-  constexpr int kChunk = (int)(kTmSplit / sizeof(int));
+  constexpr int kChunk = (int)(Tm::kSplit / sizeof(int));
   int* s_n = blk.aux;
   if (w == 0) tmem_alloc(blk.tmem, kTmCols);
   tmem_sync_block();
@@ -1278,7 +1280,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_goal_edges(PlanDev D,
       int g0 = 0, gs = 0;
       if (lane == 0) {
         const int seen = atomicAdd(blk.next, 0);
-        gs = min(8, max(1, (nl - seen) / (2 * TM_WARPS)));
+        gs = min(8, max(1, (nl - seen) / (2 * Tm::kWarps)));
         g0 = atomicAdd(blk.next, gs);
       }
       g0 = __shfl_sync(0xffffffffu, g0, 0);
@@ -1365,11 +1367,11 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_goal_edges(PlanDev D,
 // where an iteration's edges are few enough that the stages' chain of
 // launches, not their work, sets the time.  The CTA that finishes last
 // empties the dynamics list for the next body.
-__global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_edges_tm(PlanDev D, ArmK A,
+__global__ void __launch_bounds__(32 * Tm::kWarps, 1) k_plan_edges_tm(PlanDev D, ArmK A,
                                                                    GridKP Gr) {
   pdl_begin();
   extern __shared__ float4 tm_smem[];
-  const TmBlock blk(tm_smem);
+  const Tm blk(tm_smem);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   Sched* S = D.sched;
   const int E = min(S->n_dyn, D.Emax);
@@ -1388,7 +1390,7 @@ __global__ void __launch_bounds__(32 * TM_WARPS, 1) k_plan_edges_tm(PlanDev D, A
   unsigned nsplit = 0, nscan = 0;
   for (;;) {
     int n;
-    const int first = tm_claim(blk.next, r_hi - r_lo, n);
+    const int first = tm_claim<Tm::kWarps>(blk.next, r_hi - r_lo, n);
     if (n == 0) break;                               // warp-uniform
     const int32_t* run = D.dyn_list + r_lo + first;
     unsigned fin = 0u;
@@ -2862,9 +2864,9 @@ static bool plan_tm_ready() {
   std::call_once(once[dev & 63], [&] {
     ok[dev & 63] =
         cudaFuncSetAttribute(k_plan_edges_tm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kTmSmem) == cudaSuccess &&
+                             (int)Tm::kSmem) == cudaSuccess &&
         cudaFuncSetAttribute(k_plan_goal_edges, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)kTmSmem) == cudaSuccess &&
+                             (int)Tm::kSmem) == cudaSuccess &&
         cudaFuncSetAttribute(k_plan_knn_mins, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              kPlanKnnSmem) == cudaSuccess;
   });
@@ -2909,7 +2911,7 @@ static void enqueue_front(fn_planner* pl, unsigned flags, cudaStream_t st, Mark&
   };
   auto goal_edges = [&](cudaStream_t s) {   // after the goal queries' parent search
     if (!D.goal_split) return;
-    pl_launch_pdl(s != pl->side, k_plan_goal_edges, num_sms(), 32 * TM_WARPS, kTmSmem, s, D,
+    pl_launch_pdl(s != pl->side, k_plan_goal_edges, num_sms(), 32 * Tm::kWarps, Tm::kSmem, s, D,
                   pl->arm);
     trace(pl, s, "k_plan_goal_edges");
   };
@@ -3033,7 +3035,7 @@ static void enqueue_edges(fn_planner* pl, int v, int blocks, cudaStream_t st, Ma
   }
   if (v == kPairEdgeVariant && plan_tm_ready()) {   // the warp-per-edge body
     mark(4);
-    pl_launch(k_plan_edges_tm, num_sms(), 32 * TM_WARPS, kTmSmem, st, D, pl->arm, pl->grid);
+    pl_launch(k_plan_edges_tm, num_sms(), 32 * Tm::kWarps, Tm::kSmem, st, D, pl->arm, pl->grid);
     trace(pl, st, "k_plan_edges_tm");
     mark(5);
     return;

@@ -4,9 +4,10 @@
 // of 32 bits); warp w may access only lane quarter w % 4 (lanes 32 (w % 4)
 // .. 32 (w % 4) + 31), so thread t of the warp owns row 32 (w % 4) + t of
 // every allocated column.  The paired torque evaluation keeps its per-link
-// records there instead of in shared memory: 7 links x 10 float2 = 140
-// columns per warp, link j's first 16 words at column 16 j and its last 4 at
-// 112 + 4 j, so every access is aligned to its own width.
+// records there instead of in shared memory: the first six links (the last
+// one's record stays in registers) x 10 float2 = 120 columns per warp, link j's
+// first 16 words at column 16 j and its last 4 at 96 + 4 j, so every access is
+// aligned to its own width.
 #pragma once
 
 #include <stdint.h>
@@ -15,7 +16,7 @@
 
 namespace fn {
 
-#define FN_TM_COLS_PER_WARP 144   // 140 used, rounded to a multiple of 16
+#define FN_TM_COLS_PER_WARP 128   // 120 used, rounded to a multiple of 16
 
 // alloc / dealloc are warp-collective: one warp of the CTA calls both
 __device__ __forceinline__ void tmem_alloc(uint32_t* s_addr, uint32_t ncols) {
@@ -41,7 +42,7 @@ __device__ __forceinline__ void tmem_sync_block() {
 struct TmemStash {
   uint32_t base;   // lane-quarter row and first column of this warp's block
   __device__ __forceinline__ void store(int j, const float2 (&r)[FN_REC2]) const {
-    const uint32_t a = base + 16u * (uint32_t)j, b = base + 112u + 4u * (uint32_t)j;
+    const uint32_t a = base + 16u * (uint32_t)j, b = base + 96u + 4u * (uint32_t)j;
     asm volatile(
         "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
         "{%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16};\n" ::"r"(a),
@@ -58,7 +59,7 @@ struct TmemStash {
     asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
   }
   __device__ __forceinline__ void load(int j, float2 (&r)[FN_REC2]) const {
-    const uint32_t a = base + 16u * (uint32_t)j, b = base + 112u + 4u * (uint32_t)j;
+    const uint32_t a = base + 16u * (uint32_t)j, b = base + 96u + 4u * (uint32_t)j;
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
         "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n"
