@@ -7,8 +7,11 @@
 //   fn_check_edges_full   the full-resolution recheck of a plan's edges at
 //                         their own durations: all three ratios of Def.
 //                         "Feasibility Check" over S samples and the
-//                         clearance over S_clear points; one warp per edge.
+//                         clearance over S_clear points; one to eight warps
+//                         per edge.
 #include <cuda_runtime.h>
+
+#include <mutex>
 
 #include "edge_core.cuh"
 #include "fn_internal.h"
@@ -115,52 +118,71 @@ __global__ void __launch_bounds__(128) k_controller(ArmK A, CtrlK L, int B,
   }
 }
 
-#define CHECK_WARPS 3  // as the grid scan: static shared memory within 48 KB
-
-// one warp per edge: the exact fixed-duration check (all S samples), rho_v,
-// then the clearance (lane = point)
-__global__ void __launch_bounds__(32 * CHECK_WARPS, 3)
+// The exact fixed-duration check (all S samples), rho_v, then the clearance
+// (lane = point), by `group` warps of the CTA to an edge: warp r of a group
+// takes the batches of 32 samples r, r + group, ... and of points likewise from
+// the other end, and the maxima meet in shared memory.  A recheck is a few
+// edges at a high resolution, so the chain of an edge's passes sets its time: 16
+// edges at S = 256 with five obstacles take 13 us with eight warps each, and
+// took 26 with one.
+#define CHECK_WARPS 8
+constexpr size_t kCheckWarp = (FN_CUBIC_WORDS + FN_LINK_WORDS + 1) * 32 * sizeof(float);
+constexpr size_t kCheckSmem = CHECK_WARPS * (kCheckWarp + 4 * sizeof(float)) +
+                              7 * FN_LINK_F4 * sizeof(float4);
+__global__ void __launch_bounds__(32 * CHECK_WARPS, 2)
     k_check_edges(ArmK A, fn_problem_t P, int E, const int* __restrict__ E_dev, int S,
-                  int S_clear, float margin, const float* __restrict__ s0,
+                  int S_clear, float margin, int group, const float* __restrict__ s0,
                   const float* __restrict__ s1, const float* __restrict__ Tv,
                   float* __restrict__ rho3, float* __restrict__ clearance,
                   uint8_t* __restrict__ ok) {
-  __shared__ float sEdge[CHECK_WARPS][32];
-  __shared__ float sCoef[CHECK_WARPS][FN_CUBIC_WORDS * 32];
-  __shared__ float sWr[CHECK_WARPS][FN_LINK_WORDS * 32];
-  __shared__ float4 sLink[7 * FN_LINK_F4];
+  extern __shared__ float4 check_smem[];
+  float4* sLink = check_smem;
+  float* sPart = reinterpret_cast<float*>(sLink + 7 * FN_LINK_F4);   // [CHECK_WARPS][4]
   fill_links(A, sLink);
   __syncthreads();
   if (E_dev) E = min(E, max(*E_dev, 0));
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  float* es = sEdge[w];
-  const CubicLane cb{&sCoef[w][lane]};
-  const LaneLink wr{&sWr[w][lane]};
-  const LinkTab L{sLink};
-  unsigned nsamp = 0;
-  for (long e = (long)blockIdx.x * CHECK_WARPS + w; e < E; e += (long)gridDim.x * CHECK_WARPS) {
+  const int r = w % group, g = w / group, ng = CHECK_WARPS / group;
+  float* mine = sPart + 4 * CHECK_WARPS + (kCheckWarp / sizeof(float)) * w;
+  float* es = mine + (FN_CUBIC_WORDS + FN_LINK_WORDS) * 32;
+  const CubicLane cb{mine + lane};
+  const ScalarCore core{LinkTab{sLink}, cb, LaneLink{mine + FN_CUBIC_WORDS * 32 + lane}};
+  auto group_sync = [&] {
+    if (group == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;\n" ::"r"(1 + g), "r"(32 * group) : "memory");
+  };
+  for (long e = (long)blockIdx.x * ng + g; e < E; e += (long)gridDim.x * ng) {   // group-uniform
     const bool finite = stage_rows(s0 + 16 * e, s1 + 16 * e, es);
     const float T = Tv[e];
     if (!finite || !(isfinite(T) && T > 0.f)) {
-      if (lane == 0) {
+      if (r == 0 && lane == 0) {
         rho3[3 * e] = rho3[3 * e + 1] = rho3[3 * e + 2] = NAN;
         clearance[e] = NAN;
         ok[e] = 0;
       }
       continue;
     }
-    float rt = NAN, rp = NAN;
-    if (edge_scan(A, ScalarCore{L, cb, wr}, es, nullptr, nullptr, 0, S, true, T, true, rt, rp, nsamp) ==
-        FN_SCAN_ABORT)
-      rt = rp = NAN;   // the scan's pass bound (never expected): not ok
-    const float rv = warp_rho_v(A, es, T);
-    float cl = INFINITY;
+    float mt = 0.f, mp = 0.f, mc = INFINITY;
+    cubic_store_shared<true>(cb, es, T, 32);
+#pragma unroll 1
+    for (int b = r; 32 * b < S; b += group) {
+      const int s = 32 * b + lane;
+      float rx = 0.f, px = 0.f;
+      core.eval(A, dup2(sample_u(s, S)), dup2(1.f), dup2(1.f),
+                [&](int, float2 tau, float2 v, float inv_tau) {
+                  rx = fmaxf(rx, fabsf(tau.x) * inv_tau);
+                  px = fmaf(tau.x, v.x, px);
+                }, lane);
+      if (s < S) {
+        mt = fmaxf(mt, rx);
+        mp = fmaxf(mp, fabsf(px) * A.inv_w);
+      }
+    }
     if (P.n_obs > 0) {
       Cubic c;
       cubic_coef_sh<true>(es, T, c);
-      float mc = INFINITY;
 #pragma unroll 1
-      for (int s = lane; s < S_clear; s += 32) {
+      for (int s = 32 * (group - 1 - r) + lane; s < S_clear; s += 32 * group) {
         const float u = sample_u(s, S_clear);
         float q[7];
 #pragma unroll
@@ -170,15 +192,33 @@ __global__ void __launch_bounds__(32 * CHECK_WARPS, 3)
         }
         mc = fminf(mc, config_clearance(A, q, P));
       }
-      cl = -warp_max(-mc);
     }
+    mt = warp_max(mt);
+    mp = warp_max(mp);
+    mc = -warp_max(-mc);
     if (lane == 0) {
-      rho3[3 * e] = rt;
-      rho3[3 * e + 1] = rp;
-      rho3[3 * e + 2] = rv;
-      clearance[e] = cl;
-      ok[e] = (rt <= 1.f && rp <= 1.f && rv <= 1.f && (P.n_obs == 0 || cl >= margin)) ? 1 : 0;
+      sPart[4 * w] = mt;
+      sPart[4 * w + 1] = mp;
+      sPart[4 * w + 2] = mc;
     }
+    group_sync();
+    if (r == 0) {
+      float rt = 0.f, rp = 0.f, cl = INFINITY;
+      for (int i = 0; i < group; ++i) {
+        rt = fmaxf(rt, sPart[4 * (w + i)]);
+        rp = fmaxf(rp, sPart[4 * (w + i) + 1]);
+        cl = fminf(cl, sPart[4 * (w + i) + 2]);
+      }
+      const float rv = warp_rho_v(A, es, T);
+      if (lane == 0) {
+        rho3[3 * e] = rt;
+        rho3[3 * e + 1] = rp;
+        rho3[3 * e + 2] = rv;
+        clearance[e] = cl;
+        ok[e] = (rt <= 1.f && rp <= 1.f && rv <= 1.f && (P.n_obs == 0 || cl >= margin)) ? 1 : 0;
+      }
+    }
+    group_sync();   // the partial maxima are read
   }
 }
 
@@ -232,9 +272,22 @@ extern "C" fn_status fn_check_edges_full(const fn_arm_t* arm, const float* s0, c
   if (E == 0) return FN_OK;
   if (!s0 || !s1 || !T || !rho3 || !clearance || !ok) return FN_EINVAL;
   if (!aligned16(s0) || !aligned16(s1)) return FN_EINVAL;
-  const long want = ((long)E + CHECK_WARPS - 1) / CHECK_WARPS;
-  const int blocks = (int)std::max<long>(1, std::min<long>(want, 3L * num_sms()));
-  k_check_edges<<<blocks, 32 * CHECK_WARPS, 0, (cudaStream_t)stream>>>(
-      A, P, E, E_dev, S, S_clear, margin, s0, s1, T, rho3, clearance, ok);
+  static std::once_flag once[64];
+  static bool attr_ok[64];
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::call_once(once[dev & 63], [&] {
+    attr_ok[dev & 63] = cudaFuncSetAttribute(k_check_edges,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)kCheckSmem) == cudaSuccess;
+  });
+  if (!attr_ok[dev & 63]) return FN_ECUDA;
+  // as many warps to an edge as it has batches of 32 samples
+  int group = 1;
+  while (group < CHECK_WARPS && 32 * group < S) group *= 2;
+  const long want = ((long)E * group + CHECK_WARPS - 1) / CHECK_WARPS;
+  const int blocks = (int)std::max<long>(1, std::min<long>(want, 2L * num_sms()));
+  k_check_edges<<<blocks, 32 * CHECK_WARPS, kCheckSmem, (cudaStream_t)stream>>>(
+      A, P, E, E_dev, S, S_clear, margin, group, s0, s1, T, rho3, clearance, ok);
   return launch_status();
 }

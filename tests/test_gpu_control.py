@@ -230,3 +230,19 @@ def test_incumbent_path_and_recheck(orc, arm):
     res = {k: path[k][:L] for k in ("rho3", "clearance", "ok")}
     ref = _check_recheck(orc, arm, s0, s1, T, 256, 64, obs, 0.02, res)
     assert ref["ok"][0] == 0 and np.isfinite(ref["rho3"][1]).all()
+
+
+@pytest.mark.parametrize("E", [1, 5, 700])
+@pytest.mark.parametrize("S", [2, 32, 33, 64, 65, 129, 200, 256])
+def test_recheck_is_the_fixed_check(ops, arm, E, S):
+    """One, two, four and eight warps to an edge, with whole and partial batches
+    of samples: the ratios of the fixed-duration check bit for bit, and the
+    clearance of fewer points is never below that of all of them."""
+    s0, s1 = synth.random_edges(arm, E, 71 + S)
+    T = np.random.default_rng(S).uniform(0.1, 1.6, E).astype(np.float32)
+    obs = synth.obstacles(5, 3)
+    r = ops.check_edges_full(arm, dev(s0), dev(s1), dev(T), S, 65, obs, 0.02)
+    f = ops.time_edges(arm, dev(s0), dev(s1), S=S, mode=ops.FN_MODE_FIXED, T_fixed=dev(T))
+    assert r["rho3"].cpu().numpy().tobytes() == f["rho3"].cpu().numpy().tobytes()
+    half = ops.check_edges_full(arm, dev(s0), dev(s1), dev(T), S, 33, obs, 0.02)
+    assert (half["clearance"] >= r["clearance"]).all()   # every second one of the 65
