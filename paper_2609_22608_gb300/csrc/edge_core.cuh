@@ -335,7 +335,9 @@ __device__ __forceinline__ void split_group(const ArmK& A, const Core& core, flo
 //              lowest survivors not yet probed there: packed (wmode 0), the
 //              lowest eight survivors x 4 NS samples in one pass, lane = 4 i +
 //              j (x: sample j, y: sample j + 4); otherwise lanes = durations,
-//              four samples, NS per pass
+//              four samples, NS per pass (the paired core takes up to 16
+//              survivors x 4 samples in one, lane = 2 i + j, x: sample j, y:
+//              sample j + 2)
 //   PROBE_W  : (wmode 2) one sample, the witness, at the remaining survivors
 //              (plain coefficients): after a failed verify, that duration's
 //              first violating sample; on the first chunk, the caller's w_in
@@ -454,6 +456,10 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
         ay = NS == 2 && ax;
         sx = mid_probe_index(lane & 3, S, nmid);
         sy = mid_probe_index((lane & 3) + 4, S, nmid);
+      } else if (mode == PROBE_MID && mj < 0) {   // up to 16 survivors x 4 samples
+        ax = ay = cdur >= 0;
+        sx = mid_probe_index(lane & 1, S, nmid);
+        sy = mid_probe_index((lane & 1) + 2, S, nmid);
       } else if (mode == PROBE_MID) {   // lanes = durations, NS samples per pass
         ax = ((sel & cand) >> lane) & 1u;
         ay = NS == 2 && ax;
@@ -512,6 +518,16 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
         for (int i = 0; i < ns; ++i)
           if (((okb >> (4 * i)) & 0xFu) != 0xFu) failed |= 1u << nth_bit(sel, i);
         cand &= ~failed;
+        mpr |= sel;
+        decide = true;
+      } else if (mode == PROBE_MID && mj < 0) {
+        // this lane's duration: the first of its four samples that fails
+        const int i = 2 * __popc(sel & ((1u << lane) - 1u)) & 31;
+        const int f = !((ok_x >> i) & 1u) ? 0 : !((ok_x >> (i + 1)) & 1u) ? 1
+                      : !((ok_y >> i) & 1u) ? 2 : !((ok_y >> (i + 1)) & 1u) ? 3 : -1;
+        const bool out = ((sel >> lane) & 1u) && f >= 0;
+        if (out) kill = mid_probe_index(f, S, nmid);
+        cand &= ~__ballot_sync(0xffffffffu, out);
         mpr |= sel;
         decide = true;
       } else if (mode == PROBE_MID) {
@@ -584,7 +600,13 @@ __device__ __forceinline__ int edge_scan(const ArmK& A, const Core& core, float*
         cdur = i < __popc(sel) ? base + nth_bit(sel, i) : -1;
       } else {
         sel = cand & ~mpr;
-        cdur = ((sel >> lane) & 1u) ? base + lane : -1;
+        if (NS == 2 && __popc(sel) <= 16) {   // the same samples in one pass
+          mj = -1;
+          const int i = lane >> 1;
+          cdur = i < __popc(sel) ? base + nth_bit(sel, i) : -1;
+        } else {
+          cdur = ((sel >> lane) & 1u) ? base + lane : -1;
+        }
       }
       coef = COEF_PLAIN;
       continue;
