@@ -128,7 +128,7 @@ typedef struct {
  *   ok         u8: 1 iff the edge is feasible at T_star including rho_v.
  * Schedule: unless fn_autotune_time_edges chose otherwise for the shape, one
  * warp per edge with two samples per lane (paired FP32 arithmetic) and the
- * torque recursion's per-link records in tensor memory (one CTA of 12 warps
+ * torque recursion's per-link records in tensor memory (one CTA of 16 warps
  * per SM, which allocates all of the SM's 512 tensor-memory columns for the
  * duration of the call; a kernel of another stream holding columns on the
  * same SM delays it until they are released).

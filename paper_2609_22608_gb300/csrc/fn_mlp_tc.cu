@@ -7,8 +7,9 @@
 //   columns) in tensor memory; after each layer sixteen warps read it back
 //   (tcgen05.ld; warp w takes lane quarter w % 4 and 64 of the 256 columns),
 //   add the bias, apply ReLU, round to bf16 and write the next A operand;
-//   layer 4 (256 -> 2) runs on the CUDA cores in the last epilogue.  Same rounding points as the mma.sync path (bf16
-//   operands, FP32 accumulation, bias then ReLU then bf16).
+//   layer 4 (256 -> 2) runs on the CUDA cores in the last epilogue.  Same
+//   rounding points as the layer-by-layer reference (bf16 operands, FP32
+//   accumulation, bias then ReLU then bf16).
 //
 // One thread issues the copies and the MMAs; completion is tracked by
 // mbarriers (transaction bytes for the copies, tcgen05.commit for the MMAs).
