@@ -1190,9 +1190,11 @@ __global__ void __launch_bounds__(128, PL_VSEL_BLOCKS) k_plan_vselect(PlanDev D,
 // Goal edges (Algorithm 1's goal branch: the cubic from parent p to a
 // decoded goal at the fixed duration T_p = T_req - t(p)) checked apart from
 // the packed body: every (goal candidate, parent slot) of the round, on the
-// paired core with its records in tensor memory (tm_scan.cuh).  CTA b owns a
-// contiguous range of the queue's goal part (goal_off).  Its threads decode
-// the range a chunk at a time, one edge each: an edge whose parent is
+// paired core with its records in tensor memory (tm_scan.cuh).  CTA b owns
+// every gridDim.x-th run of 32 of the queue's goal part (goal_off): the live
+// edges cluster by problem and parent slot, and a contiguous range each left the
+// fullest SM twice the work of the mean (64 problems: 112 us, now 62).  Its
+// threads decode the runs a chunk at a time, one edge each: an edge whose parent is
 // missing, whose candidate did not decode, or whose T_p is not positive and
 // finite is decided there without dynamics (as k_plan_eprep decides it), the
 // others join the CTA's list of live edges.  The warps then claim the live
@@ -1244,8 +1246,9 @@ __global__ void __launch_bounds__(32 * Tm::kWarps, 1) k_plan_goal_edges(PlanDev 
   const Sched* S = D.sched;
   const int E = S->goal_off[D.P];
   fill_links2(A, blk.link);
-  const int per = (E + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int r_lo = min((int)blockIdx.x * per, E), r_hi = min(r_lo + per, E);
+  // the CTA's edges: every gridDim.x-th run of 32
+  const int runs = (E + 31) / 32, bx = (int)blockIdx.x, nb = (int)gridDim.x;
+  const int len = bx < runs ? 32 * ((runs - 1 - bx) / nb + 1) : 0;
   int* list = reinterpret_cast<int*>(blk.split);   // the live edges (the splits' room)
   constexpr int kChunk = (int)(Tm::kSplit / sizeof(int));
   int* s_n = blk.aux;
@@ -1255,14 +1258,14 @@ __global__ void __launch_bounds__(32 * Tm::kWarps, 1) k_plan_goal_edges(PlanDev 
   const PairCore<TmemStash> core = blk.core(tmem, w, lane);
   float* es_g = blk.edges_of(w);
   unsigned nscan = 0;
-  for (int c0 = r_lo; c0 < r_hi; c0 += kChunk) {     // CTA-uniform
-    const int c1 = min(c0 + kChunk, r_hi);
+  for (int c0 = 0; c0 < len; c0 += kChunk) {         // CTA-uniform
+    const int c1 = min(c0 + kChunk, len);
     if (threadIdx.x == 0) *s_n = 0;
     __syncthreads();
     for (int base = c0; base < c1; base += blockDim.x) {
-      const int x = base + threadIdx.x;
+      const int it = base + threadIdx.x, x = 32 * ((it >> 5) * nb + bx) + (it & 31);
       bool lv = false;
-      if (x < c1) {
+      if (it < c1 && x < E) {
         const GoalEdge g = decode_goal_edge(D, S, x);
         lv = g.live;
         if (!lv) goal_edge_fail(D, g);
