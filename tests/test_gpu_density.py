@@ -185,3 +185,46 @@ def test_density_arguments(P, arm):
     th0, _, _ = pl.get_density(0)
     assert th0["C"] == 0 and th0["w_u"] == pytest.approx(0.25)
     pl.close()
+
+
+@pytest.mark.parametrize("n_fit", [1, 31, 33, 64])
+def test_archive_of_a_round_of_many_plans(P, orc, arm, n_fit):
+    """A round that appends more rendezvous nodes than the archive's insertion
+    looks at in one turn, many of equal J, into archives of less than, about and
+    twice a warp's lanes: best first, an earlier node before an equal one."""
+    from tests.test_gpu_planner import K_GRID, S_COLL, make_case
+    case = make_case(arm, orc, 41, N=150, n_free=32)
+    states, t, parent = case["tree"]
+    G = case["n_goal"]
+    g = case["cand"][:G].astype(np.float64)
+    appr = g.copy()
+    appr[:, :7] = g[:, :7] - 0.1 * g[:, 8:15]
+    states = np.concatenate([states, appr.astype(np.float32)])
+    t = np.concatenate([t, (case["T_req"] - np.float32(0.1)).astype(np.float32)])
+    parent = np.concatenate([parent, np.zeros(G, parent.dtype)])
+    N, B = states.shape[0], 8192
+    rng = np.random.default_rng(7)
+    pick = np.arange(B) % G
+    cand = np.ascontiguousarray(case["cand"][:G][pick])
+    vrel = rng.choice(np.linspace(0.5, 2.0, 40).astype(np.float32), B)
+    zs = rng.uniform(0, 1, (B, 9)).astype(np.float32)
+    pl = P.Planner(arm, P=1, n_cap=N + B + 8, b_max=B, k=5, K=K_GRID, S=S_COLL, S_clear=8)
+    pl.set_sampler(n_fit=n_fit)
+    prob = P.problem_struct(case["pr"], B, B, root=case["root"])
+    pl.reset([prob])
+    pl.load_tree(0, states, t, parent)
+    pl.set_candidates(0, cand, B, case["T_req"][pick], vrel)
+    pl.set_candidate_params(0, zs)
+    pl.iterate([prob], 0, P.FN_PLAN_EXTERNAL | P.FN_PLAN_DENSITY)
+    _, aJ, aZ = pl.get_density(0)
+    tree = pl.get_tree(0)
+    pl.close()
+    J = tree["J"][N:tree["n"]]
+    attached = {x.tobytes() for x in tree["states"][N:tree["n"]]}
+    of = [b for b in range(B) if cand[b].tobytes() in attached]   # copies of a goal fare alike
+    assert len(of) == len(J) > 1024
+    arc = []
+    for Jv, b in zip(J, of):
+        arc = OD.archive_insert(arc, float(Jv), zs[b], n_fit)
+    assert np.array_equal(aJ, np.array([j for j, _ in arc], np.float32))
+    assert np.array_equal(aZ, np.array([z for _, z in arc], np.float32))
