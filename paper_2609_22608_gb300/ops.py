@@ -7,6 +7,7 @@ returns the output tensors.  All arithmetic runs in the library's kernels.
 from __future__ import annotations
 
 import ctypes as C
+from contextlib import nullcontext
 
 import numpy as np
 import torch
@@ -26,6 +27,12 @@ def _ptr(t):
 def _stream(stream=None):
     s = stream if stream is not None else torch.cuda.current_stream()
     return C.c_void_p(s.cuda_stream)
+
+
+def _torch_stream(stream, device):
+    if isinstance(stream, torch.cuda.Stream):
+        return stream
+    return torch.cuda.ExternalStream(stream.cuda_stream, device=device)
 
 
 def _states(x, name):
@@ -220,7 +227,8 @@ def knn_workspace_bytes(B, N, k) -> int:
 def knn_tree(tree, queries, k, w_vel, first=1, N=None, workspace=None, out=None, stream=None):
     """fn_knn_tree: (idx i32 [B][k], d2 f32 [B][k]).  `workspace` may be a
     uint8 CUDA tensor of knn_workspace_bytes(B, N, k) bytes; by default one is
-    allocated with torch for the call."""
+    allocated with torch for the call, as memory of the stream that the call
+    runs on."""
     _states(queries, "queries")
     B = queries.shape[0]
     if N is None:
@@ -228,9 +236,16 @@ def knn_tree(tree, queries, k, w_vel, first=1, N=None, workspace=None, out=None,
     if out is None:
         out = (torch.empty(B, k, dtype=torch.int32, device=queries.device),
                torch.empty(B, k, dtype=torch.float32, device=queries.device))
+        if stream is not None:   # a result dropped early is still written to
+            for o in out:
+                o.record_stream(_torch_stream(stream, queries.device))
     need = knn_workspace_bytes(B, N, k)
     if workspace is None and need > 0:
-        workspace = torch.empty(need + 256, dtype=torch.uint8, device=queries.device)
+        # its last reference goes on return: as memory of the call's own stream
+        # it is given to nobody else before the search is done with it
+        side = None if stream is None else _torch_stream(stream, queries.device)
+        with torch.cuda.stream(side) if side else nullcontext():
+            workspace = torch.empty(need + 256, dtype=torch.uint8, device=queries.device)
     ws_ptr, ws_bytes = None, 0
     if workspace is not None:
         base = workspace.data_ptr()

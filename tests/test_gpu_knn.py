@@ -116,3 +116,28 @@ def test_knn_filter_is_the_scan(ops, arm, kind, B, N, k, first):
     ri, rd = _scan(t, q, k, first)
     assert torch.equal(idx, ri)
     assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
+
+
+def test_knn_on_side_streams(ops, arm):
+    """Searches queued on two busy side streams, their workspaces left to the
+    call: what the current stream and the other side stream allocate and write
+    meanwhile must not be theirs."""
+    B, N, k = 300, 700, 8                     # a tree that the filter takes
+    t = [dev(synth.random_states(arm, N, 70 + i)) for i in range(2)]
+    q = [dev(synth.random_states(arm, B, 80 + i)) for i in range(2)]
+    ref = [_scan(t[i], q[i], k, 1) for i in range(2)]
+    need = ops.knn_workspace_bytes(B, N, k)
+    assert need > 0
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    got = []
+    for _ in range(4):
+        for i, s in enumerate(streams):
+            with torch.cuda.stream(s):
+                torch.cuda._sleep(1_000_000)  # the search waits; the host goes on
+            got.append((i, ops.knn_tree(t[i], q[i], k, 0.1, stream=s)))
+            torch.full((need + 256,), 0xFF, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    for i, (idx, d2) in got:
+        assert torch.equal(idx, ref[i][0])
+        assert torch.equal(d2.view(torch.int32), ref[i][1].view(torch.int32))
