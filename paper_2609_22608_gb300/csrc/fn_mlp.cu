@@ -188,12 +188,11 @@ struct fn_mlp {
   float* grads;   // gW, gb and the loss in one piece
   size_t n_grads;
   float* loss;    // [1]
-  // the weights packed for tcgen05 (refreshed lazily after any weight change;
-  // `packed` matrices: 3, with the transposes 5) and the kernels' error flag
+  // the weights packed for tcgen05 (with every change of the weights, on its
+  // stream) and the kernels' error flag
   bf16* W1p;      // [16 KB]
   bf16* Wp;       // [512 KB]
   int* tc_err;    // [1]
-  int packed;
   std::vector<void*> allocs;
 };
 
@@ -208,6 +207,14 @@ extern "C" fn_status fn_mlp_destroy(fn_mlp_t* m) {
   for (void* p : m->allocs) cudaFree(p);
   delete m;
   return FN_OK;
+}
+
+// The packed copies of the weights, after every change of these on the stream
+// of the change: whoever may use the new weights may use them packed, on any
+// stream.  (Packed at their first use instead, they were written on that
+// call's stream, of which a use on another one knew nothing.)
+static void mlp_pack(fn_mlp* m, cudaStream_t st) {
+  mlp_tc_pack(m->Wb[0], m->Wb[1], m->Wb[2], m->W1p, m->Wp, st);
 }
 
 extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_mlp_t** out) {
@@ -248,7 +255,6 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
   A((void**)&m->dYb, n * 2 * 2);
   A((void**)&m->Y, n * 2 * 4);
   A((void**)&m->W1p, kTcW1Bytes); A((void**)&m->Wp, kTcWpBytes); A((void**)&m->tc_err, 4);
-  m->packed = 0;
   if (rc != FN_OK) {
     fn_mlp_destroy(m);
     return rc;
@@ -271,6 +277,7 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
     cudaMemset(m->mb[l], 0, nout * 4); cudaMemset(m->vb[l], 0, nout * 4);
     k_to_bf16<<<(unsigned)((nw + 255) / 256), 256>>>(m->W[l], m->Wb[l], (long)nw);
   }
+  mlp_pack(m, nullptr);
   if (rc != FN_OK || cudaDeviceSynchronize() != cudaSuccess) {
     fn_mlp_destroy(m);
     return FN_ECUDA;
@@ -286,14 +293,6 @@ static void mlp_forward(fn_mlp* m, int n, cudaStream_t st) {
             m->Hb[l], 256, m->tc_err, st);
   k_gemm_bf16<<<dim3(1, (n + 63) / 64), 128, 0, st>>>(n, 2, 256, m->Hb[2], 256, m->Wb[3], 2,
                                                       m->b[3], m->Y, 2);
-}
-
-// the packed weights up to date on the stream (the transposes for training)
-static void mlp_pack(fn_mlp* m, bool transposed, cudaStream_t st) {
-  const int want = transposed ? 5 : 3;
-  if (m->packed >= want) return;
-  mlp_tc_pack(m->Wb[0], m->Wb[1], m->Wb[2], transposed, m->W1p, m->Wp, st);
-  m->packed = want;
 }
 
 static fn_status mlp_features(fn_mlp* m, const fn_arm_t* arm, const float* s0, const float* s1,
@@ -314,7 +313,6 @@ extern "C" fn_status fn_mlp_predict(fn_mlp_t* m, const fn_arm_t* arm, const floa
   ArmK A;
   if (!make_armk(arm, &A)) return FN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
-  mlp_pack(m, false, st);
   return mlp_tc_forward(A, s0, s1, E, m->W1p, m->Wp, m->b[0], m->b[1], m->b[2], m->Wb[3],
                         m->b[3], Y, m->tc_err, st);
 }
@@ -324,7 +322,6 @@ fn_status mlp_forward_rows(fn_mlp* m, const ArmK& A, const float* s0, const floa
                            const int* E_dev, float* Y, cudaStream_t st) {
   if (!m || E_max < 0) return FN_EINVAL;
   if (E_max == 0) return FN_OK;
-  mlp_pack(m, false, st);
   return mlp_tc_forward(A, s0, s1, E_max, m->W1p, m->Wp, m->b[0], m->b[1], m->b[2], m->Wb[3],
                         m->b[3], Y, m->tc_err, st, E_dev);
 }
@@ -371,7 +368,6 @@ extern "C" fn_status fn_mlp_backward(fn_mlp_t* m, const fn_arm_t* arm, const flo
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone)
     return FN_ECUDA;
-  mlp_pack(m, true, st);
   if (cudaMemsetAsync(m->grads, 0, m->n_grads * 4, st) != cudaSuccess) return FN_ECUDA;
   MlpTrain p;
   p.s0 = s0; p.s1 = s1; p.kstar = k_star; p.E = E;
@@ -400,7 +396,6 @@ extern "C" fn_status fn_mlp_adam_step(fn_mlp_t* m, float lr, void* stream) {
   if (!m || !(lr >= 0.f)) return FN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   m->step += 1;
-  m->packed = 0;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = (float)(1.0 - std::pow(0.9, m->step));
   const float c2 = (float)(1.0 - std::pow(0.999, m->step));
@@ -411,6 +406,7 @@ extern "C" fn_status fn_mlp_adam_step(fn_mlp_t* m, float lr, void* stream) {
     k_mlp_adam<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(m->b[l], m->mb[l], m->vb[l], m->gb[l],
                                                             nullptr, nb, lr, b1, b2, eps, c1, c2);
   }
+  mlp_pack(m, st);
   return launch_status();
 }
 
@@ -446,7 +442,7 @@ extern "C" fn_status fn_mlp_set_params(fn_mlp_t* m, int l, const float* W, const
   if (W && cudaMemcpy(m->W[l], W, nw * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
   if (b && cudaMemcpy(m->b[l], b, nb * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
   k_to_bf16<<<(unsigned)((nw + 255) / 256), 256>>>(m->W[l], m->Wb[l], (long)nw);
-  m->packed = 0;
+  mlp_pack(m, nullptr);
   return cudaDeviceSynchronize() == cudaSuccess ? FN_OK : FN_ECUDA;
 }
 

@@ -28,7 +28,7 @@
 namespace fn {
 
 // bf16 weights -> packed chunks (mlp_pack): blockIdx.y picks the matrix, W1,
-// W2, W3 and for training W3^T, W2^T
+// W2, W3, W3^T, W2^T
 __global__ void k_mlp_tc_pack(const bf16* __restrict__ W1, const bf16* __restrict__ W2,
                               const bf16* __restrict__ W3, bf16* __restrict__ W1p,
                               bf16* __restrict__ Wp) {
@@ -413,9 +413,9 @@ void gemm_tc(int M, int N, int K, const bf16* A, int lda, const bf16* B, int ldb
       M, N, K, A, lda, B, ldb, bias, relu ? 1 : 0, C, ldc, err);
 }
 
-void mlp_tc_pack(const bf16* W1, const bf16* W2, const bf16* W3, bool transposed, bf16* W1p,
-                 bf16* Wp, cudaStream_t st) {
-  k_mlp_tc_pack<<<dim3(256, transposed ? 5 : 3), 256, 0, st>>>(W1, W2, W3, W1p, Wp);
+void mlp_tc_pack(const bf16* W1, const bf16* W2, const bf16* W3, bf16* W1p, bf16* Wp,
+                 cudaStream_t st) {
+  k_mlp_tc_pack<<<dim3(256, 5), 256, 0, st>>>(W1, W2, W3, W1p, Wp);
 }
 
 fn_status mlp_tc_forward(const ArmK& A, const float* s0, const float* s1, int E, const bf16* W1p,

@@ -23,10 +23,10 @@ constexpr int kTcW1Bytes = kTcN * kTcK1 * 2;            // 16 KB
 constexpr int kTcWpBytes = 4 * 4 * kTcChunkBytes;       // W2, W3, W3^T, W2^T: 16 chunks
 
 // Pack the bf16 weights W [K][256] (row-major over the outputs): layer 1 as
-// one chunk of 32 columns, layers 2 and 3 and, with `transposed`, W3^T and
-// W2^T (the backward pass) as chunks of kTcKc columns.
+// one chunk of 32 columns, layers 2 and 3, W3^T and W2^T (the backward pass)
+// as chunks of kTcKc columns.
 void mlp_tc_pack(const __nv_bfloat16* W1, const __nv_bfloat16* W2, const __nv_bfloat16* W3,
-                 bool transposed, __nv_bfloat16* W1p, __nv_bfloat16* Wp, cudaStream_t st);
+                 __nv_bfloat16* W1p, __nv_bfloat16* Wp, cudaStream_t st);
 
 // Y[e] = MLP(features(s0[e], s1[e])) for e < E with the packed layers 1-3,
 // the bf16 layer-4 weights W4b [256][2] and the FP32 biases.  *err is set
@@ -71,8 +71,7 @@ struct fn_mlp;
 namespace fn {
 
 // The model's tensor-core forward over rows counted on the device (for a
-// caller inside a captured sequence): refreshes the packed weights first if
-// they changed.  Stream-ordered, no host synchronisation.
+// caller inside a captured sequence).  Stream-ordered, no host synchronisation.
 fn_status mlp_forward_rows(fn_mlp* m, const ArmK& A, const float* s0, const float* s1, int E_max,
                            const int* E_dev, float* Y, cudaStream_t st);
 

@@ -301,3 +301,40 @@ def test_trained_window_saves_work(S, arm):
     assert (w_un["k_star"] == full["k_star"]).float().mean().item() > 0.99
     assert n_tr < n_un, (n_tr, n_un)
     assert n_tr < n_full, (n_tr, n_full)
+
+
+def _call(fn, *args):
+    import ctypes as C
+    return fn(*[C.c_void_p(a.data_ptr()) if torch.is_tensor(a) else a for a in args])
+
+
+@pytest.mark.parametrize("change", ["create", "set_params", "adam"])
+def test_weights_packed_for_every_stream(S, arm, change):
+    """After a change of the weights, a gradient queued on one busy stream (the
+    loss not asked for) and a prediction on another at the same time: both see
+    the new weights, whatever the first one has not come to yet."""
+    import ctypes as C
+    E, grid = 300, synth.duration_grid(16)
+    s0, s1 = synth.random_edges(arm, E, 31)
+    d0, d1 = dev(s0), dev(s1)
+    lab = dev(np.random.default_rng(32).integers(-1, 16, E).astype(np.int32))
+    from paper_2609_22608_gb300._lib import arm_struct, lib
+    mlp = S.MLP(max_batch=512, seed=4)
+    if change == "set_params":
+        load(mlp, seeded_params(33))
+    elif change == "adam":
+        mlp.backward(arm, d0, d1, lab, grid)
+        mlp.adam_step(1e-2)
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(a):
+        torch.cuda._sleep(2_000_000)
+    A = arm_struct(arm)
+    assert _call(lib().fn_mlp_backward, mlp.h, C.byref(A), d0, d1, lab,
+                 grid.ctypes.data_as(C.c_void_p), 16, E, None, C.c_void_p(a.cuda_stream)) == 0
+    with torch.cuda.stream(b):
+        Y = mlp.predict(arm, d0, d1, stream=b)
+    torch.cuda.synchronize()
+    Yr = mlp.predict_ref(arm, d0, d1).cpu().numpy()
+    assert relerr(Y.cpu().numpy(), Yr) < 1e-3     # the two forwards' tolerance, as above
+    mlp.close()
