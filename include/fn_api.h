@@ -866,8 +866,8 @@ fn_status fn_mlp_destroy(fn_mlp_t* m);
 
 /* Y[e] = (log T*_pred, feasibility logit) for E edges (device s0, s1 [E][16],
  * 16-byte aligned; device Y [E][2]), any E.  Runs on the 5th-generation
- * tensor cores (tcgen05, accumulators in tensor memory), one fused launch;
- * the packed weights are refreshed on the stream after any weight change.
+ * tensor cores (tcgen05, accumulators in tensor memory), one fused launch on
+ * weights packed on the stream of their last change.
  * A timeout inside the kernel raises the flag read by fn_mlp_error. */
 fn_status fn_mlp_predict(fn_mlp_t* m, const fn_arm_t* arm, const float* s0, const float* s1,
                          int E, float* Y, void* stream);
@@ -881,6 +881,12 @@ fn_status fn_mlp_predict_ref(fn_mlp_t* m, const fn_arm_t* arm, const float* s0, 
 /* Error flag of the tensor-core kernel (1 after a timed-out wait); reset
  * != 0 clears it.  Synchronous. */
 fn_status fn_mlp_error(fn_mlp_t* m, int* flag, int reset);
+
+/* Longest wait of the fused kernels for a copy or the tensor core, in clock
+ * cycles (default 2e9, about a second); a kernel that gives up raises the
+ * error flag, waits for what it has in flight and returns.  cycles < 0: every
+ * wait gives up at once, which lets a caller try its own handling of it. */
+fn_status fn_mlp_set_wait(fn_mlp_t* m, long long cycles);
 
 /* Loss and gradients of one batch (E <= max_batch; k_star device [E] from
  * the exact scan over the host grid T_grid [K]); *loss (host, may be NULL)

@@ -26,6 +26,7 @@
 #include "edge_core.cuh"
 #include "fn_internal.h"
 #include "fn_mlp_tc.h"
+#include "fn_umma.cuh"
 
 namespace fn {
 
@@ -193,6 +194,7 @@ struct fn_mlp {
   bf16* W1p;      // [16 KB]
   bf16* Wp;       // [512 KB]
   int* tc_err;    // [1]
+  long long wait; // limit of their waits, clock cycles
   std::vector<void*> allocs;
 };
 
@@ -221,6 +223,7 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
   if (!out || max_batch < 1 || max_batch > (1 << 22)) return FN_EINVAL;
   fn_mlp* m = new fn_mlp();
   m->max_batch = max_batch;
+  m->wait = kWaitCycles;
   m->step = 0;
   fn_status rc = FN_OK;
   auto A = [&](void** p, size_t bytes) {
@@ -314,7 +317,7 @@ extern "C" fn_status fn_mlp_predict(fn_mlp_t* m, const fn_arm_t* arm, const floa
   if (!make_armk(arm, &A)) return FN_EINVAL;
   cudaStream_t st = (cudaStream_t)stream;
   return mlp_tc_forward(A, s0, s1, E, m->W1p, m->Wp, m->b[0], m->b[1], m->b[2], m->Wb[3],
-                        m->b[3], Y, m->tc_err, st);
+                        m->b[3], Y, m->tc_err, m->wait, st);
 }
 
 namespace fn {
@@ -323,9 +326,15 @@ fn_status mlp_forward_rows(fn_mlp* m, const ArmK& A, const float* s0, const floa
   if (!m || E_max < 0) return FN_EINVAL;
   if (E_max == 0) return FN_OK;
   return mlp_tc_forward(A, s0, s1, E_max, m->W1p, m->Wp, m->b[0], m->b[1], m->b[2], m->Wb[3],
-                        m->b[3], Y, m->tc_err, st, E_dev);
+                        m->b[3], Y, m->tc_err, m->wait, st, E_dev);
 }
 }  // namespace fn
+
+extern "C" fn_status fn_mlp_set_wait(fn_mlp_t* m, long long cycles) {
+  if (!m) return FN_EINVAL;
+  m->wait = cycles;
+  return FN_OK;
+}
 
 // the same forward layer by layer, E <= max_batch per internal batch
 extern "C" fn_status fn_mlp_predict_ref(fn_mlp_t* m, const fn_arm_t* arm, const float* s0,
@@ -381,7 +390,7 @@ extern "C" fn_status fn_mlp_backward(fn_mlp_t* m, const fn_arm_t* arm, const flo
     p.img[4 + l] = m->dZ[l];
   }
   p.dy = m->dYb; p.dy_pitch = (long)m->rows;
-  p.loss = m->loss; p.err = m->tc_err;
+  p.loss = m->loss; p.err = m->tc_err; p.wait = m->wait;
   const fn_status rc = mlp_tc_train(A, logT, p, st);
   if (rc != FN_OK) return rc;
   if (loss) {

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
              const float* __restrict__ b1, const float* __restrict__ b2,
              const float* __restrict__ b3, const bf16* __restrict__ W4b,
              const float* __restrict__ b4, float* __restrict__ Y, int* __restrict__ err,
-             const int* __restrict__ E_dev) {
+             long long wait, const int* __restrict__ E_dev) {
   extern __shared__ __align__(1024) uint8_t smem[];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int lq = warp & 3, cg = warp >> 2;          // TMEM lane quarter, column group
@@ -69,7 +69,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   volatile int* s_fail = reinterpret_cast<volatile int*>(smem + kSBar + 84);
   const uint32_t a_base = su32(sA), b_base = su32(smem + kSB), w1_base = su32(smem + kSW1);
   const uint32_t bar_base = su32(bars);
-  const uint32_t bar_layer = bar_base + 64u, bar_w1 = bar_base + 72u;
+  const uint32_t bar_layer = bar_base + 64u, bar_w1 = bar_base + 72u, bar_drain = bar_base + 88u;
 
   for (int i = tid; i < 768; i += blockDim.x)
     sBias[i] = i < 256 ? b1[i] : (i < 512 ? b2[i - 256] : b3[i - 512]);
@@ -83,6 +83,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
   if (tid == 0) {
     for (int b = 0; b < 10; ++b) mbar_init(bar_base + 8u * b, 1);
+    mbar_init(bar_drain, 1);
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -92,7 +93,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = *s_tmem;
   const uint32_t tmem_lane = tmem + ((uint32_t)(lq * 32) << 16);   // this warp's 32 lanes
 
-  TcRing ring(bar_base, b_base, W23p, 8, my_tiles);   // thread 0: layers 2 and 3 of every tile
+  TcRing ring(bar_base, b_base, W23p, 8, my_tiles, wait);   // thread 0: layers 2 and 3 of every tile
   uint32_t ph_layer = 0;
   bool fail = false;
   if (tid == 0) {
@@ -111,7 +112,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     // ---- layer 1
     if (tid == 0 && !fail) {
       tc_fence_after();
-      if (it == 0 && !mbar_wait(bar_w1, 0)) fail = true;
+      if (it == 0 && !mbar_wait(bar_w1, 0, wait)) fail = true;
       if (!fail) {
 #pragma unroll
         for (int s = 0; s < kTcK1 / 16; ++s)
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
       __syncthreads();
       // wait for this layer's accumulator (all threads; a block vote keeps
       // the decision uniform, so no thread is left at a barrier)
-      const bool lf = *s_fail || !mbar_wait(bar_layer, ph_layer);
+      const bool lf = *s_fail || !mbar_wait(bar_layer, ph_layer, wait);
       ph_layer ^= 1;
       tc_fence_after();
       if (__syncthreads_or(lf)) {
@@ -201,12 +202,14 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     }
     if (*s_fail) break;
   }
-  // ---- exit: on failure, wait (bounded) for this CTA's copies still in flight
+  // ---- exit: on failure, wait (bounded) for this CTA's copies and MMAs still in flight
   __syncthreads();
   if (*s_fail || fail) {
     if (tid == 0) {
       atomicExch(err, 1);
+      mbar_wait(bar_w1, 0);
       ring.drain();
+      umma_drain(bar_drain);
     }
     __syncthreads();
   }
@@ -330,8 +333,7 @@ __global__ void __launch_bounds__(128, 1)
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
   if (tid == 0) {
-    mbar_init(bar0, 1);
-    mbar_init(bar0 + 8, 1);
+    for (int i = 0; i < 3; ++i) mbar_init(bar0 + 8 * i, 1);   // the stages, the drain
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -392,7 +394,13 @@ __global__ void __launch_bounds__(128, 1)
   }
   tc_fence_before();
   __syncthreads();
-  if (*s_fail && tid == 0) atomicExch(err, 1);
+  if (*s_fail) {
+    if (tid == 0) {
+      atomicExch(err, 1);
+      umma_drain(bar0 + 16);
+    }
+    __syncthreads();
+  }
   tc_fence_after();
   if (warp == 0)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem),
@@ -420,8 +428,8 @@ void mlp_tc_pack(const bf16* W1, const bf16* W2, const bf16* W3, bf16* W1p, bf16
 
 fn_status mlp_tc_forward(const ArmK& A, const float* s0, const float* s1, int E, const bf16* W1p,
                          const bf16* W23p, const float* b1, const float* b2, const float* b3,
-                         const bf16* W4b, const float* b4, float* Y, int* err, cudaStream_t st,
-                         const int* E_dev) {
+                         const bf16* W4b, const float* b4, float* Y, int* err, long long wait,
+                         cudaStream_t st, const int* E_dev) {
   if (E <= 0) return FN_OK;
   static bool attr[64] = {false};
   int dev = 0;
@@ -435,7 +443,7 @@ fn_status mlp_tc_forward(const ArmK& A, const float* s0, const float* s1, int E,
   const int ntiles = (E + kTcM - 1) / kTcM;
   const int grid = ntiles < num_sms() ? ntiles : num_sms();
   k_mlp_tc<<<grid, kTcThreads, kTcSmem, st>>>(A, s0, s1, E, W1p, W23p, b1, b2, b3, W4b, b4, Y,
-                                               err, E_dev);
+                                               err, wait, E_dev);
   return launch_status();
 }
 

@@ -30,12 +30,13 @@ void mlp_tc_pack(const __nv_bfloat16* W1, const __nv_bfloat16* W2, const __nv_bf
 
 // Y[e] = MLP(features(s0[e], s1[e])) for e < E with the packed layers 1-3,
 // the bf16 layer-4 weights W4b [256][2] and the FP32 biases.  *err is set
-// to 1 if a wait on the tensor core or a copy timed out.  Y: device [E][2].
+// to 1 if a wait on the tensor core or a copy took more than `wait` cycles.
+// Y: device [E][2].
 // E_dev (device, may be NULL): the rows actually present, at most E.
 fn_status mlp_tc_forward(const ArmK& A, const float* s0, const float* s1, int E,
                          const __nv_bfloat16* W1p, const __nv_bfloat16* W23p, const float* b1,
                          const float* b2, const float* b3, const __nv_bfloat16* W4b,
-                         const float* b4, float* Y, int* err, cudaStream_t st,
+                         const float* b4, float* Y, int* err, long long wait, cudaStream_t st,
                          const int* E_dev = nullptr);
 
 // C = A B (+ bias, ReLU) in BF16 with FP32 accumulation on the tensor cores
@@ -60,6 +61,7 @@ struct MlpTrain {
   long dy_pitch;
   float *gW[4], *gb[4], *loss;
   int* err;
+  long long wait;                             // limit of a wait in cycles
 };
 struct MlpLogT { float v[FN_MAX_GRID]; };     // log of the grid's durations
 fn_status mlp_tc_train(const ArmK& A, const MlpLogT& logT, const MlpTrain& p, cudaStream_t st);

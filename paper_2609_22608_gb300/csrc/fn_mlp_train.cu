@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   volatile int* s_fail = reinterpret_cast<volatile int*>(smem + kSBar + 84);
   const uint32_t a_base = su32(sA), b_base = su32(smem + kSB), w1_base = su32(smem + kSW1);
   const uint32_t bar_base = su32(smem + kSBar);   // the ring's 8, layer done, W1 arrived
-  const uint32_t bar_layer = bar_base + 64u, bar_w1 = bar_base + 72u;
+  const uint32_t bar_layer = bar_base + 64u, bar_w1 = bar_base + 72u, bar_drain = bar_base + 88u;
 
   for (int i = tid; i < 768; i += blockDim.x)
     sBias[i] = i < 256 ? p.b[0][i] : (i < 512 ? p.b[1][i - 256] : p.b[2][i - 512]);
@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   }
   if (tid == 0) {
     for (int b = 0; b < 10; ++b) mbar_init(bar_base + 8u * b, 1);
+    mbar_init(bar_drain, 1);
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   const uint32_t tmem = *s_tmem;
   const uint32_t tmem_lane = tmem + ((uint32_t)(lq * 32) << 16);   // this warp's 32 lanes
 
-  TcRing ring(bar_base, b_base, p.Wp, 16, my_tiles);   // thread 0: W2, W3, W3^T, W2^T
+  TcRing ring(bar_base, b_base, p.Wp, 16, my_tiles, p.wait);   // thread 0: W2, W3, W3^T, W2^T
   uint32_t ph_layer = 0;
   bool fail = false;
   if (tid == 0) {
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     __syncthreads();
     if (tid == 0) {
       tc_fence_after();
-      if (it == 0 && !mbar_wait(bar_w1, 0)) fail = true;
+      if (it == 0 && !mbar_wait(bar_w1, 0, p.wait)) fail = true;
       if (!fail) {
         bulk_s2g(p.img[0] + tile * (kTcM * kTcK1), a_base, kTcM * kTcK1 * 2);
 #pragma unroll
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
         bulk_read_wait();   // A is free once its image has been read (and its MMAs are done)
       }
       __syncthreads();
-      const bool lf = *s_fail || !mbar_wait(bar_layer, ph_layer);
+      const bool lf = *s_fail || !mbar_wait(bar_layer, ph_layer, p.wait);
       ph_layer ^= 1;
       tc_fence_after();
       if (__syncthreads_or(lf)) {
@@ -338,13 +339,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (*s_fail) break;   // written before the phases' last barrier, or by every thread
   }
   // ---- exit: the images are complete; on failure, wait (bounded) for this
-  // CTA's copies still in flight
+  // CTA's copies and MMAs still in flight
   if (tid == 0) bulk_wait();
   __syncthreads();
   if (*s_fail || fail) {
     if (tid == 0) {
       atomicExch(p.err, 1);
+      mbar_wait(bar_w1, 0);
       ring.drain();
+      umma_drain(bar_drain);
     }
     __syncthreads();
   }
@@ -451,8 +454,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
   const uint32_t bytesB = kDwRows * wB * 2;
   volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + kDwBar + 64);
   volatile int* s_fail = reinterpret_cast<volatile int*>(smem + kDwBar + 68);
-  const uint32_t base = su32(smem), bar = base + kDwBar;   // arrived (3), consumed (3), done
-  const uint32_t bar_done = bar + 8u * (2 * kDwStages);
+  const uint32_t base = su32(smem), bar = base + kDwBar;   // arrived (3), consumed (3), done, drain
+  const uint32_t bar_done = bar + 8u * (2 * kDwStages), bar_drain = bar_done + 8u;
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
                      su32((const void*)s_tmem)),
@@ -461,7 +464,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
   }
   if (tid == 0) {
-    for (int b = 0; b < 2 * kDwStages + 1; ++b) mbar_init(bar + 8u * b, 1);
+    for (int b = 0; b < 2 * kDwStages + 2; ++b) mbar_init(bar + 8u * b, 1);
     *s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
@@ -482,7 +485,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
     for (int i = 0; i < filled; ++i) fill(i, i);
     for (; done < n; ++done) {
       const int st = done % kDwStages;
-      if (!mbar_wait(bar + 8u * st, (done / kDwStages) & 1)) break;
+      if (!mbar_wait(bar + 8u * st, (done / kDwStages) & 1, p.wait)) break;
       const uint32_t a = base + st * kDwStage, b = a + kDwA;
 #pragma unroll
       for (int j = 0; j < kDwRows / 16; ++j)
@@ -494,7 +497,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
       // refill the stage of the block before (its MMAs are queued before these)
       if (done >= 1 && done - 1 + kDwStages < n) {
         const int pb = (done - 1) % kDwStages;
-        if (!mbar_wait(bar + 8u * (kDwStages + pb), ((done - 1) / kDwStages) & 1)) break;
+        if (!mbar_wait(bar + 8u * (kDwStages + pb), ((done - 1) / kDwStages) & 1, p.wait)) break;
         fill(pb, filled);
         ++filled;
       }
@@ -508,9 +511,12 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
     }
   }
   __syncthreads();
-  const bool bad = *s_fail || !mbar_wait(bar_done, 0);
+  const bool bad = *s_fail || !mbar_wait(bar_done, 0, p.wait);
   if (__syncthreads_or(bad)) {
-    if (tid == 0) atomicExch(p.err, 1);
+    if (tid == 0) {
+      atomicExch(p.err, 1);
+      umma_drain(bar_drain);
+    }
   } else {
     tc_fence_after();
     // warp w: lanes of quarter w % 4, accumulator half w / 4

@@ -45,11 +45,14 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// bounded wait for phase `parity` of the barrier to complete
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+// bounded wait for phase `parity` of the barrier to complete (limit in clock
+// cycles; below zero: gives up at once)
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity,
+                                          long long limit = kWaitCycles) {
+  if (limit < 0) return false;
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity))
-    if (clock64() - t0 > kWaitCycles) return false;
+    if (clock64() - t0 > limit) return false;
   return true;
 }
 // the same among threads that give up together: returns at once when another
@@ -100,6 +103,13 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile(
       "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
       : "memory");
+}
+// After a wait that ran out: the MMAs that this thread has issued end before
+// the operands and tensor memory go away.  bar: a barrier that nothing else
+// uses (bounded, as every wait).
+__device__ __forceinline__ void umma_drain(uint32_t bar) {
+  umma_commit(bar);
+  mbar_wait(bar, 0);
 }
 __device__ __forceinline__ void tc_fence_before() {
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");

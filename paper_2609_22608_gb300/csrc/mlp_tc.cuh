@@ -81,11 +81,13 @@ struct TcRing {
   const bf16* W;
   int period;
   long total, g;                        // chunks to multiply, the next one
+  long long limit;                      // of a wait
   uint32_t in_flight, ph_w, ph_free;    // a bit per slot
 
-  __device__ TcRing(uint32_t bar_, uint32_t b_, const bf16* W_, int period_, int tiles)
+  __device__ TcRing(uint32_t bar_, uint32_t b_, const bf16* W_, int period_, int tiles,
+                    long long limit_)
       : bar(bar_), b_base(b_), W(W_), period(period_), total((long)tiles * period_), g(0),
-        in_flight(0), ph_w(0), ph_free(0) {}
+        limit(limit_), in_flight(0), ph_w(0), ph_free(0) {}
   __device__ void fill(int b, long chunk) {
     mbar_expect_tx(bar + 8u * b, kTcChunkBytes);
     bulk_g2s(b_base + b * kTcChunkBytes, W + (chunk % period) * (kTcChunkBytes / 2),
@@ -100,7 +102,7 @@ struct TcRing {
   __device__ bool layer(uint32_t tmem, uint32_t a_base) {
 #pragma unroll
     for (int c = 0; c < 4; ++c, ++g) {
-      if (!mbar_wait(bar + 8u * c, ph_w >> c & 1u)) return false;
+      if (!mbar_wait(bar + 8u * c, ph_w >> c & 1u, limit)) return false;
       ph_w ^= 1u << c;
       in_flight &= ~(1u << c);
       const uint32_t bb = b_base + c * kTcChunkBytes;
@@ -113,7 +115,7 @@ struct TcRing {
       // this chunk's) with the chunk kRing - 1 ahead of this one
       if (g >= 1 && g + kRing - 1 < total) {
         const int pb = (c + kRing - 1) % kRing;
-        if (!mbar_wait(bar + 8u * (4 + pb), ph_free >> pb & 1u)) return false;
+        if (!mbar_wait(bar + 8u * (4 + pb), ph_free >> pb & 1u, limit)) return false;
         ph_free ^= 1u << pb;
         fill(pb, g + kRing - 1);
       }

@@ -24,6 +24,7 @@ def _bind():
     L.fn_mlp_destroy.argtypes = [vp]
     L.fn_mlp_predict.argtypes = [vp, vp, vp, vp, i32, vp, vp]
     L.fn_mlp_predict_ref.argtypes = [vp, vp, vp, vp, i32, vp, vp]
+    L.fn_mlp_set_wait.argtypes = [vp, C.c_longlong]
     L.fn_mlp_error.argtypes = [vp, C.POINTER(C.c_int), i32]
     L.fn_mlp_backward.argtypes = [vp, vp, vp, vp, vp, vp, i32, i32, vp, vp]
     L.fn_mlp_adam_step.argtypes = [vp, f32, vp]
@@ -35,7 +36,7 @@ def _bind():
     L.fn_time_edges_window.argtypes = [vp, vp, vp, i32, vp, i32, i32, vp, i32, vp, vp, vp, vp, vp,
                                        vp, vp]
     for n in ("fn_mlp_create", "fn_mlp_destroy", "fn_mlp_predict", "fn_mlp_predict_ref",
-              "fn_mlp_error", "fn_mlp_backward",
+              "fn_mlp_error", "fn_mlp_set_wait", "fn_mlp_backward",
               "fn_mlp_adam_step", "fn_mlp_train_step", "fn_mlp_get_params", "fn_mlp_set_params",
               "fn_mlp_get_grads", "fn_mlp_set_grads", "fn_mlp_save", "fn_mlp_load",
               "fn_time_edges_window"):
@@ -101,6 +102,10 @@ class MLP:
         f = C.c_int()
         check(lib().fn_mlp_error(self.h, C.byref(f), int(bool(reset))), "fn_mlp_error")
         return int(f.value)
+
+    def set_wait(self, cycles):
+        """fn_mlp_set_wait: the longest wait inside the kernels."""
+        check(lib().fn_mlp_set_wait(self.h, int(cycles)), "fn_mlp_set_wait")
 
     def backward(self, arm, s0, s1, k_star, T_grid, stream=None):
         A = arm_struct(arm)

@@ -338,3 +338,46 @@ def test_weights_packed_for_every_stream(S, arm, change):
     Yr = mlp.predict_ref(arm, d0, d1).cpu().numpy()
     assert relerr(Y.cpu().numpy(), Yr) < 1e-3     # the two forwards' tolerance, as above
     mlp.close()
+
+
+def test_wait_that_runs_out(S, arm):
+    """Kernels that give up at their first wait, with the copies of the weights
+    in flight: they raise the flag and end cleanly, and with the usual limit the
+    same model gives the same results as before."""
+    E, grid = 152 * 128 + 77, synth.duration_grid(16)
+    s0, s1 = synth.random_edges(arm, E, 41)
+    d0, d1 = dev(s0), dev(s1)
+    lab = dev(np.random.default_rng(42).integers(-1, 16, E).astype(np.int32))
+    mlp = S.MLP(max_batch=E)
+    load(mlp, seeded_params(43))
+    Y = mlp.predict(arm, d0, d1)
+    mlp.backward(arm, d0, d1, lab, grid)
+    g = [mlp.get_grads(l) for l in range(4)]
+    assert mlp.error() == 0
+    for call in ("predict", "backward"):
+        mlp.set_wait(-1)
+        if call == "predict":
+            mlp.predict(arm, d0, d1)
+        else:
+            _call_backward(mlp, arm, d0, d1, lab, grid)
+        torch.cuda.synchronize()
+        assert mlp.error(reset=True) == 1
+        mlp.set_wait(2_000_000_000)
+        assert torch.equal(mlp.predict(arm, d0, d1), Y)
+        mlp.backward(arm, d0, d1, lab, grid)
+        assert mlp.error() == 0
+        for l in range(4):           # sums in another order: FP32's 2^-24 on 2e4 rows
+            for a, b in zip(mlp.get_grads(l), g[l]):
+                assert relerr(a, b) < 1e-5
+    mlp.close()
+
+
+def _call_backward(mlp, arm, d0, d1, lab, grid):
+    """fn_mlp_backward without the loss: its status."""
+    import ctypes as C
+
+    from paper_2609_22608_gb300._lib import arm_struct, lib
+    A = arm_struct(arm)
+    return _call(lib().fn_mlp_backward, mlp.h, C.byref(A), d0, d1, lab,
+                 grid.ctypes.data_as(C.c_void_p), len(grid), d0.shape[0], None,
+                 C.c_void_p(torch.cuda.current_stream().cuda_stream))
