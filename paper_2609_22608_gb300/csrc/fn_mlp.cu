@@ -143,10 +143,13 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K,
         }
 }
 
-// Adam on FP32 master weights; bf16 copy refreshed
+// Adam on FP32 master weights; bf16 copy refreshed.  *fail: the gradient was
+// given up halfway, nothing is changed.
 __global__ void k_mlp_adam(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                           const float* __restrict__ g, bf16* __restrict__ pb, long n, float lr,
-                           float b1, float b2, float eps, float c1, float c2) {
+                           const float* __restrict__ g, const int* __restrict__ fail,
+                           bf16* __restrict__ pb, long n, float lr, float b1, float b2, float eps,
+                           float c1, float c2) {
+  if (*fail) return;
   for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (long)gridDim.x * blockDim.x) {
     const float gi = g[i];
@@ -189,6 +192,7 @@ struct fn_mlp {
   float* grads;   // gW, gb and the loss in one piece
   size_t n_grads;
   float* loss;    // [1]
+  int* fail;      // [1] the last gradient was given up (with the gradients: zeroed before one)
   // the weights packed for tcgen05 (with every change of the weights, on its
   // stream) and the kernels' error flag
   bf16* W1p;      // [16 KB]
@@ -249,6 +253,7 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
       g += (kDims[l + 1] + 3) / 4 * 4;
     }
     m->loss = g;
+    m->fail = reinterpret_cast<int*>(g + 1);
   }
   const size_t n = ((size_t)max_batch + kTcM - 1) / kTcM * kTcM;
   m->rows = n;
@@ -263,6 +268,7 @@ extern "C" fn_status fn_mlp_create(int max_batch, unsigned long long seed, fn_ml
     return rc;
   }
   cudaMemset(m->tc_err, 0, 4);
+  cudaMemset(m->fail, 0, 4);
   // He-uniform initial weights (inputs 28 of 32 used), zero biases, zero moments
   std::mt19937_64 rng(seed);
   for (int l = 0; l < MLP_LAYERS; ++l) {
@@ -360,6 +366,18 @@ extern "C" fn_status fn_mlp_error(fn_mlp_t* m, int* flag, int reset) {
   return FN_OK;
 }
 
+// the loss of the gradient enqueued on st, and whether it was given up
+static fn_status mlp_read_loss(fn_mlp* m, float* loss, cudaStream_t st) {
+  float h[2];   // loss, fail
+  if (cudaMemcpyAsync(h, m->loss, sizeof(h), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return FN_ECUDA;
+  int fail;
+  std::memcpy(&fail, h + 1, sizeof(fail));
+  *loss = h[0];
+  return fail ? FN_ECUDA : FN_OK;
+}
+
 extern "C" fn_status fn_mlp_backward(fn_mlp_t* m, const fn_arm_t* arm, const float* s0,
                                      const float* s1, const int32_t* k_star, const float* T_grid,
                                      int K, int E, float* loss, void* stream) {
@@ -390,15 +408,10 @@ extern "C" fn_status fn_mlp_backward(fn_mlp_t* m, const fn_arm_t* arm, const flo
     p.img[4 + l] = m->dZ[l];
   }
   p.dy = m->dYb; p.dy_pitch = (long)m->rows;
-  p.loss = m->loss; p.err = m->tc_err; p.wait = m->wait;
+  p.loss = m->loss; p.err = m->tc_err; p.fail = m->fail; p.wait = m->wait;
   const fn_status rc = mlp_tc_train(A, logT, p, st);
   if (rc != FN_OK) return rc;
-  if (loss) {
-    if (cudaMemcpyAsync(loss, m->loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return FN_ECUDA;
-  }
-  return FN_OK;
+  return loss ? mlp_read_loss(m, loss, st) : FN_OK;
 }
 
 extern "C" fn_status fn_mlp_adam_step(fn_mlp_t* m, float lr, void* stream) {
@@ -410,9 +423,9 @@ extern "C" fn_status fn_mlp_adam_step(fn_mlp_t* m, float lr, void* stream) {
   const float c2 = (float)(1.0 - std::pow(0.999, m->step));
   for (int l = 0; l < MLP_LAYERS; ++l) {
     const long nw = (long)kDims[l] * kDims[l + 1], nb = kDims[l + 1];
-    k_mlp_adam<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(m->W[l], m->mW[l], m->vW[l], m->gW[l],
+    k_mlp_adam<<<(unsigned)((nw + 255) / 256), 256, 0, st>>>(m->W[l], m->mW[l], m->vW[l], m->gW[l], m->fail,
                                                             m->Wb[l], nw, lr, b1, b2, eps, c1, c2);
-    k_mlp_adam<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(m->b[l], m->mb[l], m->vb[l], m->gb[l],
+    k_mlp_adam<<<(unsigned)((nb + 255) / 256), 256, 0, st>>>(m->b[l], m->mb[l], m->vb[l], m->gb[l], m->fail,
                                                             nullptr, nb, lr, b1, b2, eps, c1, c2);
   }
   mlp_pack(m, st);
@@ -426,13 +439,10 @@ extern "C" fn_status fn_mlp_train_step(fn_mlp_t* m, const fn_arm_t* arm, const f
   fn_status rc = fn_mlp_backward(m, arm, s0, s1, k_star, T_grid, K, E, nullptr, stream);
   if (rc != FN_OK) return rc;
   if ((rc = fn_mlp_adam_step(m, lr, stream)) != FN_OK) return rc;
-  if (loss) {
-    cudaStream_t st = (cudaStream_t)stream;
-    if (cudaMemcpyAsync(loss, m->loss, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-      return FN_ECUDA;
-  }
-  return FN_OK;
+  if (!loss) return FN_OK;
+  rc = mlp_read_loss(m, loss, (cudaStream_t)stream);
+  if (rc != FN_OK) m->step -= 1;   // the step was left out
+  return rc;
 }
 
 // parameter / gradient / moment access (host arrays, layer l, W [in][out])
@@ -469,7 +479,7 @@ extern "C" fn_status fn_mlp_set_grads(fn_mlp_t* m, int l, const float* gW, const
   const size_t nw = (size_t)kDims[l] * kDims[l + 1], nb = kDims[l + 1];
   if (gW && cudaMemcpy(m->gW[l], gW, nw * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
   if (gb && cudaMemcpy(m->gb[l], gb, nb * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
-  return FN_OK;
+  return cudaMemset(m->fail, 0, 4) == cudaSuccess ? FN_OK : FN_ECUDA;   // the caller's gradient
 }
 
 // binary file: "FNMLP1\0\0", step, then per layer W (f32 [in][out]) and b

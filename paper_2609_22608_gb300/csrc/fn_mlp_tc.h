@@ -49,7 +49,8 @@ void gemm_tc(int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bf
 // tiles, X (8 KB a tile), h1, h2, h3, dz3, dz2, dz1 (64 KB a tile); row r, column
 // c of a tile of width w at byte ((r / 8) * (w / 8) + c / 8) * 128 +
 // (r % 8) * 16 + (c % 8) * 2.  loss, gW and gb are added
-// to (zero before a gradient).
+// to (zero before a gradient).  A wait that ran out sets *err, which stays, and
+// *fail (zero before a gradient): the gradient is not one then.
 struct MlpTrain {
   const float *s0, *s1;                       // [E][16]
   const int32_t* kstar;                       // [E]
@@ -60,7 +61,7 @@ struct MlpTrain {
   __nv_bfloat16* dy;                          // dL/dy by columns, dy_pitch (whole tiles) apart
   long dy_pitch;
   float *gW[4], *gb[4], *loss;
-  int* err;
+  int *err, *fail;
   long long wait;                             // limit of a wait in cycles
 };
 struct MlpLogT { float v[FN_MAX_GRID]; };     // log of the grid's durations

@@ -345,6 +345,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
   if (*s_fail || fail) {
     if (tid == 0) {
       atomicExch(p.err, 1);
+      atomicExch(p.fail, 1);
       mbar_wait(bar_w1, 0);
       ring.drain();
       umma_drain(bar_drain);
@@ -515,6 +516,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
   if (__syncthreads_or(bad)) {
     if (tid == 0) {
       atomicExch(p.err, 1);
+      atomicExch(p.fail, 1);
       umma_drain(bar_drain);
     }
   } else {

@@ -381,3 +381,42 @@ def _call_backward(mlp, arm, d0, d1, lab, grid):
     return _call(lib().fn_mlp_backward, mlp.h, C.byref(A), d0, d1, lab,
                  grid.ctypes.data_as(C.c_void_p), len(grid), d0.shape[0], None,
                  C.c_void_p(torch.cuda.current_stream().cuda_stream))
+
+
+def test_gradient_given_up(S, arm):
+    """A gradient whose wait ran out is reported where its loss is read and is
+    never applied; the caller's own gradients and the next backward are."""
+    from paper_2609_22608_gb300._lib import FnError
+    E, grid = 500, synth.duration_grid(16)
+    s0, s1 = synth.random_edges(arm, E, 51)
+    d0, d1 = dev(s0), dev(s1)
+    lab = dev(np.random.default_rng(52).integers(-1, 16, E).astype(np.int32))
+    mlp = S.MLP(max_batch=E)
+    load(mlp, seeded_params(53))
+    mlp.backward(arm, d0, d1, lab, grid)          # images of an earlier batch
+    before = [mlp.get_params(l) for l in range(4)]
+
+    def unchanged():
+        return all(np.array_equal(x, y) for l in range(4)
+                   for x, y in zip(mlp.get_params(l), before[l]))
+    mlp.set_wait(-1)
+    with pytest.raises(FnError):
+        mlp.backward(arm, d0, d1, lab, grid)
+    mlp.adam_step(1e-2)
+    assert unchanged()
+    assert _call_backward(mlp, arm, d0, d1, lab, grid) == 0     # nothing read back
+    mlp.adam_step(1e-2)
+    assert unchanged()
+    with pytest.raises(FnError):
+        mlp.train_step(arm, d0, d1, lab, grid, 1e-2)
+    assert unchanged() and mlp.error(reset=True) == 1
+    for l in range(4):
+        W, b = mlp.get_params(l)
+        mlp.set_grads(l, np.ones_like(W), np.ones_like(b))
+    mlp.adam_step(1e-2)
+    assert not unchanged()
+    mlp.set_wait(2_000_000_000)
+    after = [mlp.get_params(l)[0] for l in range(4)]
+    assert np.isfinite(mlp.train_step(arm, d0, d1, lab, grid, 1e-2)) and mlp.error() == 0
+    assert not np.array_equal(mlp.get_params(1)[0], after[1])
+    mlp.close()
