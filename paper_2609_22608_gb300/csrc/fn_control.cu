@@ -126,12 +126,30 @@ __global__ void __launch_bounds__(128) k_controller(ArmK A, CtrlK L, int B,
 // edges at S = 256 with five obstacles take 13 us with eight warps each, and
 // took 26 with one.
 #define CHECK_WARPS 8
+#define CHECK_BLOCKS 2   // of an SM
 constexpr size_t kCheckWarp = (FN_CUBIC_WORDS + FN_LINK_WORDS + 1) * 32 * sizeof(float);
 constexpr size_t kCheckSmem = CHECK_WARPS * (kCheckWarp + 4 * sizeof(float)) +
                               7 * FN_LINK_F4 * sizeof(float4);
-__global__ void __launch_bounds__(32 * CHECK_WARPS, 2)
+// Warps to an edge, `warps` being what the chip holds at once: as many as it has
+// batches of 32 samples and as keep all edges on the chip together.  With more
+// edges than that warps that share one wait for one another: then one, or two
+// where they end the last wave earlier (a wave of pairs takes 0.55 of a wave of
+// single warps: S = 256, five obstacles 23.1 us against 43.8; S = 64 12.8
+// against 23.0).  At S = 256 with five obstacles 608, 1216 and 3500 edges take 20.6,
+// 28.7 and 75.8 us with four, two and two warps; 26.8, 49.2 and 135 with eight;
+// 32.8, 33.0 and 92.2 with one.  65536 edges take 1180 us with one, 2352 with eight
+// (and took 1758 with one in smaller blocks).
+__host__ __device__ __forceinline__ int check_group(long E, int S, int warps) {
+  int group = 1;
+  while (group < CHECK_WARPS && 32 * group < S && E * 2 * group <= warps) group *= 2;
+  const long waves1 = (E + warps - 1) / warps, waves2 = (2 * E + warps - 1) / warps;
+  if (E > warps && S > 32 && 11 * waves2 < 20 * waves1) group = 2;
+  return group;
+}
+
+__global__ void __launch_bounds__(32 * CHECK_WARPS, CHECK_BLOCKS)
     k_check_edges(ArmK A, fn_problem_t P, int E, const int* __restrict__ E_dev, int S,
-                  int S_clear, float margin, int group, const float* __restrict__ s0,
+                  int S_clear, float margin, int warps, const float* __restrict__ s0,
                   const float* __restrict__ s1, const float* __restrict__ Tv,
                   float* __restrict__ rho3, float* __restrict__ clearance,
                   uint8_t* __restrict__ ok) {
@@ -142,6 +160,7 @@ __global__ void __launch_bounds__(32 * CHECK_WARPS, 2)
   __syncthreads();
   if (E_dev) E = min(E, max(*E_dev, 0));
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int group = check_group(E, S, warps);   // of the edges there are
   const int r = w % group, g = w / group, ng = CHECK_WARPS / group;
   float* mine = sPart + 4 * CHECK_WARPS + (kCheckWarp / sizeof(float)) * w;
   float* es = mine + (FN_CUBIC_WORDS + FN_LINK_WORDS) * 32;
@@ -282,12 +301,11 @@ extern "C" fn_status fn_check_edges_full(const fn_arm_t* arm, const float* s0, c
                                              (int)kCheckSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
-  // as many warps to an edge as it has batches of 32 samples
-  int group = 1;
-  while (group < CHECK_WARPS && 32 * group < S) group *= 2;
-  const long want = ((long)E * group + CHECK_WARPS - 1) / CHECK_WARPS;
-  const int blocks = (int)std::max<long>(1, std::min<long>(want, 2L * num_sms()));
+  const int fit = CHECK_BLOCKS * num_sms(), warps = fit * CHECK_WARPS;
+  // an edge count on the device may be any up to E: a block for each of the first
+  const long want = E_dev ? E : ((long)E * check_group(E, S, warps) + CHECK_WARPS - 1) / CHECK_WARPS;
+  const int blocks = (int)std::max<long>(1, std::min<long>(want, fit));
   k_check_edges<<<blocks, 32 * CHECK_WARPS, kCheckSmem, (cudaStream_t)stream>>>(
-      A, P, E, E_dev, S, S_clear, margin, group, s0, s1, T, rho3, clearance, ok);
+      A, P, E, E_dev, S, S_clear, margin, warps, s0, s1, T, rho3, clearance, ok);
   return launch_status();
 }

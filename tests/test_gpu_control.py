@@ -246,3 +246,25 @@ def test_recheck_is_the_fixed_check(ops, arm, E, S):
     assert r["rho3"].cpu().numpy().tobytes() == f["rho3"].cpu().numpy().tobytes()
     half = ops.check_edges_full(arm, dev(s0), dev(s1), dev(T), S, 33, obs, 0.02)
     assert (half["clearance"] >= r["clearance"]).all()   # every second one of the 65
+
+
+@pytest.mark.parametrize("E", [304, 305, 609, 1217, 2432, 2433, 3500, 5000])
+def test_recheck_of_many_edges(ops, arm, E):
+    """Numbers of edges around the steps of the warps-per-edge rule (152 SMs):
+    every edge's results are those of a call with a few edges, bit for bit, and
+    the same with the count on the device."""
+    S = 256
+    s0, s1 = synth.random_edges(arm, E, 75)
+    T = np.random.default_rng(E).uniform(0.1, 1.6, E).astype(np.float32)
+    obs = synth.obstacles(5, 3)
+    d0, d1, dT = dev(s0), dev(s1), dev(T)
+    r = ops.check_edges_full(arm, d0, d1, dT, S, 64, obs, 0.02)
+    few = torch.from_numpy(np.unique(np.r_[0:20, np.random.default_rng(1).integers(0, E, 60), E - 20:E])).cuda()
+    n = torch.tensor([len(few)], dtype=torch.int32, device="cuda")
+    f0, f1, fT = d0[few].contiguous(), d1[few].contiguous(), dT[few].contiguous()
+    a = ops.check_edges_full(arm, f0, f1, fT, S, 64, obs, 0.02)
+    d0[:len(few)], d1[:len(few)], dT[:len(few)] = f0, f1, fT
+    b = ops.check_edges_full(arm, d0, d1, dT, S, 64, obs, 0.02, E_dev=n)
+    for k in ("rho3", "clearance", "ok"):
+        assert torch.equal(r[k][few], a[k])
+        assert torch.equal(b[k][:len(few)], a[k])
