@@ -156,19 +156,24 @@ __global__ void __launch_bounds__(KT_THREADS, 1) k_knn_tc_mins(KnnTcWork W, long
   knn_mins(kt_smem, W, units * b / G, units * (b + 1) / G, err);
 }
 
+// team warps to a query, of which the first searches alone and all share an
+// exact scan (knn_wide)
 __global__ void __launch_bounds__(256, 4)
     k_knn_tc_select(const float2* __restrict__ soa, int n, int first,
                     const float4* __restrict__ queries, int B, int k, float w, float sw,
                     const float* __restrict__ gmin, int ntiles, const int* __restrict__ err,
-                    float* __restrict__ out_d, int32_t* __restrict__ out_i) {
-  __shared__ unsigned long long list[8][KT_LIST];
-  const long b = (long)blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (b >= B) return;
-  const KeyList r = knn_select(soa, n, first, queries + 4 * b, k, w, sw,
-                               gmin + b * 4 * kt_row_f4(ntiles), ntiles, *err != 0,
-                               list[threadIdx.x >> 5]);
-  const int lane = threadIdx.x & 31;
-  if (lane < k) {
+                    int team, float* __restrict__ out_d, int32_t* __restrict__ out_i) {
+  __shared__ KnnWide<8> sh;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long b = ((long)blockIdx.x * 8 + warp) / team;
+  const bool mine = warp % team == 0 && b < B;
+  KeyList r;
+  bool wide = false;
+  if (mine)
+    r = knn_select<true>(soa, n, first, queries + 4 * b, k, w, sw, gmin + b * 4 * kt_row_f4(ntiles),
+                   ntiles, *err != 0, sh.list[warp], &wide);
+  r = knn_wide(sh, r, wide, team, soa, n, first, queries + 4 * b, k, w);
+  if (mine && lane < k) {
     out_d[b * k + lane] = __uint_as_float((unsigned)(r.key >> 32));
     out_i[b * k + lane] = r.key >= KT_NONE ? -1 : (int)(unsigned)r.key;
   }
@@ -182,8 +187,12 @@ constexpr size_t kKtGminBytes = (size_t)64 << 20;   // group minima of one batch
 // filter is the faster one at every batch and k measured (1 to 8192 queries:
 // 1.2x at 256 nodes and one query, 2x at 32, 15x at 65536 nodes, 8192
 // queries and k = 16, 1906 -> 128 us).  States closer to one another than
-// the score's error (a tree of identical nodes) leave every group in reach:
-// the exact scoring of all of them takes up to 2.4x the scan's time.
+// the score's error, or outside its range, leave every group in reach; the
+// exact scan of all nodes in the select step (knn_wide) then takes about the
+// scan's time and the filter's.  8192 queries, 65536 nodes, k = 16: equal nodes
+// 1145 -> 1319 us, four clusters 1902 -> 1350, states in degrees 1913 -> 1276;
+// 2048 queries, 4096 nodes, k = 8: 45 -> 79, 80 -> 78, 82 -> 96; one query,
+// 65536 nodes: 130 -> 199, 140 -> 215, 140 -> 126.
 static bool knn_tc_wanted(int N) { return N >= 256; }
 
 struct KnnTcPlan {
@@ -236,9 +245,11 @@ static fn_status knn_tc_launch(const float* tree, int N, int first, const float*
     const KnnTcWork W{ws + p.qimg, ws + p.nimg, gmin, ntiles, nb};
     k_knn_tc_mins<<<(unsigned)std::min<long>(units, num_sms()), KT_THREADS, kKtSmem, st>>>(W, units,
                                                                                            err);
-    k_knn_tc_select<<<(nb + 7) / 8, 256, 0, st>>>(soa, N - first, first, q, nb, k, w_vel, sw, gmin,
-                                                  ntiles, err, d2 + (long)b0 * k,
-                                                  idx + (long)b0 * k);
+    int team = 8;   // warps to a query, up to what the chip holds
+    while (team > 1 && (long)nb * team > 32L * num_sms()) team /= 2;
+    k_knn_tc_select<<<(unsigned)(((long)nb * team + 7) / 8), 256, 0, st>>>(
+        soa, N - first, first, q, nb, k, w_vel, sw, gmin, ntiles, err, team, d2 + (long)b0 * k,
+        idx + (long)b0 * k);
   }
   return launch_status();
 }

@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(32 * PL_KNN_SEL_WARPS, 4) k_plan_knn_select(Pl
     }
     const int n = D.n_nodes[p] - 1;
     const KeyList best =
-        knn_select(D.soa + (long)p * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA, n, 1,
+        knn_select<false>(D.soa + (long)p * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA, n, 1,
                    reinterpret_cast<const float4*>(D.cand) + 4 * ci, D.KN, D.w_vel, D.sw_vel,
                    D.gmin[kind] + ((long)(t - t0) * KT_QT + r) * stride, knn_node_tiles(D, p), all,
                    list[w]);

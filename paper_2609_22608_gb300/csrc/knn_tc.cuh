@@ -417,24 +417,35 @@ __device__ __forceinline__ float knn_unorder(unsigned u) {
 }
 
 // Exact scores read the nodes from a second image: per group of 32 nodes
-// [7][32] float2, component pair by component pair, so that a warp's seven
+// [7][32] float2, joint by joint (position, velocity), so that a warp's seven
 // loads of a group are contiguous (from the 64-byte rows of the tree a load
 // touches sixteen lines).
 constexpr int KT_SOA = 7 * KT_GROUP;   // float2 per group
 __device__ __forceinline__ void knn_store_soa(float2* soa, long node, const float* x) {
   float2* p = soa + node / KT_GROUP * KT_SOA + node % KT_GROUP;
 #pragma unroll
-  for (int c = 0; c < 7; ++c) p[KT_GROUP * c] = make_float2(x[2 * c], x[2 * c + 1]);
+  for (int c = 0; c < 7; ++c) p[KT_GROUP * c] = make_float2(x[c], x[7 + c]);
 }
 __device__ __forceinline__ float knn_dist(const float* qv, const float2 (&x)[7], float w) {
   float dq = 0.f, dv = 0.f;
 #pragma unroll
-  for (int j = 0; j < 14; ++j) {
-    const float t = qv[j] - ((j & 1) ? x[j >> 1].y : x[j >> 1].x);
-    if (j < 7) dq = fmaf(t, t, dq);
-    else dv = fmaf(t, t, dv);
+  for (int c = 0; c < 7; ++c) {
+    const float t = qv[c] - x[c].x, u = qv[7 + c] - x[c].y;
+    dq = fmaf(t, t, dq);
+    dv = fmaf(u, u, dv);
   }
   return fmaf(w, dv, dq);
+}
+// the same with the two sums as the halves of paired operations, from the negated
+// query ((x - q)^2 is (q - x)^2): half the instructions, for a loop they bound
+__device__ __forceinline__ float knn_dist2(const float2 (&nq)[7], const float2 (&x)[7], float w) {
+  float2 d = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int c = 0; c < 7; ++c) {
+    const float2 t = __fadd2_rn(x[c], nq[c]);
+    d = __ffma2_rn(t, t, d);
+  }
+  return fmaf(w, d.y, d.x);
 }
 
 // The k nearest of n nodes (their image soa, ids from id0 on) to a query
@@ -446,17 +457,29 @@ __device__ __forceinline__ float knn_dist(const float* qv, const float2 (&x)[7],
 // registers: the loads' latency is hidden by 32 warps an SM rather than by
 // several groups in flight (8192 queries, 65536 nodes, k = 16: 50 us; two
 // groups at a time with 16 warps an SM 69 us).
-constexpr int KT_LIST = 160;
+// kWide: *wide is set when the scores do not tell the nodes apart, which is looked
+// at once when KT_TRIAL groups have been gone through: a quarter of all groups are in
+// reach still.  The list is then empty but for its bound, and knn_wide does the
+// search.  (A query that stays here may still score up to that quarter.)  Without
+// kWide such a query scores the groups one by one, a warp for itself.
+constexpr int KT_LIST = 160, KT_TRIAL = 64;
+template <bool kWide>
 __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, int n, int id0,
                                               const float4* __restrict__ query, int k, float w,
                                               float sw, const float* __restrict__ g, int ntiles,
-                                              bool all, unsigned long long* list) {
+                                              bool all, unsigned long long* list,
+                                              bool* wide = nullptr) {
   const int lane = threadIdx.x & 31;
   float qv[14], q2;
   load_query(query, qv);
   {
     float sq[14];
     all |= !knn_scaled(qv, sw, sq, q2);
+  }
+  KeyList best;
+  if (kWide && all) {
+    *wide = true;
+    return best;
   }
   const float4* g4 = reinterpret_cast<const float4*>(g);
   const int n4 = kt_row_f4(ntiles);
@@ -489,16 +512,36 @@ __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, in
   // largest score of a node at distance at most D
   auto reach = [&](float D) { return fmaf(D, 1.f + 2.f * KT_C, slack - q2) + 1e-6f * q2; };
   float lim = INFINITY;
-  KeyList best;
   if (!all && tau < KT_EMPTY) {
     // (rounded up by the last factor) at least k nodes are this near
     const float dmax = (fmaxf(tau + q2, 0.f) + slack) / (1.f - 2.f * KT_C) * (1.f + 1e-6f);
     lim = reach(dmax);
     best.kth = knn_key(dmax, 0x7fffffff);   // farther nodes need not enter the list
   }
-  int cnt = 0;   // groups collected
+  int cnt = 0, scored = 0;   // groups collected, gone through
+  bool tried = false, give_up = false;
+  auto useless = [&]() {     // do the scores leave a quarter of the groups in reach?
+    int in = 0;
+#pragma unroll 1
+    for (int b = 0; b < n4; b += 32) {
+      float x[4];
+      load4(b + lane, x);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) in += __popc(__ballot_sync(0xffffffffu, x[c] <= lim));
+    }
+    return in > ntiles;
+  };
   auto flush = [&]() {
     __syncwarp();
+    if (kWide && scored >= KT_TRIAL && !tried) {
+      tried = true;
+      give_up = useless();
+      if (give_up) {
+        lim = -INFINITY;     // nothing more is collected
+        cnt = 0;
+      }
+    }
+    scored += cnt;
     for (int f = 0; f < cnt; f += 32) {
       const int ne = min(32, cnt - f);
       unsigned long long e = lane < ne ? list[f + lane] : ~0ull;
@@ -551,6 +594,92 @@ __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, in
     }
   }
   if (cnt) flush();
+  if (kWide) *wide = give_up;
+  if (give_up) {       // start again; the k-th key so far is one of those to find
+    best.key = KT_NONE;
+    best.kth += best.kth < KT_NONE;
+  }
+  return best;
+}
+
+// The exact scan of all nodes, for the queries whose scores are of no use: node
+// states that nearly coincide, states outside the filter's range.  Every warp of a
+// block of NW calls this (it synchronises) and gets its list, best unless wide is set.
+// The block copies KT_STAGE groups at a time into shared memory (cp.async, a ring of
+// KT_STAGES) and each of its wide queries scores them from there; `team`
+// neighbouring warps share a query (the first one's wide and best count), a group
+// in turn each.  The loop is bound by issue, hence the paired distance.  A warp
+// reading every group for itself took, 8192 queries of a tree of 65536 equal nodes,
+// 2780 us (L2 bandwidth), one such query 1280 us (latency); now 1319 and 199 (the
+// scan of fn_knn.cu, without the filter before it, 1145 and 130).
+constexpr int KT_STAGE = 8, KT_STAGES = 3;
+template <int NW>
+struct KnnWide {
+  union {
+    unsigned long long list[NW][KT_LIST];            // knn_select's
+    float4 stage[KT_STAGES][KT_STAGE * KT_SOA / 2];
+    unsigned long long key[NW][16];
+  };
+  int wide[NW];
+};
+template <int NW>
+__device__ __forceinline__ KeyList knn_wide(KnnWide<NW>& sh, KeyList best, bool wide, int team,
+                                            const float2* soa, int n, int id0,
+                                            const float4* query, int k, float w) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = warp % team;
+  if (!__syncthreads_or(rank == 0 && wide)) return best;
+  if (lane == 0 && rank == 0) sh.wide[warp] = wide;
+  if (rank != 0) best = KeyList{};
+  __syncthreads();
+  const bool mine = sh.wide[warp - rank] != 0;
+  float2 nq[7];
+  if (mine) {
+    float qv[14];
+    load_query(query, qv);
+#pragma unroll
+    for (int c = 0; c < 7; ++c) nq[c] = make_float2(-qv[c], -qv[7 + c]);
+  }
+  constexpr int kF4 = KT_SOA / 2;              // of a group
+  const int groups = (n + KT_GROUP - 1) / KT_GROUP, chunks = (groups + KT_STAGE - 1) / KT_STAGE;
+  auto copy = [&](int c) {                     // one commit group, empty past the end
+    if (c < chunks) {
+      const int have = min(KT_STAGE, groups - c * KT_STAGE) * kF4;
+      const float4* src = reinterpret_cast<const float4*>(soa) + (long)c * KT_STAGE * kF4;
+      const uint32_t dst = su32(sh.stage[c % KT_STAGES]);
+      for (int i = threadIdx.x; i < have; i += 32 * NW)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16 * i),
+                     "l"(src + i)
+                     : "memory");
+    }
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+  };
+  for (int c = 0; c < KT_STAGES - 1; ++c) copy(c);
+  for (int c = 0; c < chunks; ++c) {
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(KT_STAGES - 2) : "memory");
+    __syncthreads();                           // chunk c is there, c - 1 is scored
+    copy(c + KT_STAGES - 1);
+    if (!mine) continue;
+    const float2* st = reinterpret_cast<const float2*>(sh.stage[c % KT_STAGES]) + lane;
+    const int have = min(KT_STAGE, groups - c * KT_STAGE);
+    for (int i = rank; i < have; i += team) {
+      const int node = (c * KT_STAGE + i) * KT_GROUP + lane;
+      float2 x[7];
+#pragma unroll
+      for (int j = 0; j < 7; ++j) x[j] = st[i * KT_SOA + KT_GROUP * j];
+      const float d = knn_dist2(nq, x, w);
+      const unsigned long long key =
+          node < n && d <= INFINITY ? knn_key(d, id0 + node) : KT_NONE;
+      if (__any_sync(0xffffffffu, key < best.kth)) best.offer(key, k);
+    }
+  }
+  asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+  if (team > 1) {
+    __syncthreads();                           // the last chunk is scored
+    if (lane < 16) sh.key[warp][lane] = best.key;
+    __syncthreads();
+    if (rank == 0 && mine)
+      for (int r = 1; r < team; ++r) best.offer(lane < 16 ? sh.key[warp + r][lane] : KT_NONE, k);
+  }
   return best;
 }
 

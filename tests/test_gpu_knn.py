@@ -141,3 +141,28 @@ def test_knn_on_side_streams(ops, arm):
     for i, (idx, d2) in got:
         assert torch.equal(idx, ref[i][0])
         assert torch.equal(d2.view(torch.int32), ref[i][1].view(torch.int32))
+
+
+@pytest.mark.parametrize("kind", ["same", "tight", "degrees", "one_out"])
+@pytest.mark.parametrize("B,N,k", [(1, 20003, 8), (3, 4099, 16), (130, 9000, 5), (2500, 1030, 16),
+                                   (5003, 2100, 8)])
+def test_knn_without_help_of_the_filter(ops, arm, kind, B, N, k):
+    """Queries whose scores tell nothing apart (eight to one warps each): coinciding
+    nodes, clusters below the scores' error, states outside their range, and one
+    such query among ordinary ones.  The scan's lists bit for bit."""
+    t, q = synth.random_states(arm, N, N), synth.random_states(arm, B, N + B)
+    rng = np.random.default_rng(N)
+    if kind == "same":
+        t[:] = t[0]
+    elif kind == "tight":
+        t = t[rng.integers(0, 4, N)] + 1e-4 * rng.standard_normal((N, 16)).astype(np.float32)
+        q[::2] = t[rng.integers(0, N, len(q[::2]))]
+    elif kind == "degrees":
+        t, q = t * np.float32(57.3), q * np.float32(57.3)
+    else:
+        q[B // 2] *= 1000
+    t, q = dev(t.astype(np.float32)), dev(q.astype(np.float32))
+    idx, d2 = ops.knn_tree(t, q, k, 0.1)
+    ri, rd = _scan(t, q, k, 1)
+    assert torch.equal(idx, ri)
+    assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))

@@ -635,3 +635,31 @@ def test_goal_draws_do_not_depend_on_the_batch(P, arm, goals):
     for p, g in enumerate(goals):
         for f in ("states", "T_req", "v_rel", "valid"):
             assert got[p][f][:g].tobytes() == ref[p][f][:g].tobytes(), (p, f)
+
+
+@pytest.mark.parametrize("w_vel", [0.1, 1e4])
+def test_parent_lists_without_help_of_the_filter(P, arm, w_vel):
+    """Trees whose nodes coincide beside ordinary ones (one block's queries then
+    want different trees scanned), and a velocity weight that takes the states out
+    of the filter's range: the FP32 scan's lists bit for bit."""
+    Ns, Bs, goals = [5000, 300, 2500, 4400], [300, 40, 9, 257], [37, 11, 4, 60]
+    root = synth.random_states(arm, 1, 77)[0]
+    pr = synth.make_problem(synth.random_toss(arm, 21), root=root)
+    n, k = len(Ns), 9
+    pl = P.Planner(arm, P=n, n_cap=6000, b_max=300, k=k, K=4, S=4, w_vel=w_vel)
+    probs = [P.problem_struct(pr, Bs[p], goals[p], root=root) for p in range(n)]
+    pl.reset(probs)
+    trees = []
+    for p in range(n):
+        states, parent, t = synth.random_tree(arm, Ns[p], 31 + p, root=root)
+        cand = synth.random_states(arm, Bs[p], 50 + p)
+        if p != 3:
+            states[1:] = states[1 + np.arange(Ns[p] - 1) % (1 + 2 * p)]   # one state; three; five
+        pl.load_tree(p, states, t, parent)
+        pl.set_candidates(p, cand, goals[p], np.full(goals[p], 0.5, np.float32),
+                          np.full(goals[p], 4.0, np.float32))
+        trees.append((states, cand))
+    pl.iterate(probs, 0, P.FN_PLAN_EXTERNAL)
+    for p, (states, cand) in enumerate(trees):
+        assert np.array_equal(pl.get_parents(p, Bs[p]), _scan_lists(states, cand, k - 1, w_vel)), p
+    pl.close()
