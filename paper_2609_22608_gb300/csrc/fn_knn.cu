@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(256) k_knn_merge(int B, int nsplit, int k,
 __global__ void __launch_bounds__(128) k_knn_tc_pack(const float4* __restrict__ tree, int N,
                                                      int first, int node_rows,
                                                      const float4* __restrict__ queries, int B,
-                                                     float sw, uint8_t* __restrict__ nimg,
+                                                     float2 sc, uint8_t* __restrict__ nimg,
                                                      float2* __restrict__ soa,
                                                      uint8_t* __restrict__ qimg,
                                                      int* __restrict__ err) {
@@ -128,12 +128,12 @@ __global__ void __launch_bounds__(128) k_knn_tc_pack(const float4* __restrict__ 
       load_query(tree + 4 * (long)(first + i), x);
       knn_store_soa(soa, i, x);
     }
-    knn_pack_node(nimg + (long)(i / KT_ROWS) * KT_TILE, i % KT_ROWS, x, sw, have);
+    knn_pack_node(nimg + (long)(i / KT_ROWS) * KT_TILE, i % KT_ROWS, x, sc, have);
   } else {
     const int b = i - node_rows;   // the grid ends with the last query tile
     const bool have = b < B;
     if (have) load_query(queries + 4 * (long)b, x);
-    knn_pack_query(qimg + (long)(b / KT_ROWS) * KT_TILE, b % KT_ROWS, x, sw, have);
+    knn_pack_query(qimg + (long)(b / KT_ROWS) * KT_TILE, b % KT_ROWS, x, sc, have);
   }
 }
 
@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(KT_THREADS, 1) k_knn_tc_mins(KnnTcWork W, long
 // exact scan (knn_wide)
 __global__ void __launch_bounds__(256, 4)
     k_knn_tc_select(const float2* __restrict__ soa, int n, int first,
-                    const float4* __restrict__ queries, int B, int k, float w, float sw,
+                    const float4* __restrict__ queries, int B, int k, float w, float2 sc,
                     const float* __restrict__ gmin, int ntiles, const int* __restrict__ err,
                     int team, float* __restrict__ out_d, int32_t* __restrict__ out_i) {
   __shared__ KnnWide<8> sh;
@@ -170,7 +170,7 @@ __global__ void __launch_bounds__(256, 4)
   KeyList r;
   bool wide = false;
   if (mine)
-    r = knn_select<true>(soa, n, first, queries + 4 * b, k, w, sw, gmin + b * 4 * kt_row_f4(ntiles),
+    r = knn_select<true>(soa, n, first, queries + 4 * b, k, w, sc, gmin + b * 4 * kt_row_f4(ntiles),
                    ntiles, *err != 0, sh.list[warp], &wide);
   r = knn_wide(sh, r, wide, team, soa, n, first, queries + 4 * b, k, w);
   if (mine && lane < k) {
@@ -231,7 +231,7 @@ static fn_status knn_tc_launch(const float* tree, int N, int first, const float*
   int* err = (int*)ws;
   float2* soa = (float2*)(ws + p.soa);
   float* gmin = (float*)(ws + p.gmin);
-  const float sw = std::sqrt(w_vel);
+  const float2 sc = knn_scales(w_vel, 7 * 16.0 * (1.0 + w_vel));   // of joints up to 4 rad, 4 rad/s
   // tiles of the nodes actually searched (the plan holds room for all N)
   const int ntiles = (N - first + KT_ROWS - 1) / KT_ROWS;
   for (int b0 = 0; b0 < B; b0 += p.batch) {
@@ -240,7 +240,7 @@ static fn_status knn_tc_launch(const float* tree, int N, int first, const float*
     const int nrows = b0 == 0 ? ntiles * KT_ROWS : 0;   // the node image serves every batch
     const float4* q = (const float4*)queries + 4 * (long)b0;
     k_knn_tc_pack<<<nrows / 128 + 2 * qtiles, 128, 0, st>>>((const float4*)tree, N, first, nrows, q,
-                                                            nb, sw, ws + p.nimg, soa, ws + p.qimg, err);
+                                                            nb, sc, ws + p.nimg, soa, ws + p.qimg, err);
     const long units = (long)qtiles * ntiles;
     const KnnTcWork W{ws + p.qimg, ws + p.nimg, gmin, ntiles, nb};
     k_knn_tc_mins<<<(unsigned)std::min<long>(units, num_sms()), KT_THREADS, kKtSmem, st>>>(W, units,
@@ -248,7 +248,7 @@ static fn_status knn_tc_launch(const float* tree, int N, int first, const float*
     int team = 8;   // warps to a query, up to what the chip holds
     while (team > 1 && (long)nb * team > 32L * num_sms()) team /= 2;
     k_knn_tc_select<<<(unsigned)(((long)nb * team + 7) / 8), 256, 0, st>>>(
-        soa, N - first, first, q, nb, k, w_vel, sw, gmin, ntiles, err, team, d2 + (long)b0 * k,
+        soa, N - first, first, q, nb, k, w_vel, sc, gmin, ntiles, err, team, d2 + (long)b0 * k,
         idx + (long)b0 * k);
   }
   return launch_status();

@@ -178,7 +178,7 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   int32_t* packed;    // [P] leading nodes whose images are current
   int NT;             // node tiles per problem
   int knn_tiles;      // query tiles of one launch
-  float sw_vel;       // sqrt(w_vel)
+  float2 knn_sc;      // knn_scales of w_vel and the arm's limits
 };
 
 // Programmatic dependent launch: a kernel launched with programmatic
@@ -390,7 +390,7 @@ __device__ __forceinline__ void pack_query_row(const PlanDev& D, int kind, int p
     x[7 + j] = qd[j];
   }
   knn_pack_query(D.qimg[kind] + ((long)t * 2 + (r % KT_QT) / KT_ROWS) * KT_TILE, r % KT_ROWS, x,
-                 D.sw_vel, true);
+                 D.knn_sc, true);
 }
 
 // Free candidate (p, b): uniform in the box, |qd| <= vel_frac qdbar.
@@ -549,7 +549,11 @@ __global__ void __launch_bounds__(32) k_plan_goals(PlanDev D, ArmK A, int dens) 
 // 8192 queries on 28 k nodes (k = 16) 770 -> 96 us, 2048 queries on 4096
 // nodes 57 -> 34 us (four launches' latency, of which half runs beside the
 // inverse kinematics).  Planners of all sizes take them; a window of query
-// tiles bounds the minima's memory.
+// tiles bounds the minima's memory.  In a tree whose nodes coincide within the
+// filter's error, or lie far outside the arm's limits, a query scores every node
+// on its own warp: 8192 queries on 28 k equal nodes 610 -> 1105 us, 256 on 60 k
+// 65 -> 1175 (a scan by blocks, as fn_knn_tree has it, would cost every search 4 to
+// 8 us in these kernels, or a launch).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int knn_rows(const PlanDev& D, int kind, int p) {
   if (D.n_nodes[p] <= 1) return 0;
@@ -650,7 +654,7 @@ __global__ void __launch_bounds__(32 * PL_KNN_SEL_WARPS, 4) k_plan_knn_select(Pl
     const int n = D.n_nodes[p] - 1;
     const KeyList best =
         knn_select<false>(D.soa + (long)p * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA, n, 1,
-                   reinterpret_cast<const float4*>(D.cand) + 4 * ci, D.KN, D.w_vel, D.sw_vel,
+                   reinterpret_cast<const float4*>(D.cand) + 4 * ci, D.KN, D.w_vel, D.knn_sc,
                    D.gmin[kind] + ((long)(t - t0) * KT_QT + r) * stride, knn_node_tiles(D, p), all,
                    list[w]);
     if (lane < D.KN)
@@ -681,7 +685,7 @@ __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stri
       load_query(reinterpret_cast<const float4*>(D.st) + 4 * ((long)p * D.NC + row + 1), v);
       knn_store_soa(D.soa + (long)p * D.NT * (KT_ROWS / KT_GROUP) * KT_SOA, row, v);
     }
-    knn_pack_node(D.nimg + ((long)p * D.NT + row / KT_ROWS) * KT_TILE, row % KT_ROWS, v, D.sw_vel,
+    knn_pack_node(D.nimg + ((long)p * D.NT + row / KT_ROWS) * KT_TILE, row % KT_ROWS, v, D.knn_sc,
                   have);
   }
 }
@@ -3151,7 +3155,13 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
   D.surv_cap = (int)std::min<long>((long)D.Emax * 16, 1L << 26);
   A_(D.surv, (size_t)D.surv_cap);
   D.NT = (c.n_cap - 1 + KT_ROWS - 1) / KT_ROWS;
-  D.sw_vel = std::sqrt(c.w_vel);
+  {
+    double r2 = 0.;
+    for (int j = 0; j < 7; ++j)
+      r2 += std::pow(std::max(std::fabs((double)arm->q_lo[j]), std::fabs((double)arm->q_hi[j])), 2) +
+            (double)c.w_vel * arm->qd_max[j] * arm->qd_max[j];
+    D.knn_sc = knn_scales(c.w_vel, r2);
+  }
   {
     const size_t tiles = P * ((BM + KT_QT - 1) / KT_QT);
     const size_t per = (size_t)KT_QT * kt_row_f4(D.NT) * sizeof(float4);

@@ -3,7 +3,8 @@
 //
 // The squared distance of query q and node n under the velocity weight w is
 // |q'|^2 + (|n'|^2 - 2 q'.n') with x' = (positions, sqrt(w) velocities).  The
-// bracket, the pair's score, is a contraction: each value is split into two
+// bracket, the pair's score, is a contraction (knn_scales may shrink x' by a power
+// of two, which changes no digit of it): each value is split into two
 // f16 terms (hi + lo, 22 bits), the cross products hi hi, hi lo and lo hi of
 // the 14 components and the node's squared norm in three f16 terms make a
 // row of KT_K = 48 columns, and tcgen05.mma scores 128 nodes against 128
@@ -36,6 +37,8 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+
+#include <cmath>
 
 #include "fn_umma.cuh"
 #include "knn_core.cuh"
@@ -81,25 +84,38 @@ __device__ __forceinline__ void knn_store_row(uint8_t* tile, int r, const __half
                    h2(v[8 * c + 4], v[8 * c + 5]), h2(v[8 * c + 6], v[8 * c + 7]));
 }
 
+// Scales (position, velocity) = c (1, sqrt(w)) of x', c the largest power of two up
+// to 1 that brings states with |q|^2 + w |qd|^2 <= r2 into the split's range (not
+// below 2^-50: distances of states in range stay finite in FP32, as those that
+// overflow tie).
+// A weight of 1e4 without it leaves every node to the exact scores: 60000 nodes and
+// 256 queries 1175 us, now 44.
+inline float2 knn_scales(float w, double r2) {
+  float c = 1.f;
+  if (r2 < INFINITY)
+    while (c > 1e-15f && (double)c * c * r2 > KT_MAX2) c *= 0.5f;
+  return make_float2(c, c * std::sqrt(w));
+}
+
 // x' and |x'|^2 of a state; returns whether the split covers it
-__device__ __forceinline__ bool knn_scaled(const float* x, float sw, float (&s)[14], float& n2) {
+__device__ __forceinline__ bool knn_scaled(const float* x, float2 sc, float (&s)[14], float& n2) {
   n2 = 0.f;
 #pragma unroll
   for (int j = 0; j < 14; ++j) {
-    s[j] = j < 7 ? x[j] : sw * x[j];
+    s[j] = (j < 7 ? sc.x : sc.y) * x[j];
     n2 = fmaf(s[j], s[j], n2);
   }
   return n2 <= KT_MAX2;   // false for NaN
 }
 
 // present = false: a row past the last node (x unused)
-__device__ __forceinline__ void knn_pack_node(uint8_t* tile, int r, const float* x, float sw,
+__device__ __forceinline__ void knn_pack_node(uint8_t* tile, int r, const float* x, float2 sc,
                                               bool present) {
   __half v[KT_K];
 #pragma unroll
   for (int j = 0; j < KT_K; ++j) v[j] = __float2half_rn(0.f);
   float s[14], n2 = 0.f;
-  const bool in = present && knn_scaled(x, sw, s, n2);
+  const bool in = present && knn_scaled(x, sc, s, n2);
   if (in) {
 #pragma unroll
     for (int j = 0; j < 14; ++j) {
@@ -117,13 +133,13 @@ __device__ __forceinline__ void knn_pack_node(uint8_t* tile, int r, const float*
   }
   knn_store_row(tile, r, v);
 }
-__device__ __forceinline__ void knn_pack_query(uint8_t* tile, int r, const float* x, float sw,
+__device__ __forceinline__ void knn_pack_query(uint8_t* tile, int r, const float* x, float2 sc,
                                                bool present) {
   __half v[KT_K];
 #pragma unroll
   for (int j = 0; j < KT_K; ++j) v[j] = __float2half_rn(0.f);
   float s[14], n2;
-  if (present && knn_scaled(x, sw, s, n2)) {
+  if (present && knn_scaled(x, sc, s, n2)) {
 #pragma unroll
     for (int j = 0; j < 14; ++j) {
       const float a = -2.f * s[j];
@@ -466,7 +482,7 @@ constexpr int KT_LIST = 160, KT_TRIAL = 64;
 template <bool kWide>
 __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, int n, int id0,
                                               const float4* __restrict__ query, int k, float w,
-                                              float sw, const float* __restrict__ g, int ntiles,
+                                              float2 sc, const float* __restrict__ g, int ntiles,
                                               bool all, unsigned long long* list,
                                               bool* wide = nullptr) {
   const int lane = threadIdx.x & 31;
@@ -474,7 +490,7 @@ __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, in
   load_query(query, qv);
   {
     float sq[14];
-    all |= !knn_scaled(qv, sw, sq, q2);
+    all |= !knn_scaled(qv, sc, sq, q2);
   }
   KeyList best;
   if (kWide && all) {
@@ -509,14 +525,15 @@ __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, in
     }
   const float tau = __shfl_sync(0xffffffffu, m, k - 1);
   const float slack = fmaf(8.f * KT_C, q2, KT_ABS);
-  // largest score of a node at distance at most D
+  const float c2 = sc.x * sc.x;   // of a scaled squared distance
+  // largest score of a node at (scaled) distance at most D
   auto reach = [&](float D) { return fmaf(D, 1.f + 2.f * KT_C, slack - q2) + 1e-6f * q2; };
   float lim = INFINITY;
   if (!all && tau < KT_EMPTY) {
     // (rounded up by the last factor) at least k nodes are this near
     const float dmax = (fmaxf(tau + q2, 0.f) + slack) / (1.f - 2.f * KT_C) * (1.f + 1e-6f);
     lim = reach(dmax);
-    best.kth = knn_key(dmax, 0x7fffffff);   // farther nodes need not enter the list
+    best.kth = knn_key(dmax / c2, 0x7fffffff);   // farther nodes need not enter the list
   }
   int cnt = 0, scored = 0;   // groups collected, gone through
   bool tried = false, give_up = false;
@@ -567,7 +584,7 @@ __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, in
           if (d <= INFINITY) key = knn_key(d, id0 + node);   // a NaN distance never enters
         }
         best.offer(key, k);
-        if (!all) lim = fminf(lim, reach(__uint_as_float((unsigned)(best.kth >> 32))));
+        if (!all) lim = fminf(lim, reach(c2 * __uint_as_float((unsigned)(best.kth >> 32))));
       }
     }
     cnt = 0;

@@ -65,7 +65,7 @@ def test_knn_full_size_sampled(ops, orc, arm):
     assert not knn_mismatches(ig[sel], dg[sel], ri, rd)
 
 
-def _scan(tree, q, k, first):
+def _scan(tree, q, k, first, w=0.1):
     """fn_knn_tree without a workspace: the FP32 scan of every node."""
     import ctypes as C
 
@@ -74,7 +74,7 @@ def _scan(tree, q, k, first):
     idx = torch.empty(B, k, dtype=torch.int32, device="cuda")
     d2 = torch.empty(B, k, device="cuda")
     st = lib().fn_knn_tree(C.c_void_p(tree.data_ptr()), tree.shape[0], first,
-                           C.c_void_p(q.data_ptr()), B, k, 0.1, C.c_void_p(idx.data_ptr()),
+                           C.c_void_p(q.data_ptr()), B, k, w, C.c_void_p(idx.data_ptr()),
                            C.c_void_p(d2.data_ptr()), None, 0,
                            C.c_void_p(torch.cuda.current_stream().cuda_stream))
     assert st == 0
@@ -164,5 +164,16 @@ def test_knn_without_help_of_the_filter(ops, arm, kind, B, N, k):
     t, q = dev(t.astype(np.float32)), dev(q.astype(np.float32))
     idx, d2 = ops.knn_tree(t, q, k, 0.1)
     ri, rd = _scan(t, q, k, 1)
+    assert torch.equal(idx, ri)
+    assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
+
+
+@pytest.mark.parametrize("w", [0.0, 1e-20, 1.0, 80.0, 3e3, 1e4, 1e30, 3e38])
+def test_knn_velocity_weights(ops, arm, w):
+    """Weights that need the filter's operands scaled, up to FP32's largest: the
+    scan's lists bit for bit."""
+    t, q = dev(synth.random_states(arm, 5000, 3)), dev(synth.random_states(arm, 333, 4))
+    idx, d2 = ops.knn_tree(t, q, 9, w)
+    ri, rd = _scan(t, q, 9, 1, w)
     assert torch.equal(idx, ri)
     assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))

@@ -637,11 +637,11 @@ def test_goal_draws_do_not_depend_on_the_batch(P, arm, goals):
             assert got[p][f][:g].tobytes() == ref[p][f][:g].tobytes(), (p, f)
 
 
-@pytest.mark.parametrize("w_vel", [0.1, 1e4])
+@pytest.mark.parametrize("w_vel", [0.1, 0.0, 1e4, 1e30])
 def test_parent_lists_without_help_of_the_filter(P, arm, w_vel):
-    """Trees whose nodes coincide beside ordinary ones (one block's queries then
-    want different trees scanned), and a velocity weight that takes the states out
-    of the filter's range: the FP32 scan's lists bit for bit."""
+    """Trees whose nodes coincide beside ordinary ones, and velocity weights that
+    take the states out of the filter's range unless it is scaled: the FP32 scan's
+    lists bit for bit."""
     Ns, Bs, goals = [5000, 300, 2500, 4400], [300, 40, 9, 257], [37, 11, 4, 60]
     root = synth.random_states(arm, 1, 77)[0]
     pr = synth.make_problem(synth.random_toss(arm, 21), root=root)
