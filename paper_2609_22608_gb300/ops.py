@@ -7,7 +7,6 @@ returns the output tensors.  All arithmetic runs in the library's kernels.
 from __future__ import annotations
 
 import ctypes as C
-from contextlib import nullcontext
 
 import numpy as np
 import torch
@@ -243,9 +242,11 @@ def knn_tree(tree, queries, k, w_vel, first=1, N=None, workspace=None, out=None,
     if workspace is None and need > 0:
         # its last reference goes on return: as memory of the call's own stream
         # it is given to nobody else before the search is done with it
-        side = None if stream is None else _torch_stream(stream, queries.device)
-        with torch.cuda.stream(side) if side else nullcontext():
+        if stream is None:
             workspace = torch.empty(need + 256, dtype=torch.uint8, device=queries.device)
+        else:
+            with torch.cuda.stream(_torch_stream(stream, queries.device)):
+                workspace = torch.empty(need + 256, dtype=torch.uint8, device=queries.device)
     ws_ptr, ws_bytes = None, 0
     if workspace is not None:
         base = workspace.data_ptr()
