@@ -16,7 +16,9 @@
 // takes a slice of the rows, 64 at a time (one bulk copy per operand, three
 // stages), into the whole 256 x 256 FP32 accumulator (all 512 columns of tensor
 // memory), and adds it to the gradient in 16-byte reductions.  dW1 is summed as
-// dz1^T X (256 x 32), because the tensor core's M is 128.  dW4 (two columns) is
+// dz1^T X (256 x 32), because the tensor core's M is 128; its few CTAs take the
+// blocks in turn into kDw1Sets accumulators, so that a chain of additions on the
+// tensor core (which does not round to nearest) is no longer than dW2's.  dW4 (two columns) is
 // a chain of mma.sync over all rows in order, 16 of h3's columns to a CTA
 // beside the others: one sum per element, whatever the batch and the grid.
 //
@@ -367,6 +369,7 @@ constexpr int kDwA = kDwRows * 256 * 2;             // 32 KB: 64 rows of a 256-w
 constexpr int kDwStage = 2 * kDwA;
 constexpr int kDwBar = kDwStages * kDwStage;
 constexpr int kDwSmem = kDwBar + 128;
+constexpr int kDw1Sets = 4;                         // accumulators of dW1, 32 columns each
 // dW4: CTAs of 16 columns of h3, 512 rows to a stage (16 KB of h3, 2 KB of dy)
 constexpr int kDw4Ctas = 16, kDw4Rows = 512, kDw4Stages = 4;
 constexpr int kDw4H = kDw4Rows * 16 * 2, kDw4Stage = kDw4H + kDw4Rows * 2 * 2;
@@ -453,6 +456,7 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
   const bf16* gB = layer ? p.img[6 - layer] : p.img[0];
   const int wB = layer ? 256 : kTcK1;                // B's width
   const uint32_t bytesB = kDwRows * wB * 2;
+  const int sets = layer ? 1 : kDw1Sets;
   volatile uint32_t* s_tmem = reinterpret_cast<volatile uint32_t*>(smem + kDwBar + 64);
   volatile int* s_fail = reinterpret_cast<volatile int*>(smem + kDwBar + 68);
   const uint32_t base = su32(smem), bar = base + kDwBar;   // arrived (3), consumed (3), done, drain
@@ -492,8 +496,8 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
       for (int j = 0; j < kDwRows / 16; ++j)
 #pragma unroll
         for (int h = 0; h < 2; ++h)
-          umma_f16(tmem + 256 * h, sdesc(a + j * 8192 + h * 2048, 4096, 128),
-                   sdesc(b + j * 2 * kB, kB, 128), idesc, (done | j) != 0);
+          umma_f16(tmem + 256 * h + 32 * (done % sets), sdesc(a + j * 8192 + h * 2048, 4096, 128),
+                   sdesc(b + j * 2 * kB, kB, 128), idesc, done >= sets || j != 0);
       umma_commit(bar + 8u * (kDwStages + st));
       // refill the stage of the block before (its MMAs are queued before these)
       if (done >= 1 && done - 1 + kDwStages < n) {
@@ -537,10 +541,18 @@ __global__ void __launch_bounds__(kDwThreads, 1) k_mlp_dw(MlpTrain p, int S) {
                                 __uint_as_float(v[j + 2]), __uint_as_float(v[j + 3])));
       }
     } else {
-      uint32_t v[32];
-      tmem_ld32(src, v);
+      float t[32];
 #pragma unroll
-      for (int j = 0; j < 32; ++j) atomicAdd(p.gW[0] + 256 * j + m, __uint_as_float(v[j]));
+      for (int j = 0; j < 32; ++j) t[j] = 0.f;
+#pragma unroll 1
+      for (int i = 0; i < min(n, sets); ++i) {
+        uint32_t v[32];
+        tmem_ld32(src + 32 * i, v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) t[j] += __uint_as_float(v[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < 32; ++j) atomicAdd(p.gW[0] + 256 * j + m, t[j]);
     }
   }
   tc_fence_before();

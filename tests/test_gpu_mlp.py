@@ -420,3 +420,24 @@ def test_gradient_given_up(S, arm):
     assert np.isfinite(mlp.train_step(arm, d0, d1, lab, grid, 1e-2)) and mlp.error() == 0
     assert not np.array_equal(mlp.get_params(1)[0], after[1])
     mlp.close()
+
+
+def test_gradient_sum_of_many_rows(S, arm):
+    """2^17 equal rows: every term of the first layer's weight gradient is the same
+    and scales exactly with the batch, so the sum is that of 128 rows but for what
+    the additions lose.  A chain on the tensor core loses at most 2^-23 a step of 16
+    rows (it need not round to nearest): 76 steps to each of 4 x 27 accumulators,
+    then 31 FP32 additions."""
+    E, grid = 1 << 17, synth.duration_grid(16)
+    s0, s1 = synth.random_edges(arm, 1, 5)
+    mlp = S.MLP(max_batch=E)
+    load(mlp, seeded_params(61))
+    g = []
+    for n in (128, E):
+        mlp.backward(arm, dev(np.repeat(s0, n, 0)), dev(np.repeat(s1, n, 0)),
+                     torch.full((n,), 7, dtype=torch.int32, device="cuda"), grid)
+        g.append(mlp.get_grads(0)[0].astype(np.float64))
+    mlp.close()
+    some = g[0] != 0
+    assert some.any() and np.array_equal(g[1] != 0, some)
+    assert np.abs(g[1][some] / g[0][some] - 1).max() < 76 * 2.0 ** -23 + 31 * 2.0 ** -24
