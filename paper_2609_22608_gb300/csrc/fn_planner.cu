@@ -155,7 +155,7 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   int32_t* pend;      // [2][E] edges pending verification (ping-pong lists)
   int2* surv;         // [surv_cap] probe survivors (edge, grid index)
   int32_t* dyn_list;  // [Emax] edges with probe items (order of listing)
-  int Emax, Kmax, surv_cap;
+  int Emax, surv_cap;
   // duration surrogate: free edges with admissible durations routed to the
   // window pass (sur != 0), listed in sur_list (count *sur_n)
   int sur;
@@ -291,7 +291,7 @@ __global__ void k_plan_schedule(PlanDev D) {
     S->gq_cnt[p] = 0;
     fo += (B - G) * D.KP;
     go += G * D.KP;
-    const int N = D.n_nodes[p];
+    const int N = D.KP > 1 ? D.n_nodes[p] : 0;   // k = 1: no search, nothing to pack
     if (N > 1) {
       qf += (B - G + KT_QT - 1) / KT_QT;
       qg += (G + KT_QT - 1) / KT_QT;
@@ -3147,7 +3147,6 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
   A_(D.e_klo, (size_t)D.Emax);
   A_(D.e_j, (size_t)D.Emax); A_(D.e_cnt, (size_t)D.Emax);
   A_(D.mask, (size_t)D.Emax * 8);
-  D.Kmax = c.K;
   A_(D.dyn_list, (size_t)D.Emax);
   A_(D.cur_k, (size_t)D.Emax);
   A_(D.fail, (size_t)D.Emax);
@@ -3162,7 +3161,7 @@ extern "C" fn_status fn_planner_create(const fn_planner_cfg_t* cfg, const fn_arm
             (double)c.w_vel * arm->qd_max[j] * arm->qd_max[j];
     D.knn_sc = knn_scales(c.w_vel, r2);
   }
-  {
+  if (c.k > 1) {   // the parent search's: with k = 1 only the root is a parent
     const size_t tiles = P * ((BM + KT_QT - 1) / KT_QT);
     const size_t per = (size_t)KT_QT * kt_row_f4(D.NT) * sizeof(float4);
     D.knn_tiles = (int)std::max<size_t>(1, std::min(tiles, PL_KNN_BYTES / per));

@@ -663,3 +663,29 @@ def test_parent_lists_without_help_of_the_filter(P, arm, w_vel):
     for p, (states, cand) in enumerate(trees):
         assert np.array_equal(pl.get_parents(p, Bs[p]), _scan_lists(states, cand, k - 1, w_vel)), p
     pl.close()
+
+
+def test_search_buffers_only_with_a_search(P, arm):
+    """With k = 1 only the root is a parent: the parent search's buffers (here more
+    than a gigabyte of group minima) are not held, and rounds run without them."""
+    import torch
+
+    def held(k):
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        pl = P.Planner(arm, P=1, n_cap=1 << 20, b_max=4096, k=k, K=16, S=8)
+        return pl, free - torch.cuda.mem_get_info()[0]
+    pl, two = held(2)
+    pl.close()
+    pl, one = held(1)
+    minima = 2 * 16 * 256 * 8192 * 16          # two kinds of query, 16 tiles of 256, 8192 float4
+    assert two - one > minima
+    root = synth.random_states(arm, 1, 77)[0]
+    pr = synth.make_problem(synth.random_toss(arm, 21), root=root)
+    prob = P.problem_struct(pr, 4096, 700, root=root)
+    pl.reset([prob])
+    for it in range(3):
+        out = pl.iterate([prob], it, 0)[0]
+        tree = pl.get_tree(0)
+        assert np.all(tree["parent"][1:] == 0) and len(tree["t"]) > 1
+    pl.close()
