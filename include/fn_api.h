@@ -311,8 +311,9 @@ fn_status fn_rnea_dump(const fn_arm_t* arm, const float* s0, const float* s1, co
  *              With it, searches of 256 nodes and more filter the nodes on
  *              the tensor cores and score only those that can be among the
  *              k nearest in FP32; the results are the same bit for bit.  At
- *              most 68 MiB plus 150 bytes a node, except past 131072 nodes,
- *              where 256 queries' group minima (N / 8 bytes each) exceed it.
+ *              most 64 MiB and 256 bytes plus 152 bytes a node (the nodes
+ *              rounded up to 128), except from 2 000 000 nodes on, where 256
+ *              queries (24 KiB and 32 bytes a node) take more than 64 MiB.
  */
 size_t fn_knn_workspace_bytes(int B, int N, int k);
 fn_status fn_knn_tree(const float* tree, int N, int first, const float* queries, int B, int k,

@@ -179,8 +179,8 @@ __global__ void __launch_bounds__(256, 4)
   }
 }
 
-constexpr size_t kKtGminBytes = (size_t)64 << 20;   // group minima of one batch of queries, at most
-                                                    // (one tile of 256 queries if that is more)
+constexpr size_t kKtBatchBytes = (size_t)64 << 20;   // images and group minima of one batch of queries,
+                                                     // at most (one tile of 256 queries if that is more)
 // Three launches cost about 17 us whatever they search; the scan in one or two
 // takes as long at 128 nodes (k = 8: 25 us for 32 queries or more, 15 us for
 // one) and 42 us at 256, where the filter takes 19.  From 256 nodes on the
@@ -203,7 +203,7 @@ static KnnTcPlan knn_tc_plan(int B, int N) {
   KnnTcPlan p;
   p.ntiles = (N + KT_ROWS - 1) / KT_ROWS;
   const size_t row = (size_t)kt_row_f4(p.ntiles) * sizeof(float4);
-  const long fit = std::max<long>(1, (long)(kKtGminBytes / row / KT_QT)) * KT_QT;
+  const long fit = std::max<long>(1, (long)(kKtBatchBytes / (row * KT_QT + 2 * KT_TILE))) * KT_QT;
   p.batch = (int)std::min<long>(fit, ((long)B + KT_QT - 1) / KT_QT * KT_QT);
   p.nimg = 256;
   p.soa = p.nimg + (size_t)p.ntiles * KT_TILE;

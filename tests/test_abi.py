@@ -65,3 +65,17 @@ def test_arm_struct_forms(form):
         assert bytes(_lib.arm_struct(arm)) == bytes(_lib._arm_struct_by_item(arm))
     with pytest.raises(ValueError):
         _lib.arm_struct(dict(synth.make_arm(0), dh_a=np.zeros(5, np.float32)))
+
+
+def test_knn_workspace_bound():
+    """The workspace of the parent search stays within what the header states, for
+    few and many queries on small and large trees."""
+    from paper_2609_22608_gb300 import ops
+    for N in (1, 255, 256, 257, 2047, 2048, 2049, 4096, 65536, 131073, 10 ** 6, 1999999, 3 * 10 ** 6):
+        for B in (1, 255, 257, 8192, 65536, 200000, 262144, 10 ** 6):
+            for k in (1, 8, 16):
+                nodes = (N + 127) // 128 * 128
+                batch = max(64 << 20, (24 << 10) + 32 * (nodes + 2048) if N >= 2 * 10 ** 6 else 0)
+                need = ops.knn_workspace_bytes(B, N, k)
+                assert need <= batch + 256 + 152 * nodes, (B, N, k, need)
+                assert N < 256 or need >= 152 * nodes + 1024
