@@ -9,7 +9,6 @@ from __future__ import annotations
 
 import ctypes as C
 import os
-import struct
 
 import numpy as np
 
@@ -44,7 +43,6 @@ class FnError(RuntimeError):
 
 
 _lib = None
-_I32 = struct.Struct("i")
 
 
 def lib():
@@ -89,6 +87,7 @@ def check(status: int, what: str) -> None:
 
 
 # the float fields of FnArm after dof, in the struct's order, with their shapes
+# (the scalars are whatever float() takes)
 _ARM_FLOATS = tuple(
     (name, (7, 3) if name in ("com", "inertia", "fric") else (3,) if name in (
         "gravity", "blade_base", "blade_axis", "blade_normal") else () if name in (
@@ -103,12 +102,13 @@ def arm_struct(arm) -> FnArm:
     ctypes arrays item by item took 55."""
     if isinstance(arm, FnArm):
         return arm
-    parts = [np.asarray(arm[name], np.float32) for name, _ in _ARM_FLOATS]
+    parts = [np.asarray(arm[name] if shape else float(arm[name]), np.float32)
+             for name, shape in _ARM_FLOATS]
     for (name, shape), part in zip(_ARM_FLOATS, parts):
         if part.shape != shape:
             return _arm_struct_by_item(arm)
     flat = np.concatenate([part.ravel() for part in parts])
-    return FnArm.from_buffer_copy(_I32.pack(int(arm["dof"])) + flat.tobytes())
+    return FnArm.from_buffer_copy(bytes(C.c_int(int(arm["dof"]))) + flat.tobytes())
 
 
 def _arm_struct_by_item(arm) -> FnArm:

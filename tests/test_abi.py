@@ -79,3 +79,19 @@ def test_knn_workspace_bound():
                 need = ops.knn_workspace_bytes(B, N, k)
                 assert need <= batch + 256 + 152 * nodes, (B, N, k, need)
                 assert N < 256 or need >= 152 * nodes + 1024
+
+
+def test_arm_struct_scalars():
+    """Scalar fields may be anything that float() takes, as in the item-wise
+    conversion, and dof any integer that a C int holds in its way."""
+    import torch
+
+    from paper_2609_22608_gb300 import _lib, synth
+    arm = synth.make_arm(1)
+    arm = dict(arm, w_max=torch.tensor(float(arm["w_max"]), requires_grad=True),
+               blade_len=str(float(arm["blade_len"])), flange_d=np.float64(arm["flange_d"]))
+    assert bytes(_lib.arm_struct(arm)) == bytes(_lib._arm_struct_by_item(arm))
+    arm["dof"] = 2 ** 32 + 7
+    assert _lib.arm_struct(arm).dof == 7
+    with pytest.raises((TypeError, ValueError)):
+        _lib.arm_struct(dict(arm, w_max="wide"))
