@@ -378,7 +378,9 @@ def whole_job_rate(units_per_rank, world, ms):
 # iterations of (FK 475, residual 48, Jacobian 72, J^T J 237, J^T e 72,
 # Gauss-Jordan over the six rows 246, update 6) plus a final FK and residual
 # (523)
-FLOP_PER_PAIR = 44             # one (query, node) distance of the parent search
+FLOP_PER_PAIR = 96             # one (query, node) score of the parent search: a row of 48
+                               # f16 products on the tensor cores (the exact FP32 scores of
+                               # the few nodes in reach are not counted)
 FLOP_PER_IK_START = 28267      # one damped-least-squares start, 24 iterations + final check
 
 # DRAM bytes (read + written) per launch from one ncu capture of the kernel on
@@ -407,7 +409,8 @@ def kernel_table(traced):
 def roofline_from_trace(traced, work, workload="iteration"):
     """Roofline object for the kernel with the largest share of the traced
     iteration: its algorithmic FLOP (work counter x FLOP per unit) over its
-    own event-timed duration, against the derived FP32 peak."""
+    own event-timed duration, against the derived FP32 peak or, for the parent
+    search, the measured 16-bit tensor rate."""
     tab = kernel_table(traced)
     units = {"k_plan_probe": (work["probe"], FLOP_PER_SAMPLE,
                               "torque evaluations (the end-sample split, three per edge end)"),
@@ -415,19 +418,23 @@ def roofline_from_trace(traced, work, workload="iteration"):
              "k_plan_edges_tm": (work["probe"] + work["mprobe"] + work["verify"], FLOP_PER_SAMPLE,
                                  "torque evaluations (splits, probes and checks)"),
              "k_plan_vstage": (None, FLOP_PER_SAMPLE, "torque evaluations"),
-             "k_plan_knn": (work["knn_pairs"], FLOP_PER_PAIR, "(query, node) pairs, most of them scored on "
-                                                          "the tensor cores"),
+             "k_plan_knn": (work["knn_pairs"], FLOP_PER_PAIR,
+                            "(query, node) pairs scored on the tensor cores; the time is that of "
+                            "the filter's and the selection's launches together"),
              "k_plan_sample": (work["ik_starts"], FLOP_PER_IK_START,
                                "IK starts (the goal chart's; the uniform draws and the node "
-                               "images' update in the same launch are not credited)")}
+                               "images' update are k_plan_prep)")}
     dom = max(tab, key=lambda k: tab[k]["ms"])
-    peak = fp32_peak_tflops()
+    tensor = dom == "k_plan_knn"
+    peak = tensor_peak_tflops() if tensor else fp32_peak_tflops()
     total = sum(t["ms"] for t in tab.values())
     traffic = MEASURED_DRAM_BYTES.get(dom) if workload == "iteration" else None
-    out = {"bound": "alu", "peak": peak, "unit": "TFLOP/s", "traffic": traffic, "kernel": dom,
+    out = {"bound": "tensor" if tensor else "alu", "peak": peak, "unit": "TFLOP/s",
+           "traffic": traffic, "kernel": dom,
            "launches": tab[dom]["launches"], "kernel_ms": tab[dom]["ms"] / tab[dom]["launches"],
            "share_of_traced_iteration": tab[dom]["ms"] / total,
-           "peak_note": "FP32 FMA peak derived: 152 SMs x 128 lanes x 2 FLOP x max SM clock (of derived)",
+           "peak_note": "16-bit GEMM rate (of measured, or of fallback without the file)" if tensor else
+                        "FP32 FMA peak derived: 152 SMs x 128 lanes x 2 FLOP x max SM clock (of derived)",
            "traffic_note": "dram__bytes_read.sum + dram__bytes_write.sum per launch, one ncu "
                            "capture of this kernel on this workload (L2-resident inputs)"}
     n, f, what = units.get(dom, (None, None, None))
@@ -459,6 +466,13 @@ def roofline_from_trace(traced, work, workload="iteration"):
                              "note": "the tree and its images are L2-resident: the search is "
                                      "bound by latency, not by HBM"}
     return out
+
+
+def tensor_peak_tflops():
+    try:
+        return float(json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))["bf16_tflops"])
+    except (OSError, ValueError, KeyError):
+        return 1900.0
 
 
 def fp32_peak_tflops():

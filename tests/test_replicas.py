@@ -67,3 +67,17 @@ def test_reference_arm_runs_on_rank_zero_only():
     class A:
         seed, steps, warmup = 0, 1, 0
     assert bench.run_reference(A(), rank=1, world=2) is None
+
+
+def test_roofline_credits_the_unit_that_works():
+    """The parent search's pairs are scored on the tensor cores and held against
+    their rate; a kernel of torque evaluations against the FP32 peak."""
+    import bench
+    work = dict(probe=10 ** 6, mprobe=10 ** 6, verify=10 ** 6, knn_pairs=10 ** 10, ik_starts=4096)
+    traced = [("k_plan_knn", 0.05)] * 4 + [("k_plan_probe", 0.06)]
+    r = bench.roofline_from_trace(traced, work, "batched")
+    assert r["kernel"] == "k_plan_knn" and r["bound"] == "tensor"
+    assert r["peak"] == bench.tensor_peak_tflops()
+    assert r["achieved"] == pytest.approx(10 ** 10 * 96 / 0.2e-3 / 1e12)
+    r = bench.roofline_from_trace(traced + [("k_plan_probe", 0.3)], work, "batched")
+    assert r["bound"] == "alu" and r["peak"] == bench.fp32_peak_tflops()
