@@ -181,7 +181,8 @@ fn_status fn_time_edges_counted(const fn_arm_t* arm, const float* s0, const floa
  *   rounds      device [E] i32 or NULL: rounds run.
  *   sample_count device, one u64 or NULL: torque evaluations are ADDED.
  *   stream      cudaStream_t or NULL.
- * Ownership: all device buffers are the caller's; nothing is allocated.
+ * Ownership: all device buffers are the caller's; nothing is allocated.  The
+ * kernel holds an SM's tensor-memory columns as fn_time_edges's does.
  * Errors: FN_EINVAL for a bad argument (nothing launched), FN_ECUDA on a
  * launch error.  Non-finite states give k_star = -2 for that edge only.
  */
@@ -314,6 +315,11 @@ fn_status fn_rnea_dump(const fn_arm_t* arm, const float* s0, const float* s1, co
  *              most 64 MiB and 256 bytes plus 152 bytes a node (the nodes
  *              rounded up to 128), except from 2 000 000 nodes on, where 256
  *              queries (24 KiB and 32 bytes a node) take more than 64 MiB.
+ *              The filter's kernel holds all of an SM's tensor-memory columns
+ *              while it runs, as fn_time_edges's does.  Where the filter cannot
+ *              tell the nodes apart (states that nearly coincide, or far from
+ *              the ranges of joints in radians) all nodes are scored, in about
+ *              the time of the search without a workspace.
  */
 size_t fn_knn_workspace_bytes(int B, int N, int k);
 fn_status fn_knn_tree(const float* tree, int N, int first, const float* queries, int B, int k,
@@ -392,7 +398,9 @@ typedef struct {
   int S;              /* collocation points of the dynamics check            */
   int S_clear;        /* collocation points of the clearance check (>= 2)    */
   int reach_grid;     /* points of the Eq. (reach) grid (>= 2)               */
-  float w_vel;        /* velocity weight of the parent distance              */
+  float w_vel;        /* velocity weight of the parent distance (a tree whose
+                         nodes nearly coincide makes the parent search score all
+                         of them: several times slower)                      */
   float vel_frac;     /* free samples: |qd_j| <= vel_frac * qdbar_j(q_j)     */
   float clear_margin; /* minimum clearance of an edge, metres                */
   int edge_blocks;    /* persistent blocks of the edge kernel (0 = auto)     */
@@ -565,7 +573,7 @@ fn_status fn_planner_set_schedule(fn_planner_t* pl, int variant);
 
 /* Durations in ms of the last fn_plan_iteration's phases, from CUDA events
  * recorded on its stream: [0] schedule, [1] sample, [2] parents (kNN),
- * [3] edge prep + item scan, [4] probe (the end-sample torque split of every
+ * [3] edge prep, [4] probe (the end-sample torque split of every
  * edge with admissible durations, then both end samples of every admissible
  * (edge, duration) item), [5] verify (surviving durations, rho_v, Clear),
  * [6] attach + score, [7] prune, [8] output.  ms: host [9].  FN_EINVAL
@@ -869,7 +877,9 @@ fn_status fn_mlp_destroy(fn_mlp_t* m);
  * 16-byte aligned; device Y [E][2]), any E.  Runs on the 5th-generation
  * tensor cores (tcgen05, accumulators in tensor memory), one fused launch on
  * weights packed on the stream of their last change.
- * A timeout inside the kernel raises the flag read by fn_mlp_error. */
+ * The kernel holds half of an SM's tensor-memory columns while it runs (the
+ * gradient's second one all of them).  A timeout inside it raises the flag read
+ * by fn_mlp_error. */
 fn_status fn_mlp_predict(fn_mlp_t* m, const fn_arm_t* arm, const float* s0, const float* s1,
                          int E, float* Y, void* stream);
 

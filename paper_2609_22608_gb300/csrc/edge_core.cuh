@@ -7,9 +7,8 @@
 // FN_SPLIT_WORDS floats for the end-sample torque split.
 //   split : once per edge, lanes 0..5 = (end, part) evaluate Eq. (torque) at
 //           the edge's two end states: tau(T) = alpha / T^2 + beta / T + gamma
-//           at u = 0 and u = 1 (end_torque_part's decomposition), because the
-//           end states do not depend on T and the acceleration enters
-//           Eq. (torque) affinely;
+//           at u = 0 and u = 1 (split_cubic), because the end states do not
+//           depend on T and the acceleration enters Eq. (torque) affinely;
 //   probe : lanes take 32 consecutive grid durations and check both end
 //           samples from the split (no torque evaluation), then four
 //           interior samples (plain FP32 coefficients); a violation at any
@@ -257,10 +256,20 @@ struct PairCore {
   }
 };
 
-// The end-sample split cubic of item (end, part) of a staged edge: its
-// u = 0 sample is (q, qd, qdd) exactly (iT = iT2 = 1, b1 = qd, b2 = qdd / 2):
-// part 0 the end state with zero acceleration, parts 1 and 2 the two
-// acceleration vectors of end_torque_part at zero velocity.
+// Eq. (torque) at an end of the cubic as a function of the duration T.  At
+// u = 0 and u = 1 the position and velocity are the edge's end state,
+// whatever T; only the acceleration depends on T, and it is
+//   u = 0:  qdd = 6 (q1 - q0) / T^2 - (4 qd0 + 2 qd1) / T,
+//   u = 1:  qdd = -6 (q1 - q0) / T^2 + (4 qd1 + 2 qd0) / T.
+// Eq. (torque) is affine in qdd (mass matrix plus armature times qdd, plus
+// the velocity, gravity and friction terms at the end state), so
+//   tau(T) = alpha / T^2 + beta / T + gamma
+// with alpha = (M(q) + I_m) a and beta = (M(q) + I_m) b for the two vectors
+// above, and gamma = tau(q, qd, 0).
+// The split cubic of item (end, part) of a staged edge has (q, qd, qdd) as its
+// u = 0 sample exactly (iT = iT2 = 1, b1 = qd, b2 = qdd / 2): part 0 the end
+// state with zero acceleration (gamma), parts 1 and 2 the vectors a and b at zero
+// velocity (alpha, beta; the caller scales gravity and friction to zero).
 __device__ __forceinline__ void split_cubic(const float* es, int end, int part, Cubic& c) {
   c.iT = 1.f;
   c.iT2 = 1.f;

@@ -190,9 +190,9 @@ constexpr size_t kKtBatchBytes = (size_t)64 << 20;   // images and group minima 
 // the score's error, or outside its range, leave every group in reach; the
 // exact scan of all nodes in the select step (knn_wide) then takes about the
 // scan's time and the filter's.  8192 queries, 65536 nodes, k = 16: equal nodes
-// 1145 -> 1319 us, four clusters 1902 -> 1350, states in degrees 1913 -> 1276;
-// 2048 queries, 4096 nodes, k = 8: 45 -> 79, 80 -> 78, 82 -> 96; one query,
-// 65536 nodes: 130 -> 199, 140 -> 215, 140 -> 126.
+// 1145 -> 1319 us, four clusters 1902 -> 1323, states in degrees 1913 -> 1276;
+// 2048 queries, 4096 nodes, k = 8: 45 -> 79, 80 -> 70, 82 -> 96; one query,
+// 65536 nodes: 130 -> 199, 140 -> 220, 140 -> 126.
 static bool knn_tc_wanted(int N) { return N >= 256; }
 
 struct KnnTcPlan {

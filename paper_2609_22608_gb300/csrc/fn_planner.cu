@@ -693,8 +693,8 @@ __device__ __forceinline__ void parents_prep(const PlanDev& D, long i, long stri
 #define PL_EDGE_WARPS 4
 
 // ---------------------------------------------------------------------------
-// packed edge phase: prep -> item scan -> probe (lanes = (edge, duration)
-// items) -> verify (warp per edge, lanes = samples)
+// packed edge phase: prep -> split and probe (five edges to a warp) -> interior
+// probe (lane per survivor and sample) -> verification (packed stages, leftovers)
 // ---------------------------------------------------------------------------
 #define PL_SCAN 256
 #define PL_PRUNE_T 256   // threads (and nodes) per block of the multi-block prune
@@ -828,8 +828,7 @@ __global__ void __launch_bounds__(PL_SCAN) k_plan_eprep(PlanDev D, GridKP Gr) {
 }
 
 // Split and probe of the listed edges, five to a warp at a time.  Lanes
-// (edge, end, part) evaluate the end-sample torque split (end_torque_part's
-// decomposition: three torque evaluations per end instead of two per
+// (edge, end, part) evaluate the end-sample torque split (split_cubic: three torque evaluations per end instead of two per
 // duration) with the rolled recursion, whose one-link body is fetched once
 // where each lane evaluates Eq. (torque) about once; then, edge by edge, the
 // lanes take 32 grid durations each and check both end samples (u = 0, 1)
@@ -1370,7 +1369,7 @@ __global__ void __launch_bounds__(32 * Tm::kWarps, 1) k_plan_goal_edges(PlanDev 
 // admissible prefix (free edges: T_k <= the cap T_p) or the check at its
 // fixed duration T_p (goal edges, Algorithm 1), and finish_edge's velocity
 // and clearance tests.  One launch stands for the packed body's stages
-// (expand, probes, verification stages, leftovers); the autotuner takes it
+// (probes, verification stages, leftovers); the autotuner takes it
 // where an iteration's edges are few enough that the stages' chain of
 // launches, not their work, sets the time.  The CTA that finishes last
 // empties the dynamics list for the next body.

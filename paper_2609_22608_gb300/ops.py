@@ -85,7 +85,7 @@ def autotune_time_edges(arm, s0, s1, T_grid, S, reps=3, T_cap=None, stream=None)
     """fn_autotune_time_edges (FULL mode): times every schedule variant of the
     edge kernels on this workload (three register budgets of the scalar scan,
     then the paired scan with tensor-memory records) and keeps the fastest for
-    its shape (the N-ary refinement follows a scalar choice).  Returns
+    its shape (the N-ary refinement follows the choice).  Returns
     (variant, ms[4])."""
     _states(s0, "s0"); _states(s1, "s1")
     E = s0.shape[0]
