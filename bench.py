@@ -388,7 +388,7 @@ FLOP_PER_IK_START = 28267      # one damped-least-squares start, 24 iterations +
 # its launches in one iteration, as `achieved` is).  An entry holds only
 # while the kernel and the workload are the ones captured; it is removed
 # when either changes, and the roofline then reports null.
-MEASURED_DRAM_BYTES = {}
+MEASURED_DRAM_BYTES = {"k_plan_knn": 559232}
 # algorithmic bytes of one parent-search launch on this workload: the 4096
 # tree rows and the 2048 queries at 56 B (14 floats), the 2048 lists of 7
 # parents at 8 B per entry, over the iteration's four launches (group minima
