@@ -179,8 +179,9 @@ __global__ void __launch_bounds__(256, 4)
   }
 }
 
-constexpr size_t kKtBatchBytes = (size_t)64 << 20;   // images and group minima of one batch of queries,
-                                                     // at most (one tile of 256 queries if that is more)
+// images and group minima of one batch of queries, at most (one tile of 256 queries
+// if that is more): 64 MiB of minima and their queries' images at every tree size
+constexpr size_t kKtBatchBytes = (size_t)88 << 20;
 // Three launches cost about 17 us whatever they search; the scan in one or two
 // takes as long at 128 nodes (k = 8: 25 us for 32 queries or more, 15 us for
 // one) and 42 us at 256, where the filter takes 19.  From 256 nodes on the

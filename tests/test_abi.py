@@ -71,14 +71,16 @@ def test_knn_workspace_bound():
     """The workspace of the parent search stays within what the header states, for
     few and many queries on small and large trees."""
     from paper_2609_22608_gb300 import ops
-    for N in (1, 255, 256, 257, 2047, 2048, 2049, 4096, 65536, 131073, 10 ** 6, 1999999, 3 * 10 ** 6):
+    for N in (1, 255, 256, 257, 2047, 2048, 2049, 4096, 65536, 131073, 10 ** 6, 2799999, 3 * 10 ** 6):
         for B in (1, 255, 257, 8192, 65536, 200000, 262144, 10 ** 6):
             for k in (1, 8, 16):
                 nodes = (N + 127) // 128 * 128
-                batch = max(64 << 20, (24 << 10) + 32 * (nodes + 2048) if N >= 2 * 10 ** 6 else 0)
+                batch = max(88 << 20, (24 << 10) + 32 * (nodes + 2048) if N >= 2800000 else 0)
                 need = ops.knn_workspace_bytes(B, N, k)
                 assert need <= batch + 256 + 152 * nodes, (B, N, k, need)
                 assert N < 256 or need >= 152 * nodes + 1024
+    # the largest planner's search is one batch: 8192 queries' minima of 65536 nodes
+    assert ops.knn_workspace_bytes(8192, 65536, 16) >= 8192 * 8192 + 152 * 65536
 
 
 def test_arm_struct_scalars():
