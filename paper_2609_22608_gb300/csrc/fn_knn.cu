@@ -197,18 +197,22 @@ constexpr size_t kKtBatchBytes = (size_t)88 << 20;
 static bool knn_tc_wanted(int N) { return N >= 256; }
 
 struct KnnTcPlan {
-  int ntiles, batch;
+  int ntiles, batch;                     // batch 0: not even one tile of queries fits
   size_t nimg, soa, qimg, gmin, total;   // offsets into the workspace
 };
-static KnnTcPlan knn_tc_plan(int B, int N) {
+// as many queries to a batch as `bytes` hold: the workspace of a larger tree or of
+// fewer queries still serves, in more batches
+static KnnTcPlan knn_tc_plan(int B, int N, size_t bytes = SIZE_MAX) {
   KnnTcPlan p;
   p.ntiles = (N + KT_ROWS - 1) / KT_ROWS;
   const size_t row = (size_t)kt_row_f4(p.ntiles) * sizeof(float4);
-  const long fit = std::max<long>(1, (long)(kKtBatchBytes / (row * KT_QT + 2 * KT_TILE))) * KT_QT;
-  p.batch = (int)std::min<long>(fit, ((long)B + KT_QT - 1) / KT_QT * KT_QT);
+  const size_t tile = row * KT_QT + 2 * KT_TILE;   // of KT_QT queries
   p.nimg = 256;
   p.soa = p.nimg + (size_t)p.ntiles * KT_TILE;
   p.qimg = p.soa + (size_t)p.ntiles * (KT_ROWS / KT_GROUP) * KT_SOA * sizeof(float2);
+  const size_t room = bytes > p.qimg ? (bytes - p.qimg) / tile : 0;
+  const size_t fit = std::min(room, std::max<size_t>(1, kKtBatchBytes / tile)) * KT_QT;
+  p.batch = (int)std::min<size_t>(fit, ((size_t)B + KT_QT - 1) / KT_QT * KT_QT);
   p.gmin = p.qimg + (size_t)(p.batch / KT_ROWS) * KT_TILE;
   p.total = p.gmin + (size_t)p.batch * row;
   return p;
@@ -216,7 +220,7 @@ static KnnTcPlan knn_tc_plan(int B, int N) {
 
 static fn_status knn_tc_launch(const float* tree, int N, int first, const float* queries, int B,
                                int k, float w_vel, int32_t* idx, float* d2, void* workspace,
-                               cudaStream_t st) {
+                               const KnnTcPlan& p, cudaStream_t st) {
   static std::once_flag once[64];
   static bool attr_ok[64];
   int dev = 0;
@@ -227,7 +231,6 @@ static fn_status knn_tc_launch(const float* tree, int N, int first, const float*
                                              kKtSmem) == cudaSuccess;
   });
   if (!attr_ok[dev & 63]) return FN_ECUDA;
-  const KnnTcPlan p = knn_tc_plan(B, N);
   uint8_t* ws = (uint8_t*)workspace;
   int* err = (int*)ws;
   float2* soa = (float2*)(ws + p.soa);
@@ -315,13 +318,16 @@ extern "C" fn_status fn_knn_tree(const float* tree, int N, int first, const floa
   int nsplit = 1;
   float* part_d = nullptr;
   int32_t* part_i = nullptr;
-  // the tensor-core filter where its workspace is given; a workspace that
-  // only holds the split pass still gets that
-  if (workspace && aligned256(workspace) && N > first && knn_tc_wanted(N - first) &&
-      workspace_bytes >= knn_tc_plan(B, N).total)
-    return knn_tc_launch(tree, N, first, queries, B, k, w_vel, idx, d2, workspace,
-                         (cudaStream_t)stream);
   const size_t need = knn_split_bytes(B, N, k);
+  // the tensor-core filter where the workspace holds a tile of queries beside the
+  // nodes; one that does not still gets the split pass
+  if (workspace && aligned256(workspace) && N > first && knn_tc_wanted(N - first) &&
+      workspace_bytes >= std::min(need, knn_tc_plan(B, N).total)) {
+    const KnnTcPlan p = knn_tc_plan(B, N, workspace_bytes);
+    if (p.batch > 0)
+      return knn_tc_launch(tree, N, first, queries, B, k, w_vel, idx, d2, workspace, p,
+                           (cudaStream_t)stream);
+  }
   if (workspace && need > 0) {
     if (workspace_bytes < need || !aligned256(workspace)) return FN_EINVAL;
     nsplit = knn_nsplit(B, N);

@@ -177,3 +177,20 @@ def test_knn_velocity_weights(ops, arm, w):
     ri, rd = _scan(t, q, 9, 1, w)
     assert torch.equal(idx, ri)
     assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
+
+
+@pytest.mark.parametrize("tiles", [0, 1, 2, 5])
+def test_knn_in_a_smaller_workspace(ops, arm, tiles):
+    """A workspace that holds the nodes and only some tiles of 256 queries: the same
+    lists in more batches; with no tile, the scan's split pass."""
+    B, N, k = 1500, 3000, 6
+    t, q = dev(synth.random_states(arm, N, 5)), dev(synth.random_states(arm, B, 6))
+    ri, rd = _scan(t, q, k, 1)
+    one, two = (ops.knn_workspace_bytes(b, N, k) for b in (256, 512))
+    size = one + (tiles - 1) * (two - one) if tiles else one - 256
+    ws = torch.full((size + 256 + 1024,), 0x7F, dtype=torch.uint8, device="cuda")
+    off = -ws.data_ptr() % 256
+    idx, d2 = ops.knn_tree(t, q, k, 0.1, workspace=ws[off:off + size])
+    assert torch.equal(idx, ri)
+    assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
+    assert (ws[off + size:] == 0x7F).all()
