@@ -479,7 +479,9 @@ extern "C" fn_status fn_mlp_set_grads(fn_mlp_t* m, int l, const float* gW, const
   const size_t nw = (size_t)kDims[l] * kDims[l + 1], nb = kDims[l + 1];
   if (gW && cudaMemcpy(m->gW[l], gW, nw * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
   if (gb && cudaMemcpy(m->gb[l], gb, nb * 4, cudaMemcpyHostToDevice) != cudaSuccess) return FN_ECUDA;
-  return cudaMemset(m->fail, 0, 4) == cudaSuccess ? FN_OK : FN_ECUDA;   // the caller's gradient
+  // the caller's gradient, in place before any stream's next step
+  if (cudaMemset(m->fail, 0, 4) != cudaSuccess) return FN_ECUDA;
+  return cudaDeviceSynchronize() == cudaSuccess ? FN_OK : FN_ECUDA;
 }
 
 // binary file: "FNMLP1\0\0", step, then per layer W (f32 [in][out]) and b
