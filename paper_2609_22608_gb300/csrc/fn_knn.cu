@@ -17,6 +17,7 @@
 #include <mutex>
 
 #include "fn_internal.h"
+#include "fn_pdl.cuh"
 #include "knn_core.cuh"
 #include "knn_tc.cuh"
 
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(128) k_knn_tc_pack(const float4* __restrict__ 
                                                      float2* __restrict__ soa,
                                                      uint8_t* __restrict__ qimg,
                                                      int* __restrict__ err) {
+  pdl_trigger();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) *err = 0;
   float x[14];
@@ -152,18 +154,21 @@ struct KnnTcWork {
 
 __global__ void __launch_bounds__(KT_THREADS, 1) k_knn_tc_mins(KnnTcWork W, long units, int* err) {
   extern __shared__ __align__(1024) uint8_t kt_smem[];
+  pdl_begin();
   const long G = gridDim.x, b = blockIdx.x;
   knn_mins(kt_smem, W, units * b / G, units * (b + 1) / G, err);
 }
 
 // team warps to a query, of which the first searches alone and all share an
 // exact scan (knn_wide)
+template <int kGroups, int kStages>
 __global__ void __launch_bounds__(256, 4)
     k_knn_tc_select(const float2* __restrict__ soa, int n, int first,
                     const float4* __restrict__ queries, int B, int k, float w, float2 sc,
                     const float* __restrict__ gmin, int ntiles, const int* __restrict__ err,
                     int team, float* __restrict__ out_d, int32_t* __restrict__ out_i) {
-  __shared__ KnnWide<8> sh;
+  __shared__ KnnWide<8, kGroups, kStages> sh;
+  pdl_begin();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long b = ((long)blockIdx.x * 8 + warp) / team;
   const bool mine = warp % team == 0 && b < B;
@@ -191,9 +196,9 @@ constexpr size_t kKtBatchBytes = (size_t)88 << 20;
 // the score's error, or outside its range, leave every group in reach; the
 // exact scan of all nodes in the select step (knn_wide) then takes about the
 // scan's time and the filter's.  8192 queries, 65536 nodes, k = 16: equal nodes
-// 1145 -> 1319 us, four clusters 1902 -> 1323, states in degrees 1913 -> 1276;
-// 2048 queries, 4096 nodes, k = 8: 45 -> 79, 80 -> 70, 82 -> 96; one query,
-// 65536 nodes: 130 -> 199, 140 -> 220, 140 -> 126.
+// 1145 -> 1441 us, four clusters 1902 -> 1437, states in degrees 1913 -> 1405;
+// 2048 queries, 4096 nodes, k = 8: 45 -> 80, 80 -> 70, 82 -> 98; one query,
+// 65536 nodes: 130 -> 199, 140 -> 220, 140 -> 128.
 static bool knn_tc_wanted(int N) { return N >= 256; }
 
 struct KnnTcPlan {
@@ -247,13 +252,15 @@ static fn_status knn_tc_launch(const float* tree, int N, int first, const float*
                                                             nb, sc, ws + p.nimg, soa, ws + p.qimg, err);
     const long units = (long)qtiles * ntiles;
     const KnnTcWork W{ws + p.qimg, ws + p.nimg, gmin, ntiles, nb};
-    k_knn_tc_mins<<<(unsigned)std::min<long>(units, num_sms()), KT_THREADS, kKtSmem, st>>>(W, units,
-                                                                                           err);
+    // (launched while the step before drains: 100 queries on 600 nodes 10.9 us, with
+    // plain launches 16.8)
+    pl_launch(k_knn_tc_mins, (unsigned)std::min<long>(units, num_sms()), KT_THREADS, kKtSmem, st, W,
+              units, err);
     int team = 8;   // warps to a query, up to what the chip holds
     while (team > 1 && (long)nb * team > 32L * num_sms()) team /= 2;
-    k_knn_tc_select<<<(unsigned)(((long)nb * team + 7) / 8), 256, 0, st>>>(
-        soa, N - first, first, q, nb, k, w_vel, sc, gmin, ntiles, err, team, d2 + (long)b0 * k,
-        idx + (long)b0 * k);
+    const auto select = team > 1 ? k_knn_tc_select<8, 3> : k_knn_tc_select<4, 2>;
+    pl_launch(select, (unsigned)(((long)nb * team + 7) / 8), 256, 0, st, soa, N - first, first, q, nb,
+              k, w_vel, sc, gmin, ntiles, err, team, d2 + (long)b0 * k, idx + (long)b0 * k);
   }
   return launch_status();
 }

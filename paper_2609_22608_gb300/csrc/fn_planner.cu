@@ -36,6 +36,7 @@
 #include "fn_kin.cuh"
 #include "nary_core.cuh"
 #include "fn_mlp_tc.h"
+#include "fn_pdl.cuh"
 #include "fn_tune.h"
 #include "knn_tc.cuh"
 
@@ -180,21 +181,6 @@ struct PlanDev {  // device pointers, passed by value to the kernels
   int knn_tiles;      // query tiles of one launch
   float2 knn_sc;      // knn_scales of w_vel and the arm's limits
 };
-
-// Programmatic dependent launch: a kernel launched with programmatic
-// stream serialization may be scheduled while its predecessor drains; it
-// touches nothing the predecessor writes before this wait (a no-op for a
-// plain launch), and then lets its own successor be scheduled.
-__device__ __forceinline__ void pdl_begin() {
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
-__device__ __forceinline__ void pdl_trigger() {
-  asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-}
-__device__ __forceinline__ void pdl_wait() {
-  asm volatile("griddepcontrol.wait;\n" ::: "memory");
-}
 
 // A slot in a list that every thread appends to: the lanes of a warp that
 // call this together get consecutive slots from one atomic on the counter
@@ -2835,29 +2821,6 @@ static int plan_edge_blocks(fn_planner* pl, int v) {
   return std::min(resident(plan_mprobe_variant(v)),
                   std::min(resident_stage(plan_vstage_variant(v)),
                            resident_stage(plan_vseq_variant(v))));
-}
-
-// Launch with programmatic stream serialization (see pdl_begin): the
-// kernel may be scheduled while the previous kernel on the stream drains.
-template <class... KArgs, class... Args>
-static void pl_launch_pdl(bool pdl, void (*k)(KArgs...), unsigned grid, unsigned block,
-                          size_t smem, cudaStream_t st, Args... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = pdl ? 1 : 0;
-  cudaLaunchKernelEx(&cfg, k, args...);
-}
-template <class... KArgs, class... Args>
-static void pl_launch(void (*k)(KArgs...), unsigned grid, unsigned block, size_t smem,
-                      cudaStream_t st, Args... args) {
-  pl_launch_pdl(true, k, grid, block, smem, st, args...);
 }
 
 // the shared-memory request of the planner's tensor-memory kernels (the

@@ -622,26 +622,29 @@ __device__ __forceinline__ KeyList knn_select(const float2* __restrict__ soa, in
 // The exact scan of all nodes, for the queries whose scores are of no use: node
 // states that nearly coincide, states outside the filter's range.  Every warp of a
 // block of NW calls this (it synchronises) and gets its list, best unless wide is set.
-// The block copies KT_STAGE groups at a time into shared memory (cp.async, a ring of
-// KT_STAGES) and each of its wide queries scores them from there; `team`
+// The block copies kGroups groups at a time into shared memory (cp.async, a ring of
+// kStages) and each of its wide queries scores them from there; `team`
 // neighbouring warps share a query (the first one's wide and best count), a group
 // in turn each.  The loop is bound by issue, hence the paired distance.  A warp
 // reading every group for itself took, 8192 queries of a tree of 65536 equal nodes,
-// 2780 us (L2 bandwidth), one such query 1280 us (latency); now 1319 and 199 (the
+// 2780 us (L2 bandwidth), one such query 1280 us (latency); now 1441 and 199 (the
 // scan of fn_knn.cu, without the filter before it, 1145 and 130).
-constexpr int KT_STAGE = 8, KT_STAGES = 3;
-template <int NW>
+// kStages, kGroups: for a query to a warp two stages of four groups, 15 KB a block
+// that leave ordinary searches of small trees their L1 (three of eight, 44 KB: 20000
+// queries on 2000 nodes 89 us, so 86); three of eight for shared queries, whose scan
+// is bound by latency (one query on 65536 nodes 257 -> 150 us).
+template <int NW, int kGroups, int kStages>
 struct KnnWide {
   union {
     unsigned long long list[NW][KT_LIST];            // knn_select's
-    float4 stage[KT_STAGES][KT_STAGE * KT_SOA / 2];
+    float4 stage[kStages][kGroups * KT_SOA / 2];
     unsigned long long key[NW][16];
   };
   int wide[NW];
 };
-template <int NW>
-__device__ __forceinline__ KeyList knn_wide(KnnWide<NW>& sh, KeyList best, bool wide, int team,
-                                            const float2* soa, int n, int id0,
+template <int NW, int kGroups, int kStages>
+__device__ __forceinline__ KeyList knn_wide(KnnWide<NW, kGroups, kStages>& sh, KeyList best,
+                                            bool wide, int team, const float2* soa, int n, int id0,
                                             const float4* query, int k, float w) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rank = warp % team;
   if (!__syncthreads_or(rank == 0 && wide)) return best;
@@ -657,12 +660,12 @@ __device__ __forceinline__ KeyList knn_wide(KnnWide<NW>& sh, KeyList best, bool 
     for (int c = 0; c < 7; ++c) nq[c] = make_float2(-qv[c], -qv[7 + c]);
   }
   constexpr int kF4 = KT_SOA / 2;              // of a group
-  const int groups = (n + KT_GROUP - 1) / KT_GROUP, chunks = (groups + KT_STAGE - 1) / KT_STAGE;
+  const int groups = (n + KT_GROUP - 1) / KT_GROUP, chunks = (groups + kGroups - 1) / kGroups;
   auto copy = [&](int c) {                     // one commit group, empty past the end
     if (c < chunks) {
-      const int have = min(KT_STAGE, groups - c * KT_STAGE) * kF4;
-      const float4* src = reinterpret_cast<const float4*>(soa) + (long)c * KT_STAGE * kF4;
-      const uint32_t dst = su32(sh.stage[c % KT_STAGES]);
+      const int have = min(kGroups, groups - c * kGroups) * kF4;
+      const float4* src = reinterpret_cast<const float4*>(soa) + (long)c * kGroups * kF4;
+      const uint32_t dst = su32(sh.stage[c % kStages]);
       for (int i = threadIdx.x; i < have; i += 32 * NW)
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst + 16 * i),
                      "l"(src + i)
@@ -670,16 +673,16 @@ __device__ __forceinline__ KeyList knn_wide(KnnWide<NW>& sh, KeyList best, bool 
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
-  for (int c = 0; c < KT_STAGES - 1; ++c) copy(c);
+  for (int c = 0; c < kStages - 1; ++c) copy(c);
   for (int c = 0; c < chunks; ++c) {
-    asm volatile("cp.async.wait_group %0;\n" ::"n"(KT_STAGES - 2) : "memory");
+    asm volatile("cp.async.wait_group %0;\n" ::"n"(kStages - 2) : "memory");
     __syncthreads();                           // chunk c is there, c - 1 is scored
-    copy(c + KT_STAGES - 1);
+    copy(c + kStages - 1);
     if (!mine) continue;
-    const float2* st = reinterpret_cast<const float2*>(sh.stage[c % KT_STAGES]) + lane;
-    const int have = min(KT_STAGE, groups - c * KT_STAGE);
+    const float2* st = reinterpret_cast<const float2*>(sh.stage[c % kStages]) + lane;
+    const int have = min(kGroups, groups - c * kGroups);
     for (int i = rank; i < have; i += team) {
-      const int node = (c * KT_STAGE + i) * KT_GROUP + lane;
+      const int node = (c * kGroups + i) * KT_GROUP + lane;
       float2 x[7];
 #pragma unroll
       for (int j = 0; j < 7; ++j) x[j] = st[i * KT_SOA + KT_GROUP * j];
