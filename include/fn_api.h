@@ -316,7 +316,8 @@ fn_status fn_rnea_dump(const fn_arm_t* arm, const float* s0, const float* s1, co
  *              rounded up to 128), except from 2 800 000 nodes on, where 256
  *              queries (24 KiB and 32 bytes a node) take more than 88 MiB.
  *              One that holds fewer queries (for another B or N) serves in
- *              more batches.
+ *              more batches while these are few (one, and one for every 2^22
+ *              pairs of a query and a node).
  *              The filter's kernel holds all of an SM's tensor-memory columns
  *              while it runs, as fn_time_edges's does.  Where the filter cannot
  *              tell the nodes apart (states that nearly coincide, or far from

@@ -223,6 +223,15 @@ static KnnTcPlan knn_tc_plan(int B, int N, size_t bytes = SIZE_MAX) {
   return p;
 }
 
+// Whether the filter still pays in the batches of a workspace that does not hold
+// the plan: a batch takes about 15 us whatever it searches, the scan, split or not,
+// 15 us and as much again for 2^22 pairs (more where its threads are few).  16384 nodes
+// and 8192 queries in 32 batches 526 us, the scan 1096; past the line 256 nodes, 8192
+// queries in 32 batches 460, the scan 44.
+static bool knn_tc_batches_pay(int B, int n, int batch) {
+  return ((long)B + batch - 1) / batch <= 1 + ((long)B * n >> 22);
+}
+
 static fn_status knn_tc_launch(const float* tree, int N, int first, const float* queries, int B,
                                int k, float w_vel, int32_t* idx, float* d2, void* workspace,
                                const KnnTcPlan& p, cudaStream_t st) {
@@ -326,12 +335,13 @@ extern "C" fn_status fn_knn_tree(const float* tree, int N, int first, const floa
   float* part_d = nullptr;
   int32_t* part_i = nullptr;
   const size_t need = knn_split_bytes(B, N, k);
-  // the tensor-core filter where the workspace holds a tile of queries beside the
-  // nodes; one that does not still gets the split pass
-  if (workspace && aligned256(workspace) && N > first && knn_tc_wanted(N - first) &&
-      workspace_bytes >= std::min(need, knn_tc_plan(B, N).total)) {
+  // the tensor-core filter where the workspace holds its plan, or so many queries
+  // beside the nodes that the batches are few; one that does not still gets the
+  // split pass
+  if (workspace && aligned256(workspace) && N > first && knn_tc_wanted(N - first)) {
     const KnnTcPlan p = knn_tc_plan(B, N, workspace_bytes);
-    if (p.batch > 0)
+    if (workspace_bytes >= knn_tc_plan(B, N).total ||
+        (workspace_bytes >= need && p.batch > 0 && knn_tc_batches_pay(B, N - first, p.batch)))
       return knn_tc_launch(tree, N, first, queries, B, k, w_vel, idx, d2, workspace, p,
                            (cudaStream_t)stream);
   }

@@ -194,3 +194,22 @@ def test_knn_in_a_smaller_workspace(ops, arm, tiles):
     assert torch.equal(idx, ri)
     assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
     assert (ws[off + size:] == 0x7F).all()
+
+
+@pytest.mark.parametrize("N,B,rows,filtered", [
+    (257, 40000, 13568, True), (257, 40000, 10240, False),       # 3 batches pay, 4 do not
+    (700, 40000, 5888, True), (700, 40000, 5632, False)])        # 7 and 8
+def test_knn_batches_that_pay(ops, arm, N, B, rows, filtered):
+    """A workspace of `rows` queries serves the filter while the batches are few, and is
+    left alone where the scan in one launch is faster.  The same lists either way."""
+    k = 4
+    t, q = dev(synth.random_states(arm, N, 7)), dev(synth.random_states(arm, B, 8))
+    ri, rd = _scan(t, q, k, 1)
+    one, two = (ops.knn_workspace_bytes(b, N, k) for b in (32768, 33024))
+    size = one + (rows - 32768) // 256 * (two - one)
+    ws = torch.full((size + 256,), 0x7F, dtype=torch.uint8, device="cuda")
+    off = -ws.data_ptr() % 256
+    idx, d2 = ops.knn_tree(t, q, k, 0.1, workspace=ws[off:off + size])
+    assert torch.equal(idx, ri)
+    assert torch.equal(d2.view(torch.int32), rd.view(torch.int32))
+    assert bool((ws != 0x7F).any()) == filtered
