@@ -187,12 +187,17 @@ __global__ void __launch_bounds__(256, 4)
 // images and group minima of one batch of queries, at most (one tile of 256 queries
 // if that is more): 64 MiB of minima and their queries' images at every tree size
 constexpr size_t kKtBatchBytes = (size_t)88 << 20;
-// Three launches cost about 17 us whatever they search; the scan in one or two
-// takes as long at 128 nodes (k = 8: 25 us for 32 queries or more, 15 us for
-// one) and 42 us at 256, where the filter takes 19.  From 256 nodes on the
-// filter is the faster one at every batch and k measured (1 to 8192 queries:
-// 1.2x at 256 nodes and one query, 2x at 32, 15x at 65536 nodes, 8192
-// queries and k = 16, 1906 -> 128 us).  States closer to one another than
+// Three overlapping launches cost about 11 us whatever they search (one after the
+// other 17); the scan in one or two takes as long at 128 nodes (k = 8: 25 us for 32
+// queries or more, 15 us for one) and 42 us at 256.  From 256 nodes on the
+// filter is the faster one at every batch up to 16384 queries and every k measured
+// (8192 queries: 44 -> 25 us at 256 nodes and k = 8, 1906 -> 123 at 65536 and
+// k = 16).  Larger batches on a few hundred nodes are bound by the selection, whose
+// time goes with k: with k = 1 the filter stays ahead (a million queries, 256 nodes
+// 986 -> 820 us), with k = 8 the scan is ahead from 24576 queries at 256 nodes (52
+// against 54 us, 269 against 459 for 262144), 65536 at 384 (121, 131) and 262144 at 576
+// (496, 525), with k = 16 from 131072 at 256 only (275, 288): left with the filter, as a
+// planning batch is far smaller and the line would run through B, N and k.  States closer to one another than
 // the score's error, or outside its range, leave every group in reach; the
 // exact scan of all nodes in the select step (knn_wide) then takes about the
 // scan's time and the filter's.  8192 queries, 65536 nodes, k = 16: equal nodes
