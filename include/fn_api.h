@@ -906,8 +906,8 @@ fn_status fn_mlp_set_wait(fn_mlp_t* m, long long cycles);
  * the exact scan over the host grid T_grid [K]); *loss (host, may be NULL)
  * receives the loss.  Gradients stay on the device (fn_mlp_get_grads).  If a
  * wait inside ran out there is no gradient: FN_ECUDA where the loss is read,
- * fn_mlp_error in any case, and fn_mlp_adam_step changes nothing until the
- * next backward or fn_mlp_set_grads. */
+ * fn_mlp_error in any case, and fn_mlp_adam_step changes no parameter or moment
+ * until the next backward or fn_mlp_set_grads (it still counts as a step). */
 fn_status fn_mlp_backward(fn_mlp_t* m, const fn_arm_t* arm, const float* s0, const float* s1,
                           const int32_t* k_star, const float* T_grid, int K, int E,
                           float* loss, void* stream);
